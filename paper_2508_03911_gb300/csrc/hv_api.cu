@@ -58,7 +58,6 @@ struct hv_handle {
   size_t s1_bytes = 0, s2_bytes = 0;
   uint32_t chunk = 0;
   int sp_cluster = 0;         // 1: whole-frame cluster kernel
-  int sp_pp = 0;              // 1: persistent multi-pass kernels
   int sp_fused = 0;           // 1: fused transform (s1 / s2 are rings of kFusedRing frames)
   int inject = HV_INJECT_NONE;  // pending fault injection (hv_debug_inject)
   int stft_kernel = STFT_AUTO;  // STFT kernel for windows that do not overlap (autotuner's choice)
@@ -372,7 +371,11 @@ hv_status apply_pending(hv_handle* h) {
   Q = std::max(Q, d.T);
   s = ensure(h, reinterpret_cast<void**>(&h->tq), &h->tq_bytes, size_t(Q) * fbytes);
   if (s != HV_OK) return s;
-  uint32_t chunk = p.spatial_chunk ? p.spatial_chunk : std::max<uint32_t>(1, uint32_t((size_t(32) << 20) / fbytes));
+  // frames per launch: 256 MB of fields (at 256 x 256 ASP 0.55, 0.46, 0.41, 0.37 us a frame
+  // for 32, 48, 160 and 512 MB: a launch's ramp and tail weigh more than the L2 hits that
+  // a small launch's intermediates get)
+  uint32_t chunk = p.spatial_chunk ? p.spatial_chunk : std::max<uint32_t>(1, uint32_t((size_t(256) << 20) / fbytes));
+  if (p.spatial_chunk == 0) chunk = std::min(chunk, Q);
   chunk = std::min<uint32_t>(chunk, 1024);
   const bool fused = p.spatial_kernel == HV_SK_FUSED;
   const size_t sbytes = size_t(fused ? std::max(chunk, kFusedRing) : chunk) * fbytes;
@@ -522,7 +525,6 @@ hv_status apply_pending(hv_handle* h) {
   h->Q = Q;
   h->chunk = chunk;
   h->sp_cluster = p.spatial_kernel == HV_SK_CLUSTER ? 1 : 0;
-  h->sp_pp = p.spatial_kernel == HV_SK_PERSISTENT ? 1 : 0;
   h->sp_fused = fused ? 1 : 0;
   h->tuning = hv_tuning{};
   h->tuning.spatial_chunk = chunk;
@@ -625,7 +627,6 @@ hv_status propagate_run(hv_handle* h, uint64_t r0, uint64_t r1, RingRef raw) {
     sa.chirp_x = h->chirp;
     sa.chirp_y = h->chirp + h->W;
     sa.use_cluster = h->sp_cluster;
-    sa.use_pp = h->sp_pp;
     sa.use_fused = h->sp_fused;
     sa.ring = kFusedRing;
     sa.fused_ctr = h->fused_ctr;
@@ -701,7 +702,8 @@ hv_status tune_spatial(hv_handle* h) {
   for (int ci = 0; ci < 11; ++ci) {
     const Cand c = cands[ci];
     if (c.kind == 2 && !cluster_ok(h)) continue;
-    if (c.kind == 3 && !pp_ok) continue;
+    // from 64 up kinds 1 and 3 are the same passes: each launch size is timed once
+    if (c.kind == 3 && (!pp_ok || c.chunk <= 256)) continue;
     if (c.kind == 4 && !fused_ok) continue;
     const uint32_t ch = (c.kind == 2 || c.kind == 4) ? n : std::min(c.chunk, n);
     if (c.kind == 4 && ensure(h, reinterpret_cast<void**>(&h->fused_ctr), &h->fused_ctr_bytes,
@@ -715,7 +717,6 @@ hv_status tune_spatial(hv_handle* h) {
         continue;
     }
     h->sp_cluster = c.kind == 2;
-    h->sp_pp = c.kind == 3;
     h->sp_fused = c.kind == 4;
     h->chunk = (c.kind == 2 || c.kind == 4) ? h->chunk : ch;
     const uint64_t before = h->st.frames_propagated;
@@ -742,7 +743,6 @@ hv_status tune_spatial(hv_handle* h) {
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   h->sp_cluster = best_kind == 2;
-  h->sp_pp = best_kind == 3;
   h->sp_fused = best_kind == 4;
   h->chunk = best_chunk;
   // the chosen kernels' scratch: chunk frames (multi-pass), the rings (fused)

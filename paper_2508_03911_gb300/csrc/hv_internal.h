@@ -33,7 +33,6 @@ struct SpatialArgs {
   const float2* chirp_x;// Fresnel chirp factors along x (length W), fftshift folded in
   const float2* chirp_y;// along y (length H)
   int use_cluster;      // 1: whole-frame cluster kernel when the size allows it
-  int use_pp;           // 1: persistent prefetching multi-pass kernels when the size allows
   double* tam_acc;      // focus sweep: frame i adds (sum |u|, sum |u|^2) at tam_acc + i * tam_stride
   uint32_t tam_stride;
   int discard_inputs;   // persistent passes: scratch1/scratch2 are read once, drop their L2 lines after staging
@@ -51,7 +50,9 @@ struct SpatialArgs {
 cudaError_t launch_spatial(const SpatialArgs& a, cudaStream_t s, int* launches);
 bool spatial_cluster_supported(const SpatialArgs& a);
 bool spatial_pp_supported(const SpatialArgs& a);
-cudaError_t launch_spatial_pp(const SpatialArgs& a, cudaStream_t s, int* launches);
+// Register-direct passes for sides 64 .. 1024 (ASP needs asp_h).
+bool spatial_strip_supported(const SpatialArgs& a);
+cudaError_t launch_spatial_strip(const SpatialArgs& a, cudaStream_t s, int* launches);
 cudaError_t launch_spatial_cluster(const SpatialArgs& a, cudaStream_t s, int* launches);
 // Fused transform: frames of 256 x 256, ASP or Fresnel; needs ring >= kFusedRing
 // frames in scratch1 (and scratch2 for ASP), fused_ctr and err.

@@ -83,9 +83,10 @@ struct TableArgs {
   uint32_t W, H;
   double z, lam, dx, dy;
   double highpass;  // cutoff in cycles per pixel, 0 = off
+  int transposed;   // layout of h
 };
 
-// Twiddles, chirp factors and the transposed transfer function, in float64 on
+// Twiddles, chirp factors and the transfer function, in float64 on
 // the device (same definitions as the tables the handle path builds on the host).
 __global__ void k_static_tables(TableArgs a) {
   const size_t ntw = packed_offset(2048);
@@ -119,8 +120,8 @@ __global__ void k_static_tables(TableArgs a) {
       }
       a.chirp[j] = v;
     } else if (a.spatial == HV_SPATIAL_ASP) {
-      const size_t q = e - ntw - a.W - a.H;  // [kx][ky]
-      const uint32_t kx = uint32_t(q / a.H), ky = uint32_t(q % a.H);
+      const size_t q = e - ntw - a.W - a.H;  // [ky][kx], transposed with a side below 64
+      const uint32_t kx = uint32_t(a.transposed ? q / a.H : q % a.W), ky = uint32_t(a.transposed ? q % a.H : q / a.W);
       const double k = 2.0 * M_PI / a.lam;
       const double mx = kx < a.W / 2 ? double(kx) : double(kx) - a.W;
       const double my = ky < a.H / 2 ? double(ky) : double(ky) - a.H;
@@ -196,7 +197,7 @@ extern "C" hv_status hv_spatial_static(const void* frames, uint32_t pixel_bits, 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
 
   TableArgs ta{tw, chirp, htab, p->spatial, p->fftshift, W, H, p->z_m, p->lambda_m, p->pitch_x_m,
-               p->pitch_y_m, p->highpass_cpp};
+               p->pitch_y_m, p->highpass_cpp, (W < 64 || H < 64) ? 1 : 0};
   k_static_tables<<<256, 256, 0, s>>>(ta);
   // no error was pending before the launch, so one now is this launch's
   if (cudaGetLastError() != cudaSuccess) return HV_ERR_CUDA;
@@ -213,7 +214,8 @@ extern "C" hv_status hv_spatial_static(const void* frames, uint32_t pixel_bits, 
   sa.scratch2 = s2;
   sa.tw_w = tw + packed_offset(W);
   sa.tw_h = tw + packed_offset(H);
-  sa.asp_ht = htab;
+  sa.asp_ht = ta.transposed ? htab : nullptr;
+  sa.asp_h = ta.transposed ? nullptr : htab;
   sa.chirp_x = chirp;
   sa.chirp_y = chirp + W;
   int launches = 0;

@@ -199,16 +199,21 @@ static cudaError_t spatial_fixed(const SpatialArgs& a, cudaStream_t s, int* laun
   return e;
 }
 
+// A side of 16 or 32 (both sides from 64 up: the register-direct passes).
 template <int LH>
 static cudaError_t spatial_w(const SpatialArgs& a, cudaStream_t s, int* launches) {
   switch (a.W) {
     case 16: return spatial_fixed<LH, 16>(a, s, launches);
     case 32: return spatial_fixed<LH, 32>(a, s, launches);
-    case 64: return spatial_fixed<LH, 64>(a, s, launches);
-    case 128: return spatial_fixed<LH, 128>(a, s, launches);
-    case 256: return spatial_fixed<LH, 256>(a, s, launches);
-    case 512: return spatial_fixed<LH, 512>(a, s, launches);
-    case 1024: return spatial_fixed<LH, 1024>(a, s, launches);
+  }
+  if constexpr (LH <= 32) {
+    switch (a.W) {
+      case 64: return spatial_fixed<LH, 64>(a, s, launches);
+      case 128: return spatial_fixed<LH, 128>(a, s, launches);
+      case 256: return spatial_fixed<LH, 256>(a, s, launches);
+      case 512: return spatial_fixed<LH, 512>(a, s, launches);
+      case 1024: return spatial_fixed<LH, 1024>(a, s, launches);
+    }
   }
   return cudaErrorInvalidValue;
 }
@@ -224,7 +229,7 @@ cudaError_t launch_spatial(const SpatialArgs& a, cudaStream_t s, int* launches) 
   }
   if (a.use_fused && spatial_fused_supported(a)) return launch_spatial_fused(a, s, launches);
   if (a.use_cluster && spatial_cluster_supported(a)) return launch_spatial_cluster(a, s, launches);
-  if (a.use_pp && spatial_pp_supported(a)) return launch_spatial_pp(a, s, launches);
+  if (spatial_strip_supported(a)) return launch_spatial_strip(a, s, launches);
   switch (a.H) {
     case 16: return spatial_w<16>(a, s, launches);
     case 32: return spatial_w<32>(a, s, launches);

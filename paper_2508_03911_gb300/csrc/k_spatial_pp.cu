@@ -1,30 +1,12 @@
-// k_spatial_pp.cu -- the spatial transform (Sec. III-B.1) as persistent kernels, one
-// per pass, that prefetch their next work item and keep the integer work per
-// pixel small.
-//
-// A CTA stays resident and loops over work items (frame, strip of 16 lines of
-// the pass; 8 at line length 1024). While it transforms one item, the input of its next item streams
-// into a second buffer with cp.async. Each pass reads its input in whatever
-// order makes the global loads coalesced and writes its output straight from
-// the registers of the last FFT stage; the intermediate layouts are chosen so
-// that those stores are coalesced too (lanes of a warp hold 16 neighbouring
-// lines):
-//   P1  column FFT (length H) of 16 columns: the first FFT stage reads the raw
-//       strip (uint8/uint16, staged by cp.async) and converts it in registers
-//       (Fresnel: times the chirp) -> S1[ky][x]
-//   P2a row FFT (length W) of 16 rows ky of S1, x H^T (1/(WH) and the optional
-//       high-pass folded in), row IFFT -> S2[x][ky]
-//   P3a column IFFT (length H) of 16 columns x of S2 -> time queue [y][x]
-//   P2f row FFT of 16 rows ky of S1 -> time queue [ky][kx]; its last stage maps
-//       threads along kx (twiddles from a per-stage table), so the store of
-//       each row is coalesced straight from registers
-//   P3t as P3a, but instead of storing the field it adds sum |u| and sum |u|^2 of
-//       the strip to the frame's two float64 accumulators (focus sweep)
-// Twiddles of the pass length are copied to shared memory once per CTA. In the
-// full transform the intermediates S1 and S2 are read exactly once: once a strip
-// is staged, its L2 lines are discarded (no write-back of dead data when a
-// chunk's intermediates fit in L2). Single passes (the focus sweep re-reads S1
-// for every distance) keep them.
+// k_spatial_pp.cu -- single passes of the spatial transform (Sec. III-B.1) for the focus
+// sweep and the network input, as persistent kernels that prefetch their next strip of 16
+// lines (8 at line length 1024) with cp.async, and the fused transform of 256 x 256 frames:
+//   P1  column FFT (length H) of 16 columns, converted in the first stage -> S1[ky][x]
+//   P2a row FFT (length W) of 16 rows ky of S1, x H^T, row IFFT -> S2[x][ky]
+//   P3t column IFFT of 16 columns x of S2, adding sum |u| and sum |u|^2 of the strip to the
+//       frame's two float64 accumulators
+//   P2f row FFT of 16 rows ky of S1 -> [ky][kx]
+//   P2c row FFT of 16 rows, its last stage forming the network's input cells
 #include <cuda.h>
 
 #include "fft_dev.cuh"
@@ -476,19 +458,7 @@ static cudaError_t launch_pp(const SpatialArgs& a, uint32_t lines, cudaStream_t 
   return cudaGetLastError();
 }
 
-// ------------------------------------------------- row FFT, one warp per 2 rows
-//
-// The Fresnel row pass at L = 256 with the STFT's warp-private layout: 16 lanes
-// carry one row, so the 256-point FFT (16 x 16 Stockham) needs only __syncwarp
-// between its stages. A CTA of 8 warps takes strips of 16 rows of S1 [ky][x]; one
-// TMA tensor load per strip (16 x 256 complex64, dense rows) lands in one of two
-// tiles and completes on the tile's mbarrier, the next strip's load in flight
-// while the current one is transformed. Stage 1 reads samples jl + 16 m
-// (consecutive lanes) and writes its output m back into the row at 16 jl +
-// (m ^ jl) (an XOR swizzle: conflict-free without padding); stage 2 reads
-// 16 m + (jl ^ m), applies w_256^(jl m) from a table laid out by (m, jl) and leaves
-// bin jl + 16 m in lane jl, stored to the time queue row (coalesced).
-constexpr int RW_L = 256, RW_BT = 16, RW_NT = 256;
+constexpr int RW_L = 256;  // side of the fused transform's frames
 
 __device__ __forceinline__ uint32_t rw_smem(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -507,353 +477,6 @@ __device__ __forceinline__ bool rw_wait(uint32_t mbar, uint32_t parity) {
     if (ok) return true;
     if (clock64() - t0 > (1ll << 32)) return false;
   }
-}
-
-__global__ void __launch_bounds__(RW_NT, 3)
-    k_row_warp(SpatialArgs a, int nitems, int strip_log2, const __grid_constant__ CUtensorMap s1map) {
-  extern __shared__ __align__(128) unsigned char smem_tma[];  // TMA destinations: 128-byte aligned
-  __shared__ __align__(8) unsigned long long full[2];
-  float2* tile0 = reinterpret_cast<float2*>(smem_tma);
-  float2* tile1 = tile0 + RW_BT * RW_L;
-  float2* tw2 = tile1 + RW_BT * RW_L;  // stage 2: w_256^(j m) at (m - 1) 16 + j
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int b = 2 * warp + (lane >> 4), jl = lane & 15;  // row of the strip, lane within the row
-  const int smask = (1 << strip_log2) - 1;
-  for (int e = tid; e < 15 * 16; e += RW_NT) {
-    const int m = e / 16 + 1, j = e % 16;
-    tw2[e] = __ldg(&a.tw_w[j * m]);
-  }
-  if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(rw_smem(&full[0])) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(rw_smem(&full[1])) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  }
-  __syncthreads();
-  // one thread: the strip of item `it` (rows i H + s0 .. + 15 of S1) into tile `k`
-  auto issue = [&](int it, int k) {
-    const int i = it >> strip_log2, s0 = (it & smask) * RW_BT;
-    const uint32_t mb = rw_smem(&full[k]);
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(mb), "r"(RW_BT * RW_L * 8)
-                 : "memory");
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-        "[%4];\n" ::"r"(rw_smem(k ? tile1 : tile0)),
-        "l"(reinterpret_cast<uint64_t>(&s1map)), "r"(0), "r"(int(i * a.H + s0)), "r"(mb)
-        : "memory");
-  };
-  int item = blockIdx.x;
-  if (tid == 0 && item < nitems) issue(item, 0);
-  bool ok = true;
-  for (int k = 0; item < nitems && ok; ++k, item += gridDim.x) {
-    const int cur = k & 1;
-    float2* tile = cur ? tile1 : tile0;
-    const int i = item >> strip_log2, s0 = (item & smask) * RW_BT;
-    ok = rw_wait(rw_smem(&full[cur]), uint32_t(k >> 1) & 1u);
-    // every warp is done with the other tile (two strips ago) and sees this one
-    ok = __syncthreads_and(ok) != 0;
-    if (!ok) break;
-    const int nxt = item + gridDim.x;
-    if (tid == 0 && nxt < nitems) {
-      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-      issue(nxt, cur ^ 1);
-    }
-    if (a.discard_inputs) {
-      const char* st = reinterpret_cast<const char*>(a.scratch1 + (size_t(i) * a.H + s0) * RW_L);
-      for (int e = tid; e < RW_BT * RW_L * 8 / 128; e += RW_NT)
-        asm volatile("discard.global.L2 [%0], 128;\n" ::"l"(st + size_t(e) * 128) : "memory");
-    }
-    float2* row = tile + b * RW_L;
-    float2 v[16];
-#pragma unroll
-    for (int m = 0; m < 16; ++m) v[m] = row[jl + 16 * m];
-    dft<16, -1>(v);
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < 16; ++m) row[16 * jl + (m ^ jl)] = v[m];
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < 16; ++m) {
-      v[m] = row[16 * m + (jl ^ m)];
-      if (m > 0) v[m] = cmul(v[m], tw2[(m - 1) * 16 + jl]);
-    }
-    dft<16, -1>(v);
-    // time queue [ky][kx]: bin kx = jl + 16 m of row s0 + b
-    const size_t tslot = (a.tq.slot0 + uint32_t(i)) % a.tq.cap;
-    float2* out = static_cast<float2*>(a.tq.base) + (tslot * a.H + s0 + b) * size_t(RW_L);
-#pragma unroll
-    for (int m = 0; m < 16; ++m) out[jl + 16 * m] = v[m];
-  }
-  if (!ok && tid == 0 && a.err) atomicOr(a.err, 8u);
-}
-
-static cudaError_t launch_row_warp(const SpatialArgs& a, cudaStream_t s) {
-  const size_t smem = (2 * size_t(RW_BT) * RW_L + 15 * 16) * sizeof(float2);
-  CUtensorMap map{};
-  if (!encode_map_2d_u64(&map, a.scratch1, RW_L, uint64_t(a.n) * a.H, RW_L * 8, RW_L, RW_BT, false))
-    return cudaErrorNotSupported;
-  cudaError_t e = cudaFuncSetAttribute(k_row_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-  if (e != cudaSuccess) return e;
-  int per_sm = 0, dev = 0, nsm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_row_warp, RW_NT, smem);
-  if (e != cudaSuccess) return e;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  int strip_log2 = 0;
-  while ((uint32_t(RW_BT) << strip_log2) < a.H) ++strip_log2;
-  const int nitems = int(a.n) << strip_log2;
-  int grid = per_sm * nsm;
-  if (grid > nitems) grid = nitems;
-  if (grid < 1) grid = 1;
-  k_row_warp<<<grid, RW_NT, smem, s>>>(a, nitems, strip_log2, map);
-  return cudaGetLastError();
-}
-
-// ASP row pass at W = 256, warp-private like k_row_warp: forward row FFT, bins
-// times the transfer function H[ky][kx] (row-major copy, 1/(W H) folded in), then
-// the inverse row FFT, whose first stage takes the bins the forward FFT left in
-// the lane's registers (butterfly jl of the inverse is bins jl + 16 m). S2 is
-// written row-major [ky][x], coalesced.
-__global__ void __launch_bounds__(RW_NT, 3)
-    k_row_asp(SpatialArgs a, int nitems, int strip_log2, const __grid_constant__ CUtensorMap s1map) {
-  extern __shared__ __align__(128) unsigned char smem_tma[];  // TMA destinations: 128-byte aligned
-  __shared__ __align__(8) unsigned long long full[2];
-  float2* tile0 = reinterpret_cast<float2*>(smem_tma);
-  float2* tile1 = tile0 + RW_BT * RW_L;
-  float2* tw2 = tile1 + RW_BT * RW_L;  // w_256^(j m) at (m - 1) 16 + j
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int b = 2 * warp + (lane >> 4), jl = lane & 15;
-  const int smask = (1 << strip_log2) - 1;
-  for (int e = tid; e < 15 * 16; e += RW_NT) {
-    const int m = e / 16 + 1, j = e % 16;
-    tw2[e] = __ldg(&a.tw_w[j * m]);
-  }
-  if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(rw_smem(&full[0])) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(rw_smem(&full[1])) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  }
-  __syncthreads();
-  auto issue = [&](int it, int k) {
-    const int i = it >> strip_log2, s0 = (it & smask) * RW_BT;
-    const uint32_t mb = rw_smem(&full[k]);
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(mb), "r"(RW_BT * RW_L * 8)
-                 : "memory");
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-        "[%4];\n" ::"r"(rw_smem(k ? tile1 : tile0)),
-        "l"(reinterpret_cast<uint64_t>(&s1map)), "r"(0), "r"(int(i * a.H + s0)), "r"(mb)
-        : "memory");
-  };
-  int item = blockIdx.x;
-  if (tid == 0 && item < nitems) issue(item, 0);
-  bool ok = true;
-  for (int k = 0; item < nitems && ok; ++k, item += gridDim.x) {
-    const int cur = k & 1;
-    float2* tile = cur ? tile1 : tile0;
-    const int i = item >> strip_log2, s0 = (item & smask) * RW_BT;
-    ok = rw_wait(rw_smem(&full[cur]), uint32_t(k >> 1) & 1u);
-    ok = __syncthreads_and(ok) != 0;
-    if (!ok) break;
-    const int nxt = item + gridDim.x;
-    if (tid == 0 && nxt < nitems) {
-      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-      issue(nxt, cur ^ 1);
-    }
-    if (a.discard_inputs) {
-      const char* st = reinterpret_cast<const char*>(a.scratch1 + (size_t(i) * a.H + s0) * RW_L);
-      for (int e = tid; e < RW_BT * RW_L * 8 / 128; e += RW_NT)
-        asm volatile("discard.global.L2 [%0], 128;\n" ::"l"(st + size_t(e) * 128) : "memory");
-    }
-    float2* row = tile + b * RW_L;
-    const int ky = s0 + b;
-    float2 v[16];
-    // forward row FFT
-#pragma unroll
-    for (int m = 0; m < 16; ++m) v[m] = row[jl + 16 * m];
-    dft<16, -1>(v);
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < 16; ++m) row[16 * jl + (m ^ jl)] = v[m];
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < 16; ++m) {
-      v[m] = row[16 * m + (jl ^ m)];
-      if (m > 0) v[m] = cmul(v[m], tw2[(m - 1) * 16 + jl]);
-    }
-    dft<16, -1>(v);
-    // bins kx = jl + 16 m times H[ky][kx]
-    const float2* hrow = a.asp_h + size_t(ky) * RW_L;
-#pragma unroll
-    for (int m = 0; m < 16; ++m) v[m] = cmul(v[m], __ldg(&hrow[jl + 16 * m]));
-    // inverse row FFT: its first butterfly jl takes the inputs jl + 16 m, here already
-    dft<16, +1>(v);
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < 16; ++m) row[16 * jl + (m ^ jl)] = v[m];
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < 16; ++m) {
-      v[m] = row[16 * m + (jl ^ m)];
-      if (m > 0) {
-        float2 w = tw2[(m - 1) * 16 + jl];
-        w.y = -w.y;
-        v[m] = cmul(v[m], w);
-      }
-    }
-    dft<16, +1>(v);
-    // S2 [ky][x]: sample x = jl + 16 m of row ky
-    float2* out = a.scratch2 + (size_t(i) * a.H + ky) * RW_L;
-#pragma unroll
-    for (int m = 0; m < 16; ++m) out[jl + 16 * m] = v[m];
-  }
-  if (!ok && tid == 0 && a.err) atomicOr(a.err, 8u);
-}
-
-// Column IFFT (length L = H <= 256) of 16-column strips of a row-major S2 [ky][x]:
-// one TMA tensor load per strip (H rows x 16 columns, dense: the block-wide FFT's
-// lines-fastest layout with row stride 16), the next strip in flight; samples
-// stored to the time queue [y][x] from the last stage's registers.
-template <int L>
-__global__ void __launch_bounds__(PpCfg<L>::NT, (L <= 256 ? 768 / L : 1))
-    k_col_ifft_tma(SpatialArgs a, int nitems, int strip_log2, const __grid_constant__ CUtensorMap s2map) {
-  using C = PpCfg<L>;
-  static_assert(C::BT == 16, "16-column strips");
-  extern __shared__ __align__(128) unsigned char smem_tma[];  // TMA destinations: 128-byte aligned
-  __shared__ __align__(8) unsigned long long full[2];
-  float2* buf0 = reinterpret_cast<float2*>(smem_tma);
-  float2* buf1 = buf0 + L * 16;
-  float2* tws = buf1 + L * 16;
-  const int tid = threadIdx.x;
-  const int smask = (1 << strip_log2) - 1;
-  for (int e = tid; e < L; e += C::NT) tws[e] = __ldg(&a.tw_h[e]);
-  if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(rw_smem(&full[0])) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(rw_smem(&full[1])) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  }
-  __syncthreads();
-  auto issue = [&](int it, int k) {
-    const int i = it >> strip_log2, s0 = (it & smask) * 16;
-    const uint32_t mb = rw_smem(&full[k]);
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(mb), "r"(L * 16 * 8) : "memory");
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-        "[%4];\n" ::"r"(rw_smem(k ? buf1 : buf0)),
-        "l"(reinterpret_cast<uint64_t>(&s2map)), "r"(s0), "r"(int(i * L)), "r"(mb)
-        : "memory");
-  };
-  int item = blockIdx.x;
-  if (tid == 0 && item < nitems) issue(item, 0);
-  bool ok = true;
-  for (int k = 0; item < nitems && ok; ++k, item += gridDim.x) {
-    const int cur = k & 1;
-    float2* buf = cur ? buf1 : buf0;
-    const int i = item >> strip_log2, s0 = (item & smask) * 16;
-    ok = rw_wait(rw_smem(&full[cur]), uint32_t(k >> 1) & 1u);
-    ok = __syncthreads_and(ok) != 0;
-    if (!ok) break;
-    const int nxt = item + gridDim.x;
-    if (tid == 0 && nxt < nitems) {
-      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-      issue(nxt, cur ^ 1);
-    }
-    if (a.discard_inputs)  // the strip's 128-byte row segments of S2 are dead once staged
-      for (int y = tid; y < L; y += C::NT)
-        asm volatile("discard.global.L2 [%0], 128;\n" ::"l"(a.scratch2 + (size_t(i) * L + y) * a.W + s0)
-                     : "memory");
-    const size_t tslot = (a.tq.slot0 + uint32_t(i)) % a.tq.cap;
-    // time queue [y][x]: sample y of column s0 + b at tq[y W + s0 + b]
-    pp_stages<L, 1, +1, SmemSrc<16>, GlobalOut, 16>(
-        SmemSrc<16>{buf}, buf, tws, GlobalOut{static_cast<float2*>(a.tq.base) + tslot * size_t(a.W) * L + s0, a.W});
-  }
-  if (!ok && tid == 0 && a.err) atomicOr(a.err, 8u);
-}
-
-template <int LH>
-static cudaError_t launch_asp_rows(const SpatialArgs& a, cudaStream_t s, int* launches) {
-  CUtensorMap m1{}, m2{};
-  if (!encode_map_2d_u64(&m1, a.scratch1, RW_L, uint64_t(a.n) * a.H, RW_L * 8, RW_L, RW_BT, false) ||
-      !encode_map_2d_u64(&m2, a.scratch2, RW_L, uint64_t(a.n) * a.H, RW_L * 8, 16, LH, false))
-    return cudaErrorNotSupported;
-  int dev = 0, nsm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  // row pass
-  {
-    const size_t smem = (2 * size_t(RW_BT) * RW_L + 15 * 16) * sizeof(float2);
-    cudaError_t e = cudaFuncSetAttribute(k_row_asp, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_row_asp, RW_NT, smem);
-    if (e != cudaSuccess) return e;
-    int sl = 0;
-    while ((uint32_t(RW_BT) << sl) < a.H) ++sl;
-    const int nitems = int(a.n) << sl;
-    int grid = per_sm * nsm;
-    grid = grid > nitems ? nitems : (grid < 1 ? 1 : grid);
-    k_row_asp<<<grid, RW_NT, smem, s>>>(a, nitems, sl, m1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  // column IFFT
-  {
-    using C = PpCfg<LH>;
-    const size_t smem = (2 * size_t(LH) * 16 + LH) * sizeof(float2);
-    auto kern = k_col_ifft_tma<LH>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, C::NT, smem);
-    if (e != cudaSuccess) return e;
-    int sl = 0;
-    while ((16u << sl) < a.W) ++sl;
-    const int nitems = int(a.n) << sl;
-    int grid = per_sm * nsm;
-    grid = grid > nitems ? nitems : (grid < 1 ? 1 : grid);
-    kern<<<grid, C::NT, smem, s>>>(a, nitems, sl, m2);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  *launches += 2;
-  return cudaSuccess;
-}
-
-template <int LH, int LW>
-static cudaError_t pp_fixed(const SpatialArgs& a, cudaStream_t s, int* launches) {
-  cudaError_t e = launch_pp<LH, PK_P1>(a, a.W, s);
-  if (e != cudaSuccess) return e;
-  ++*launches;
-  if (a.spatial == HV_SPATIAL_ASP) {
-    // rows of 256 with the row-major transfer function: warp-private row pass and
-    // TMA-staged column IFFT (the block-wide passes when a tensor map cannot be built)
-    if constexpr (LW == RW_L && LH <= 256) {
-      if (a.asp_h) {
-        e = launch_asp_rows<LH>(a, s, launches);
-        if (e != cudaErrorNotSupported) return e;
-      }
-    }
-    e = launch_pp<LW, PK_P2A>(a, a.H, s);
-    if (e != cudaSuccess) return e;
-    e = launch_pp<LH, PK_P3A>(a, a.W, s);
-    *launches += 2;
-  } else {
-    // rows of 256: the warp-private row pass (H a multiple of its 16-row strips;
-    // the block-wide pass when the tensor map cannot be encoded)
-    e = (LW == RW_L && a.H % RW_BT == 0) ? launch_row_warp(a, s) : cudaErrorNotSupported;
-    if (e == cudaErrorNotSupported) e = launch_pp<LW, PK_P2F>(a, a.H, s);
-    ++*launches;
-  }
-  return e;
-}
-
-template <int LH>
-static cudaError_t pp_w(const SpatialArgs& a, cudaStream_t s, int* launches) {
-  switch (a.W) {
-    case 64: return pp_fixed<LH, 64>(a, s, launches);
-    case 128: return pp_fixed<LH, 128>(a, s, launches);
-    case 256: return pp_fixed<LH, 256>(a, s, launches);
-    case 512: return pp_fixed<LH, 512>(a, s, launches);
-    case 1024: return pp_fixed<LH, 1024>(a, s, launches);
-  }
-  return cudaErrorInvalidValue;
 }
 
 template <int PK>
@@ -1356,20 +979,6 @@ cudaError_t launch_pp_pass(const SpatialArgs& a, int pass, cudaStream_t s) {
 bool spatial_pp_supported(const SpatialArgs& a) {
   auto ok = [](uint32_t v) { return v >= 64 && v <= 1024; };  // two strip buffers must fit
   return ok(a.W) && ok(a.H) && (a.spatial == HV_SPATIAL_ASP || a.spatial == HV_SPATIAL_FRESNEL);
-}
-
-cudaError_t launch_spatial_pp(const SpatialArgs& a0, cudaStream_t s, int* launches) {
-  if (a0.n == 0) return cudaSuccess;
-  SpatialArgs a = a0;
-  a.discard_inputs = 1;  // the full transform reads each intermediate exactly once
-  switch (a.H) {
-    case 64: return pp_w<64>(a, s, launches);
-    case 128: return pp_w<128>(a, s, launches);
-    case 256: return pp_w<256>(a, s, launches);
-    case 512: return pp_w<512>(a, s, launches);
-    case 1024: return pp_w<1024>(a, s, launches);
-  }
-  return cudaErrorInvalidValue;
 }
 
 bool spatial_fused_supported(const SpatialArgs& a) {

@@ -1,0 +1,468 @@
+// k_spatial_strip.cu -- the spatial transform (Sec. III-B.1) of frames with sides 64
+// .. 1024 as three (ASP) or two (Fresnel) passes of 1-D FFTs whose operands go from
+// global memory straight to registers and back:
+//
+//   columns  raw [y][x] -> column FFT -> S1 [ky][x]. ASP: two real columns are one
+//            complex line, the two spectra separated in registers after, and only
+//            ky = 0 .. H/2 stored (a real column's spectrum is Hermitian). Fresnel:
+//            one column times the chirp per line, every ky stored.
+//   rows     ASP: S1 row ky -> row FFT W(kx); IFFT(W H) is row ky of S2, and row H - ky
+//            is conj(IFFT(W conj(H))): the spectrum there is conj(W(-kx)), and H(ky, kx)
+//            depends on kx^2 and ky^2 only. So H/2 + 1 forward and H inverse row FFTs a
+//            frame. Fresnel: S1 row ky -> row FFT -> time queue [ky][kx].
+//   columns  ASP: S2 [ky][x] -> column IFFT -> time queue [y][x].
+//
+// Every FFT is two register stages (radices 8 x 8 .. 32 x 32) with one exchange
+// through shared memory between them. A column CTA takes BT neighbouring lines, lines
+// fastest across lanes, so that a load or store of one row is BT x 8 contiguous
+// bytes; a row FFT is carried by 8, 16 or 32 lanes of one warp, which then needs no
+// CTA barrier. Nothing is staged: the up to 32 loads that feed a thread's first stage
+// are all in flight at once, and several CTAs per SM overlap one another's loads,
+// arithmetic and stores.
+//
+// Bound by memory: ASP moves 2 + 4 | 4 + 8 | 8 + 8 bytes per 16-bit pixel (34 against the
+// 42 of passes over full spectra). Us a frame in large launches, against the persistent
+// block-wide passes that staged each strip of 16 lines in shared memory (two strips per
+// CTA, so one or two CTAs per SM from 512 points on): 256 x 256 ASP 0.53 -> 0.37, Fresnel
+// 0.33 -> 0.31; 512 x 512 3.14 -> 2.04 and 1.65 -> 1.40; 1024 x 1024 17.0 -> 8.7 and
+// 8.4 -> 6.4; 128 x 128 0.139 -> 0.107 and 0.081 -> 0.083.
+#include "fft_dev.cuh"
+#include "hv_internal.h"
+#include "../../include/hv.h"
+
+namespace hv {
+
+namespace {
+
+// Column CTAs: L = R1 x R2, BT lines, NT threads. A thread holds I1 first-stage and I2
+// second-stage butterflies of one line.
+template <int L>
+struct ColCfg {
+  static constexpr int R1 = L >= 512 ? 32 : (L >= 128 ? 16 : 8);
+  static constexpr int R2 = L / R1;
+  static constexpr int BT = L >= 512 ? 8 : 16;
+  static constexpr int NT = L == 64 ? 64 : (L == 1024 ? 256 : 128);
+  static constexpr int NJ = NT / BT;          // threads per line
+  static constexpr int I1 = (L / R1) / NJ;    // first-stage butterflies per thread
+  static constexpr int I2 = (L / R2) / NJ;    // second-stage butterflies per thread
+  static constexpr int NTW = (R2 - 1) * R1;   // second-stage twiddles
+  static constexpr int PAD = BT == 8 ? 1 : 0; // padding rows per R1 rows of the exchange buffer
+  static constexpr int ROWS = L + PAD * R2;
+  static constexpr size_t SMEM = (size_t(ROWS) * BT + NTW) * sizeof(float2);
+  static constexpr int CTAS = L == 1024 ? 2 : (L == 512 ? 5 : (L == 64 ? 12 : 5));
+  static_assert(I1 >= 1 && I2 >= 1 && I2 <= 2 && L / R2 == R1, "two-stage plan");
+};
+
+// Second-stage twiddles w_L^{j m} at (m - 1) R1 + j, from the length-L table.
+template <int R1, int NTW, int NT>
+__device__ __forceinline__ void load_stage_twiddles(float2* tw, const float2* __restrict__ table) {
+  for (int e = threadIdx.x; e < NTW; e += NT) tw[e] = __ldg(&table[(e / R1 + 1) * (e % R1)]);
+}
+
+// The exchange buffer holds row r at r + PAD (r / R1). With 8 lines a half-warp covers
+// two rows: the padding keeps the two of a first-stage store (r and r + R1) in different
+// bank halves, at addresses that stay a register plus a constant (an XOR swizzle here
+// and in the row FFTs left 32 and more addresses live across the loop, and spilled).
+
+// First stage of a thread's line b (butterflies j = t + NJ it, inputs in v), exchange.
+template <int L, int DIR>
+__device__ __forceinline__ void col_stage1(float2 (&v)[ColCfg<L>::I1][ColCfg<L>::R1], float2* buf, int t, int b) {
+  using C = ColCfg<L>;
+#pragma unroll
+  for (int it = 0; it < C::I1; ++it) dft<C::R1, DIR>(v[it]);
+  __syncthreads();  // the previous item's second stage has read the buffer
+#pragma unroll
+  for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+    for (int m = 0; m < C::R1; ++m) buf[((t + C::NJ * it) * (C::R1 + C::PAD) + m) * C::BT + b] = v[it][m];
+  __syncthreads();
+}
+
+// Butterfly of item `it` of the second stage: with two per thread, t and its mirror
+// R1 - t (0 and R1 / 2 for t = 0), so that bins k and L - k of a line meet in a thread.
+template <int L>
+__device__ __forceinline__ int col_j2(int t, int it) {
+  using C = ColCfg<L>;
+  if (C::I2 == 1 || it == 0) return t;
+  return t == 0 ? C::R1 / 2 : C::R1 - t;
+}
+
+// Second stage: bins j + R1 m of butterfly j end in u[it][m].
+template <int L, int DIR>
+__device__ __forceinline__ void col_stage2(float2 (&u)[ColCfg<L>::I2][ColCfg<L>::R2], const float2* buf,
+                                           const float2* tw, int t, int b) {
+  using C = ColCfg<L>;
+#pragma unroll
+  for (int it = 0; it < C::I2; ++it) {
+    const int j = col_j2<L>(t, it);
+#pragma unroll
+    for (int m = 0; m < C::R2; ++m) {
+      u[it][m] = buf[(j + (C::R1 + C::PAD) * m) * C::BT + b];
+      if (m > 0) {
+        float2 w = tw[(m - 1) * C::R1 + j];
+        if (DIR > 0) w.y = -w.y;
+        u[it][m] = cmul(u[it][m], w);
+      }
+    }
+    dft<C::R2, DIR>(u[it]);
+  }
+}
+
+// Spectra of the two real columns packed in one line, from Z(k) and Z(L - k):
+// A(k) = (Z(k) + conj Z(-k)) / 2, B(k) = (Z(k) - conj Z(-k)) / 2i.
+__device__ __forceinline__ float4 unpack_pair(float2 z, float2 w) {
+  return make_float4(0.5f * (z.x + w.x), 0.5f * (z.y - w.y), 0.5f * (z.y + w.y), 0.5f * (w.x - z.x));
+}
+
+// Column FFT of raw strips. ASP: BT lines of two columns, S1 [0 .. H/2][W];
+// Fresnel: BT lines of one column, S1 [H][W].
+template <int L, bool ASP>
+__global__ void __launch_bounds__(ColCfg<L>::NT, ColCfg<L>::CTAS) k_strip_cols(SpatialArgs a, uint32_t nitems,
+                                                                              uint32_t strips) {
+  using C = ColCfg<L>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  float2* buf = reinterpret_cast<float2*>(smem);
+  float2* tw = buf + C::ROWS * C::BT;
+  load_stage_twiddles<C::R1, C::NTW, C::NT>(tw, a.tw_h);
+  const int b = threadIdx.x % C::BT, t = threadIdx.x / C::BT;
+  const uint32_t W = a.W;
+  const bool u8 = a.in_kind == IN_U8;
+  for (uint32_t item = blockIdx.x; item < nitems; item += gridDim.x) {
+    const uint32_t i = item / strips, s = item % strips;
+    const size_t frame = ((a.raw.slot0 + i) % a.raw.cap) * size_t(W) * L;
+    float2 v[C::I1][C::R1];
+    if constexpr (ASP) {
+      const size_t x = size_t(s) * (2 * C::BT) + 2 * b;
+      const size_t at = frame + x;
+      if (u8) {
+        const unsigned char* p = static_cast<const unsigned char*>(a.raw.base) + at;
+        if ((reinterpret_cast<uintptr_t>(a.raw.base) & 1) == 0) {
+#pragma unroll
+          for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+            for (int m = 0; m < C::R1; ++m) {
+              const uint32_t q =
+                  *reinterpret_cast<const uint16_t*>(p + size_t(t + C::NJ * it + (L / C::R1) * m) * W);
+              v[it][m] = make_float2(float(q & 0xffu), float(q >> 8));
+            }
+        } else {
+#pragma unroll
+          for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+            for (int m = 0; m < C::R1; ++m) {
+              const unsigned char* q = p + size_t(t + C::NJ * it + (L / C::R1) * m) * W;
+              v[it][m] = make_float2(float(q[0]), float(q[1]));
+            }
+        }
+      } else {
+        const uint16_t* p = static_cast<const uint16_t*>(a.raw.base) + at;
+        if ((reinterpret_cast<uintptr_t>(a.raw.base) & 3) == 0) {
+#pragma unroll
+          for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+            for (int m = 0; m < C::R1; ++m) {
+              const uint32_t q =
+                  *reinterpret_cast<const uint32_t*>(p + size_t(t + C::NJ * it + (L / C::R1) * m) * W);
+              v[it][m] = make_float2(float(q & 0xffffu), float(q >> 16));
+            }
+        } else {
+#pragma unroll
+          for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+            for (int m = 0; m < C::R1; ++m) {
+              const uint16_t* q = p + size_t(t + C::NJ * it + (L / C::R1) * m) * W;
+              v[it][m] = make_float2(float(q[0]), float(q[1]));
+            }
+        }
+      }
+    } else {
+      const size_t x = size_t(s) * C::BT + b;
+      const float2 cx = __ldg(&a.chirp_x[x]);
+      float r[C::I1][C::R1];
+      if (u8) {
+        const unsigned char* p = static_cast<const unsigned char*>(a.raw.base) + frame + x;
+#pragma unroll
+        for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+          for (int m = 0; m < C::R1; ++m) r[it][m] = float(p[size_t(t + C::NJ * it + (L / C::R1) * m) * W]);
+      } else {
+        const uint16_t* p = static_cast<const uint16_t*>(a.raw.base) + frame + x;
+#pragma unroll
+        for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+          for (int m = 0; m < C::R1; ++m) r[it][m] = float(p[size_t(t + C::NJ * it + (L / C::R1) * m) * W]);
+      }
+#pragma unroll
+      for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+        for (int m = 0; m < C::R1; ++m)
+          v[it][m] = cscale(cmul(__ldg(&a.chirp_y[t + C::NJ * it + (L / C::R1) * m]), cx), r[it][m]);
+    }
+    col_stage1<L, -1>(v, buf, t, b);
+    float2 u[C::I2][C::R2];
+    col_stage2<L, -1>(u, buf, tw, t, b);
+    if constexpr (!ASP) {
+      float2* out = a.scratch1 + size_t(i) * L * W + size_t(s) * C::BT + b;
+#pragma unroll
+      for (int it = 0; it < C::I2; ++it)
+#pragma unroll
+        for (int m = 0; m < C::R2; ++m) out[size_t(col_j2<L>(t, it) + C::R1 * m) * W] = u[it][m];
+    } else {
+      float2* out = a.scratch1 + size_t(i) * (L / 2 + 1) * W + size_t(s) * (2 * C::BT) + 2 * b;
+      auto put = [&](int k, float2 z, float2 w) {
+        *reinterpret_cast<float4*>(out + size_t(k) * W) = unpack_pair(z, w);
+      };
+      if constexpr (C::I2 == 2) {
+        if (t != 0) {
+          // bins t + R1 m in u[0][m], their mirrors (R1 - t) + R1 (R2 - 1 - m) in u[1]
+#pragma unroll
+          for (int m = 0; m < C::R2 / 2; ++m) {
+            put(t + C::R1 * m, u[0][m], u[1][C::R2 - 1 - m]);
+            put(C::R1 - t + C::R1 * m, u[1][m], u[0][C::R2 - 1 - m]);
+          }
+        } else {
+          // bins R1 m mirror R1 (R2 - m); bins R1 / 2 + R1 m mirror R1 / 2 + R1 (R2 - 1 - m)
+          put(0, u[0][0], u[0][0]);
+#pragma unroll
+          for (int m = 1; m <= C::R2 / 2; ++m) put(C::R1 * m, u[0][m], u[0][C::R2 - m]);
+#pragma unroll
+          for (int m = 0; m < C::R2 / 2; ++m) put(C::R1 / 2 + C::R1 * m, u[1][m], u[1][C::R2 - 1 - m]);
+        }
+      } else {
+        __syncthreads();  // every second-stage read is done
+#pragma unroll
+        for (int m = 0; m < C::R2; ++m) buf[(t + C::R1 * m) * C::BT + b] = u[0][m];
+        __syncthreads();
+#pragma unroll 4
+        for (int k = t; k <= L / 2; k += C::NJ) put(k, buf[k * C::BT + b], buf[((L - k) & (L - 1)) * C::BT + b]);
+      }
+    }
+  }
+}
+
+// Column IFFT of strips of S2 [ky][x] -> time queue [y][x].
+template <int L>
+__global__ void __launch_bounds__(ColCfg<L>::NT, ColCfg<L>::CTAS) k_strip_icols(SpatialArgs a, uint32_t nitems,
+                                                                               uint32_t strips) {
+  using C = ColCfg<L>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  float2* buf = reinterpret_cast<float2*>(smem);
+  float2* tw = buf + C::ROWS * C::BT;
+  load_stage_twiddles<C::R1, C::NTW, C::NT>(tw, a.tw_h);
+  const int b = threadIdx.x % C::BT, t = threadIdx.x / C::BT;
+  const uint32_t W = a.W;
+  for (uint32_t item = blockIdx.x; item < nitems; item += gridDim.x) {
+    const uint32_t i = item / strips, s = item % strips;
+    const float2* in = a.scratch2 + size_t(i) * L * W + size_t(s) * C::BT + b;
+    float2 v[C::I1][C::R1];
+#pragma unroll
+    for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+      for (int m = 0; m < C::R1; ++m) v[it][m] = in[size_t(t + C::NJ * it + (L / C::R1) * m) * W];
+    col_stage1<L, +1>(v, buf, t, b);
+    float2 u[C::I2][C::R2];
+    col_stage2<L, +1>(u, buf, tw, t, b);
+    float2* out = static_cast<float2*>(a.tq.base) + ((a.tq.slot0 + i) % a.tq.cap) * size_t(L) * W + size_t(s) * C::BT + b;
+#pragma unroll
+    for (int it = 0; it < C::I2; ++it)
+#pragma unroll
+      for (int m = 0; m < C::R2; ++m) __stcs(&out[size_t(col_j2<L>(t, it) + C::R1 * m) * W], u[it][m]);
+  }
+}
+
+// Row FFTs: LP lanes carry a row (lane jl holds elements jl + LP m in v[m]), RPW rows
+// per warp, four warps per CTA.
+template <int L>
+struct RowCfg {
+  static constexpr int R1 = ColCfg<L>::R1, R2 = ColCfg<L>::R2;
+  static constexpr int LP = L / R1, RPW = 32 / LP, NW = 4, NT = 32 * NW;
+  static constexpr int I2 = R1 / LP;
+  static constexpr int NTW = (R2 - 1) * R1;
+  static constexpr int RS = L + L / R1;  // exchange row: element e at e + e / R1
+  static constexpr size_t SMEM = (size_t(NW) * RPW * RS + NTW) * sizeof(float2);
+  static constexpr bool STASH = L >= 512;  // k_strip_rows_asp
+  static constexpr size_t ASP_SMEM = SMEM + (STASH ? size_t(NT) * R1 * sizeof(float2) : 0);
+  static constexpr int ASP_CTAS = L >= 512 ? 3 : (L == 64 ? 5 : 4);
+};
+
+// L-point FFT of a row through its exchange buffer rowp (padded: the 16 lanes of a
+// half-warp always meet 16 different bank pairs, two rows of 8 lanes too). On return
+// bin jl + LP m is in v[m].
+template <int L, int DIR>
+__device__ __forceinline__ void strip_row_fft(float2 (&v)[RowCfg<L>::R1], float2* rowp, const float2* tw, int jl) {
+  using C = RowCfg<L>;
+  dft<C::R1, DIR>(v);
+  __syncwarp();
+#pragma unroll
+  for (int m = 0; m < C::R1; ++m) rowp[(C::R1 + 1) * jl + m] = v[m];
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < C::I2; ++i) {
+    const int j = jl + C::LP * i;
+    float2 u[C::R2];
+#pragma unroll
+    for (int m = 0; m < C::R2; ++m) {
+      u[m] = rowp[(C::R1 + 1) * m + j];
+      if (m > 0) {
+        float2 w = tw[(m - 1) * C::R1 + j];
+        if (DIR > 0) w.y = -w.y;
+        u[m] = cmul(u[m], w);
+      }
+    }
+    dft<C::R2, DIR>(u);
+#pragma unroll
+    for (int m = 0; m < C::R2; ++m) v[i + C::I2 * m] = u[m];
+  }
+}
+
+// ASP rows: S1 rows 0 .. H/2 of n frames -> S2 rows 0 .. H - 1. Rows 0 and H / 2 are
+// their own mirrors (their W is Hermitian in kx, so both products give the same row);
+// a last warp with a row too many repeats the last row. Neither needs a branch. From
+// 512 points on W waits in shared memory while the first inverse FFT runs (each lane
+// its own words): held in registers it spilled.
+template <int L>
+__global__ void __launch_bounds__(RowCfg<L>::NT, RowCfg<L>::ASP_CTAS) k_strip_rows_asp(SpatialArgs a, uint32_t nrows) {
+  using C = RowCfg<L>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  float2* tw = reinterpret_cast<float2*>(smem);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, jl = lane % C::LP, sub = lane / C::LP;
+  float2* rowp = tw + C::NTW + (warp * C::RPW + sub) * C::RS;
+  float2* stash = tw + C::NTW + C::NW * C::RPW * C::RS + threadIdx.x;
+  load_stage_twiddles<C::R1, C::NTW, C::NT>(tw, a.tw_w);
+  __syncthreads();
+  const uint32_t H = a.H, HR = H / 2 + 1;
+  for (uint32_t r0 = (blockIdx.x * C::NW + warp) * C::RPW; r0 < nrows; r0 += gridDim.x * C::NW * C::RPW) {
+    const uint32_t row = r0 + sub < nrows ? r0 + sub : nrows - 1;
+    const uint32_t i = row / HR, ky = row % HR;
+    const float2* in = a.scratch1 + size_t(row) * L + jl;
+    float2 v[C::R1], u[C::R1];
+#pragma unroll
+    for (int m = 0; m < C::R1; ++m) v[m] = in[C::LP * m];
+    strip_row_fft<L, -1>(v, rowp, tw, jl);
+    const float2* h = a.asp_h + size_t(ky) * L + jl;
+    float2* out = a.scratch2 + size_t(i) * H * L + jl;
+#pragma unroll
+    for (int m = 0; m < C::R1; ++m) {
+      if (C::STASH) stash[m * C::NT] = v[m];
+      u[m] = cmul(v[m], __ldg(&h[C::LP * m]));
+    }
+    strip_row_fft<L, +1>(u, rowp, tw, jl);
+#pragma unroll
+    for (int m = 0; m < C::R1; ++m) out[size_t(ky) * L + C::LP * m] = u[m];
+#pragma unroll
+    for (int m = 0; m < C::R1; ++m) {
+      // read again (an L1 hit): kept from the first product it would cost 2 R1 registers
+      float2 w;
+      asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];\n" : "=f"(w.x), "=f"(w.y) : "l"(&h[C::LP * m]) : "memory");
+      w.y = -w.y;
+      u[m] = cmul(C::STASH ? stash[m * C::NT] : v[m], w);
+    }
+    strip_row_fft<L, +1>(u, rowp, tw, jl);
+#pragma unroll
+    for (int m = 0; m < C::R1; ++m)
+      out[size_t((H - ky) & (H - 1)) * L + C::LP * m] = make_float2(u[m].x, -u[m].y);
+  }
+}
+
+// Fresnel rows: S1 rows -> row FFT -> time queue [ky][kx].
+template <int L>
+__global__ void __launch_bounds__(RowCfg<L>::NT, (L >= 512 ? 4 : 6)) k_strip_rows_fft(SpatialArgs a, uint32_t nrows) {
+  using C = RowCfg<L>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  float2* tw = reinterpret_cast<float2*>(smem);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, jl = lane % C::LP, sub = lane / C::LP;
+  float2* rowp = tw + C::NTW + (warp * C::RPW + sub) * C::RS;
+  load_stage_twiddles<C::R1, C::NTW, C::NT>(tw, a.tw_w);
+  __syncthreads();
+  // H is a multiple of the rows of a warp: its rows are all valid and of one frame
+  for (uint32_t r0 = (blockIdx.x * C::NW + warp) * C::RPW; r0 < nrows; r0 += gridDim.x * C::NW * C::RPW) {
+    const uint32_t row = r0 + sub, i = row / a.H, ky = row % a.H;
+    const float2* in = a.scratch1 + size_t(row) * L + jl;
+    float2 v[C::R1];
+#pragma unroll
+    for (int m = 0; m < C::R1; ++m) v[m] = in[C::LP * m];
+    strip_row_fft<L, -1>(v, rowp, tw, jl);
+    float2* out = static_cast<float2*>(a.tq.base) + (((a.tq.slot0 + i) % a.tq.cap) * a.H + ky) * size_t(L) + jl;
+#pragma unroll
+    for (int m = 0; m < C::R1; ++m) __stcs(&out[C::LP * m], v[m]);
+  }
+}
+
+// Persistent grid: every CTA that fits at once, no more than the items.
+template <class K, class... Args>
+cudaError_t launch_resident(K kern, int nt, size_t smem, uint32_t ctas, cudaStream_t s, Args... args) {
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  if (e != cudaSuccess) return e;
+  int per_sm = 0, dev = 0, nsm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem);
+  if (e != cudaSuccess) return e;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const uint32_t most = uint32_t(per_sm > 0 ? per_sm : 1) * uint32_t(nsm);
+  kern<<<ctas < most ? ctas : most, nt, smem, s>>>(args...);
+  return cudaGetLastError();
+}
+
+template <int L, bool ASP>
+cudaError_t cols(const SpatialArgs& a, cudaStream_t s) {
+  using C = ColCfg<L>;
+  const uint32_t strips = a.W / (ASP ? 2 * C::BT : C::BT), items = strips * a.n;
+  return launch_resident(k_strip_cols<L, ASP>, C::NT, C::SMEM, items, s, a, items, strips);
+}
+
+template <int L>
+cudaError_t icols(const SpatialArgs& a, cudaStream_t s) {
+  using C = ColCfg<L>;
+  const uint32_t strips = a.W / C::BT, items = strips * a.n;
+  return launch_resident(k_strip_icols<L>, C::NT, C::SMEM, items, s, a, items, strips);
+}
+
+template <int L>
+cudaError_t rows(const SpatialArgs& a, cudaStream_t s) {
+  using C = RowCfg<L>;
+  constexpr uint32_t per = C::NW * C::RPW;
+  if (a.spatial == HV_SPATIAL_ASP) {
+    const uint32_t nrows = a.n * (a.H / 2 + 1);
+    return launch_resident(k_strip_rows_asp<L>, C::NT, C::ASP_SMEM, (nrows + per - 1) / per, s, a, nrows);
+  }
+  const uint32_t nrows = a.n * a.H;
+  return launch_resident(k_strip_rows_fft<L>, C::NT, C::SMEM, (nrows + per - 1) / per, s, a, nrows);
+}
+
+#define HV_BY_SIDE(side, fn)             \
+  switch (side) {                        \
+    case 64: e = fn(64); break;          \
+    case 128: e = fn(128); break;        \
+    case 256: e = fn(256); break;        \
+    case 512: e = fn(512); break;        \
+    case 1024: e = fn(1024); break;      \
+    default: e = cudaErrorInvalidValue;  \
+  }
+
+}  // namespace
+
+bool spatial_strip_supported(const SpatialArgs& a) {
+  auto ok = [](uint32_t v) { return v >= 64 && v <= 1024; };
+  return ok(a.W) && ok(a.H) &&
+         (a.spatial == HV_SPATIAL_FRESNEL || (a.spatial == HV_SPATIAL_ASP && a.asp_h != nullptr));
+}
+
+cudaError_t launch_spatial_strip(const SpatialArgs& a, cudaStream_t s, int* launches) {
+  if (a.n == 0) return cudaSuccess;
+  if (!spatial_strip_supported(a)) return cudaErrorInvalidValue;
+  const bool asp = a.spatial == HV_SPATIAL_ASP;
+  cudaError_t e;
+#define HV_COLS(L) (asp ? cols<L, true>(a, s) : cols<L, false>(a, s))
+#define HV_ROWS(L) rows<L>(a, s)
+#define HV_ICOLS(L) icols<L>(a, s)
+  HV_BY_SIDE(a.H, HV_COLS)
+  if (e != cudaSuccess) return e;
+  HV_BY_SIDE(a.W, HV_ROWS)
+  *launches += 2;
+  if (e != cudaSuccess || !asp) return e;
+  HV_BY_SIDE(a.H, HV_ICOLS)
+  ++*launches;
+  return e;
+}
+
+}  // namespace hv

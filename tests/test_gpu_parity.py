@@ -118,15 +118,32 @@ def test_cluster_spatial_field_parity(N, spatial, bits):
                                               (64, 256, "asp", 8), (128, 256, "asp", 12),
                                               (64, 256, "fresnel", 8), (128, 256, "fresnel", 12)])
 def test_persistent_multipass_parity(H, W, spatial, bits):
-    """Persistent prefetching multi-pass kernels (frames and strips looped per CTA;
-    8-line strips at side 1024, 8-byte raw copies for uint8 there). Width 256 takes
-    the warp-private row passes (Fresnel; ASP with the TMA column IFFT for H <= 256)."""
+    """The passes with a small launch size: frames and strips looped per CTA, several
+    launches per render."""
     n = 7
     fr = synth.random_frames(n, H, W, bits, seed=H + 3 * W)
     p = oracle_params(spatial=spatial, z_m=0.3, pitch_y_m=17e-6, temporal="none", T=1, stride=1,
                       H=H, W=W)
     img, _ = gpu_render(fr, p, extra=dict(spatial_kernel="persistent", spatial_chunk=3),
                         packets=[2, 5])
+    ref = oracle_fields(fr, p)
+    for i in range(n):
+        assert rel_l2(img[i], ref[i]) <= FIELD_TOL, (i, rel_l2(img[i], ref[i]))
+
+
+@pytest.mark.parametrize("H,W,spatial,bits,n", [(64, 1024, "asp", 8, 1), (1024, 128, "asp", 12, 3),
+                                                (512, 64, "fresnel", 8, 2), (512, 512, "asp", 8, 2),
+                                                (1024, 256, "fresnel", 12, 2), (64, 64, "asp", 12, 1),
+                                                (128, 64, "asp", 8, 3)])
+def test_strip_passes_parity(H, W, spatial, bits, n):
+    """Register-direct passes at lengths 64 .. 1024 along either axis: a last warp with
+    fewer rows than it holds (33 or 99 rows of 4 per warp), the rows that are their own
+    mirrors, 8-bit column pairs, a high-pass filter."""
+    fr = synth.random_frames(n, H, W, bits, seed=H + 5 * W)
+    p = oracle_params(spatial=spatial, z_m=0.3, pitch_y_m=17e-6, temporal="none", T=1, stride=1, H=H, W=W)
+    if spatial == "asp":
+        p["highpass"] = 0.05
+    img, _ = gpu_render(fr, p, extra=dict(spatial_chunk=2))
     ref = oracle_fields(fr, p)
     for i in range(n):
         assert rel_l2(img[i], ref[i]) <= FIELD_TOL, (i, rel_l2(img[i], ref[i]))

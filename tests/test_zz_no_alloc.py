@@ -157,3 +157,22 @@ def test_static_refuses_misaligned_pointers_and_highpass_without_asp():
     assert f(dev.data_ptr(), 16, 1, ctypes.byref(p), out.data_ptr(), None) == hv.HV_OK
     torch.cuda.synchronize()
     assert torch.isfinite(out[: 64 * 64 * 2]).all()
+
+
+@pytest.mark.parametrize("bits,offset", [(8, 1), (16, 2)])
+def test_static_reads_frames_at_the_alignment_of_a_pixel(bits, offset):
+    """Column pairs are read as one word where the frames allow it, else pixel by pixel."""
+    import torch
+    f = _entry()
+    H, W = 64, 128
+    fr = synth.random_frames(1, H, W, 8 if bits == 8 else 12, seed=11)
+    p = oracle_params(spatial="asp", temporal="none", T=1, stride=1, H=H, W=W)
+    ref = _cplx(_handle_fields(fr, p), 1, H, W)
+    raw = torch.zeros(fr.nbytes + offset, dtype=torch.uint8, device="cuda")
+    raw[offset:] = torch.from_numpy(np.ascontiguousarray(fr).reshape(-1).view(np.uint8)).cuda()
+    out = torch.zeros(H * W * 2, dtype=torch.float32, device="cuda")
+    prm = to_hv(p)
+    torch.cuda.synchronize()
+    assert f(raw.data_ptr() + offset, bits, 1, ctypes.byref(prm), out.data_ptr(), None) == hv.HV_OK
+    torch.cuda.synchronize()
+    assert rel_l2(_cplx(out.cpu().numpy(), 1, H, W)[0], ref[0]) <= FIELD_TOL
