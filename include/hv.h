@@ -100,8 +100,8 @@ typedef struct {
   int32_t tuned;              /* 1 = tuned form (spatial kernels chosen by timing)    */
   uint32_t spatial_chunk;     /* frames per spatial launch (0 = automatic)             */
   uint32_t spatial_kernel;    /* HV_SK_*: which spatial kernels (default automatic):
-                                 multi-pass (one strip per CTA), persistent multi-pass
-                                 (CTAs loop over strips, prefetching the next), the
+                                 multi-pass, persistent multi-pass (sides from 64 up,
+                                 where both are the same register-direct passes), the
                                  whole-frame cluster kernel, or the fused transform
                                  (256 x 256 frames: every pass of every frame in one
                                  persistent launch, intermediates in L2-resident rings) */
@@ -209,7 +209,8 @@ typedef struct {
                                        _WINDOW_TMA_PIPELINED                          */
   float candidate_us_per_frame[12]; /* measured us per frame: multi-pass with 16, 32, 64,
                                        128, 256 frames per launch; persistent
-                                       multi-pass with 64, 128, 256, 512; the cluster
+                                       multi-pass with 64, 128, 256 (0: the same passes
+                                       as multi-pass) and 512; the cluster
                                        kernel; the fused transform (0 where not
                                        applicable)                                    */
   float stft_us_per_window[6];      /* measured us per window of the STFT kernels:
