@@ -577,13 +577,7 @@ def roofline(w, res, peaks):
     if t_tm < t_sp and w["N"] == 256 and w["spatial"] == "asp":
         kern = "k_spatial_fused (every spatial pass, one launch per render)" if tun.get("spatial_kernel") == 4 \
             else kern
-        if tun.get("spatial_kernel") == 3 and tun.get("spatial_chunk") == 512:
-            # the three persistent passes of one 512-frame launch set, scaled to a render
-            parts = [profiled_traffic("spatial_pp_asp_256.md", ["k_spatial_pp.cu", "fft_dev.cuh"], i)
-                     for i in range(3)]
-            if all(v is not None for v in parts):
-                traffic = int(sum(parts) * frames_per_render / 512)
-        elif tun.get("spatial_kernel") == 4 and w["bits"] > 8:
+        if tun.get("spatial_kernel") == 4 and w["bits"] > 8:
             v = profiled_traffic("spatial_fused_asp_256.md", ["k_spatial_pp.cu", "fft_dev.cuh"])
             if v is not None:
                 traffic = int(v * frames_per_render / 1024)
