@@ -209,8 +209,8 @@ typedef struct {
                                        _WINDOW_TMA_PIPELINED                          */
   float candidate_us_per_frame[12]; /* measured us per frame: multi-pass with 16, 32, 64,
                                        128, 256 frames per launch; persistent
-                                       multi-pass with 64, 128, 256 (0: the same passes
-                                       as multi-pass) and 512; the cluster
+                                       multi-pass with 64, 128, 256 (the same passes as
+                                       multi-pass, not timed again) and 512; the cluster
                                        kernel; the fused transform (0 where not
                                        applicable)                                    */
   float stft_us_per_window[6];      /* measured us per window of the STFT kernels:

@@ -702,8 +702,11 @@ hv_status tune_spatial(hv_handle* h) {
   for (int ci = 0; ci < 11; ++ci) {
     const Cand c = cands[ci];
     if (c.kind == 2 && !cluster_ok(h)) continue;
-    // from 64 up kinds 1 and 3 are the same passes: each launch size is timed once
-    if (c.kind == 3 && (!pp_ok || c.chunk <= 256)) continue;
+    if (c.kind == 3 && !pp_ok) continue;
+    if (c.kind == 3 && c.chunk <= 256) {  // from 64 up kind 1's passes: its time for this launch size
+      t.candidate_us_per_frame[ci] = t.candidate_us_per_frame[ci - 3];
+      continue;
+    }
     if (c.kind == 4 && !fused_ok) continue;
     const uint32_t ch = (c.kind == 2 || c.kind == 4) ? n : std::min(c.chunk, n);
     if (c.kind == 4 && ensure(h, reinterpret_cast<void**>(&h->fused_ctr), &h->fused_ctr_bytes,
