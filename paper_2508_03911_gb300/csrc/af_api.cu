@@ -74,7 +74,6 @@ hv_status hv_af_open(const hv_af_desc* d, hv_af** out) {
   }
   const size_t B = d->max_batch;
   Net& t = a->t;
-  t.dw_chunks = 256;
   // one allocation, carved in 256-byte aligned pieces
   struct Piece {
     void** p;
@@ -92,8 +91,7 @@ hv_status hv_af_open(const hv_af_desc* d, hv_af** out) {
       {reinterpret_cast<void**>(&t.dbuf0), B * 32 * 32 * 32 * 4},
       {reinterpret_cast<void**>(&t.dbuf1), B * 16 * 64 * 64 * 4},
       {reinterpret_cast<void**>(&t.head), B * 130 * 4},
-      {reinterpret_cast<void**>(&t.part), dw_part_floats(t.dw_chunks) * 4},
-      {reinterpret_cast<void**>(&t.partb), size_t(t.dw_chunks) * 64 * 4},
+      {reinterpret_cast<void**>(&t.part), dw_part_floats() * 4},
       {reinterpret_cast<void**>(&t.err), 16},
   };
   size_t total = 0;

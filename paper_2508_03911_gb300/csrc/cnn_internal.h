@@ -28,9 +28,7 @@ struct Net {
   float* dbuf0;             // [n][32][32][32] floats (dZ4, then dZ2)
   float* dbuf1;             // [n][16][64][64] floats (dZ3, then dZ1)
   float* head;              // [n][130] head scratch
-  float* part;              // weight-gradient partials, dw_part_floats(dw_chunks)
-  float* partb;             // [dw_chunks][64] bias-gradient partials
-  uint32_t dw_chunks;       // pixel chunks of the weight-gradient reduction
+  float* part;              // weight- and bias-gradient partials, dw_part_floats()
   unsigned* err;            // device flags: bit 2 set when a tensor-core convolution gave up a bounded wait
 };
 
@@ -51,7 +49,7 @@ cudaError_t net_backward(const Net& t, const void* x, uint32_t n, float* loss, c
 cudaError_t net_adam(const Net& t, float lr, float b1, float b2, float eps, float c1, float c2, cudaStream_t s);
 // Refresh the bfloat16 mirror from the float32 parameters.
 cudaError_t net_sync_bf16(const Net& t, cudaStream_t s);
-size_t dw_part_floats(uint32_t nchunks);
+size_t dw_part_floats();
 
 }  // namespace cnn
 }  // namespace hv

@@ -77,6 +77,33 @@ def test_gradients_match_oracle():
         o += k
 
 
+@pytest.mark.parametrize("n,offset", [(1, 0), (19, 0), (3, 1)])
+def test_gradients_of_other_batches(n, offset):
+    """Fewer and more bands and images than CTAs of a layer's weight gradient share
+    evenly; inputs at an odd bfloat16 of a buffer (layer 1 reads 16 bytes where aligned)."""
+    import torch
+    flat, x, z, xd, zd = _setup(n, 5 + n)
+    buf = torch.zeros(xd.numel() + offset, dtype=torch.bfloat16, device="cuda")
+    buf[offset:] = xd.reshape(-1)
+    xo = buf[offset:].reshape(xd.shape)
+    with _net(n) as net:
+        net.set_params(flat)
+        loss = torch.zeros(1, device="cuda")
+        grad = torch.zeros(A.n_params(), device="cuda")
+        torch.cuda.synchronize()
+        net.loss_grad(xo, zd, loss, grad)
+        torch.cuda.synchronize()
+        g = grad.cpu().numpy().astype(np.float64)
+    Lr, gr = A.gradients(flat, x, z.astype(np.float32).astype(np.float64), bf16_acts=True)
+    assert abs(float(loss.item()) - Lr) <= 1e-3 * Lr
+    o = 0
+    for name, s in A.param_shapes():
+        k = int(np.prod(s))
+        e = np.linalg.norm(g[o:o + k] - gr[o:o + k]) / max(np.linalg.norm(gr[o:o + k]), 1e-30)
+        assert e <= 1e-2, (name, e)
+        o += k
+
+
 def test_adam_update_matches_oracle():
     import torch
     flat, x, z, xd, zd = _setup(4, 3)
