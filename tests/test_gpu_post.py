@@ -128,3 +128,57 @@ def test_invalid_post_settings_and_temporal_none():
         assert ei.value.status == hv.HV_ERR_UNSUPPORTED
     finally:
         r.close()
+
+
+@pytest.mark.parametrize("H,W,K,shift", [(16, 16, 3, 0), (48 - 16, 32, 31, 0), (32, 64, 1, 1), (16, 128, 7, 3),
+                                         (64, 256, 15, 0)])
+def test_convolution_widths_and_kernel_sizes(H, W, K, shift):
+    """Tiles of 16, 32 and 64 columns, kernels of 1 to 31 (wider than the image too: it is
+    periodic), outputs at any float of a buffer, a short accumulation."""
+    import torch
+    T, S = 16, 16
+    fr = synth.random_frames(5 * T, H, W, 12, seed=K + W)
+    p = oracle_params(spatial="none", T=T, stride=S, fs_hz=20000.0, band_lo_bin=1, band_hi_bin=7,
+                      moments=("M0", "M1N"), H=H, W=W)
+    kern = np.random.default_rng(K).standard_normal((K, K)) / K + 0.5 / (K * K)
+    ref = oracle_post(fr, p, kern.astype(np.float32).astype(np.float64), True, 3)
+    r = hv.Renderer(W, H, 16, len(fr))
+    try:
+        hv.hv_set_params(r.h, to_hv(p))
+        hv.hv_set_postprocess(r.h, kernel=kern, renormalize=True, accumulate=3)
+        wf = r.window_floats()
+        out = torch.zeros(5 * wf + shift, dtype=torch.float32, device="cuda")
+        torch.cuda.synchronize()
+        assert r.push(to_device(fr)) == hv.HV_OK
+        assert r.render(out[shift:]) == 5
+        torch.cuda.synchronize()
+        check(out[shift:].cpu().numpy().reshape(5, 2, H, W), ref)
+    finally:
+        r.close()
+
+
+def test_an_infinite_pixel_stays_within_the_kernels_reach():
+    """No tap outside the K x K kernel is formed (0 x infinity is not 0), and the sums of an
+    image with an infinity come from the float64 path: its mean is infinite."""
+    import torch
+    H = W = 64
+    fr = synth.random_frames(16, H, W, 12, seed=5)
+    p = oracle_params(spatial="none", T=16, stride=16, fs_hz=1.6e20, band_lo_bin=1, band_hi_bin=7,
+                      moments=("M2",), H=H, W=W)
+    # M2 is about 3e9 (squared bins) times (1e16)^2 kHz^2: past the largest float; rows from
+    # 20 on are constant in time, their bins and moments exactly 0
+    fr[:, 20:, :] = 100
+    r = hv.Renderer(W, H, 16, 16)
+    try:
+        hv.hv_set_params(r.h, to_hv(p))
+        hv.hv_set_postprocess(r.h, kernel=np.full((5, 5), 0.04, np.float32))
+        out = torch.zeros(H * W, dtype=torch.float32, device="cuda")
+        torch.cuda.synchronize()
+        assert r.push(to_device(fr)) == hv.HV_OK
+        assert r.render(out) == 1
+        torch.cuda.synchronize()
+        img = out.cpu().numpy().reshape(H, W)
+        assert np.all(np.isposinf(img[2:18])) and not np.any(np.isnan(img))
+        assert np.all(np.isfinite(img[24:60]))
+    finally:
+        r.close()
