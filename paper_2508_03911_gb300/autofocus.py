@@ -76,7 +76,7 @@ class Pipeline:
             fr = torch.from_numpy(frames[a:b].view(np.int16)).to(self.dev)
             hv.hv_focus_sweep(self.r.h, fr, self.zs, metric[a:b])
             hv.hv_af_features(self.r.h, fr, feats[a:b])
-        self.r.synchronize()
+            self.r.synchronize()  # the calls are queued on the handle's stream: before fr is freed
         m = metric.cpu().numpy()
         j = np.argmax(m, axis=1)
         return j, self.zs[j], m, feats

@@ -690,11 +690,7 @@ hv_status tune_spatial(hv_handle* h) {
   struct Cand { int kind; uint32_t chunk; };  // kind: 1 multi-pass, 3 persistent, 2 cluster, 4 fused
   static const Cand cands[] = {{1, 16}, {1, 32}, {1, 64}, {1, 128}, {1, 256},
                                {3, 64}, {3, 128}, {3, 256}, {3, 512}, {2, 0}, {4, 0}};
-  SpatialArgs probe{};
-  probe.spatial = h->cur.spatial;
-  probe.W = h->W;
-  probe.H = h->H;
-  const bool pp_ok = spatial_pp_supported(probe);
+  const bool pp_ok = h->W >= 64 && h->H >= 64;
   const bool fused_ok = h->W == 256 && h->H == 256;  // ASP or Fresnel (checked above)
   float best = 1e30f;
   int best_kind = 1;
@@ -1522,11 +1518,7 @@ static hv_status af_prepare(hv_handle* h, const void* frames, uint32_t n, uint32
   HV_CU(h, cudaSetDevice(h->device));
   hv_status s = apply_pending(h);
   if (s != HV_OK) return s;
-  SpatialArgs probe{};
-  probe.spatial = HV_SPATIAL_ASP;
-  probe.W = h->W;
-  probe.H = h->H;
-  if (!spatial_pp_supported(probe)) return fail(h, HV_ERR_UNSUPPORTED, "autofocus needs sides in [64, 1024]");
+  if (h->W < 64 || h->H < 64) return fail(h, HV_ERR_UNSUPPORTED, "autofocus needs sides in [64, 1024]");
   const size_t need = size_t(chunk) * h->W * h->H * sizeof(float2);
   s = ensure(h, reinterpret_cast<void**>(&h->s1), &h->s1_bytes, need);
   if (s == HV_OK) s = ensure(h, reinterpret_cast<void**>(&h->s2), &h->s2_bytes, need);
@@ -1536,24 +1528,29 @@ static hv_status af_prepare(hv_handle* h, const void* frames, uint32_t n, uint32
 hv_status hv_focus_sweep(hv_handle* h, const void* frames, uint32_t n, const double* z, uint32_t nz, float* metric) {
   if (!h) return HV_ERR_ARG;
   if (!z || !metric || nz == 0 || nz > 1024) return fail(h, HV_ERR_ARG, "bad distances or output");
-  const uint32_t chunk = 64;
-  hv_status s = af_prepare(h, frames, n, std::min(n, chunk));
+  // holograms whose spectra are held at once, and (distance, hologram) images per launch
+  const uint32_t chunk = std::min<uint32_t>(n, 64);
+  hv_status s = af_prepare(h, frames, n, chunk);
   if (s != HV_OK) return s;
   const uint32_t W = h->W, H = h->H;
+  const size_t fbytes = size_t(W) * H * sizeof(float2);
+  const uint32_t images = std::max(chunk, uint32_t((size_t(128) << 20) / fbytes));
+  s = ensure(h, reinterpret_cast<void**>(&h->s2), &h->s2_bytes, images * fbytes);
+  if (s != HV_OK) return s;
   const hv_params& p = h->cur;
-  // transfer functions H_j (transposed [kx][ky], 1/(W H) folded in, DC bin zero)
+  // transfer functions H_j, rows ky = 0 .. H/2 (1/(W H) folded in, DC bin zero)
+  const size_t per = size_t(W) * (H / 2 + 1);
   std::vector<double> key = {double(W), double(H), p.lambda_m, p.pitch_x_m, p.pitch_y_m};
   key.insert(key.end(), z, z + nz);
   if (key != h->sw_key) {
-    const size_t per = size_t(W) * H;
     s = ensure(h, reinterpret_cast<void**>(&h->sw_tables), &h->sw_bytes, per * nz * sizeof(float2));
     if (s != HV_OK) return s;
     std::vector<float2> host(per * nz);
     const double k = 2.0 * M_PI / p.lambda_m, scale = 1.0 / (double(W) * double(H));
     for (uint32_t kx = 0; kx < W; ++kx) {
       const double fx = 2.0 * M_PI * (kx < W / 2 ? double(kx) : double(kx) - W) / (W * p.pitch_x_m);
-      for (uint32_t ky = 0; ky < H; ++ky) {
-        const double fy = 2.0 * M_PI * (ky < H / 2 ? double(ky) : double(ky) - H) / (H * p.pitch_y_m);
+      for (uint32_t ky = 0; ky <= H / 2; ++ky) {
+        const double fy = 2.0 * M_PI * double(ky) / (H * p.pitch_y_m);
         const double kz2 = k * k - fx * fx - fy * fy;
         for (uint32_t j = 0; j < nz; ++j) {
           float2 v = make_float2(0.f, 0.f);
@@ -1561,7 +1558,7 @@ hv_status hv_focus_sweep(hv_handle* h, const void* frames, uint32_t n, const dou
             const double ph = z[j] * std::sqrt(kz2);
             v = make_float2(float(std::cos(ph) * scale), float(std::sin(ph) * scale));
           }
-          host[j * per + size_t(kx) * H + ky] = v;
+          host[j * per + size_t(ky) * W + kx] = v;
         }
       }
     }
@@ -1577,16 +1574,16 @@ hv_status hv_focus_sweep(hv_handle* h, const void* frames, uint32_t n, const dou
     SpatialArgs sa = af_args(h, frames, n);
     sa.raw.slot0 = a;
     sa.n = std::min(chunk, n - a);
-    cudaError_t e = launch_pp_pass(sa, PASS_COL_FFT, h->stream);
-    for (uint32_t j = 0; j < nz && e == cudaSuccess; ++j) {
-      sa.asp_ht = h->sw_tables + size_t(j) * W * H;
-      e = launch_pp_pass(sa, PASS_ROW_ASP, h->stream);
+    cudaError_t e = launch_strip_spectrum(sa, h->stream);
+    h->st.kernel_launches += 2;
+    const uint32_t zc = std::max<uint32_t>(1, images / sa.n);
+    for (uint32_t j = 0; j < nz && e == cudaSuccess; j += zc) {
       sa.tam_acc = h->sw_acc + (size_t(a) * nz + j) * 2;
       sa.tam_stride = nz * 2;
-      if (e == cudaSuccess) e = launch_pp_pass(sa, PASS_COL_IFFT_TAMURA, h->stream);
+      e = launch_strip_sweep(sa, h->sw_tables + j * per, std::min(zc, nz - j), h->stream);
+      h->st.kernel_launches += 2;
     }
     if (e != cudaSuccess) return cuda_fail(h, e, "focus sweep passes");
-    h->st.kernel_launches += 1 + 2 * nz;
   }
   cudaError_t e = launch_tamura_finish(h->sw_acc, n * nz, W * H, metric, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "tamura");
@@ -1603,30 +1600,18 @@ hv_status hv_af_features(hv_handle* h, const void* frames, uint32_t n, void* out
   hv_status s = af_prepare(h, frames, n, std::min(n, chunk));
   if (s != HV_OK) return s;
   const size_t cells = size_t(h->W / 2) * (h->H / 2);
-  // widths up to 256: the row pass forms the cells in its epilogue (no spectrum in
-  // memory); wider frames store the spectra and bin them in a second kernel
-  const bool fused = h->W <= 256;
   for (uint32_t a = 0; a < n; a += chunk) {
     SpatialArgs sa = af_args(h, frames, n);
     sa.raw.slot0 = a;
     sa.n = std::min(chunk, n - a);
-    sa.discard_inputs = 1;  // the column pass output is read once
-    cudaError_t e = launch_pp_pass(sa, PASS_COL_FFT, h->stream);
     uint16_t* dst = static_cast<uint16_t*>(out_bf16) + a * cells;
-    if (fused) {
-      // s2 holds this chunk's cells [n][H/2][W/2] (floats), then its (sum, sum of squares)
-      sa.cells = reinterpret_cast<float*>(h->s2);
-      sa.tam_acc = reinterpret_cast<double*>(h->s2 + (size_t(sa.n) * cells + 1) / 2);
-      sa.tam_stride = 2;
-      if (e == cudaSuccess) e = cudaMemsetAsync(sa.tam_acc, 0, size_t(sa.n) * 2 * sizeof(double), h->stream);
-      if (e == cudaSuccess) e = launch_pp_pass(sa, PASS_ROW_CELLS, h->stream);
-      if (e == cudaSuccess)
-        e = launch_af_standardize(sa.cells, sa.tam_acc, 2, sa.n, uint32_t(cells), dst, h->stream);
-    } else {
-      sa.tq = RingRef{h->s2, sa.n, 0};  // spectra [ky][kx] of this chunk
-      if (e == cudaSuccess) e = launch_pp_pass(sa, PASS_ROW_FFT, h->stream);
-      if (e == cudaSuccess) e = launch_af_features(h->s2, sa.n, h->W, h->H, dst, h->stream);
-    }
+    // s2 holds this chunk's cells [n][H/2][W/2] (floats), then its (sum, sum of squares)
+    sa.cells = reinterpret_cast<float*>(h->s2);
+    sa.tam_acc = reinterpret_cast<double*>(h->s2 + (size_t(sa.n) * cells + 1) / 2);
+    sa.tam_stride = 2;
+    cudaError_t e = cudaMemsetAsync(sa.tam_acc, 0, size_t(sa.n) * 2 * sizeof(double), h->stream);
+    if (e == cudaSuccess) e = launch_strip_cells(sa, h->stream);
+    if (e == cudaSuccess) e = launch_af_standardize(sa.cells, sa.tam_acc, 2, sa.n, uint32_t(cells), dst, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "feature passes");
     h->st.kernel_launches += 3;
   }

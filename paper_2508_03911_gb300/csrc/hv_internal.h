@@ -35,8 +35,7 @@ struct SpatialArgs {
   int use_cluster;      // 1: whole-frame cluster kernel when the size allows it
   double* tam_acc;      // focus sweep: frame i adds (sum |u|, sum |u|^2) at tam_acc + i * tam_stride
   uint32_t tam_stride;
-  int discard_inputs;   // persistent passes: scratch1/scratch2 are read once, drop their L2 lines after staging
-  float* cells;         // PASS_ROW_CELLS output [n][H/2][W/2]
+  float* cells;         // launch_strip_cells output [n][H/2][W/2]
   unsigned* err;        // device flags (bit 3: a row pass's wait for its staged strip gave up;
                         // bit 4: a fused-transform wait for another CTA's pass gave up); may be NULL
   // fused transform (one persistent launch for every pass of every frame, 256 x 256):
@@ -49,10 +48,19 @@ struct SpatialArgs {
 };
 cudaError_t launch_spatial(const SpatialArgs& a, cudaStream_t s, int* launches);
 bool spatial_cluster_supported(const SpatialArgs& a);
-bool spatial_pp_supported(const SpatialArgs& a);
 // Register-direct passes for sides 64 .. 1024 (ASP needs asp_h).
 bool spatial_strip_supported(const SpatialArgs& a);
 cudaError_t launch_spatial_strip(const SpatialArgs& a, cudaStream_t s, int* launches);
+// Focus sweep: the spectra of n frames, rows ky = 0 .. H/2, in scratch1 [n][H/2 + 1][W];
+// then for nz transfer functions h [nz][H/2 + 1][W] the propagated frames through scratch2
+// (nz n frames), adding (sum |u|, sum |u|^2) of frame i, function z to tam_acc + i
+// tam_stride + 2 z.
+cudaError_t launch_strip_spectrum(const SpatialArgs& a, cudaStream_t s);
+cudaError_t launch_strip_sweep(const SpatialArgs& a, const float2* h, uint32_t nz, cudaStream_t s);
+// Network-input cells [n][H/2][W/2] of n frames into cells (through scratch1): the centred
+// spectrum's 2 x 2 blocks as log1p(mean |F|) (DC bin as 0), (sum v, sum v^2) of a frame
+// added to tam_acc + frame * tam_stride.
+cudaError_t launch_strip_cells(const SpatialArgs& a, cudaStream_t s);
 cudaError_t launch_spatial_cluster(const SpatialArgs& a, cudaStream_t s, int* launches);
 // Fused transform: frames of 256 x 256, ASP or Fresnel; needs ring >= kFusedRing
 // frames in scratch1 (and scratch2 for ASP), fused_ctr and err.
@@ -60,20 +68,6 @@ constexpr uint32_t kFusedRing = 96;
 constexpr uint32_t kFusedPasses = 4;  // counter sets: ASP takes four passes, Fresnel two
 bool spatial_fused_supported(const SpatialArgs& a);
 cudaError_t launch_spatial_fused(const SpatialArgs& a, cudaStream_t s, int* launches);
-
-// Single passes of the persistent multi-pass transform (sides 64..512):
-//   PASS_COL_FFT   raw -> column FFT (chirped when spatial is Fresnel) -> scratch1 [ky][x]
-//   PASS_ROW_ASP   scratch1 -> row FFT, x asp_ht, row IFFT -> scratch2 [x][ky]
-//   PASS_COL_IFFT  scratch2 -> column IFFT -> tq ring [y][x]
-//   PASS_ROW_FFT   scratch1 -> row FFT -> tq ring [ky][kx]
-//   PASS_COL_IFFT_TAMURA  scratch2 -> column IFFT -> (sum |u|, sum |u|^2) per frame
-//   PASS_ROW_CELLS scratch1 -> row FFT -> network-input cells (sides 64..256): the
-//                  centred spectrum's 2 x 2 blocks as log1p(mean |F|) (DC bin as 0)
-//                  into cells [frame][H/2][W/2], and (sum v, sum v^2) per frame
-//                  into tam_acc + frame * tam_stride
-enum { PASS_COL_FFT = 0, PASS_ROW_ASP = 1, PASS_COL_IFFT = 2, PASS_ROW_FFT = 3, PASS_COL_IFFT_TAMURA = 4,
-       PASS_ROW_CELLS = 5 };
-cudaError_t launch_pp_pass(const SpatialArgs& a, int pass, cudaStream_t s);
 
 // STFT band moments of nwin windows (Sec. III-B.1), time-queue ring -> images.
 struct StftArgs {
@@ -174,12 +168,9 @@ cudaError_t launch_pca_eig(PcaArgs& a, cudaStream_t s, int* launches);
 cudaError_t launch_pca_proj(PcaArgs& a, float* out, cudaStream_t s, int* launches);
 
 // Autofocus: Tamura coefficients from per-(frame, distance) amplitude sums, and the
-// network input (2 x 2 binned log-magnitude spectrum, standardised, bfloat16)
-// from n unshifted spectra [ky][kx].
+// network input (2 x 2 binned log-magnitude spectrum, standardised, bfloat16).
 cudaError_t launch_tamura_finish(const double* acc, uint32_t count, uint32_t pixels, float* metric, cudaStream_t s);
-cudaError_t launch_af_features(const float2* spec, uint32_t n, uint32_t W, uint32_t H, void* out_bf16,
-                               cudaStream_t s);
-// The network input from the cells and per-frame sums of PASS_ROW_CELLS:
+// The network input from the cells and per-frame sums of launch_strip_cells:
 // (v - mean) / deviation per frame, rounded to bfloat16.
 cudaError_t launch_af_standardize(const float* cells, const double* sums, uint32_t sum_stride, uint32_t n,
                                   uint32_t ncell, void* out_bf16, cudaStream_t s);

@@ -1,12 +1,7 @@
-// k_spatial_pp.cu -- single passes of the spatial transform (Sec. III-B.1) for the focus
-// sweep and the network input, as persistent kernels that prefetch their next strip of 16
-// lines (8 at line length 1024) with cp.async, and the fused transform of 256 x 256 frames:
-//   P1  column FFT (length H) of 16 columns, converted in the first stage -> S1[ky][x]
-//   P2a row FFT (length W) of 16 rows ky of S1, x H^T, row IFFT -> S2[x][ky]
-//   P3t column IFFT of 16 columns x of S2, adding sum |u| and sum |u|^2 of the strip to the
-//       frame's two float64 accumulators
-//   P2f row FFT of 16 rows ky of S1 -> [ky][kx]
-//   P2c row FFT of 16 rows, its last stage forming the network's input cells
+// k_spatial_pp.cu -- the spatial transform (Sec. III-B.1) of 256 x 256 frames as one
+// persistent, warp-specialised launch for every pass of every frame of a render (the
+// kernel's own comment says how). First the block-wide FFT stages that its column passes
+// run on strips of 16 lines staged in shared memory.
 #include <cuda.h>
 
 #include "fft_dev.cuh"
@@ -17,34 +12,13 @@ namespace hv {
 
 namespace {
 
-constexpr int PP_BT = 16;
-enum { PK_P1 = PASS_COL_FFT, PK_P2A = PASS_ROW_ASP, PK_P3A = PASS_COL_IFFT, PK_P2F = PASS_ROW_FFT,
-       PK_P3T = PASS_COL_IFFT_TAMURA, PK_P2C = PASS_ROW_CELLS };
-
-// Lines per strip: 16, or 8 at L = 1024 (two buffers of 16 lines would not fit).
+// Strips of 16 lines of length L, NT threads.
 template <int L>
 struct PpCfg {
-  static constexpr int BT = L >= 1024 ? 8 : PP_BT;
-  static constexpr int NT = FftThreads<L, BT>::value;  // L for 64 <= L <= 512, 512 at 1024
-  static constexpr int LD = BT + 1;
-  static constexpr size_t BUF = size_t(L) * LD * sizeof(float2);
-  static constexpr size_t RAW = size_t(L) * BT * 2;    // one uint16 strip
-  static constexpr size_t TW = size_t(L) * sizeof(float2);
+  static constexpr int BT = 16;
+  static constexpr int NT = FftThreads<L, BT>::value;
   static_assert(L % NT == 0 && NT % BT == 0, "threads cover the elements of a line");
 };
-
-__device__ __forceinline__ void cpa8(void* s, const void* g) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(s))),
-               "l"(g)
-               : "memory");
-}
-__device__ __forceinline__ void cpa16(void* s, const void* g) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(s))),
-               "l"(g)
-               : "memory");
-}
-__device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cpa_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 // ------------------------------------------------ stage inputs and epilogues
 
@@ -92,7 +66,6 @@ struct PackedRawSrc {
 template <int LD>
 struct SmemOut {
   static constexpr bool kSyncFirst = true;
-  static constexpr bool kJFast = false;
   float2* buf;
   __device__ __forceinline__ void operator()(int b, int k, float2 v) const { buf[k * LD + b] = v; }
 };
@@ -100,97 +73,15 @@ struct SmemOut {
 // Bin k of line b straight to global memory at out[k * stride + b].
 struct GlobalOut {
   static constexpr bool kSyncFirst = false;
-  static constexpr bool kJFast = false;
   float2* out;
   uint32_t stride;
   __device__ __forceinline__ void operator()(int b, int k, float2 v) const { out[size_t(k) * stride + b] = v; }
 };
 
-// Sum of |v| and |v|^2 over the bins this thread holds (Tamura accumulation).
-struct AmpSums {
-  static constexpr bool kSyncFirst = false;
-  static constexpr bool kJFast = false;
-  float* s;  // s[0] += |v|, s[1] += |v|^2
-  __device__ __forceinline__ void operator()(int, int, float2 v) const {
-    const float q = fmaf(v.x, v.x, v.y * v.y);
-    s[0] += sqrtf(q);
-    s[1] += q;
-  }
-};
-
-// Bin k of line b times the transposed transfer function, back to the buffer.
-template <int LD>
-struct MulHtSmem {
-  static constexpr bool kSyncFirst = true;
-  static constexpr bool kJFast = false;
-  float2* buf;
-  const float2* ht;  // ht[k * H + line] of this strip's first line
-  uint32_t H;
-  __device__ __forceinline__ void operator()(int b, int k, float2 v) const {
-    buf[k * LD + b] = cmul(v, __ldg(&ht[size_t(k) * H + b]));
-  }
-};
-
-// Bin k of line b straight to global memory at out[b * stride + k], with the
-// last stage's threads laid out along the bins (consecutive lanes hold
-// consecutive bins of one line, so the stores are coalesced).
-struct RowOut {
-  static constexpr bool kSyncFirst = false;
-  static constexpr bool kJFast = true;
-  float2* out;
-  uint32_t stride;
-  __device__ __forceinline__ void operator()(int b, int k, float2 v) const { out[size_t(b) * stride + k] = v; }
-};
-
-// Network-input cells from bins handed out bin-fastest with 16 butterflies per
-// line (lanes 0-15: row b, lanes 16-31: row b + 1; bins j + 16 m): the 2 x 2 block
-// of unshifted bins (even ky, even kx) sits in lanes j, j ^ 1, j ^ 16, j ^ 17. The
-// lane with even j of the even row writes log1p(mean |F|) (DC bin as 0) at the
-// block's centred position and adds it to its running (sum v, sum v^2).
-struct CellsOut {
-  static constexpr bool kSyncFirst = false;
-  static constexpr bool kJFast = true;
-  float* cells;      // this frame's [H/2][W/2]
-  uint32_t ky0;      // unshifted row of the strip's first line
-  uint32_t W, H;
-  float* s;          // s[0] += v, s[1] += v^2
-  __device__ __forceinline__ void operator()(int b, int k, float2 v) const {
-    const uint32_t ky = ky0 + uint32_t(b);
-    float a = (ky | uint32_t(k)) ? sqrtf(fmaf(v.x, v.x, v.y * v.y)) : 0.f;
-    a += __shfl_xor_sync(0xffffffffu, a, 1);
-    a += __shfl_xor_sync(0xffffffffu, a, 16);
-    if (((threadIdx.x & 31) & 17) == 0) {  // even bin, even row
-      const float c = log1pf(0.25f * a);
-      const uint32_t r = ((ky + H / 2) & (H - 1)) >> 1, q = ((uint32_t(k) + W / 2) & (W - 1)) >> 1;
-      cells[size_t(r) * (W / 2) + q] = c;
-      s[0] += c;
-      s[1] = fmaf(c, c, s[1]);
-    }
-  }
-};
-
-// Span NS and radix R of the last stage of the pass (the BlockRadix chain).
-template <int L, int BT, int NT>
-struct LastStage {
-  static constexpr int radix(int rem) {
-    return (rem % 16 == 0 && (BT * (L / 16)) % NT == 0 && BT * (L / 16) >= NT) ? 16
-           : (rem % 8 == 0 ? 8 : (rem % 4 == 0 ? 4 : 2));
-  }
-  static constexpr int ns() {
-    int ns = 1;
-    while (ns * radix(L / ns) < L) ns *= radix(L / ns);
-    return ns;
-  }
-  static constexpr int NS = ns();
-  static constexpr int R = L / NS;
-};
-
-// One Stockham stage of span NS over the PP_BT lines (thread layout and index
+// One Stockham stage of span NS over the 16 lines (thread layout and index
 // rules of fft_dev.cuh), and recursively the rest. The first stage reads
 // through `src`, later ones the buffer; twiddles come from the shared table
 // tws[e] = exp(-2 pi i e / L). The last stage hands bin k of line b to epi.
-// With an epilogue of kJFast, the last stage maps threads bin-fastest (b = idx / NB,
-// j = idx % NB) and takes its twiddles from twl[(m - 1) NS + j] (contiguous in j).
 // Barrier between stages: the whole CTA (BAR = 0), or named barrier BAR over the
 // pass's NT threads (warp-specialised kernels whose other warps do not take part).
 template <int BAR, int NT>
@@ -199,32 +90,30 @@ __device__ __forceinline__ void pp_sync() {
   else asm volatile("bar.sync %0, %1;\n" ::"n"(BAR), "n"(NT) : "memory");
 }
 
-template <int L, int NS, int DIR, class Src, class Epi, int LDX = 0, int BAR = 0>
-__device__ __forceinline__ void pp_stages(const Src& src, float2* buf, const float2* tws, const Epi& epi,
-                                          const float2* twl = nullptr) {
+template <int L, int NS, int DIR, class Src, class Epi, int LD, int BAR>
+__device__ __forceinline__ void pp_stages(const Src& src, float2* buf, const float2* tws, const Epi& epi) {
   using C = PpCfg<L>;
-  // LDX > 0: buffer row stride other than the padded one (16 for TMA-staged strips:
-  // with lines fastest, a warp's stage accesses are two contiguous 128-byte runs)
-  constexpr int NT = C::NT, BT = C::BT, LD = LDX > 0 ? LDX : C::LD;
+  // row stride LD = 16 (TMA-staged strips): with lines fastest, a warp's stage accesses
+  // are two contiguous 128-byte runs
+  constexpr int NT = C::NT, BT = C::BT;
   constexpr int REM = L / NS;
   constexpr int R = BlockRadix<REM, L, BT, NT>::value;
   constexpr int NB = L / R;
   static_assert((BT * NB) % NT == 0, "thread count must divide the butterflies");
   constexpr int ITEMS = BT * NB / NT;
   constexpr bool LAST = NS * R == L;
-  constexpr bool JF = LAST && Epi::kJFast;
   float2 v[ITEMS][R];
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
     const int idx = threadIdx.x + it * NT;
-    const int b = JF ? idx / NB : idx % BT, j = JF ? idx % NB : idx / BT;
+    const int b = idx % BT, j = idx / BT;
 #pragma unroll
     for (int m = 0; m < R; ++m) v[it][m] = src(j + m * NB, b);
     if constexpr (NS > 1) {
       const int jm = j % NS;
 #pragma unroll
       for (int m = 1; m < R; ++m) {
-        float2 w = JF ? twl[(m - 1) * NS + jm] : tws[jm * m * (L / (NS * R))];
+        float2 w = tws[jm * m * (L / (NS * R))];
         if constexpr (DIR > 0) w.y = -w.y;
         v[it][m] = cmul(v[it][m], w);
       }
@@ -236,7 +125,7 @@ __device__ __forceinline__ void pp_stages(const Src& src, float2* buf, const flo
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
       const int idx = threadIdx.x + it * NT;
-      const int b = JF ? idx / NB : idx % BT, j = JF ? idx % NB : idx / BT;
+      const int b = idx % BT, j = idx / BT;
 #pragma unroll
       for (int m = 0; m < R; ++m) epi(b, j + m * NB, v[it][m]);
     }
@@ -252,210 +141,8 @@ __device__ __forceinline__ void pp_stages(const Src& src, float2* buf, const flo
     }
     pp_sync<BAR, NT>();
     SmemSrc<LD> s{buf};
-    pp_stages<L, NS * R, DIR, SmemSrc<LD>, Epi, LDX, BAR>(s, buf, tws, epi, twl);
+    pp_stages<L, NS * R, DIR, SmemSrc<LD>, Epi, LD, BAR>(s, buf, tws, epi);
   }
-}
-
-// ------------------------------------------------------------- prefetch
-
-// Raw strip of pass P1: rows 0..H-1, columns s0..s0+BT-1 of frame i -> raw_s[y][BT],
-// in 16-byte pieces (8-byte ones when a row segment is shorter: uint8 at BT = 8).
-template <int L>
-__device__ __forceinline__ void prefetch_raw(const SpatialArgs& a, int i, int s0, unsigned char* dst) {
-  using C = PpCfg<L>;
-  const int bpp = a.in_kind == IN_U8 ? 1 : 2;
-  const int seg = C::BT * bpp;  // bytes of one row segment: 8, 16 or 32
-  const size_t rslot = (a.raw.slot0 + uint32_t(i)) % a.raw.cap;
-  const unsigned char* src = static_cast<const unsigned char*>(a.raw.base) + (rslot * size_t(a.W) * L + s0) * bpp;
-  const size_t row = size_t(a.W) * bpp;
-  if (seg >= 16) {
-    const int pieces = seg / 16;
-    for (int e = threadIdx.x; e < L * pieces; e += C::NT) {
-      const int y = e / pieces, q = e % pieces;
-      cpa16(dst + y * seg + q * 16, src + y * row + q * 16);
-    }
-  } else {
-    for (int y = threadIdx.x; y < L; y += C::NT) cpa8(dst + y * seg, src + y * row);
-  }
-  cpa_commit();
-}
-
-// Complex strip: line b of the strip is src[b * L + t], t = 0..L-1 -> buf[t][b].
-template <int L>
-__device__ __forceinline__ void prefetch_lines(const float2* src, float2* dst) {
-  using C = PpCfg<L>;
-#pragma unroll
-  for (int t = threadIdx.x; t < L; t += C::NT)
-#pragma unroll
-    for (int b = 0; b < C::BT; ++b) cpa8(&dst[t * C::LD + b], &src[b * L + t]);
-  cpa_commit();
-}
-
-// ---------------------------------------------------------------- kernel
-
-template <int L, int PK>
-__global__ void __launch_bounds__(PpCfg<L>::NT, (L <= 256 ? 768 / L : 1))
-    k_pass_pp(SpatialArgs a, int nitems, int strip_log2) {
-  using C = PpCfg<L>;
-  extern __shared__ __align__(16) unsigned char smem[];
-  float2* tws = reinterpret_cast<float2*>(smem);
-  float2* cys = reinterpret_cast<float2*>(smem + C::TW);  // P1 Fresnel: chirp along y
-  float2* twl = cys;                                      // P2f: last-stage twiddles by (m, j)
-  unsigned char* body = smem + ((PK == PK_P1 || PK == PK_P2F || PK == PK_P2C) ? 2 * C::TW : C::TW);
-  float2* buf0 = reinterpret_cast<float2*>(body);
-  // P1: one FFT buffer and two raw staging buffers; other passes: two FFT buffers
-  float2* buf1 = reinterpret_cast<float2*>(body + C::BUF);
-  unsigned char* raw0 = body + C::BUF;
-  unsigned char* raw1 = body + C::BUF + C::RAW;
-  const int tid = threadIdx.x;
-  const int smask = (1 << strip_log2) - 1;
-  const bool fresnel = a.spatial == HV_SPATIAL_FRESNEL;
-  const bool u8 = a.in_kind == IN_U8;
-  // the pass length: P1 and P3a run along y (length H), P2a and P2f along x
-  const float2* twg = (PK == PK_P1 || PK == PK_P3A || PK == PK_P3T) ? a.tw_h : a.tw_w;
-  for (int e = tid; e < L; e += C::NT) {
-    tws[e] = __ldg(&twg[e]);
-    if (PK == PK_P1 && fresnel) cys[e] = __ldg(&a.chirp_y[e]);
-  }
-  if constexpr (PK == PK_P2F || PK == PK_P2C) {
-    using LS = LastStage<L, C::BT, C::NT>;
-    for (int e = tid; e < (LS::R - 1) * LS::NS; e += C::NT) {
-      const int m = e / LS::NS + 1, jm = e % LS::NS;
-      twl[e] = __ldg(&twg[jm * m * (L / (LS::NS * LS::R))]);
-    }
-  }
-  // lines per frame of the other axis: W columns (P1, P3a) or H rows (P2a, P2f)
-  const uint32_t LO = (PK == PK_P1 || PK == PK_P3A || PK == PK_P3T) ? a.W : a.H;
-
-  auto issue = [&](int it, int cur) {
-    const int i = it >> strip_log2, s0 = (it & smask) * C::BT;
-    if constexpr (PK == PK_P1) {
-      prefetch_raw<L>(a, i, s0, cur == 0 ? raw0 : raw1);
-    } else {
-      const float2* base = (PK == PK_P3A || PK == PK_P3T) ? a.scratch2 : a.scratch1;
-      prefetch_lines<L>(base + size_t(i) * L * LO + size_t(s0) * L, cur == 0 ? buf0 : buf1);
-    }
-  };
-
-  int item = blockIdx.x;
-  if (item < nitems) issue(item, 0);
-  for (int k = 0; item < nitems; ++k, item += gridDim.x) {
-    const int cur = k & 1;
-    const int i = item >> strip_log2, s0 = (item & smask) * C::BT;
-    cpa_wait_all();
-    __syncthreads();  // this item's input resident; the other buffer is free
-    const int nxt = item + gridDim.x;
-    if (nxt < nitems) issue(nxt, cur ^ 1);
-    if (PK != PK_P1 && a.discard_inputs) {
-      // the strip's intermediate is dead once staged: drop its L2 lines unwritten
-      const float2* base = (PK == PK_P3A || PK == PK_P3T) ? a.scratch2 : a.scratch1;
-      const char* st = reinterpret_cast<const char*>(base + size_t(i) * L * LO + size_t(s0) * L);
-      for (int e = tid; e < C::BT * L * 8 / 128; e += C::NT)
-        asm volatile("discard.global.L2 [%0], 128;\n" ::"l"(st + size_t(e) * 128) : "memory");
-    }
-    if constexpr (PK == PK_P1) {
-      // S1[ky][x]: bin ky of column s0 + b at s1[ky * W + s0 + b]
-      const GlobalOut out{a.scratch1 + size_t(i) * a.H * a.W + s0, a.W};
-      const unsigned char* raw = cur == 0 ? raw0 : raw1;
-      const int b = tid % C::BT;
-      if (fresnel) {
-        const float2 cx = __ldg(&a.chirp_x[s0 + b]);
-        if (u8) pp_stages<L, 1, -1>(RawSrc<true, true, C::BT>{raw, cys, cx}, buf0, tws, out);
-        else pp_stages<L, 1, -1>(RawSrc<false, true, C::BT>{raw, cys, cx}, buf0, tws, out);
-      } else {
-        if (u8) pp_stages<L, 1, -1>(RawSrc<true, false, C::BT>{raw, cys, make_float2(0.f, 0.f)}, buf0, tws, out);
-        else pp_stages<L, 1, -1>(RawSrc<false, false, C::BT>{raw, cys, make_float2(0.f, 0.f)}, buf0, tws, out);
-      }
-    } else if constexpr (PK == PK_P2A) {
-      float2* buf = cur == 0 ? buf0 : buf1;
-      const SmemSrc<C::LD> src{buf};
-      pp_stages<L, 1, -1>(src, buf, tws, MulHtSmem<C::LD>{buf, a.asp_ht + s0, a.H});
-      __syncthreads();
-      // S2[x][ky]: sample x of row s0 + b at s2[x * H + s0 + b]
-      pp_stages<L, 1, +1>(src, buf, tws, GlobalOut{a.scratch2 + size_t(i) * a.H * a.W + s0, a.H});
-    } else if constexpr (PK == PK_P3A) {
-      float2* buf = cur == 0 ? buf0 : buf1;
-      const size_t tslot = (a.tq.slot0 + uint32_t(i)) % a.tq.cap;
-      // time queue [y][x]: sample y of column s0 + b at tq[y * W + s0 + b]
-      pp_stages<L, 1, +1>(SmemSrc<C::LD>{buf}, buf, tws,
-                          GlobalOut{static_cast<float2*>(a.tq.base) + tslot * size_t(a.W) * a.H + s0, a.W});
-    } else if constexpr (PK == PK_P3T) {
-      float2* buf = cur == 0 ? buf0 : buf1;
-      float acc[2] = {0.f, 0.f};
-      pp_stages<L, 1, +1>(SmemSrc<C::LD>{buf}, buf, tws, AmpSums{acc});
-      // block sums: warp shuffles, then one partial per warp in shared memory
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
-        acc[1] += __shfl_xor_sync(0xffffffffu, acc[1], o);
-      }
-      __shared__ float red[2][C::NT / 32];
-      if ((tid & 31) == 0) {
-        red[0][tid >> 5] = acc[0];
-        red[1][tid >> 5] = acc[1];
-      }
-      __syncthreads();
-      if (tid < 2) {
-        float t = 0.f;
-#pragma unroll
-        for (int w = 0; w < C::NT / 32; ++w) t += red[tid][w];
-        atomicAdd(&a.tam_acc[size_t(i) * a.tam_stride + tid], double(t));
-      }
-    } else if constexpr (PK == PK_P2C) {
-      float2* buf = cur == 0 ? buf0 : buf1;
-      float acc[2] = {0.f, 0.f};
-      pp_stages<L, 1, -1>(SmemSrc<C::LD>{buf}, buf, tws,
-                          CellsOut{a.cells + size_t(i) * (a.H / 2) * (a.W / 2), uint32_t(s0), a.W, a.H, acc}, twl);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
-        acc[1] += __shfl_xor_sync(0xffffffffu, acc[1], o);
-      }
-      __shared__ float redc[2][C::NT / 32];
-      if ((tid & 31) == 0) {
-        redc[0][tid >> 5] = acc[0];
-        redc[1][tid >> 5] = acc[1];
-      }
-      __syncthreads();
-      if (tid < 2) {
-        double t = 0.0;
-#pragma unroll
-        for (int w = 0; w < C::NT / 32; ++w) t += redc[tid][w];
-        atomicAdd(&a.tam_acc[size_t(i) * a.tam_stride + tid], t);
-      }
-    } else {
-      float2* buf = cur == 0 ? buf0 : buf1;
-      // time queue [ky][kx]: bin kx of row s0 + b, stored from the registers of the
-      // last stage (threads along kx there)
-      const size_t tslot = (a.tq.slot0 + uint32_t(i)) % a.tq.cap;
-      float2* out = static_cast<float2*>(a.tq.base) + tslot * size_t(a.H) * a.W + size_t(s0) * a.W;
-      pp_stages<L, 1, -1>(SmemSrc<C::LD>{buf}, buf, tws, RowOut{out, a.W}, twl);
-    }
-  }
-  cpa_wait_all();
-}
-
-template <int L, int PK>
-static cudaError_t launch_pp(const SpatialArgs& a, uint32_t lines, cudaStream_t s) {
-  using C = PpCfg<L>;
-  const size_t smem = PK == PK_P1 ? 2 * C::TW + C::BUF + 2 * C::RAW
-                                   : ((PK == PK_P2F || PK == PK_P2C) ? 2 * C::TW : C::TW) + 2 * C::BUF;
-  auto kern = k_pass_pp<L, PK>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-  if (e != cudaSuccess) return e;
-  int per_sm = 0, dev = 0, nsm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, C::NT, smem);
-  if (e != cudaSuccess) return e;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  int strip_log2 = 0;
-  while ((uint32_t(C::BT) << strip_log2) < lines) ++strip_log2;
-  const int nitems = int(a.n) << strip_log2;
-  int grid = per_sm * nsm;
-  if (grid > nitems) grid = nitems;
-  if (grid < 1) grid = 1;
-  kern<<<grid, C::NT, smem, s>>>(a, nitems, strip_log2);
-  return cudaGetLastError();
 }
 
 constexpr int RW_L = 256;  // side of the fused transform's frames
@@ -479,27 +166,11 @@ __device__ __forceinline__ bool rw_wait(uint32_t mbar, uint32_t parity) {
   }
 }
 
-template <int PK>
-static cudaError_t pass_by_len(const SpatialArgs& a, cudaStream_t s) {
-  // pass length and number of lines: columns (length H, W lines) or rows (length W, H lines)
-  const bool cols = PK == PK_P1 || PK == PK_P3A || PK == PK_P3T;
-  const uint32_t L = cols ? a.H : a.W, lines = cols ? a.W : a.H;
-  switch (L) {
-    case 64: return launch_pp<64, PK>(a, lines, s);
-    case 128: return launch_pp<128, PK>(a, lines, s);
-    case 256: return launch_pp<256, PK>(a, lines, s);
-    case 512: return launch_pp<512, PK>(a, lines, s);
-    case 1024: return launch_pp<1024, PK>(a, lines, s);
-  }
-  return cudaErrorInvalidValue;
-}
-
 // ------------------------------------------- fused transform, 256 x 256 frames
 //
-// Every pass of every frame of a launch in one persistent kernel. The passes
-// above each run as a launch of their own over a chunk of frames, so their
-// intermediates (S1, S2: 512 KB per frame) go through HBM once written and once
-// read. Here work items come in a fixed global order from an atomic ticket
+// Every pass of every frame of a launch in one persistent kernel. As launches of their
+// own over a chunk of frames, the passes take their intermediates (S1, S2: up to 512 KB
+// per frame) through HBM, once written and once read. Here work items come in a fixed global order from an atomic ticket
 // counter: row r of the order holds the column items of frame r and the items of
 // each later pass of frame r - (the lags up to that pass). A Fresnel frame takes two passes of 16
 // items: 16 chirped (complex) columns per column item, 16 rows per row item,
@@ -579,7 +250,6 @@ constexpr uint32_t FZ_STOP = 0xffffffffu;
 // Bin k of line b to global memory at out[k * stride + b] with a streaming store.
 struct GlobalOutCs {
   static constexpr bool kSyncFirst = false;
-  static constexpr bool kJFast = false;
   float2* out;
   uint32_t stride;
   __device__ __forceinline__ void operator()(int b, int k, float2 v) const { __stcs(&out[size_t(k) * stride + b], v); }
@@ -958,28 +628,6 @@ __global__ void __launch_bounds__(FZ_THREADS, 3)
 }
 
 }  // namespace
-
-cudaError_t launch_pp_pass(const SpatialArgs& a, int pass, cudaStream_t s) {
-  if (a.n == 0) return cudaSuccess;
-  if (!spatial_pp_supported(a)) return cudaErrorInvalidValue;
-  switch (pass) {
-    case PASS_COL_FFT: return pass_by_len<PK_P1>(a, s);
-    case PASS_ROW_ASP: return pass_by_len<PK_P2A>(a, s);
-    case PASS_COL_IFFT: return pass_by_len<PK_P3A>(a, s);
-    case PASS_ROW_FFT: return pass_by_len<PK_P2F>(a, s);
-    case PASS_COL_IFFT_TAMURA: return pass_by_len<PK_P3T>(a, s);
-    case PASS_ROW_CELLS:
-      // the cell epilogue pairs rows and bins across lanes: 16 butterflies per line in the last stage
-      if (a.W > 256 || a.H > 1024) return cudaErrorInvalidValue;
-      return pass_by_len<PK_P2C>(a, s);
-  }
-  return cudaErrorInvalidValue;
-}
-
-bool spatial_pp_supported(const SpatialArgs& a) {
-  auto ok = [](uint32_t v) { return v >= 64 && v <= 1024; };  // two strip buffers must fit
-  return ok(a.W) && ok(a.H) && (a.spatial == HV_SPATIAL_ASP || a.spatial == HV_SPATIAL_FRESNEL);
-}
 
 bool spatial_fused_supported(const SpatialArgs& a) {
   return a.W == RW_L && a.H == RW_L && (a.spatial == HV_SPATIAL_ASP || a.spatial == HV_SPATIAL_FRESNEL) &&

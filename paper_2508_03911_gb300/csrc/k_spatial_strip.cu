@@ -388,6 +388,218 @@ __global__ void __launch_bounds__(RowCfg<L>::NT, (L >= 512 ? 4 : 6)) k_strip_row
   }
 }
 
+// ---------------------------------------------------------------- focus sweep
+//
+// The sweep needs IFFT2(W H_z) of each hologram for every distance z, W its spectrum. W is
+// formed once (column FFT, then the row FFT in place on S1 rows 0 .. H / 2); per
+// (distance, hologram) only the inverse row and column FFTs run, and many distances share
+// a launch (per distance the forward row FFT was repeated over all H rows: 17.8 + 10.4 us
+// a distance for 64 holograms of 256 x 256 in 130 launches; 7.7 + 12.5 now in 34).
+
+// Row FFT of S1 rows in place (a last warp with a row too many repeats the last row).
+template <int L>
+__global__ void __launch_bounds__(RowCfg<L>::NT, (L >= 512 ? 4 : 6)) k_strip_rows_fwd(SpatialArgs a, uint32_t nrows) {
+  using C = RowCfg<L>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  float2* tw = reinterpret_cast<float2*>(smem);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, jl = lane % C::LP, sub = lane / C::LP;
+  float2* rowp = tw + C::NTW + (warp * C::RPW + sub) * C::RS;
+  load_stage_twiddles<C::R1, C::NTW, C::NT>(tw, a.tw_w);
+  __syncthreads();
+  for (uint32_t r0 = (blockIdx.x * C::NW + warp) * C::RPW; r0 < nrows; r0 += gridDim.x * C::NW * C::RPW) {
+    float2* at = a.scratch1 + size_t(r0 + sub < nrows ? r0 + sub : nrows - 1) * L + jl;
+    float2 v[C::R1];
+#pragma unroll
+    for (int m = 0; m < C::R1; ++m) v[m] = at[C::LP * m];
+    strip_row_fft<L, -1>(v, rowp, tw, jl);
+#pragma unroll
+    for (int m = 0; m < C::R1; ++m) at[C::LP * m] = v[m];
+  }
+}
+
+// Rows of nz distances: row (z, i, ky) of nz n (H / 2 + 1): W of hologram i times H_z, inverse
+// row FFT -> S2 rows ky and H - ky of image z n + i (the mirror as in k_strip_rows_asp).
+// h: [nz][H / 2 + 1][W].
+template <int L>
+__global__ void __launch_bounds__(RowCfg<L>::NT, (L >= 512 ? 3 : 5)) k_strip_rows_inv(SpatialArgs a, const float2* h,
+                                                                                     uint32_t nrows) {
+  using C = RowCfg<L>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  float2* tw = reinterpret_cast<float2*>(smem);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, jl = lane % C::LP, sub = lane / C::LP;
+  float2* rowp = tw + C::NTW + (warp * C::RPW + sub) * C::RS;
+  load_stage_twiddles<C::R1, C::NTW, C::NT>(tw, a.tw_w);
+  __syncthreads();
+  const uint32_t H = a.H, HR = H / 2 + 1;
+  for (uint32_t r0 = (blockIdx.x * C::NW + warp) * C::RPW; r0 < nrows; r0 += gridDim.x * C::NW * C::RPW) {
+    const uint32_t row = r0 + sub < nrows ? r0 + sub : nrows - 1;
+    const uint32_t image = row / HR, ky = row % HR, z = image / a.n, i = image % a.n;
+    const float2* in = a.scratch1 + (size_t(i) * HR + ky) * L + jl;
+    const float2* hz = h + (size_t(z) * HR + ky) * L + jl;
+    float2* out = a.scratch2 + size_t(image) * H * L + jl;
+    float2 u[C::R1];
+#pragma unroll
+    for (int m = 0; m < C::R1; ++m) u[m] = cmul(in[C::LP * m], __ldg(&hz[C::LP * m]));
+    strip_row_fft<L, +1>(u, rowp, tw, jl);
+#pragma unroll
+    for (int m = 0; m < C::R1; ++m) out[size_t(ky) * L + C::LP * m] = u[m];
+#pragma unroll
+    for (int m = 0; m < C::R1; ++m) {
+      // both read again (L1 hits) rather than kept across the first inverse FFT
+      float2 v, w;
+      asm volatile("ld.global.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "l"(&in[C::LP * m]) : "memory");
+      asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];\n" : "=f"(w.x), "=f"(w.y) : "l"(&hz[C::LP * m]) : "memory");
+      w.y = -w.y;
+      u[m] = cmul(v, w);
+    }
+    strip_row_fft<L, +1>(u, rowp, tw, jl);
+#pragma unroll
+    for (int m = 0; m < C::R1; ++m)
+      out[size_t((H - ky) & (H - 1)) * L + C::LP * m] = make_float2(u[m].x, -u[m].y);
+  }
+}
+
+// Column IFFT of strips of S2; sum |u| and sum |u|^2 of image z n + i added to the float64
+// pair z of hologram i at tam_acc + i tam_stride + 2 z.
+template <int L>
+__global__ void __launch_bounds__(ColCfg<L>::NT, (L == 1024 ? 2 : 4)) k_strip_icols_sums(SpatialArgs a, uint32_t nitems,
+                                                                                    uint32_t strips) {
+  using C = ColCfg<L>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ float red[2][C::NT / 32];
+  float2* buf = reinterpret_cast<float2*>(smem);
+  float2* tw = buf + C::ROWS * C::BT;
+  load_stage_twiddles<C::R1, C::NTW, C::NT>(tw, a.tw_h);
+  const int b = threadIdx.x % C::BT, t = threadIdx.x / C::BT;
+  const uint32_t W = a.W;
+  for (uint32_t item = blockIdx.x; item < nitems; item += gridDim.x) {
+    const uint32_t image = item / strips, s = item % strips;
+    const float2* in = a.scratch2 + size_t(image) * L * W + size_t(s) * C::BT + b;
+    float2 v[C::I1][C::R1];
+#pragma unroll
+    for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+      for (int m = 0; m < C::R1; ++m) v[it][m] = in[size_t(t + C::NJ * it + (L / C::R1) * m) * W];
+    col_stage1<L, +1>(v, buf, t, b);
+    float2 u[C::I2][C::R2];
+    col_stage2<L, +1>(u, buf, tw, t, b);
+    float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+    for (int it = 0; it < C::I2; ++it)
+#pragma unroll
+      for (int m = 0; m < C::R2; ++m) {
+        const float q = fmaf(u[it][m].x, u[it][m].x, u[it][m].y * u[it][m].y);
+        s0 += sqrtf(q);
+        s1 += q;
+      }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+    }
+    // the barriers of the next item's first stage come before its sums are written here
+    if ((threadIdx.x & 31) == 0) {
+      red[0][threadIdx.x >> 5] = s0;
+      red[1][threadIdx.x >> 5] = s1;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+      float q = 0.f;
+#pragma unroll
+      for (int w = 0; w < C::NT / 32; ++w) q += red[threadIdx.x][w];
+      atomicAdd(&a.tam_acc[size_t(image % a.n) * a.tam_stride + 2 * (image / a.n) + threadIdx.x], double(q));
+    }
+  }
+}
+
+// -------------------------------------------------------------- network input
+//
+// Cells of the autofocus network's input: the centred spectrum's 2 x 2 blocks as
+// log1p(mean |F|) (DC bin as 0). |F| of a real frame is symmetric, |F(-k)| = |F(k)|, so S1
+// rows 0 .. H / 2 are enough: a CTA row-transforms rows y0 .. y0 + SR, keeps their |F| in
+// shared memory, and forms the blocks of rows (2r, 2r + 1), and of rows (H - e, H - e + 1)
+// from rows e and e - 1 with the columns mirrored, e even (over all H rows the column and
+// row passes took 64 + 144 us for 512 holograms of 256 x 256; 37 + 71 now).
+template <int L>
+struct CellCfg {
+  static constexpr int SR = L <= 256 ? 32 : 16;  // rows of a strip (one more is transformed)
+  static constexpr size_t SMEM = RowCfg<L>::SMEM + size_t(SR + 1) * L * sizeof(float);
+};
+
+template <int L>
+__global__ void __launch_bounds__(RowCfg<L>::NT) k_strip_cells(SpatialArgs a, uint32_t nitems, uint32_t strips) {
+  using C = RowCfg<L>;
+  constexpr int SR = CellCfg<L>::SR;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ float red[2][C::NW];
+  float2* tw = reinterpret_cast<float2*>(smem);
+  float* mag = reinterpret_cast<float*>(tw + C::NTW + C::NW * C::RPW * C::RS);  // [SR + 1][L]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, jl = lane % C::LP, sub = lane / C::LP;
+  float2* rowp = tw + C::NTW + (warp * C::RPW + sub) * C::RS;
+  load_stage_twiddles<C::R1, C::NTW, C::NT>(tw, a.tw_w);
+  const int H = int(a.H);
+  for (uint32_t item = blockIdx.x; item < nitems; item += gridDim.x) {
+    const uint32_t i = item / strips;
+    const int y0 = int(item % strips) * SR;
+    __syncthreads();  // twiddles loaded; the previous strip's cells formed
+    for (int r0 = warp * C::RPW; r0 <= SR; r0 += C::NW * C::RPW) {
+      const int r = r0 + sub <= SR ? r0 + sub : SR;  // a row too many repeats the last
+      const float2* in = a.scratch1 + (size_t(i) * (H / 2 + 1) + y0 + r) * L + jl;
+      float2 v[C::R1];
+#pragma unroll
+      for (int m = 0; m < C::R1; ++m) v[m] = in[C::LP * m];
+      strip_row_fft<L, -1>(v, rowp, tw, jl);
+#pragma unroll
+      for (int m = 0; m < C::R1; ++m)
+        mag[r * L + jl + C::LP * m] = sqrtf(fmaf(v[m].x, v[m].x, v[m].y * v[m].y));
+    }
+    __syncthreads();
+    if (y0 == 0 && threadIdx.x == 0) mag[0] = 0.f;  // DC bin
+    __syncthreads();
+    float* cells = a.cells + size_t(i) * (H / 2) * (L / 2);
+    float s0 = 0.f, s1 = 0.f;
+    // SR / 2 block rows of each kind, L / 2 cells each
+    for (int e = threadIdx.x; e < SR * (L / 2); e += C::NT) {
+      const int q = e % (L / 2), p = e / (L / 2), k = p >> 1;
+      int ky, ra, rb, xa, xb;
+      if (p & 1) {  // rows H - ke, H - ke + 1 from rows ke and ke - 1, ke = y0 + 2 k + 2
+        ra = 2 * k + 2;
+        rb = 2 * k + 1;
+        ky = H - (y0 + ra);
+        xa = (L - 2 * q) & (L - 1);
+        xb = L - 2 * q - 1;
+      } else {
+        ra = 2 * k;
+        rb = 2 * k + 1;
+        ky = y0 + ra;
+        xa = 2 * q;
+        xb = 2 * q + 1;
+      }
+      const float m = ((mag[ra * L + xa] + mag[ra * L + xb]) + mag[rb * L + xa]) + mag[rb * L + xb];
+      const float c = log1pf(0.25f * m);
+      cells[size_t(((ky + H / 2) & (H - 1)) >> 1) * (L / 2) + (((2 * q + L / 2) & (L - 1)) >> 1)] = c;
+      s0 += c;
+      s1 = fmaf(c, c, s1);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+    }
+    if (lane == 0) {
+      red[0][warp] = s0;
+      red[1][warp] = s1;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+      double t = 0.0;
+#pragma unroll
+      for (int w = 0; w < C::NW; ++w) t += red[threadIdx.x][w];
+      atomicAdd(&a.tam_acc[size_t(i) * a.tam_stride + threadIdx.x], t);
+    }
+  }
+}
+
 // Persistent grid: every CTA that fits at once, no more than the items.
 template <class K, class... Args>
 cudaError_t launch_resident(K kern, int nt, size_t smem, uint32_t ctas, cudaStream_t s, Args... args) {
@@ -439,6 +651,35 @@ cudaError_t rows(const SpatialArgs& a, cudaStream_t s) {
     default: e = cudaErrorInvalidValue;  \
   }
 
+template <int L>
+cudaError_t rows_fwd(const SpatialArgs& a, cudaStream_t s) {
+  using C = RowCfg<L>;
+  constexpr uint32_t per = C::NW * C::RPW;
+  const uint32_t nrows = a.n * (a.H / 2 + 1);
+  return launch_resident(k_strip_rows_fwd<L>, C::NT, C::SMEM, (nrows + per - 1) / per, s, a, nrows);
+}
+
+template <int L>
+cudaError_t rows_inv(const SpatialArgs& a, const float2* h, uint32_t nz, cudaStream_t s) {
+  using C = RowCfg<L>;
+  constexpr uint32_t per = C::NW * C::RPW;
+  const uint32_t nrows = nz * a.n * (a.H / 2 + 1);
+  return launch_resident(k_strip_rows_inv<L>, C::NT, C::SMEM, (nrows + per - 1) / per, s, a, h, nrows);
+}
+
+template <int L>
+cudaError_t icols_sums(const SpatialArgs& a, uint32_t nz, cudaStream_t s) {
+  using C = ColCfg<L>;
+  const uint32_t strips = a.W / C::BT, items = strips * a.n * nz;
+  return launch_resident(k_strip_icols_sums<L>, C::NT, C::SMEM, items, s, a, items, strips);
+}
+
+template <int L>
+cudaError_t cells(const SpatialArgs& a, cudaStream_t s) {
+  const uint32_t strips = a.H / (2 * CellCfg<L>::SR), items = strips * a.n;
+  return launch_resident(k_strip_cells<L>, RowCfg<L>::NT, CellCfg<L>::SMEM, items, s, a, items, strips);
+}
+
 }  // namespace
 
 bool spatial_strip_supported(const SpatialArgs& a) {
@@ -462,6 +703,35 @@ cudaError_t launch_spatial_strip(const SpatialArgs& a, cudaStream_t s, int* laun
   if (e != cudaSuccess || !asp) return e;
   HV_BY_SIDE(a.H, HV_ICOLS)
   ++*launches;
+  return e;
+}
+
+cudaError_t launch_strip_spectrum(const SpatialArgs& a, cudaStream_t s) {
+  cudaError_t e;
+#define HV_COLS_ASP(L) cols<L, true>(a, s)
+#define HV_ROWS_FWD(L) rows_fwd<L>(a, s)
+  HV_BY_SIDE(a.H, HV_COLS_ASP)
+  if (e != cudaSuccess) return e;
+  HV_BY_SIDE(a.W, HV_ROWS_FWD)
+  return e;
+}
+
+cudaError_t launch_strip_sweep(const SpatialArgs& a, const float2* h, uint32_t nz, cudaStream_t s) {
+  cudaError_t e;
+#define HV_ROWS_INV(L) rows_inv<L>(a, h, nz, s)
+#define HV_ICOLS_SUMS(L) icols_sums<L>(a, nz, s)
+  HV_BY_SIDE(a.W, HV_ROWS_INV)
+  if (e != cudaSuccess) return e;
+  HV_BY_SIDE(a.H, HV_ICOLS_SUMS)
+  return e;
+}
+
+cudaError_t launch_strip_cells(const SpatialArgs& a, cudaStream_t s) {
+  cudaError_t e;
+#define HV_CELLS(L) cells<L>(a, s)
+  HV_BY_SIDE(a.H, HV_COLS_ASP)
+  if (e != cudaSuccess) return e;
+  HV_BY_SIDE(a.W, HV_CELLS)
   return e;
 }
 

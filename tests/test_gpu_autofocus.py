@@ -59,6 +59,19 @@ def test_sweep_other_sizes(H, W, bits):
         assert np.max(np.abs(got[i] - ref) / ref) <= TAMURA_TOL
 
 
+@pytest.mark.parametrize("H,W,n,nz", [(64, 64, 65, 3), (512, 64, 2, 5), (64, 512, 1, 70), (256, 1024, 1, 2),
+                                      (1024, 64, 1, 2)])
+def test_sweep_across_launches(H, W, n, nz):
+    """More holograms than are held at once, more distances than share a launch, lengths
+    512 and 1024 along either axis, a last warp with fewer rows than it holds."""
+    fr = synth.random_frames(n, H, W, 12, seed=H + W + n)
+    zs = np.linspace(0.1, 0.6, nz)
+    got = gpu_sweep(fr, zs)
+    for i in sorted({0, n // 2, n - 1}):
+        ref = A.focus_sweep(fr[i], 852e-9, 20e-6, 20e-6, zs)
+        assert np.max(np.abs(got[i] - ref) / ref) <= TAMURA_TOL
+
+
 def gpu_features(frames):
     import torch
     n, H, W = frames.shape
@@ -72,10 +85,11 @@ def gpu_features(frames):
         r.close()
 
 
-@pytest.mark.parametrize("H,W,bits", [(256, 256, 16), (64, 128, 8), (128, 64, 16), (64, 512, 8)])
+@pytest.mark.parametrize("H,W,bits", [(256, 256, 16), (64, 128, 8), (128, 64, 16), (64, 512, 8), (512, 1024, 16),
+                                      (1024, 256, 8)])
 def test_features_match_oracle(H, W, bits):
-    """Widths up to 256 form the binned cells in the row pass's epilogue (lanes
-    pair bins and rows); 512 stores the spectra and bins them in a second kernel."""
+    """The cells of the half spectrum's rows and of their mirrors, strips of 32 rows (16 from
+    width 512 on)."""
     if H == 256:
         fr, _ = synth.autofocus_set(5, N=256, seed=1007)
     else:
