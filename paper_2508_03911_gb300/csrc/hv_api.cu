@@ -600,8 +600,9 @@ bool cluster_ok(const hv_handle* h) {
 }
 
 // Spatial transform of frames r0 .. r1 - 1, whose raw frames are at `raw` (frame
-// r0 at slot raw.slot0); the time queue slots follow the frame numbers.
-hv_status propagate_run(hv_handle* h, uint64_t r0, uint64_t r1, RingRef raw) {
+// r0 at slot raw.slot0). The fields go to the time queue, whose slots follow the frame
+// numbers, or to `out`, where frame out0 is slot 0.
+hv_status propagate_run(hv_handle* h, uint64_t r0, uint64_t r1, RingRef raw, float2* out, uint64_t out0) {
   // the cluster kernel needs no scratch, the fused transform keeps its intermediates
   // in rings: one persistent launch for all frames
   const bool whole = (h->sp_cluster && cluster_ok(h)) || h->sp_fused;
@@ -616,7 +617,7 @@ hv_status propagate_run(hv_handle* h, uint64_t r0, uint64_t r1, RingRef raw) {
     sa.H = h->H;
     sa.n = n;
     sa.raw = RingRef{raw.base, raw.cap, uint32_t((raw.slot0 + (a - r0)) % raw.cap)};
-    sa.tq = RingRef{h->tq, h->Q, uint32_t(a % h->Q)};
+    sa.tq = out ? RingRef{out + (a - out0) * h->W * h->H, n, 0} : RingRef{h->tq, h->Q, uint32_t(a % h->Q)};
     sa.scratch1 = h->s1;
     sa.scratch2 = h->s2;
     sa.tw_w = h->tw + tw_offset(h->W);
@@ -645,8 +646,9 @@ hv_status propagate_run(hv_handle* h, uint64_t r0, uint64_t r1, RingRef raw) {
 
 // Spatial transform of frames f0 .. f1 - 1: runs of frames read in place from the
 // caller's memory (HV_MEM_DEVICE_ASYNC) and runs in the input ring, one after the
-// other. ring_only: the input ring whatever its contents (the autotuner's timing).
-hv_status propagate(hv_handle* h, uint64_t f0, uint64_t f1, bool ring_only = false) {
+// other. ring_only: the input ring whatever its contents (the autotuner's timing). out:
+// where the fields go instead of the time queue, frame f0 first.
+hv_status propagate(hv_handle* h, uint64_t f0, uint64_t f1, bool ring_only = false, float2* out = nullptr) {
   uint64_t a = f0;
   while (a < f1) {
     uint64_t end = f1;
@@ -663,7 +665,7 @@ hv_status propagate(hv_handle* h, uint64_t f0, uint64_t f1, bool ring_only = fal
         break;
       }
     }
-    hv_status s = propagate_run(h, a, end, raw);
+    hv_status s = propagate_run(h, a, end, raw, out, f0);
     if (s != HV_OK) return s;
     a = end;
   }
@@ -905,17 +907,26 @@ hv_status wait_slots_free(hv_handle* h, uint32_t n) {
   return HV_OK;
 }
 
-// Copies n frames from device memory into the input ring on the handle's stream
-// (one copy, or two where the ring wraps). The caller has checked the capacity.
-hv_status enqueue_push_device(hv_handle* h, const void* frames, uint32_t n) {
+// Copies frames from .. n - 1 of the n frames pushed at frame number `first` from device
+// memory into the input ring on the handle's stream (one copy, or two where the ring
+// wraps). The caller has checked the capacity.
+hv_status enqueue_frames(hv_handle* h, const void* frames, uint32_t from, uint64_t first, uint32_t n) {
   const hv_params& p = h->pending ? h->pend : h->cur;
   const size_t fb = size_t(p.width) * p.height * (h->bits / 8);
-  const uint32_t slot = uint32_t(h->pushed % h->cap);
-  const uint32_t n1 = std::min(n, h->cap - slot);
-  const char* src = static_cast<const char*>(frames);
+  const uint32_t slot = uint32_t((first + from) % h->cap);
+  const uint32_t n1 = std::min(n - from, h->cap - slot);
+  const char* src = static_cast<const char*>(frames) + from * fb;
   char* ring = static_cast<char*>(h->raw);
   HV_CU(h, cudaMemcpyAsync(ring + slot * fb, src, n1 * fb, cudaMemcpyDeviceToDevice, h->stream));
-  if (n1 < n) HV_CU(h, cudaMemcpyAsync(ring, src + n1 * fb, (n - n1) * fb, cudaMemcpyDeviceToDevice, h->stream));
+  if (n1 < n - from)
+    HV_CU(h, cudaMemcpyAsync(ring, src + n1 * fb, (n - from - n1) * fb, cudaMemcpyDeviceToDevice, h->stream));
+  return HV_OK;
+}
+
+// A device push: all n frames.
+hv_status enqueue_push_device(hv_handle* h, const void* frames, uint32_t n) {
+  const hv_status s = enqueue_frames(h, frames, 0, h->pushed, n);
+  if (s != HV_OK) return s;
   h->pushed += n;
   h->st.frames_pushed += n;
   return HV_OK;
@@ -940,6 +951,11 @@ hv_status enqueue_windows(hv_handle* h, float* dst, uint32_t nw, bool capturing)
   const uint32_t T = h->T, S = h->S;
   hv_status s = HV_OK;
   const uint64_t prop_before = h->st.frames_propagated;
+  // propagated fields without temporal analysis go straight to the output (a copy out of
+  // the time queue took 83 of 384 us for 96 frames of 512 x 512); every frame of the
+  // windows is new, as T = S = 1. The kernels store 8-byte values: an output at an odd
+  // float is copied
+  const bool direct = none && (reinterpret_cast<uintptr_t>(dst) & 7) == 0 && h->propagated <= h->next_win;
   // long PCA windows, several in this render: window by window, each window's
   // spatial chunk and covariance on the handle's stream while the previous window's
   // eigensolver runs on eig_stream (below)
@@ -954,7 +970,7 @@ hv_status enqueue_windows(hv_handle* h, float* dst, uint32_t nw, bool capturing)
     const uint64_t lo = std::max(h->next_win, h->propagated);
     const uint64_t hi = h->next_win + uint64_t(nw - 1) * S + T;
     if (lo < hi) {
-      s = propagate(h, lo, hi);
+      s = propagate(h, lo, hi, false, direct ? reinterpret_cast<float2*>(dst) : nullptr);
       if (s != HV_OK) return s;
       h->propagated = hi;
     }
@@ -994,7 +1010,9 @@ hv_status enqueue_windows(hv_handle* h, float* dst, uint32_t nw, bool capturing)
     // without a convolution the STFT epilogue writes the image ring and its sums
     pa.fused = !none && h->cur.temporal != HV_TEMPORAL_PCA && pa.K == 0 ? 1 : 0;
   }
-  if (none) {
+  if (direct) {
+    e = cudaSuccess;
+  } else if (none) {
     e = launch_copy_frames(tq, nw, h->W * h->H, dst, h->stream, &launches);
   } else if (pca_pipe) {
     // pipelined long windows: spatial chunk(w), covariance(w) and projection(w - 1)
@@ -1740,11 +1758,28 @@ hv_status hv_render_group(hv_group* g, const void* const* frames, const uint32_t
         break;
       }
     }
+    // the batch's windows read its frames where they are; only frames that a later
+    // window can still read are copied into the input queue (all of them took 1.0 of
+    // 15.8 ms for 2 GB of frames). The fused transform's tensor map wants 16-byte
+    // alignment: other frames are copied first
     const uint32_t nf = n_frames ? n_frames[i] : 0;
-    if (nf) s = enqueue_push_device(h, frames[i], nf);
+    const bool in_place = nf && (reinterpret_cast<uintptr_t>(frames[i]) & 15) == 0;
+    const uint64_t first = h->pushed;
+    if (in_place) {
+      h->borrowed.push_back(hv_handle::Borrowed{first, nf, frames[i]});
+      h->pushed += nf;
+      h->st.frames_pushed += nf;
+    } else if (nf) {
+      s = enqueue_push_device(h, frames[i], nf);
+    }
     if (s != HV_OK) break;
     const uint32_t nw = outs[i] ? windows_ready(h, out_capacity_floats[i]) : 0;
     if (nw) s = enqueue_windows(h, outs[i], nw, graph);
+    if (in_place) {
+      if (!h->borrowed.empty() && h->borrowed.back().first == first) h->borrowed.pop_back();
+      const uint64_t keep = std::max(first, h->next_win);
+      if (s == HV_OK && keep < first + nf) s = enqueue_frames(h, frames[i], uint32_t(keep - first), first, nf);
+    }
     if (s != HV_OK) break;
     n_windows[i] = nw;
     cudaError_t e = cudaEventRecord(g->ev_join[i], h->stream);
