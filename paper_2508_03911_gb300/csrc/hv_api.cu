@@ -82,16 +82,15 @@ struct hv_handle {
   bool pca_has_lam = false;
   bool pca_batched = false;   // T <= 64 with FP32 covariance: many windows per launch
   uint32_t pca_last_nwin = 1;
-  // long windows, several per render: the eigensolver of one window (16 SMs) runs on
-  // eig_stream while the handle's stream runs the next window's covariance and the
-  // previous window's projection; windows alternate between two sets of C, counters,
-  // eigenvalues and sub-basis (set 0 is the one in `pca`)
-  cudaStream_t eig_stream = nullptr;
-  cudaEvent_t ev_cov[2] = {}, ev_eig[2] = {};
-  double2* pca_C[2] = {};
-  unsigned* pca_cnt[2] = {};
-  double* pca_lam[2] = {};
-  float2* pca_Vs[2] = {};
+  // long windows, several per render: the eigensolver of a window (one 16-SM cluster) runs
+  // on a stream of its own while the handle's stream runs the next windows' covariances and
+  // earlier windows' projections. Window w takes set w mod pca_sets: C, counters,
+  // eigenvalues and sub-basis, and with several lanes the eigensolver's scratch and stream
+  // (set 0 is the one in `pca`)
+  cudaStream_t eig_stream[kEigLanes] = {};
+  cudaEvent_t ev_cov[kEigLanes] = {}, ev_eig[kEigLanes] = {};
+  uint32_t pca_sets = 1, pca_lanes = 1;
+  PcaArgs pca_set[kEigLanes];
   const double* pca_lam_last = nullptr;  // eigenvalues of the last window rendered
   // stage timing
   bool prof = false;
@@ -432,10 +431,13 @@ hv_status apply_pending(hv_handle* h) {
     const size_t b_stage = stage_part * sizeof(uint16_t) * (p.precision == HV_PREC_SPLIT_BF16 ? 2 : 1);
     auto al = [](size_t v) { return (v + 255) / 256 * 256; };
     const size_t b_matf = size_t(T) * T * sizeof(float2);
-    // the second window set of the pipelined long windows: C, counters, lam, Vs
-    const size_t b_set2 = batched ? 0 : al(b_mat) + al(b_cnt) + al(b_lam) + al(b_vs);
+    // the further window sets of the pipelined long windows: C, counters, lam, Vs; each
+    // with the eigensolver's scratch where eigensolvers run side by side
+    const uint32_t lanes = batched ? 1 : pca_eig_lanes(T), sets = batched ? 1 : std::max<uint32_t>(2, lanes);
+    const size_t b_eig = lanes > 1 ? 2 * al(b_mat) + 3 * al(b_matf) + al(b_rot) : 0;
+    const size_t b_set = al(b_mat) + al(b_cnt) + al(b_lam) + al(b_vs) + b_eig;
     const size_t total = al(b_part) + (NW + 2) * al(b_mat) + 3 * al(b_matf) + al(b_rot) + al(b_cnt) + al(b_lam) +
-                         al(b_vs) + al(b_tc) + al(b_stage) + b_set2;
+                         al(b_vs) + al(b_tc) + al(b_stage) + (sets - 1) * b_set;
     s = ensure(h, &h->pca_ws, &h->pca_ws_bytes, total);
     if (s != HV_OK) return s;
     char* b = static_cast<char*>(h->pca_ws);
@@ -489,23 +491,34 @@ hv_status apply_pending(hv_handle* h) {
     std::memcpy(a.tc_tile_i, ti, sizeof(ti));
     std::memcpy(a.tc_tile_j, tj, sizeof(tj));
     b += al(b_stage);
-    h->pca_C[0] = a.C;
-    h->pca_cnt[0] = a.counters;
-    h->pca_lam[0] = a.lam;
-    h->pca_Vs[0] = a.Vs;
-    h->pca_C[1] = nullptr;
-    if (!batched) {
-      h->pca_C[1] = reinterpret_cast<double2*>(b);
-      b += al(b_mat);
-      h->pca_cnt[1] = reinterpret_cast<unsigned*>(b);
-      b += al(b_cnt);
-      h->pca_lam[1] = reinterpret_cast<double*>(b);
-      b += al(b_lam);
-      h->pca_Vs[1] = reinterpret_cast<float2*>(b);
-    }
     a.err = h->dev_err;
     a.nwin = 1;
     a.wstride = d.S;
+    h->pca_sets = sets;
+    h->pca_lanes = lanes;
+    h->pca_set[0] = a;
+    for (uint32_t k = 1; k < sets; ++k) {
+      PcaArgs& q = h->pca_set[k];
+      q = a;
+      auto take = [&](size_t bytes) {
+        char* at = b;
+        b += al(bytes);
+        return at;
+      };
+      q.C = reinterpret_cast<double2*>(take(b_mat));
+      q.counters = reinterpret_cast<unsigned*>(take(b_cnt));
+      q.cmax = reinterpret_cast<double*>(q.counters + 4);
+      q.lam = reinterpret_cast<double*>(take(b_lam));
+      q.Vs = reinterpret_cast<float2*>(take(b_vs));
+      if (lanes > 1) {
+        q.V = reinterpret_cast<double2*>(take(b_mat));
+        q.C2 = reinterpret_cast<double2*>(take(b_mat));
+        q.Cf = reinterpret_cast<float2*>(take(b_matf));
+        q.Cf2 = reinterpret_cast<float2*>(take(b_matf));
+        q.Vf = reinterpret_cast<float2*>(take(b_matf));
+        q.rot = reinterpret_cast<double*>(take(b_rot));
+      }
+    }
     h->pca_batched = batched;
     h->pca_has_lam = false;
     h->pca_lam_last = nullptr;
@@ -957,10 +970,10 @@ hv_status enqueue_windows(hv_handle* h, float* dst, uint32_t nw, bool capturing)
   // float is copied
   const bool direct = none && (reinterpret_cast<uintptr_t>(dst) & 7) == 0 && h->propagated <= h->next_win;
   // long PCA windows, several in this render: window by window, each window's
-  // spatial chunk and covariance on the handle's stream while the previous window's
-  // eigensolver runs on eig_stream (below)
+  // spatial chunk and covariance on the handle's stream while earlier windows'
+  // eigensolvers run on streams of their own (below)
   const bool pca_pipe = h->cur.temporal == HV_TEMPORAL_PCA && !h->pca_batched && !capturing && nw >= 2 &&
-                        h->pca_C[1] != nullptr;
+                        h->pca_sets >= 2;
   s = prof_mark(h, 0);
   if (s != HV_OK) return s;
   // spatial transform of every frame of these windows not yet in the queue: one
@@ -1015,28 +1028,24 @@ hv_status enqueue_windows(hv_handle* h, float* dst, uint32_t nw, bool capturing)
   } else if (none) {
     e = launch_copy_frames(tq, nw, h->W * h->H, dst, h->stream, &launches);
   } else if (pca_pipe) {
-    // pipelined long windows: spatial chunk(w), covariance(w) and projection(w - 1)
-    // on the handle's stream around eigensolver(w - 1, then w) on eig_stream; every
-    // frame of the render's windows fits in the time queue at once
+    // pipelined long windows: spatial chunk(w), covariance(w) and projection(w - sets + 1)
+    // on the handle's stream beside the eigensolvers of the windows between; every frame
+    // of the render's windows fits in the time queue at once. Set k is free again for
+    // window w: the handle's stream has waited for eigensolver(w - sets), before its
+    // projection. An eigensolver holds 16 SMs for 5.5 ms of serial rounds: two windows of
+    // 512 x 512, T = 256 took 14.3 ms one after the other, 9.2 side by side
     e = cudaSuccess;
+    const uint32_t sets = h->pca_sets, lanes = h->pca_lanes;
     auto window_args = [&](uint32_t w) {
-      PcaArgs a = h->pca;
-      const int k = int(w & 1);
-      a.nwin = 1;
-      a.wstride = S;
+      PcaArgs a = h->pca_set[w % sets];
       a.tq = RingRef{h->tq, h->Q, uint32_t((h->next_win + uint64_t(w) * S) % h->Q)};
-      a.C = h->pca_C[k];
-      a.counters = h->pca_cnt[k];
-      a.cmax = reinterpret_cast<double*>(a.counters + 4);
-      a.lam = h->pca_lam[k];
-      a.Vs = h->pca_Vs[k];
       return a;
     };
     // stage profiling: each window's eight events (start and end of its spatial
     // chunk, covariance, eigensolver and projection) on the stream that runs the
     // stage; room for all windows of the render first (the flush synchronises,
     // before anything is queued)
-    cudaEvent_t* evw[2] = {nullptr, nullptr};
+    cudaEvent_t* evw[kEigLanes] = {};
     if (h->prof && h->pca_ev_used + 8 * size_t(nw) > h->pca_ev.size()) {
       s = prof_flush(h);
       if (s != HV_OK) return s;
@@ -1046,12 +1055,13 @@ hv_status enqueue_windows(hv_handle* h, float* dst, uint32_t nw, bool capturing)
         h->pca_ev.push_back(x);
       }
     }
-    for (uint32_t w = 0; w <= nw && e == cudaSuccess; ++w) {
+    for (uint32_t w = 0; w < nw + sets - 1 && e == cudaSuccess; ++w) {
       if (w < nw) {
         PcaArgs a = window_args(w);
+        cudaStream_t eig = h->eig_stream[w % lanes];
         cudaEvent_t* ev = nullptr;
         if (h->prof) {
-          ev = evw[w & 1] = &h->pca_ev[h->pca_ev_used];
+          ev = evw[w % sets] = &h->pca_ev[h->pca_ev_used];
           h->pca_ev_used += 8;
         }
         // the window's frames not yet in the time queue
@@ -1069,25 +1079,26 @@ hv_status enqueue_windows(hv_handle* h, float* dst, uint32_t nw, bool capturing)
         if (ev) e = cudaEventRecord(ev[0], h->stream);
         if (e == cudaSuccess) e = launch_pca_cov(a, h->stream, &launches);
         if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], h->stream);
-        if (e == cudaSuccess) e = cudaEventRecord(h->ev_cov[w & 1], h->stream);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(h->eig_stream, h->ev_cov[w & 1], 0);
-        if (e == cudaSuccess && ev) e = cudaEventRecord(ev[2], h->eig_stream);
-        if (e == cudaSuccess) e = launch_pca_eig(a, h->eig_stream, &launches);
-        if (e == cudaSuccess && ev) e = cudaEventRecord(ev[3], h->eig_stream);
-        if (e == cudaSuccess && h->prof) e = launch_pca_sweeps_add(a.counters, h->pca_sweeps_dev, h->eig_stream);
-        if (e == cudaSuccess) e = cudaEventRecord(h->ev_eig[w & 1], h->eig_stream);
+        if (e == cudaSuccess) e = cudaEventRecord(h->ev_cov[w % sets], h->stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(eig, h->ev_cov[w % sets], 0);
+        if (e == cudaSuccess && ev) e = cudaEventRecord(ev[2], eig);
+        if (e == cudaSuccess) e = launch_pca_eig(a, eig, &launches);
+        if (e == cudaSuccess && ev) e = cudaEventRecord(ev[3], eig);
+        if (e == cudaSuccess && h->prof) e = launch_pca_sweeps_add(a.counters, h->pca_sweeps_dev, eig);
+        if (e == cudaSuccess) e = cudaEventRecord(h->ev_eig[w % sets], eig);
       }
-      if (w >= 1 && e == cudaSuccess) {
-        PcaArgs a = window_args(w - 1);
-        cudaEvent_t* ev = evw[(w - 1) & 1] ? evw[(w - 1) & 1] + 2 : nullptr;
-        e = cudaStreamWaitEvent(h->stream, h->ev_eig[(w - 1) & 1], 0);
+      if (w >= sets - 1 && e == cudaSuccess) {
+        const uint32_t q = w - (sets - 1);  // < nw
+        PcaArgs a = window_args(q);
+        cudaEvent_t* ev = evw[q % sets] ? evw[q % sets] + 2 : nullptr;
+        e = cudaStreamWaitEvent(h->stream, h->ev_eig[q % sets], 0);
         if (e == cudaSuccess && ev) e = cudaEventRecord(ev[4], h->stream);
-        if (e == cudaSuccess) e = launch_pca_proj(a, dst + size_t(w - 1) * h->win_floats, h->stream, &launches);
+        if (e == cudaSuccess) e = launch_pca_proj(a, dst + size_t(q) * h->win_floats, h->stream, &launches);
         if (e == cudaSuccess && ev) e = cudaEventRecord(ev[5], h->stream);
       }
     }
     h->pca_last_nwin = 1;
-    h->pca_lam_last = h->pca_lam[(nw - 1) & 1];
+    h->pca_lam_last = h->pca_set[(nw - 1) % sets].lam;
     h->pca_has_lam = true;
   } else if (h->cur.temporal == HV_TEMPORAL_PCA) {
     e = cudaSuccess;
@@ -1211,9 +1222,9 @@ hv_status hv_open(const hv_open_desc* desc, hv_handle** out) {
     h->own_stream = true;
   }
   e = cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->eig_stream, cudaStreamNonBlocking);
-  for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
-    e = cudaEventCreateWithFlags(&h->ev_cov[i], cudaEventDisableTiming);
+  for (uint32_t i = 0; i < kEigLanes && e == cudaSuccess; ++i) {
+    e = cudaStreamCreateWithFlags(&h->eig_stream[i], cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_cov[i], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_eig[i], cudaEventDisableTiming);
   }
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_pushed, cudaEventDisableTiming);
@@ -1440,11 +1451,11 @@ hv_status hv_close(hv_handle* h) {
     cudaStreamSynchronize(h->copy_stream);
     cudaStreamDestroy(h->copy_stream);
   }
-  if (h->eig_stream) {
-    cudaStreamSynchronize(h->eig_stream);
-    cudaStreamDestroy(h->eig_stream);
-  }
-  for (int i = 0; i < 2; ++i) {
+  for (uint32_t i = 0; i < kEigLanes; ++i) {
+    if (h->eig_stream[i]) {
+      cudaStreamSynchronize(h->eig_stream[i]);
+      cudaStreamDestroy(h->eig_stream[i]);
+    }
     if (h->ev_cov[i]) cudaEventDestroy(h->ev_cov[i]);
     if (h->ev_eig[i]) cudaEventDestroy(h->ev_eig[i]);
   }

@@ -164,6 +164,11 @@ cudaError_t launch_pca_sweeps_add(const unsigned* counters, unsigned long long* 
 // covariance into a.C (and the counters cleared), eigensolver (a.C, the shared
 // eigensolver scratch -> a.lam, a.Vs), projection (a.Vs, the window's frames -> out).
 cudaError_t launch_pca_cov(PcaArgs& a, cudaStream_t s, int* launches);
+// Eigensolvers of windows of T frames that may run side by side, each on its own stream with
+// its own scratch (C2, Cf, Cf2, Vf, V, rot): the 16-CTA clusters that fit the device at
+// once, at most kEigLanes; 1 where the eigensolver is a cooperative launch.
+constexpr uint32_t kEigLanes = 4;
+uint32_t pca_eig_lanes(uint32_t T);
 cudaError_t launch_pca_eig(PcaArgs& a, cudaStream_t s, int* launches);
 cudaError_t launch_pca_proj(PcaArgs& a, float* out, cudaStream_t s, int* launches);
 

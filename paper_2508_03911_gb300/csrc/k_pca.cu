@@ -745,38 +745,57 @@ __global__ void __launch_bounds__(JC_NT) k_jacobi_cluster(PcaArgs a) {
   if (rank == 0 && tid == 0) atomicAdd(&a.counters[REFINE ? 2 : 1], unsigned(sweeps));
 }
 
+// Launch of one cluster on stream s; *clusters: how many fit the device at once (0 where
+// one cannot be placed: the caller uses the cooperative kernel).
 template <int T, bool REFINE>
-static cudaError_t launch_jacobi_cluster(const PcaArgs& a, cudaStream_t s, bool* ok) {
-  *ok = false;
+static void jacobi_cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, cudaStream_t s, int* clusters) {
+  *clusters = 0;
   const size_t smem = JclSmem<T, REFINE>::bytes();
   auto kern = k_jacobi_cluster<T, REFINE>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) {
     cudaGetLastError();
-    return cudaSuccess;  // not available: the caller uses the cooperative kernel
+    return;
   }
-  cudaLaunchConfig_t cfg{};
+  cfg = cudaLaunchConfig_t{};
   cfg.gridDim = dim3(JC);
   cfg.blockDim = dim3(JC_NT);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = JC;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = JC;
+  attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  int nclusters = 0;
-  e = cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg);
-  if (e != cudaSuccess || nclusters < 1) {
+  if (cudaOccupancyMaxActiveClusters(clusters, kern, &cfg) != cudaSuccess) {
     cudaGetLastError();
-    return cudaSuccess;
+    *clusters = 0;
   }
-  e = cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+template <int T, bool REFINE>
+static cudaError_t launch_jacobi_cluster(const PcaArgs& a, cudaStream_t s, bool* ok) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr;
+  int clusters = 0;
+  jacobi_cluster_config<T, REFINE>(cfg, attr, s, &clusters);
+  *ok = false;
+  if (clusters < 1) return cudaSuccess;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_jacobi_cluster<T, REFINE>, a);
   if (e == cudaSuccess) *ok = true;
   return e;
+}
+
+template <int T>
+static uint32_t clusters_at_once() {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr;
+  int a = 0, b = 0;
+  jacobi_cluster_config<T, false>(cfg, attr, nullptr, &a);
+  jacobi_cluster_config<T, true>(cfg, attr, nullptr, &b);
+  return uint32_t(a < b ? a : b);
 }
 
 // out = op(A) B for T x T complex matrices: A float64 (op = identity) or the
@@ -1355,6 +1374,11 @@ cudaError_t launch_pca_cov(PcaArgs& a, cudaStream_t s, int* launches) {
   return cudaGetLastError();
 }
 
+uint32_t pca_eig_lanes(uint32_t T) {
+  const uint32_t n = T == 256 ? clusters_at_once<256>() : (T == 128 ? clusters_at_once<128>() : 1u);
+  return n < 1 ? 1u : (n < kEigLanes ? n : kEigLanes);
+}
+
 cudaError_t launch_pca_eig(PcaArgs& a, cudaStream_t s, int* launches) {
   cudaError_t e = cudaSuccess;
   if (a.T == 32) {
@@ -1451,8 +1475,8 @@ cudaError_t launch_pca(PcaArgs& a, float* out, cudaStream_t s, int* launches, cu
 
 // total[0] += float32 sweeps, total[1] += refinement sweeps of the last window
 __global__ void k_pca_sweeps_add(const unsigned* counters, unsigned long long* total) {
-  total[0] += counters[1];
-  total[1] += counters[2];
+  atomicAdd(&total[0], counters[1]);  // windows finish on several streams
+  atomicAdd(&total[1], counters[2]);
 }
 
 cudaError_t launch_pca_sweeps_add(const unsigned* counters, unsigned long long* total, cudaStream_t s) {
