@@ -81,6 +81,7 @@ hv_status hv_af_open(const hv_af_desc* d, hv_af** out) {
   } pieces[] = {
       {reinterpret_cast<void**>(&t.prm), NPARAMS * 4},
       {reinterpret_cast<void**>(&t.prm_bf), NPARAMS * 2},
+      {reinterpret_cast<void**>(&t.wtc), NTC * 2},
       {reinterpret_cast<void**>(&t.grad), NPARAMS * 4},
       {reinterpret_cast<void**>(&t.m), NPARAMS * 4},
       {reinterpret_cast<void**>(&t.v), NPARAMS * 4},

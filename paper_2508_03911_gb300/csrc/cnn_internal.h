@@ -14,10 +14,25 @@ constexpr int OFF_W1 = 0, OFF_B1 = 144, OFF_W2 = 160, OFF_B2 = 4768, OFF_W3 = 48
               OFF_F2B = 62336, NPARAMS = 62337;
 constexpr int IN_SIDE = 128;
 
+// Weights of layers 2-4 in the order the tensor cores read them (k_conv_tc.cu): per layer
+// no-swizzle K-major core matrices of 8 output channels x 8 values of k = tap CI + c.
+constexpr int OFF_TC2 = 0, OFF_TC3 = 32 * 144, OFF_TC4 = OFF_TC3 + 64 * 288, NTC = OFF_TC4 + 64 * 576;
+// Place of parameter i there, -1 for the others.
+__host__ __device__ inline int tc_place(int i) {
+  int off, ci, base;
+  if (i >= OFF_W2 && i < OFF_B2) off = OFF_W2, ci = 16, base = OFF_TC2;
+  else if (i >= OFF_W3 && i < OFF_B3) off = OFF_W3, ci = 32, base = OFF_TC3;
+  else if (i >= OFF_W4 && i < OFF_B4) off = OFF_W4, ci = 64, base = OFF_TC4;
+  else return -1;
+  const int e = i - off, o = e / (ci * 9), c = e / 9 % ci, t = e % 9, k = t * ci + c;
+  return base + (o >> 3) * (8 * 9 * ci) + (k >> 3) * 64 + (o & 7) * 8 + (k & 7);
+}
+
 // Device buffers of one network (sizes for max_batch images).
 struct Net {
   float* prm;               // NPARAMS float32 parameters
   __nv_bfloat16* prm_bf;    // bfloat16 mirror (the convolutions read their weights here)
+  __nv_bfloat16* wtc;       // NTC: layers 2-4 again, in the tensor cores' order
   float* grad;              // NPARAMS gradient of the last backward pass
   float* m;                 // Adam first moment
   float* v;                 // Adam second moment
@@ -33,7 +48,8 @@ struct Net {
 };
 
 // y = relu(conv3x3_stride2(x, w) + b) for [n][CI][HI][HI] bfloat16 inputs on the
-// tensor cores (k_conv_tc.cu); instantiated for the network's layers 2-4.
+// tensor cores (k_conv_tc.cu), w in their order (tc_place); instantiated for the network's
+// layers 2-4.
 template <int CI, int CO, int HI>
 cudaError_t conv_tc(const __nv_bfloat16* x, const __nv_bfloat16* w, const float* bias, __nv_bfloat16* y,
                     uint32_t n, unsigned* err, cudaStream_t s);

@@ -27,72 +27,78 @@ __device__ __forceinline__ float bf(const __nv_bfloat16 v) { return __bfloat162f
 
 // ------------------------------------------------------------------ forward
 //
-// y[n][o][i][j] = relu(b[o] + sum_{c,di,dj} w[o][c][di][dj] x[n][c][2i+di-1][2j+dj-1]).
-// A CTA covers image n, NR output rows and all CO channels; a thread owns 4
-// channels (4 cg .. 4 cg + 3) x 4 neighbouring pixels of one row. Input rows
-// and weights are staged in shared memory CK channels at a time.
-template <int CI, int CO, int HI>
-__global__ void __launch_bounds__(NT) k_conv_fwd(const __nv_bfloat16* __restrict__ x,
-                                                 const __nv_bfloat16* __restrict__ w,
-                                                 const float* __restrict__ bias, __nv_bfloat16* __restrict__ y) {
-  constexpr int WI = HI, HO = HI / 2, WO = HO;
-  constexpr int CG = CO / 4, PG = NT / CG, TPX = 4 * PG;
-  constexpr int NR = TPX / WO;
-  static_assert(TPX % WO == 0 && NR <= HO && HO % NR == 0, "tile");
-  constexpr int CK = CI < 8 ? CI : 8;
-  constexpr int SR = 2 * NR + 1, SC = WI + 2;
-  __shared__ float xs[CK][SR][SC];
-  __shared__ __align__(16) float ws[CK][9][CO];
-  constexpr int TILES = HO / NR;
-  const int n = blockIdx.x / TILES, r0 = (blockIdx.x % TILES) * NR;
-  const int tid = threadIdx.x, cg = tid % CG, pg = tid / CG;
-  const int p0 = pg * 4, il = p0 / WO, j0 = p0 % WO;
-  float acc[4][4];
+// The 3 x 9 inputs of 4 neighbouring outputs 4 q .. 4 q + 3 of row i of layer 1: columns 8 q
+// - 1 .. 8 q + 7 of rows 2 i - 1 .. 2 i + 1 (zero outside). VEC: x 16-byte aligned. The left
+// column comes from the neighbouring lane (16 lanes hold a row).
+template <bool VEC>
+__device__ __forceinline__ void load_inputs1(const __nv_bfloat16* __restrict__ xn, int i, int q, float (&xv)[3][9]) {
+  constexpr int HI = 128;
 #pragma unroll
-  for (int k = 0; k < 4; ++k)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[k][q] = 0.f;
-  for (int c0 = 0; c0 < CI; c0 += CK) {
-    __syncthreads();
-    for (int e = tid; e < CK * SR * SC; e += NT) {
-      const int c = e / (SR * SC), rr = (e / SC) % SR, cc = e % SC;
-      const int yy = 2 * r0 - 1 + rr, xx = cc - 1;
-      float v = 0.f;
-      if (yy >= 0 && yy < HI && xx >= 0 && xx < WI) v = bf(x[((size_t(n) * CI + c0 + c) * HI + yy) * WI + xx]);
-      xs[c][rr][cc] = v;
+  for (int di = 0; di < 3; ++di) {
+    const int yy = 2 * i + di - 1;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    __nv_bfloat162* p = reinterpret_cast<__nv_bfloat162*>(&v);
+    if (yy >= 0) {
+      const __nv_bfloat16* row = xn + yy * HI + 8 * q;
+      if (VEC) v = *reinterpret_cast<const uint4*>(row);
+      else
+        for (int e = 0; e < 4; ++e) p[e] = __nv_bfloat162(row[2 * e], row[2 * e + 1]);
     }
-    for (int e = tid; e < CK * 9 * CO; e += NT) {
-      const int o = e % CO, t = (e / CO) % 9, c = e / (9 * CO);
-      ws[c][t][o] = bf(w[(size_t(o) * CI + c0 + c) * 9 + t]);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float2 f = __bfloat1622float2(p[e]);
+      xv[di][1 + 2 * e] = f.x;
+      xv[di][2 + 2 * e] = f.y;
     }
-    __syncthreads();
-#pragma unroll 2
-    for (int c = 0; c < CK; ++c)
-#pragma unroll
-      for (int di = 0; di < 3; ++di)
-#pragma unroll
-        for (int dj = 0; dj < 3; ++dj) {
-          const float4 wv = *reinterpret_cast<const float4*>(&ws[c][di * 3 + dj][4 * cg]);
-          float xv[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) xv[q] = xs[c][2 * il + di][2 * (j0 + q) + dj];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            acc[0][q] = fmaf(wv.x, xv[q], acc[0][q]);
-            acc[1][q] = fmaf(wv.y, xv[q], acc[1][q]);
-            acc[2][q] = fmaf(wv.z, xv[q], acc[2][q]);
-            acc[3][q] = fmaf(wv.w, xv[q], acc[3][q]);
-          }
-        }
+    const float left = __shfl_up_sync(0xffffffffu, xv[di][8], 1);
+    xv[di][0] = q == 0 ? 0.f : left;
   }
+}
+
+// Layer 1 (one input channel): y[n][o][i][j] = relu(b[o] + sum_{di,dj} w[o][di][dj]
+// x[n][2i+di-1][2j+dj-1]). Bound by its output (67 MB at n = 512). A thread forms 4
+// neighbouring pixels of all 16 channels from inputs in registers and broadcast weights
+// (staging input rows and weights per 4 channels x 4 pixels took 39 us at n = 512; 23 now).
+template <bool VEC>
+__global__ void __launch_bounds__(NT) k_conv1(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ w,
+                                              const float* __restrict__ bias, __nv_bfloat16* __restrict__ y) {
+  constexpr int HO = 64;
+  __shared__ __align__(16) float ws[9][16];
+  __shared__ float bs[16];
+  const int tid = threadIdx.x, q = tid & 15;
+  if (tid < 144) ws[tid % 9][tid / 9] = bf(w[tid]);
+  if (tid < 16) bs[tid] = bias[tid];
+  __syncthreads();
+  const uint32_t row = blockIdx.x * (NT / 16) + tid / 16;  // 16 rows of 64 pixels per CTA
+  const uint32_t n = row / HO;
+  const int i = int(row % HO);
+  float xv[3][9];
+  load_inputs1<VEC>(x + size_t(n) * 128 * 128, i, q, xv);
+  float acc[16][4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int o = 4 * cg + k;
-    const float b = bias[o];
+  for (int o = 0; o < 16; ++o)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) acc[o][e] = 0.f;
+#pragma unroll
+  for (int t = 0; t < 9; ++t)
+#pragma unroll
+    for (int o = 0; o < 16; o += 4) {
+      const float4 wv = *reinterpret_cast<const float4*>(&ws[t][o]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float v = xv[t / 3][2 * e + t % 3];
+        acc[o][e] = fmaf(wv.x, v, acc[o][e]);
+        acc[o + 1][e] = fmaf(wv.y, v, acc[o + 1][e]);
+        acc[o + 2][e] = fmaf(wv.z, v, acc[o + 2][e]);
+        acc[o + 3][e] = fmaf(wv.w, v, acc[o + 3][e]);
+      }
+    }
+#pragma unroll
+  for (int o = 0; o < 16; ++o) {
     __align__(8) __nv_bfloat16 v[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = __float2bfloat16_rn(fmaxf(acc[k][q] + b, 0.f));
-    *reinterpret_cast<uint2*>(y + ((size_t(n) * CO + o) * HO + r0 + il) * WO + j0) = *reinterpret_cast<uint2*>(v);
+    for (int e = 0; e < 4; ++e) v[e] = __float2bfloat16_rn(fmaxf(acc[o][e] + bs[o], 0.f));
+    *reinterpret_cast<uint2*>(y + ((size_t(n) * 16 + o) * HO + i) * HO + 4 * q) = *reinterpret_cast<uint2*>(v);
   }
 }
 
@@ -359,28 +365,8 @@ __global__ void __launch_bounds__(NT, 3) k_conv_dw1(const float* __restrict__ dz
   for (uint32_t quad = blockIdx.x; quad < nquads; quad += gridDim.x) {
     const uint32_t n = quad / (HO / 4);
     const int i = 4 * int(quad % (HO / 4)) + il;
-    const __nv_bfloat16* xn = x + size_t(n) * HI * HI;
-    float xv[3][9];  // columns 2 j0 - 1 .. 2 j0 + 7
-#pragma unroll
-    for (int di = 0; di < 3; ++di) {
-      const int yy = 2 * i + di - 1;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      __nv_bfloat162* p = reinterpret_cast<__nv_bfloat162*>(&v);
-      if (yy >= 0) {
-        const __nv_bfloat16* row = xn + yy * HI + 2 * j0;
-        if (VEC) v = *reinterpret_cast<const uint4*>(row);
-        else
-          for (int e = 0; e < 4; ++e) p[e] = __nv_bfloat162(row[2 * e], row[2 * e + 1]);
-      }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 f = __bfloat1622float2(p[e]);
-        xv[di][1 + 2 * e] = f.x;
-        xv[di][2 + 2 * e] = f.y;
-      }
-      const float left = __shfl_up_sync(0xffffffffu, xv[di][8], 1);
-      xv[di][0] = j0 == 0 ? 0.f : left;
-    }
+    float xv[3][9];
+    load_inputs1<VEC>(x + size_t(n) * HI * HI, i, lane & 15, xv);
     const float* zp = dz + ((size_t(n) * 16 + 4 * og) * HO + i) * HO + j0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -564,8 +550,8 @@ __global__ void __launch_bounds__(NT) k_head_grads(const float* __restrict__ scr
 // ---------------------------------------------------------------------- Adam
 
 __global__ void k_adam(float* __restrict__ prm, const float* __restrict__ grad, float* __restrict__ m,
-                       float* __restrict__ v, __nv_bfloat16* __restrict__ prm_bf, uint32_t count, float lr,
-                       float b1, float b2, float eps, float c1, float c2) {
+                       float* __restrict__ v, __nv_bfloat16* __restrict__ prm_bf, __nv_bfloat16* __restrict__ wtc,
+                       uint32_t count, float lr, float b1, float b2, float eps, float c1, float c2) {
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
     const float g = grad[i];
     const float mi = fmaf(b1, m[i], (1.f - b1) * g);
@@ -575,23 +561,21 @@ __global__ void k_adam(float* __restrict__ prm, const float* __restrict__ grad, 
     const float p = prm[i] - lr * (mi * c1) / (sqrtf(vi * c2) + eps);
     prm[i] = p;
     prm_bf[i] = __float2bfloat16_rn(p);
+    const int k = tc_place(int(i));
+    if (k >= 0) wtc[k] = prm_bf[i];
   }
 }
 
-__global__ void k_to_bf16(const float* __restrict__ prm, __nv_bfloat16* __restrict__ out, uint32_t count) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x)
+__global__ void k_to_bf16(const float* __restrict__ prm, __nv_bfloat16* __restrict__ out,
+                          __nv_bfloat16* __restrict__ wtc, uint32_t count) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
     out[i] = __float2bfloat16_rn(prm[i]);
+    const int k = tc_place(int(i));
+    if (k >= 0) wtc[k] = out[i];
+  }
 }
 
 // ------------------------------------------------------------------ launchers
-
-template <int CI, int CO, int HI>
-cudaError_t conv_fwd(const Net& t, const __nv_bfloat16* x, int off_w, int off_b, __nv_bfloat16* y, uint32_t n,
-                     cudaStream_t s) {
-  constexpr int WO = HI / 2, CG = CO / 4, TPX = 4 * (NT / CG), NR = TPX / WO;
-  k_conv_fwd<CI, CO, HI><<<n * (HI / 2 / NR), NT, 0, s>>>(x, t.prm_bf + off_w, t.prm + off_b, y);
-  return cudaGetLastError();
-}
 
 // Partials of the weight gradients: CTAs per layer (about two per SM; layer 4 has 256
 // bands at the largest batch of the reference workload and large partials: one per SM).
@@ -622,11 +606,16 @@ cudaError_t conv_bwd(const Net& t, int layer, const float* dz, const __nv_bfloat
 
 cudaError_t net_forward(const Net& t, const void* x, uint32_t n, const float* ztarget, float* zout, cudaStream_t s) {
   const auto* xi = static_cast<const __nv_bfloat16*>(x);
-  cudaError_t e = conv_fwd<1, 16, 128>(t, xi, OFF_W1, OFF_B1, t.a1, n, s);
+  const uint32_t rows = n * 64;
+  if ((reinterpret_cast<uintptr_t>(x) & 15) == 0)
+    k_conv1<true><<<rows / 16, NT, 0, s>>>(xi, t.prm_bf + OFF_W1, t.prm + OFF_B1, t.a1);
+  else
+    k_conv1<false><<<rows / 16, NT, 0, s>>>(xi, t.prm_bf + OFF_W1, t.prm + OFF_B1, t.a1);
+  cudaError_t e = cudaGetLastError();
   // layers 2-4 (K = 144, 288, 576): implicit GEMMs on the tensor cores
-  if (e == cudaSuccess) e = conv_tc<16, 32, 64>(t.a1, t.prm_bf + OFF_W2, t.prm + OFF_B2, t.a2, n, t.err, s);
-  if (e == cudaSuccess) e = conv_tc<32, 64, 32>(t.a2, t.prm_bf + OFF_W3, t.prm + OFF_B3, t.a3, n, t.err, s);
-  if (e == cudaSuccess) e = conv_tc<64, 64, 16>(t.a3, t.prm_bf + OFF_W4, t.prm + OFF_B4, t.a4, n, t.err, s);
+  if (e == cudaSuccess) e = conv_tc<16, 32, 64>(t.a1, t.wtc + OFF_TC2, t.prm + OFF_B2, t.a2, n, t.err, s);
+  if (e == cudaSuccess) e = conv_tc<32, 64, 32>(t.a2, t.wtc + OFF_TC3, t.prm + OFF_B3, t.a3, n, t.err, s);
+  if (e == cudaSuccess) e = conv_tc<64, 64, 16>(t.a3, t.wtc + OFF_TC4, t.prm + OFF_B4, t.a4, n, t.err, s);
   if (e != cudaSuccess) return e;
   k_head<<<n, 64, 0, s>>>(t.a4, t.prm, ztarget, n, zout, t.head, t.dbuf0);
   return cudaGetLastError();
@@ -654,12 +643,12 @@ cudaError_t net_backward(const Net& t, const void* x, uint32_t n, float* loss, c
 }
 
 cudaError_t net_adam(const Net& t, float lr, float b1, float b2, float eps, float c1, float c2, cudaStream_t s) {
-  k_adam<<<(NPARAMS + 255) / 256, 256, 0, s>>>(t.prm, t.grad, t.m, t.v, t.prm_bf, NPARAMS, lr, b1, b2, eps, c1, c2);
+  k_adam<<<(NPARAMS + 255) / 256, 256, 0, s>>>(t.prm, t.grad, t.m, t.v, t.prm_bf, t.wtc, NPARAMS, lr, b1, b2, eps, c1, c2);
   return cudaGetLastError();
 }
 
 cudaError_t net_sync_bf16(const Net& t, cudaStream_t s) {
-  k_to_bf16<<<(NPARAMS + 255) / 256, 256, 0, s>>>(t.prm, t.prm_bf, NPARAMS);
+  k_to_bf16<<<(NPARAMS + 255) / 256, 256, 0, s>>>(t.prm, t.prm_bf, t.wtc, NPARAMS);
   return cudaGetLastError();
 }
 

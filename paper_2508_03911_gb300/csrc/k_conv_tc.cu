@@ -11,7 +11,15 @@
 // pixels; per tile it gathers the 9 taps one at a time (128 pixels x CI channels,
 // no-swizzle K-major core matrices) into two alternating buffers, and one thread
 // issues the tap's K = CI / 16 MMAs and commits them to the buffer's mbarrier,
-// so gathering tap t + 1 overlaps the MMAs of tap t. Every mbarrier wait is
+// so gathering tap t + 1 overlaps the MMAs of tap t.
+//
+// Bound by the gather's load instructions, and by the weights' before the first tile. The
+// three taps of an input row come from one 4-byte load per channel: a pixel's own two
+// columns 2 j, 2 j + 1, and the left neighbour's second one by a shuffle (three 2-byte
+// loads before). The next row's loads are issued before the current row's taps are
+// written. The weights are kept in the MMA's layout by the kernels that write them, and
+// copied 16 bytes at a time (288 2-byte loads a thread for layer 4 before). n = 512: layers
+// 2, 3, 4 in 45, 41, 32 us before, 35, 23, 16 now. Every mbarrier wait is
 // bounded; on timeout the kernel records an error, stops and releases its tensor
 // memory.
 #include <cuda_bf16.h>
@@ -66,8 +74,6 @@ __device__ __forceinline__ bool wait_phase(uint32_t mbar, uint32_t parity) {
   }
 }
 
-__device__ __forceinline__ uint32_t pack(uint16_t lo, uint16_t hi) { return uint32_t(lo) | (uint32_t(hi) << 16); }
-
 // core-matrix offset of element (row, k) in a K-major tile whose 8-row groups are sbo apart
 __device__ __forceinline__ int cm_off(int row, int kgroup, int sbo) { return (row >> 3) * sbo + kgroup * 128 + (row & 7) * 16; }
 
@@ -75,6 +81,7 @@ template <int CI, int CO, int HI>
 struct ConvTc {
   static_assert(CI % 16 == 0 && CO % 16 == 0 && CO >= 16 && CO <= 256, "tensor-core shapes");
   static constexpr int HO = HI / 2, K = 9 * CI;
+  static_assert(32 % HO == 0, "a warp's pixels are whole rows: a left neighbour is the lane before");
   static constexpr int SBO_A = (CI / 8) * 128, SBO_B = (K / 8) * 128;
   static constexpr int A_BYTES = CT_M * CI * 2;  // one tap of a tile
   static constexpr int B_BYTES = CO * K * 2;     // all weights
@@ -96,8 +103,6 @@ __global__ void __launch_bounds__(CT_NT) k_conv_tc(const __nv_bfloat16* __restri
   unsigned char* Bs = sm;
   unsigned char* As0 = sm + G::B_BYTES;
   const int tid = threadIdx.x, warp = tid >> 5;
-  const uint16_t* xr = reinterpret_cast<const uint16_t*>(x);
-  const uint16_t* wr = reinterpret_cast<const uint16_t*>(w);
 
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(su32(&mbar[0])) : "memory");
@@ -110,16 +115,10 @@ __global__ void __launch_bounds__(CT_NT) k_conv_tc(const __nv_bfloat16* __restri
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
   }
-  // weights: B[o][k = t CI + c] = w[o][c][t], 8 consecutive k (channels of one tap) per 16 bytes
-  for (int e = tid; e < CO * (G::K / 8); e += CT_NT) {
-    const int o = e / (G::K / 8), kg = e % (G::K / 8);
-    const int t = (kg * 8) / CI, c0 = (kg * 8) % CI;
-    uint16_t v[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = wr[(size_t(o) * CI + c0 + q) * 9 + t];
-    *reinterpret_cast<uint4*>(Bs + cm_off(o, kg, G::SBO_B)) =
-        make_uint4(pack(v[0], v[1]), pack(v[2], v[3]), pack(v[4], v[5]), pack(v[6], v[7]));
-  }
+  // weights, laid out already
+#pragma unroll 8
+  for (int e = tid; e < G::B_BYTES / 16; e += CT_NT)
+    reinterpret_cast<uint4*>(Bs)[e] = __ldg(reinterpret_cast<const uint4*>(w) + e);
   asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
@@ -131,40 +130,65 @@ __global__ void __launch_bounds__(CT_NT) k_conv_tc(const __nv_bfloat16* __restri
   uint32_t q = 0;  // taps issued so far: tap q used buffer q & 1 and completes phase q >> 1 of its mbarrier
   const int ntiles = (npix + CT_M - 1) / CT_M;
 
+  // columns 2 j and 2 j + 1 of input row 2 i + di - 1, every channel, of this thread's
+  // output pixel in `tile` (zero outside the image and past the last pixel)
+  auto load_row = [&](int tile, int di, uint32_t (&u)[CI]) {
+    const int p = tile * CT_M + tid;
+    const int n = p / (HO * HO), rem = p % (HO * HO), yy = 2 * (rem / HO) + di - 1;
+    const bool in = tile < ntiles && p < npix && yy >= 0;
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(x) + (size_t(in ? n : 0) * CI * HI + (in ? yy : 0)) * (HI / 2) + rem % HO;
+#pragma unroll
+    for (int c = 0; c < CI; ++c) u[c] = in ? __ldg(src + size_t(c) * HI * (HI / 2)) : 0u;
+  };
+  uint32_t u[CI], next[CI];
+  load_row(blockIdx.x, 0, next);
+
   for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
     const int p = tile * CT_M + tid;  // this thread's output pixel = row of A and D
     const bool valid = p < npix;
     const int n = p / (HO * HO), rem = p % (HO * HO), i = rem / HO, j = rem % HO;
-    for (int t = 0; t < 9; ++t, ++q) {
-      const uint32_t b = q & 1;
-      if (q >= 2) {  // the MMAs that last read this buffer are done
-        if (tid == 0) s_ok = wait_phase(su32(&mbar[b]), ((q >> 1) - 1) & 1) ? 1 : 0;
+#pragma unroll 1
+    for (int di = 0; di < 3 && ok; ++di) {
+#pragma unroll
+      for (int c = 0; c < CI; ++c) u[c] = next[c];
+      load_row(di < 2 ? tile : tile + int(gridDim.x), di < 2 ? di + 1 : 0, next);
+#pragma unroll
+      for (int dj = 0; dj < 3; ++dj, ++q) {
+        const int t = 3 * di + dj;
+        const uint32_t b = q & 1;
+        if (q >= 2) {  // the MMAs that last read this buffer are done
+          if (tid == 0) s_ok = wait_phase(su32(&mbar[b]), ((q >> 1) - 1) & 1) ? 1 : 0;
+          __syncthreads();
+          ok = s_ok != 0;
+          if (!ok) break;
+        }
+        unsigned char* At = As0 + b * G::A_BYTES;
+#pragma unroll
+        for (int cg = 0; cg < CI / 8; ++cg) {
+          uint32_t v[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            uint32_t lo = u[cg * 8 + 2 * k], hi = u[cg * 8 + 2 * k + 1];
+            if (dj == 0) {  // column 2 j - 1: the left neighbour's second column, 0 at the edge
+              lo = __shfl_up_sync(0xffffffffu, lo, 1);
+              hi = __shfl_up_sync(0xffffffffu, hi, 1);
+            }
+            v[k] = __byte_perm(lo, hi, dj == 1 ? 0x5410 : 0x7632);
+            if (dj == 0 && j == 0) v[k] = 0u;
+          }
+          *reinterpret_cast<uint4*>(At + cm_off(tid, cg, G::SBO_A)) = make_uint4(v[0], v[1], v[2], v[3]);
+        }
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         __syncthreads();
-        ok = s_ok != 0;
-        if (!ok) break;
-      }
-      const int yy = 2 * i + t / 3 - 1, xx = 2 * j + t % 3 - 1;
-      const bool in = valid && yy >= 0 && yy < HI && xx >= 0 && xx < HI;
-      const uint16_t* src = xr + ((size_t(n) * CI) * HI + (in ? yy : 0)) * HI + (in ? xx : 0);
-      unsigned char* At = As0 + b * G::A_BYTES;
+        if (tid == 0) {
+          asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+          const uint32_t at = as0 + b * G::A_BYTES;
 #pragma unroll
-      for (int cg = 0; cg < CI / 8; ++cg) {
-        uint16_t v[8];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) v[c] = in ? src[size_t(cg * 8 + c) * HI * HI] : uint16_t(0);
-        *reinterpret_cast<uint4*>(At + cm_off(tid, cg, G::SBO_A)) =
-            make_uint4(pack(v[0], v[1]), pack(v[2], v[3]), pack(v[4], v[5]), pack(v[6], v[7]));
-      }
-      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-      __syncthreads();
-      if (tid == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        const uint32_t at = as0 + b * G::A_BYTES;
-#pragma unroll
-        for (int s = 0; s < CI / 16; ++s)
-          mma(tmem, kdesc(at + 256 * s, G::SBO_A), kdesc(bs + (t * CI / 8 + 2 * s) * 128, G::SBO_B), id,
-              (t > 0 || s > 0) ? 1u : 0u);
-        commit(su32(&mbar[b]));
+          for (int s = 0; s < CI / 16; ++s)
+            mma(tmem, kdesc(at + 256 * s, G::SBO_A), kdesc(bs + (t * CI / 8 + 2 * s) * 128, G::SBO_B), id,
+                (t > 0 || s > 0) ? 1u : 0u);
+          commit(su32(&mbar[b]));
+        }
       }
     }
     if (!ok) break;
@@ -218,11 +242,16 @@ cudaError_t conv_tc(const __nv_bfloat16* x, const __nv_bfloat16* w, const float*
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  // CTAs per SM: as many as shared memory holds (the hardware places them), at most
-  // as many as share the SM's 512 tensor-memory columns
+  // CTAs per SM: as many as shared memory and registers hold (the hardware places them),
+  // at most as many as share the SM's 512 tensor-memory columns
+  cudaFuncAttributes attr{};
+  e = cudaFuncGetAttributes(&attr, kern);
+  if (e != cudaSuccess) return e;
   const int by_smem = int((228 * 1024) / (G::SMEM + 2048));
   const int by_tmem = int(512 / G::TMEM_COLS);
-  const int per_sm = by_smem < by_tmem ? by_smem : by_tmem;
+  const int by_regs = 65536 / (CT_NT * ((attr.numRegs + 7) / 8 * 8));
+  int per_sm = by_smem < by_tmem ? by_smem : by_tmem;
+  if (per_sm > by_regs) per_sm = by_regs;
   const int npix = int(n) * G::HO * G::HO;
   const int ntiles = (npix + CT_M - 1) / CT_M;
   int grid = (per_sm > 0 ? per_sm : 1) * nsm;
