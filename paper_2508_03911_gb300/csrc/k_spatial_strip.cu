@@ -24,95 +24,15 @@
 // 42 of passes over full spectra). Us a frame in large launches, against the persistent
 // block-wide passes that staged each strip of 16 lines in shared memory (two strips per
 // CTA, so one or two CTAs per SM from 512 points on): 256 x 256 ASP 0.53 -> 0.37, Fresnel
-// 0.33 -> 0.31; 512 x 512 3.14 -> 2.04 and 1.65 -> 1.40; 1024 x 1024 17.0 -> 8.7 and
-// 8.4 -> 6.4; 128 x 128 0.139 -> 0.107 and 0.081 -> 0.083.
-#include "fft_dev.cuh"
+// 0.33 -> 0.31; 512 x 512 3.14 -> 1.89 and 1.65 -> 1.36; 1024 x 1024 17.0 -> 8.9 and
+// 8.4 -> 6.1; 128 x 128 0.139 -> 0.107 and 0.081 -> 0.083.
+#include "strip_dev.cuh"
 #include "hv_internal.h"
 #include "../../include/hv.h"
 
 namespace hv {
 
 namespace {
-
-// Column CTAs: L = R1 x R2, BT lines, NT threads. A thread holds I1 first-stage and I2
-// second-stage butterflies of one line.
-template <int L>
-struct ColCfg {
-  static constexpr int R1 = L >= 512 ? 32 : (L >= 128 ? 16 : 8);
-  static constexpr int R2 = L / R1;
-  static constexpr int BT = L >= 512 ? 8 : 16;
-  static constexpr int NT = L == 64 ? 64 : (L == 1024 ? 256 : 128);
-  static constexpr int NJ = NT / BT;          // threads per line
-  static constexpr int I1 = (L / R1) / NJ;    // first-stage butterflies per thread
-  static constexpr int I2 = (L / R2) / NJ;    // second-stage butterflies per thread
-  static constexpr int NTW = (R2 - 1) * R1;   // second-stage twiddles
-  static constexpr int PAD = BT == 8 ? 1 : 0; // padding rows per R1 rows of the exchange buffer
-  static constexpr int ROWS = L + PAD * R2;
-  static constexpr size_t SMEM = (size_t(ROWS) * BT + NTW) * sizeof(float2);
-  static constexpr int CTAS = L == 1024 ? 2 : (L == 512 ? 5 : (L == 64 ? 12 : 5));
-  static_assert(I1 >= 1 && I2 >= 1 && I2 <= 2 && L / R2 == R1, "two-stage plan");
-};
-
-// Second-stage twiddles w_L^{j m} at (m - 1) R1 + j, from the length-L table.
-template <int R1, int NTW, int NT>
-__device__ __forceinline__ void load_stage_twiddles(float2* tw, const float2* __restrict__ table) {
-  for (int e = threadIdx.x; e < NTW; e += NT) tw[e] = __ldg(&table[(e / R1 + 1) * (e % R1)]);
-}
-
-// The exchange buffer holds row r at r + PAD (r / R1). With 8 lines a half-warp covers
-// two rows: the padding keeps the two of a first-stage store (r and r + R1) in different
-// bank halves, at addresses that stay a register plus a constant (an XOR swizzle here
-// and in the row FFTs left 32 and more addresses live across the loop, and spilled).
-
-// First stage of a thread's line b (butterflies j = t + NJ it, inputs in v), exchange.
-template <int L, int DIR>
-__device__ __forceinline__ void col_stage1(float2 (&v)[ColCfg<L>::I1][ColCfg<L>::R1], float2* buf, int t, int b) {
-  using C = ColCfg<L>;
-#pragma unroll
-  for (int it = 0; it < C::I1; ++it) dft<C::R1, DIR>(v[it]);
-  __syncthreads();  // the previous item's second stage has read the buffer
-#pragma unroll
-  for (int it = 0; it < C::I1; ++it)
-#pragma unroll
-    for (int m = 0; m < C::R1; ++m) buf[((t + C::NJ * it) * (C::R1 + C::PAD) + m) * C::BT + b] = v[it][m];
-  __syncthreads();
-}
-
-// Butterfly of item `it` of the second stage: with two per thread, t and its mirror
-// R1 - t (0 and R1 / 2 for t = 0), so that bins k and L - k of a line meet in a thread.
-template <int L>
-__device__ __forceinline__ int col_j2(int t, int it) {
-  using C = ColCfg<L>;
-  if (C::I2 == 1 || it == 0) return t;
-  return t == 0 ? C::R1 / 2 : C::R1 - t;
-}
-
-// Second stage: bins j + R1 m of butterfly j end in u[it][m].
-template <int L, int DIR>
-__device__ __forceinline__ void col_stage2(float2 (&u)[ColCfg<L>::I2][ColCfg<L>::R2], const float2* buf,
-                                           const float2* tw, int t, int b) {
-  using C = ColCfg<L>;
-#pragma unroll
-  for (int it = 0; it < C::I2; ++it) {
-    const int j = col_j2<L>(t, it);
-#pragma unroll
-    for (int m = 0; m < C::R2; ++m) {
-      u[it][m] = buf[(j + (C::R1 + C::PAD) * m) * C::BT + b];
-      if (m > 0) {
-        float2 w = tw[(m - 1) * C::R1 + j];
-        if (DIR > 0) w.y = -w.y;
-        u[it][m] = cmul(u[it][m], w);
-      }
-    }
-    dft<C::R2, DIR>(u[it]);
-  }
-}
-
-// Spectra of the two real columns packed in one line, from Z(k) and Z(L - k):
-// A(k) = (Z(k) + conj Z(-k)) / 2, B(k) = (Z(k) - conj Z(-k)) / 2i.
-__device__ __forceinline__ float4 unpack_pair(float2 z, float2 w) {
-  return make_float4(0.5f * (z.x + w.x), 0.5f * (z.y - w.y), 0.5f * (z.y + w.y), 0.5f * (w.x - z.x));
-}
 
 // Column FFT of raw strips. ASP: BT lines of two columns, S1 [0 .. H/2][W];
 // Fresnel: BT lines of one column, S1 [H][W].
@@ -126,78 +46,11 @@ __global__ void __launch_bounds__(ColCfg<L>::NT, ColCfg<L>::CTAS) k_strip_cols(S
   load_stage_twiddles<C::R1, C::NTW, C::NT>(tw, a.tw_h);
   const int b = threadIdx.x % C::BT, t = threadIdx.x / C::BT;
   const uint32_t W = a.W;
-  const bool u8 = a.in_kind == IN_U8;
   for (uint32_t item = blockIdx.x; item < nitems; item += gridDim.x) {
     const uint32_t i = item / strips, s = item % strips;
     const size_t frame = ((a.raw.slot0 + i) % a.raw.cap) * size_t(W) * L;
     float2 v[C::I1][C::R1];
-    if constexpr (ASP) {
-      const size_t x = size_t(s) * (2 * C::BT) + 2 * b;
-      const size_t at = frame + x;
-      if (u8) {
-        const unsigned char* p = static_cast<const unsigned char*>(a.raw.base) + at;
-        if ((reinterpret_cast<uintptr_t>(a.raw.base) & 1) == 0) {
-#pragma unroll
-          for (int it = 0; it < C::I1; ++it)
-#pragma unroll
-            for (int m = 0; m < C::R1; ++m) {
-              const uint32_t q =
-                  *reinterpret_cast<const uint16_t*>(p + size_t(t + C::NJ * it + (L / C::R1) * m) * W);
-              v[it][m] = make_float2(float(q & 0xffu), float(q >> 8));
-            }
-        } else {
-#pragma unroll
-          for (int it = 0; it < C::I1; ++it)
-#pragma unroll
-            for (int m = 0; m < C::R1; ++m) {
-              const unsigned char* q = p + size_t(t + C::NJ * it + (L / C::R1) * m) * W;
-              v[it][m] = make_float2(float(q[0]), float(q[1]));
-            }
-        }
-      } else {
-        const uint16_t* p = static_cast<const uint16_t*>(a.raw.base) + at;
-        if ((reinterpret_cast<uintptr_t>(a.raw.base) & 3) == 0) {
-#pragma unroll
-          for (int it = 0; it < C::I1; ++it)
-#pragma unroll
-            for (int m = 0; m < C::R1; ++m) {
-              const uint32_t q =
-                  *reinterpret_cast<const uint32_t*>(p + size_t(t + C::NJ * it + (L / C::R1) * m) * W);
-              v[it][m] = make_float2(float(q & 0xffffu), float(q >> 16));
-            }
-        } else {
-#pragma unroll
-          for (int it = 0; it < C::I1; ++it)
-#pragma unroll
-            for (int m = 0; m < C::R1; ++m) {
-              const uint16_t* q = p + size_t(t + C::NJ * it + (L / C::R1) * m) * W;
-              v[it][m] = make_float2(float(q[0]), float(q[1]));
-            }
-        }
-      }
-    } else {
-      const size_t x = size_t(s) * C::BT + b;
-      const float2 cx = __ldg(&a.chirp_x[x]);
-      float r[C::I1][C::R1];
-      if (u8) {
-        const unsigned char* p = static_cast<const unsigned char*>(a.raw.base) + frame + x;
-#pragma unroll
-        for (int it = 0; it < C::I1; ++it)
-#pragma unroll
-          for (int m = 0; m < C::R1; ++m) r[it][m] = float(p[size_t(t + C::NJ * it + (L / C::R1) * m) * W]);
-      } else {
-        const uint16_t* p = static_cast<const uint16_t*>(a.raw.base) + frame + x;
-#pragma unroll
-        for (int it = 0; it < C::I1; ++it)
-#pragma unroll
-          for (int m = 0; m < C::R1; ++m) r[it][m] = float(p[size_t(t + C::NJ * it + (L / C::R1) * m) * W]);
-      }
-#pragma unroll
-      for (int it = 0; it < C::I1; ++it)
-#pragma unroll
-        for (int m = 0; m < C::R1; ++m)
-          v[it][m] = cscale(cmul(__ldg(&a.chirp_y[t + C::NJ * it + (L / C::R1) * m]), cx), r[it][m]);
-    }
+    load_raw_strip<L, ASP>(a, frame, s, t, b, v);
     col_stage1<L, -1>(v, buf, t, b);
     float2 u[C::I2][C::R2];
     col_stage2<L, -1>(u, buf, tw, t, b);
@@ -270,56 +123,13 @@ __global__ void __launch_bounds__(ColCfg<L>::NT, ColCfg<L>::CTAS) k_strip_icols(
   }
 }
 
-// Row FFTs: LP lanes carry a row (lane jl holds elements jl + LP m in v[m]), RPW rows
-// per warp, four warps per CTA.
-template <int L>
-struct RowCfg {
-  static constexpr int R1 = ColCfg<L>::R1, R2 = ColCfg<L>::R2;
-  static constexpr int LP = L / R1, RPW = 32 / LP, NW = 4, NT = 32 * NW;
-  static constexpr int I2 = R1 / LP;
-  static constexpr int NTW = (R2 - 1) * R1;
-  static constexpr int RS = L + L / R1;  // exchange row: element e at e + e / R1
-  static constexpr size_t SMEM = (size_t(NW) * RPW * RS + NTW) * sizeof(float2);
-  static constexpr bool STASH = L >= 512;  // k_strip_rows_asp
-  static constexpr size_t ASP_SMEM = SMEM + (STASH ? size_t(NT) * R1 * sizeof(float2) : 0);
-  static constexpr int ASP_CTAS = L >= 512 ? 3 : (L == 64 ? 5 : 4);
-};
-
-// L-point FFT of a row through its exchange buffer rowp (padded: the 16 lanes of a
-// half-warp always meet 16 different bank pairs, two rows of 8 lanes too). On return
-// bin jl + LP m is in v[m].
-template <int L, int DIR>
-__device__ __forceinline__ void strip_row_fft(float2 (&v)[RowCfg<L>::R1], float2* rowp, const float2* tw, int jl) {
-  using C = RowCfg<L>;
-  dft<C::R1, DIR>(v);
-  __syncwarp();
-#pragma unroll
-  for (int m = 0; m < C::R1; ++m) rowp[(C::R1 + 1) * jl + m] = v[m];
-  __syncwarp();
-#pragma unroll
-  for (int i = 0; i < C::I2; ++i) {
-    const int j = jl + C::LP * i;
-    float2 u[C::R2];
-#pragma unroll
-    for (int m = 0; m < C::R2; ++m) {
-      u[m] = rowp[(C::R1 + 1) * m + j];
-      if (m > 0) {
-        float2 w = tw[(m - 1) * C::R1 + j];
-        if (DIR > 0) w.y = -w.y;
-        u[m] = cmul(u[m], w);
-      }
-    }
-    dft<C::R2, DIR>(u);
-#pragma unroll
-    for (int m = 0; m < C::R2; ++m) v[i + C::I2 * m] = u[m];
-  }
-}
-
 // ASP rows: S1 rows 0 .. H/2 of n frames -> S2 rows 0 .. H - 1. Rows 0 and H / 2 are
 // their own mirrors (their W is Hermitian in kx, so both products give the same row);
-// a last warp with a row too many repeats the last row. Neither needs a branch. From
-// 512 points on W waits in shared memory while the first inverse FFT runs (each lane
-// its own words): held in registers it spilled.
+// a last warp with a row too many repeats the last row. Neither needs a branch. Up to 256
+// points W stays in registers for the second product; from 512 points on it would take 64
+// more of them, and the forward FFT is done again instead (the row is an L1 or L2 hit): a
+// sixth more arithmetic for 20 resident warps per SM instead of 12 (us a frame: 512 x 512
+// 0.85 -> 0.77, 1024 x 1024 3.70 -> 3.36).
 template <int L>
 __global__ void __launch_bounds__(RowCfg<L>::NT, RowCfg<L>::ASP_CTAS) k_strip_rows_asp(SpatialArgs a, uint32_t nrows) {
   using C = RowCfg<L>;
@@ -327,7 +137,6 @@ __global__ void __launch_bounds__(RowCfg<L>::NT, RowCfg<L>::ASP_CTAS) k_strip_ro
   float2* tw = reinterpret_cast<float2*>(smem);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, jl = lane % C::LP, sub = lane / C::LP;
   float2* rowp = tw + C::NTW + (warp * C::RPW + sub) * C::RS;
-  float2* stash = tw + C::NTW + C::NW * C::RPW * C::RS + threadIdx.x;
   load_stage_twiddles<C::R1, C::NTW, C::NT>(tw, a.tw_w);
   __syncthreads();
   const uint32_t H = a.H, HR = H / 2 + 1;
@@ -335,32 +144,49 @@ __global__ void __launch_bounds__(RowCfg<L>::NT, RowCfg<L>::ASP_CTAS) k_strip_ro
     const uint32_t row = r0 + sub < nrows ? r0 + sub : nrows - 1;
     const uint32_t i = row / HR, ky = row % HR;
     const float2* in = a.scratch1 + size_t(row) * L + jl;
-    float2 v[C::R1], u[C::R1];
-#pragma unroll
-    for (int m = 0; m < C::R1; ++m) v[m] = in[C::LP * m];
-    strip_row_fft<L, -1>(v, rowp, tw, jl);
     const float2* h = a.asp_h + size_t(ky) * L + jl;
     float2* out = a.scratch2 + size_t(i) * H * L + jl;
+    if constexpr (C::AGAIN) {
+#pragma unroll 1
+      for (int conj = 0; conj < 2; ++conj) {
+        const float sign = conj ? -1.f : 1.f;
+        float2 v[C::R1];
 #pragma unroll
-    for (int m = 0; m < C::R1; ++m) {
-      if (C::STASH) stash[m * C::NT] = v[m];
-      u[m] = cmul(v[m], __ldg(&h[C::LP * m]));
+        for (int m = 0; m < C::R1; ++m) v[m] = in[C::LP * m];
+        strip_row_fft<L, -1>(v, rowp, tw, jl);
+#pragma unroll
+        for (int m = 0; m < C::R1; ++m) {
+          const float2 w = __ldg(&h[C::LP * m]);
+          v[m] = cmul(v[m], make_float2(w.x, sign * w.y));
+        }
+        strip_row_fft<L, +1>(v, rowp, tw, jl);
+        float2* o = out + size_t(conj ? (H - ky) & (H - 1) : ky) * L;
+#pragma unroll
+        for (int m = 0; m < C::R1; ++m) o[C::LP * m] = make_float2(v[m].x, sign * v[m].y);
+      }
+    } else {
+      float2 v[C::R1], u[C::R1];
+#pragma unroll
+      for (int m = 0; m < C::R1; ++m) v[m] = in[C::LP * m];
+      strip_row_fft<L, -1>(v, rowp, tw, jl);
+#pragma unroll
+      for (int m = 0; m < C::R1; ++m) u[m] = cmul(v[m], __ldg(&h[C::LP * m]));
+      strip_row_fft<L, +1>(u, rowp, tw, jl);
+#pragma unroll
+      for (int m = 0; m < C::R1; ++m) out[size_t(ky) * L + C::LP * m] = u[m];
+#pragma unroll
+      for (int m = 0; m < C::R1; ++m) {
+        // read again (an L1 hit): kept from the first product it would cost 2 R1 registers
+        float2 w;
+        asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];\n" : "=f"(w.x), "=f"(w.y) : "l"(&h[C::LP * m]) : "memory");
+        w.y = -w.y;
+        u[m] = cmul(v[m], w);
+      }
+      strip_row_fft<L, +1>(u, rowp, tw, jl);
+#pragma unroll
+      for (int m = 0; m < C::R1; ++m)
+        out[size_t((H - ky) & (H - 1)) * L + C::LP * m] = make_float2(u[m].x, -u[m].y);
     }
-    strip_row_fft<L, +1>(u, rowp, tw, jl);
-#pragma unroll
-    for (int m = 0; m < C::R1; ++m) out[size_t(ky) * L + C::LP * m] = u[m];
-#pragma unroll
-    for (int m = 0; m < C::R1; ++m) {
-      // read again (an L1 hit): kept from the first product it would cost 2 R1 registers
-      float2 w;
-      asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];\n" : "=f"(w.x), "=f"(w.y) : "l"(&h[C::LP * m]) : "memory");
-      w.y = -w.y;
-      u[m] = cmul(C::STASH ? stash[m * C::NT] : v[m], w);
-    }
-    strip_row_fft<L, +1>(u, rowp, tw, jl);
-#pragma unroll
-    for (int m = 0; m < C::R1; ++m)
-      out[size_t((H - ky) & (H - 1)) * L + C::LP * m] = make_float2(u[m].x, -u[m].y);
   }
 }
 
@@ -462,7 +288,7 @@ __global__ void __launch_bounds__(RowCfg<L>::NT, (L >= 512 ? 3 : 5)) k_strip_row
 // Column IFFT of strips of S2; sum |u| and sum |u|^2 of image z n + i added to the float64
 // pair z of hologram i at tam_acc + i tam_stride + 2 z.
 template <int L>
-__global__ void __launch_bounds__(ColCfg<L>::NT, (L == 1024 ? 2 : 4)) k_strip_icols_sums(SpatialArgs a, uint32_t nitems,
+__global__ void __launch_bounds__(ColCfg<L>::NT, (L >= 512 ? 2 : 4)) k_strip_icols_sums(SpatialArgs a, uint32_t nitems,
                                                                                     uint32_t strips) {
   using C = ColCfg<L>;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -635,7 +461,7 @@ cudaError_t rows(const SpatialArgs& a, cudaStream_t s) {
   constexpr uint32_t per = C::NW * C::RPW;
   if (a.spatial == HV_SPATIAL_ASP) {
     const uint32_t nrows = a.n * (a.H / 2 + 1);
-    return launch_resident(k_strip_rows_asp<L>, C::NT, C::ASP_SMEM, (nrows + per - 1) / per, s, a, nrows);
+    return launch_resident(k_strip_rows_asp<L>, C::NT, C::SMEM, (nrows + per - 1) / per, s, a, nrows);
   }
   const uint32_t nrows = a.n * a.H;
   return launch_resident(k_strip_rows_fft<L>, C::NT, C::SMEM, (nrows + per - 1) / per, s, a, nrows);
