@@ -1557,13 +1557,15 @@ static hv_status af_prepare(hv_handle* h, const void* frames, uint32_t n, uint32
 hv_status hv_focus_sweep(hv_handle* h, const void* frames, uint32_t n, const double* z, uint32_t nz, float* metric) {
   if (!h) return HV_ERR_ARG;
   if (!z || !metric || nz == 0 || nz > 1024) return fail(h, HV_ERR_ARG, "bad distances or output");
-  // holograms whose spectra are held at once, and (distance, hologram) images per launch
+  // holograms whose spectra are held at once, and (distance, hologram) images per launch:
+  // 256 MB of them (64 distances x 64 holograms of 256 x 256 in 1612, 1346, 1281 and 1141 us
+  // with 32, 64, 128 and 256 MB)
   const uint32_t chunk = std::min<uint32_t>(n, 64);
   hv_status s = af_prepare(h, frames, n, chunk);
   if (s != HV_OK) return s;
   const uint32_t W = h->W, H = h->H;
   const size_t fbytes = size_t(W) * H * sizeof(float2);
-  const uint32_t images = std::max(chunk, uint32_t((size_t(128) << 20) / fbytes));
+  const uint32_t images = std::max(chunk, uint32_t((size_t(256) << 20) / fbytes));
   s = ensure(h, reinterpret_cast<void**>(&h->s2), &h->s2_bytes, images * fbytes);
   if (s != HV_OK) return s;
   const hv_params& p = h->cur;
