@@ -540,8 +540,8 @@ def roofline(w, res, peaks):
     if t_tm >= t_sp:
         flops = alg["stft_flops"] * frames_per_render
         byts = alg["stft_bytes"] * frames_per_render
-        names = {1: "k_stft_warp", 2: "k_stft_win", 3: "k_stft_win (wide)", 4: "k_stft_winp", 5: "k_stft_wt",
-                 6: "k_stft_wtp"}
+        win = "k_stft_px" if w["T"] <= 32 else "k_stft_cols"
+        names = {1: "k_stft_warp", 2: win, 3: win, 4: win, 5: "k_stft_wt", 6: "k_stft_wtp"}
         sk = (res.get("tuning") or {}).get("stft_kernel")
         kern, t = f"{names.get(sk, 'k_stft_warp')} (time FFT + band moments)", t_tm
     else:
@@ -566,11 +566,10 @@ def roofline(w, res, peaks):
             traffic = int(v * (frames_per_render + ov) / (1024 + ov))
             traffic_per = "launch of the STFT kernel (1,024-frame ncu capture scaled to the launch's frames)"
     if (t_tm >= t_sp and w["T"] == 512 and w["N"] == 256 and w["S"] == 512
-            and tun.get("stft_kernel") in (2, 5)):
-        # window STFT (window-per-CTA, or TMA-fed): a 1,024-frame launch captured,
-        # traffic in proportion to the frames
-        prof = "stft_wt_512_asp_256.md" if tun.get("stft_kernel") == 5 else "stft_win_512_asp_256.md"
-        v = profiled_traffic(prof, ["k_stft.cu", "fft_dev.cuh"])
+            and tun.get("stft_kernel") == 5):
+        # TMA-fed window STFT: a 1,024-frame launch captured, traffic in proportion to
+        # the frames
+        v = profiled_traffic("stft_wt_512_asp_256.md", ["k_stft.cu", "fft_dev.cuh"])
         if v is not None:
             traffic = int(v * frames_per_render / 1024)
             traffic_per = "render (the STFT launch; 1,024-frame ncu capture scaled to the render's frames)"

@@ -110,12 +110,12 @@ typedef struct {
                                  radius sqrt((m/W)^2 + (n/H)^2) in cycles per pixel is
                                  below this cutoff are zeroed; 0 = off. Folded into
                                  the transfer function. */
-  int32_t stft_kernel;        /* STFT kernel for windows that do not overlap (S >= T):
+  int32_t stft_kernel;        /* STFT kernel for windows that do not overlap (S >= T;
+                                 overlapping windows take the walking kernel unless 0):
                                  0 = automatic (the autotuner's choice when tuned = 1,
                                  else the walking kernel launched once per window),
-                                 HV_STFT_WALK, HV_STFT_WINDOW, HV_STFT_WINDOW_WIDE,
-                                 HV_STFT_WINDOW_PIPELINED (persistent CTAs that load
-                                 their next window tile while transforming one),
+                                 HV_STFT_WALK, HV_STFT_WINDOW (HV_STFT_WINDOW_WIDE and
+                                 HV_STFT_WINDOW_PIPELINED run the same kernel),
                                  HV_STFT_WINDOW_TMA or HV_STFT_WINDOW_TMA_PIPELINED
                                  (T = 512: a window tile brought in by TMA tensor
                                  loads and transformed in place; the second
@@ -215,16 +215,15 @@ typedef struct {
                                        applicable)                                    */
   float stft_us_per_window[6];      /* measured us per window of the STFT kernels:
                                        walking (CTAs walk every window of their
-                                       pixels), one CTA per (window, pixel tile), the
-                                       same with twice the pixels per CTA, persistent
-                                       double-buffered CTAs over the (window, tile)
-                                       items, the TMA-fed kernel, the same persistent
-                                       and double-buffered; 0 where not applicable
-                                       (all but the first need S >= T, the last two
-                                       T = 512)                                       */
+                                       pixels), the window kernel (its time also for
+                                       the wide and the pipelined selection), the
+                                       TMA-fed kernel, the same persistent and
+                                       double-buffered; 0 where not applicable (the
+                                       last two need S >= T = 512)                    */
 } hv_tuning;
 
-/* STFT kernels the autotuner chooses between (windows that do not overlap). */
+/* STFT kernels; the autotuner chooses between WALK and WINDOW and, where windows do not
+ * overlap and T = 512, the TMA-fed two. */
 enum { HV_STFT_WALK = 1, HV_STFT_WINDOW = 2, HV_STFT_WINDOW_WIDE = 3, HV_STFT_WINDOW_PIPELINED = 4,
        HV_STFT_WINDOW_TMA = 5, HV_STFT_WINDOW_TMA_PIPELINED = 6 };
 

@@ -60,7 +60,7 @@ struct hv_handle {
   int sp_cluster = 0;         // 1: whole-frame cluster kernel
   int sp_fused = 0;           // 1: fused transform (s1 / s2 are rings of kFusedRing frames)
   int inject = HV_INJECT_NONE;  // pending fault injection (hv_debug_inject)
-  int stft_kernel = STFT_AUTO;  // STFT kernel for windows that do not overlap (autotuner's choice)
+  int stft_kernel = STFT_WINDOW;  // the settings' STFT kernel, or the autotuner's choice
   unsigned* fused_ctr = nullptr;  // its ticket and per-slot counters
   size_t fused_ctr_bytes = 0;
   hv_tuning tuning{};
@@ -544,18 +544,16 @@ hv_status apply_pending(hv_handle* h) {
   h->tuning.spatial_kernel = p.spatial_kernel == HV_SK_AUTO ? HV_SK_MULTIPASS : int32_t(p.spatial_kernel);
   // STFT kernel for windows that do not overlap: the caller's, the autotuner's (tuned),
   // else the walking kernel launched once per window (the plain form)
-  h->stft_kernel = p.stft_kernel == HV_STFT_WINDOW ? STFT_AUTO
-                   : p.stft_kernel == HV_STFT_WINDOW_WIDE     ? STFT_WIDE
-                   : p.stft_kernel == HV_STFT_WINDOW_PIPELINED ? STFT_PIPE
-                   : p.stft_kernel == HV_STFT_WINDOW_TMA       ? STFT_TMA
+  h->stft_kernel = p.stft_kernel == 0 || p.stft_kernel == HV_STFT_WALK     ? STFT_WALK
+                   : p.stft_kernel == HV_STFT_WINDOW_TMA           ? STFT_TMA
                    : p.stft_kernel == HV_STFT_WINDOW_TMA_PIPELINED ? STFT_TMA_PIPE
-                                                               : STFT_WALK;
+                                                                   : STFT_WINDOW;
   if (p.tuned && p.spatial_kernel == HV_SK_AUTO) {
     s = tune_spatial(h);  // rewrites the tuning record
     if (s != HV_OK) return s;
   }
   h->tuning.stft_kernel = p.stft_kernel == 0 ? HV_STFT_WALK : p.stft_kernel;
-  if (p.tuned && p.stft_kernel == 0 && p.temporal == HV_TEMPORAL_STFT && d.S >= d.T) {
+  if (p.tuned && p.stft_kernel == 0 && p.temporal == HV_TEMPORAL_STFT) {
     s = tune_temporal(h);
     if (s != HV_OK) return s;
   }
@@ -774,16 +772,21 @@ hv_status tune_spatial(hv_handle* h) {
   return HV_OK;
 }
 
-// Autotuner of the STFT for windows that do not overlap (S >= T): times the
-// walking kernel (CTAs walk every window of their pixels), the kernels with one
-// CTA per (window, pixel tile) (plain, wide, persistent double-buffered) and, at
-// T = 512, the TMA-fed ones (one CTA per item, persistent double-buffered) on the
-// handle's time queue (its contents are being flushed, so any values do) and
-// keeps the fastest.
+// Autotuner of the STFT: times the walking kernel (CTAs walk every window of their
+// pixels), the window kernel and, at T = 512 and S >= T, the TMA-fed ones (one CTA per
+// item, persistent double-buffered) on the handle's time queue (its contents are being
+// flushed, so any values do) and keeps the fastest. The wide and the pipelined selections
+// run the window kernel and carry its time.
 hv_status tune_temporal(hv_handle* h) {
   const uint32_t T = h->T, S = h->S;
-  const uint32_t nwin = std::min<uint32_t>(16, (h->Q - T) / S + 1);
+  const bool overlap = S < T;
   const size_t hw = size_t(h->W) * h->H;
+  // 16 windows; where they overlap as many as a render has (the walking kernel's first
+  // window weighs less then), within 256 MB of images
+  uint32_t nwin = std::min<uint32_t>(16, (h->Q - T) / S + 1);
+  if (overlap)
+    nwin = std::min<uint32_t>((h->Q - T) / S + 1,
+                              std::max<uint32_t>(nwin, std::min<uint32_t>(64, uint32_t((size_t(64) << 20) / (h->nout * hw)))));
   float* out = nullptr;
   HV_CU(h, cudaMalloc(&out, size_t(nwin) * h->nout * hw * sizeof(float)));
   cudaEvent_t e0, e1;
@@ -804,14 +807,17 @@ hv_status tune_temporal(hv_handle* h) {
   sa.nout = h->nout;
   sa.out = out;
   sa.err = h->dev_err;
-  const int kinds[6] = {STFT_WALK, STFT_AUTO, STFT_WIDE, STFT_PIPE, STFT_TMA, STFT_TMA_PIPE};
+  const int window = overlap ? STFT_OVERLAP : STFT_WINDOW;
+  const int kinds[6] = {STFT_WALK, window, window, window, STFT_TMA, STFT_TMA_PIPE};
   float best = 1e30f;
-  int best_kind = STFT_AUTO;
+  int best_kind = STFT_WALK;
   hv_status st = HV_OK;
   for (int ci = 0; ci < 6 && st == HV_OK; ++ci) {
-    // the TMA-fed kernels exist for T = 512 only (elsewhere they would time the
-    // window-per-CTA kernel again)
-    if ((kinds[ci] == STFT_TMA || kinds[ci] == STFT_TMA_PIPE) && T != 512) continue;
+    if (ci == 2 || ci == 3) {
+      h->tuning.stft_us_per_window[ci] = h->tuning.stft_us_per_window[1];
+      continue;
+    }
+    if (ci > 3 && (T != 512 || overlap)) continue;  // no such kernels there
     sa.kernel = kinds[ci];
     int launches = 0;
     cudaError_t e = launch_stft(sa, h->stream, &launches);  // warm-up
@@ -838,8 +844,6 @@ hv_status tune_temporal(hv_handle* h) {
   if (st != HV_OK) return st;
   h->stft_kernel = best_kind;
   h->tuning.stft_kernel = best_kind == STFT_WALK       ? HV_STFT_WALK
-                          : best_kind == STFT_WIDE     ? HV_STFT_WINDOW_WIDE
-                          : best_kind == STFT_PIPE     ? HV_STFT_WINDOW_PIPELINED
                           : best_kind == STFT_TMA      ? HV_STFT_WINDOW_TMA
                           : best_kind == STFT_TMA_PIPE ? HV_STFT_WINDOW_TMA_PIPELINED
                                                        : HV_STFT_WINDOW;

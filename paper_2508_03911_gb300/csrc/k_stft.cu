@@ -3,7 +3,7 @@
 // For every pixel p and window w (frames wS .. wS+T-1 of the time queue):
 //   S_k(p) = sum_t U_{wS+t}(p) exp(-2 pi i k t / T),   P_k = |S_k|^2,
 //   M0 = sum_{k=klo..khi} P_k,  M1 = sum f_k P_k,  M2 = sum f_k^2 P_k  (f_k in kHz),
-//   M1N = M1 / M0 and M2N = sqrt(M2 / M0) in float64 (0 where M0 = 0).
+//   M1N = M1 / M0 and M2N = sqrt(M2 / M0) to float64's float32 results (0 where M0 = 0).
 //
 // One CTA owns BT adjacent pixels and walks all windows of the launch, so
 // overlapping windows (S < T) load each propagated frame from HBM once per
@@ -14,9 +14,8 @@
 #include <cudaTypedefs.h>
 
 #include <mutex>
-#include <type_traits>
 
-#include "fft_dev.cuh"
+#include "strip_dev.cuh"
 #include "hv_internal.h"
 #include "../../include/hv.h"
 
@@ -57,8 +56,6 @@ __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 // all but the newest N committed groups complete
-template <int N>
-__device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 __device__ __forceinline__ int wpad(int i) { return i + (i >> 4); }
 
@@ -185,7 +182,7 @@ __device__ __forceinline__ void add_moments(const float2* v, int it, float kb, M
 // of its group (jl = lane within the group): stage 1 reads the window (T
 // samples from `win`, in order), later stages the pixel's work row; the last
 // stage feeds the moment sums.
-template <int T, int NS, int LP, bool WP = false>
+template <int T, int NS, int LP>
 __device__ __forceinline__ void warp_fft(const float2* win, float2* work, const float2* tw, int jl,
                                          MomAcc& acc, bool lower) {
   // WP: the window itself is stored padded (sample t at t + t / 16)
@@ -200,7 +197,7 @@ __device__ __forceinline__ void warp_fft(const float2* win, float2* work, const 
 #pragma unroll
     for (int m = 0; m < R; ++m) {
       const int t = j + m * NB;
-      if constexpr (NS == 1) v[it][m] = WP ? win[wpad(t)] : win[t];
+      if constexpr (NS == 1) v[it][m] = win[t];
       else v[it][m] = work[wpad(t)];
     }
     if constexpr (NS > 1) {
@@ -238,7 +235,7 @@ __device__ __forceinline__ void warp_fft(const float2* win, float2* work, const 
       for (int m = 0; m < R; ++m) work[wpad(base + m * NS)] = v[it][m];
     }
     __syncwarp();
-    warp_fft<T, NS * R, LP, WP>(win, work, tw, jl, acc, lower);
+    warp_fft<T, NS * R, LP>(win, work, tw, jl, acc, lower);
   }
 }
 
@@ -288,9 +285,29 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity) {
   }
 }
 
+// float(double(a) / double(b)): the float32 quotient is the same number, since float64 keeps
+// more than twice float32's digits and two bits (results below the normal range apart, which
+// float64 rounds twice). Float64 instructions run at 1/64 of the float32 rate, and one lane
+// in 4 to 16 writes: M1N and M2N took 0.1 ms per window of 1024 x 512 in float64.
+__device__ __forceinline__ float quotient(float a, float b) { return __fdiv_rn(a, b); }
+
+// float(sqrt(double(a) / double(b))) for a >= 0, b > 0: the quotient as a float32 pair (its
+// remainder exact by fma), one Newton step of the root on the pair; the float64 form
+// outside the range where the pair holds.
+__device__ __forceinline__ float root_of_quotient(float a, float b) {
+  const float q = __fdiv_rn(a, b);
+  if (!(a > 1e-25f && b > 1e-25f && b < 1e25f && q > 1e-25f && q < 1e25f)) {
+    const double r = double(a) / double(b);
+    return float(sqrt(r > 0.0 ? r : 0.0));
+  }
+  const float lo = __fdiv_rn(fmaf(-q, b, a), b);
+  const float s = __fsqrt_rn(q);
+  return fmaf(0.5f * __frcp_rn(s), fmaf(-s, s, q) + lo, s);
+}
+
 // Post-processing fused into the moment epilogue: the moments of pixel `pix` for
 // window w, from the lane group's reduced sums (held by its lane jl = 0, the
-// writer) -- M0, M1, M2 (bins -> kHz), then M1N and M2N in float64, in that order
+// writer) -- M0, M1, M2 (bins -> kHz), then M1N and M2N, in that order
 // among those the mask asks for -- to the image ring slot of the window (or to
 // out [w][image][pixel] without a ring), adding each image's sum over the warp's
 // pixels into one of the slot's partial sums. Called by every lane of the warp
@@ -305,14 +322,8 @@ __device__ __forceinline__ void emit_moments(const StftArgs& a, uint32_t w, size
   v[0] = acc.m0;
   v[1] = acc.m1 * a.fscale;
   v[2] = acc.m2 * (a.fscale * a.fscale);
-  const double d0 = acc.m0;
-  v[3] = 0.f;
-  v[4] = 0.f;
-  if (a.mask & HV_MOM_M1N) v[3] = d0 > 0.0 ? float(double(v[1]) / d0) : 0.f;
-  if (a.mask & HV_MOM_M2N) {
-    const double r = d0 > 0.0 ? double(v[2]) / d0 : 0.0;
-    v[4] = float(sqrt(r > 0.0 ? r : 0.0));
-  }
+  v[3] = (a.mask & HV_MOM_M1N) && v[0] > 0.f ? quotient(v[1], v[0]) : 0.f;
+  v[4] = (a.mask & HV_MOM_M2N) && v[0] > 0.f ? root_of_quotient(v[2], v[0]) : 0.f;
   uint32_t slot = 0;
   float* o;
   if (a.post_ring) {
@@ -516,235 +527,172 @@ __global__ void __launch_bounds__(WarpLayout<T>::NT, (T <= 512 ? 3 : 1))
       if (a.mask & HV_MOM_M0) o[HW * q++] = acc.m0;
       if (a.mask & HV_MOM_M1) o[HW * q++] = m1;
       if (a.mask & HV_MOM_M2) o[HW * q++] = m2;
-      const double d0 = acc.m0;
-      if (a.mask & HV_MOM_M1N) o[HW * q++] = d0 > 0.0 ? float(double(m1) / d0) : 0.f;
-      if (a.mask & HV_MOM_M2N) {
-        const double r = d0 > 0.0 ? double(m2) / d0 : 0.0;
-        o[HW * q++] = float(sqrt(r > 0.0 ? r : 0.0));
-      }
+      if (a.mask & HV_MOM_M1N) o[HW * q++] = acc.m0 > 0.f ? quotient(m1, acc.m0) : 0.f;
+      if (a.mask & HV_MOM_M2N) o[HW * q++] = acc.m0 > 0.f ? root_of_quotient(m2, acc.m0) : 0.f;
     }
   }
 }
 
-// Windows that do not overlap (S >= T): one CTA per (window, tile of BT pixels),
-// so that many windows are in flight per SM instead of one CTA walking all
-// windows of its pixels. The window's T frames of the CTA's pixels land by
-// cp.async straight in the pixels' padded work rows (sample t at t + t / 16; the
-// row stride adds two more values so that the eight rows of a CTA start in
-// different banks), and the FFT runs in place there: the first stage reads the
-// whole row into registers before any lane of the pixel writes. A CTA holds one
-// window, so its shared memory is a quarter of the walking kernel's and several
-// CTAs share an SM.
-template <int T, bool WIDE = false>
-struct WinCfg {
-  using Lw = WarpLayout<T>;
-  // warps per CTA: 8 for short windows (a warp's fetch covers 32 pixels, 256
-  // contiguous bytes of a frame), else the walking kernel's count; WIDE doubles
-  // it (twice the pixels per CTA: longer contiguous runs of each frame)
-  static constexpr int NW = (T <= 128 ? 8 : Lw::NW) * (WIDE ? 2 : 1);
-  static constexpr int NT = 32 * NW;
-  static constexpr int BT = NW * Lw::PW;  // pixels per CTA
-  // row stride (float2): the padded row, rounded to 1 mod 16 so that the rows of
-  // consecutive pixels start in consecutive bank pairs
-  static constexpr int WR = (T + T / 16 + 15) / 16 * 16 + 1;
-  static constexpr int OCC = WIDE ? (T >= 512 ? 2 : 2) : (T >= 1024 ? 1 : (T >= 512 ? 4 : (T >= 256 ? 6 : 4)));
-  static constexpr size_t bytes() { return (size_t(BT) * WR + (T - WarpPlan<T>::R1)) * sizeof(float2); }
-};
-
-template <int T, bool WIDE, bool POST>
-__global__ void __launch_bounds__(WinCfg<T, WIDE>::NT, WinCfg<T, WIDE>::OCC) k_stft_win(StftArgs a) {
-  using Lw = WarpLayout<T>;
-  using Wc = WinCfg<T, WIDE>;
-  constexpr int NT = Wc::NT, LP = Lw::LP, PW = Lw::PW, BT = Wc::BT, WR = Wc::WR;
-  extern __shared__ __align__(16) unsigned char smem_win[];
-  float2* rows = reinterpret_cast<float2*>(smem_win);
-  float2* tw = rows + BT * WR;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int pl = lane / LP, jl = lane % LP;
-  const int px = warp * PW + pl;
+// Writes the moments of one pixel (sums in bins) of window w.
+__device__ __forceinline__ void store_moments(const StftArgs& a, uint32_t w, size_t pix, const MomAcc& acc) {
   const size_t HW = size_t(a.W) * a.H;
-  const uint32_t ntile = uint32_t(HW / BT);
-  const uint32_t w = blockIdx.x / ntile;
-  const uint32_t p0 = (blockIdx.x % ntile) * BT;
-  const float2* tq = static_cast<const float2*>(a.tq.base);
-  const uint32_t cap = a.tq.cap;
-  // the window's frames: queue slots slot0 + w S + f (one wrap at most)
-  {
-    constexpr int FS = NT / BT;  // frames per pass of the CTA
-    const int b = tid % BT;
-    int f = tid / BT;
-    uint32_t g = a.tq.slot0 + w * a.S + uint32_t(f);
-    while (g >= cap) g -= cap;
-    for (; f < T; f += FS) {
-      cp_async8(&rows[b * WR + wpad(f)], &tq[size_t(g) * HW + p0 + b]);
-      g += FS;
-      if (g >= cap) g -= cap;
-    }
-    cp_async_commit();
-  }
-  {  // stage twiddles (the walking kernel's table layout)
-    constexpr int R1 = WarpPlan<T>::R1;
-    int NS = R1;
-    while (NS < T) {
-      const int rem = T / NS;
-      const int R = WarpPlan<T>::R2 != 0 ? WarpPlan<T>::R2 : (rem % 8 == 0 ? 8 : (rem % 4 == 0 ? 4 : 2));
-      for (int idx = tid; idx < (R - 1) * NS; idx += NT) {
-        const int m = idx / NS + 1, jm = idx % NS;
-        tw[(NS - R1) + idx] = a.tw_t[jm * m * (T / (NS * R))];
-      }
-      NS *= R;
-    }
-  }
-  uint32_t band = 0;
-  {
-    constexpr int RL = Lw::RL, NBL = T / RL;
-#pragma unroll
-    for (int it = 0; it < Lw::ITL; ++it)
-#pragma unroll
-      for (int m = 0; m < RL; ++m) {
-        const uint32_t k = uint32_t(jl + LP * it + m * NBL);
-        if (k - a.klo <= a.khi - a.klo) band |= 1u << (it * RL + m);
-      }
-  }
-  cp_async_wait_all();
-  __syncthreads();
-  const bool lower = a.khi < uint32_t(T / 2);
-  MomAcc acc{band, 0.f, 0.f, 0.f};
-  float2* row = rows + px * WR;
-  warp_fft<T, 1, LP, true>(row, row, tw, jl, acc, lower);
-#pragma unroll
-  for (int o = LP / 2; o > 0; o >>= 1) {
-    acc.m0 += __shfl_xor_sync(0xffffffffu, acc.m0, o);
-    acc.m1 += __shfl_xor_sync(0xffffffffu, acc.m1, o);
-    acc.m2 += __shfl_xor_sync(0xffffffffu, acc.m2, o);
-  }
-  if constexpr (POST) {
-    emit_moments(a, w, p0 + px, acc, jl == 0, true);
-  } else if (jl == 0) {
-    const float m1 = acc.m1 * a.fscale, m2 = acc.m2 * (a.fscale * a.fscale);  // bins -> kHz
-    float* o = a.out + size_t(w) * a.nout * HW + p0 + px;
-    int q = 0;
-    if (a.mask & HV_MOM_M0) __stcs(&o[HW * q++], acc.m0);
-    if (a.mask & HV_MOM_M1) __stcs(&o[HW * q++], m1);
-    if (a.mask & HV_MOM_M2) __stcs(&o[HW * q++], m2);
-    const double d0 = acc.m0;
-    if (a.mask & HV_MOM_M1N) __stcs(&o[HW * q++], d0 > 0.0 ? float(double(m1) / d0) : 0.f);
-    if (a.mask & HV_MOM_M2N) {
-      const double r = d0 > 0.0 ? double(m2) / d0 : 0.0;
-      __stcs(&o[HW * q++], float(sqrt(r > 0.0 ? r : 0.0)));
-    }
-  }
+  const float m1 = acc.m1 * a.fscale, m2 = acc.m2 * (a.fscale * a.fscale);  // bins -> kHz
+  float* o = a.out + size_t(w) * a.nout * HW + pix;
+  int q = 0;
+  if (a.mask & HV_MOM_M0) __stcs(&o[HW * q++], acc.m0);
+  if (a.mask & HV_MOM_M1) __stcs(&o[HW * q++], m1);
+  if (a.mask & HV_MOM_M2) __stcs(&o[HW * q++], m2);
+  if (a.mask & HV_MOM_M1N) __stcs(&o[HW * q++], acc.m0 > 0.f ? quotient(m1, acc.m0) : 0.f);
+  if (a.mask & HV_MOM_M2N) __stcs(&o[HW * q++], acc.m0 > 0.f ? root_of_quotient(m2, acc.m0) : 0.f);
 }
 
-// The window-per-CTA kernel made persistent and double-buffered: CTA c takes the
-// (window, pixel tile) items c, c + grid, ... and issues the cp.async copies of its
-// next item's frames into the other buffer before it transforms the current one,
-// so that its loads overlap its own FFT instead of only other CTAs'. Two padded
-// buffers per CTA: fewer CTAs per SM than the one-item kernel (3 at T = 512).
+// In-band bits of bins kb + NB m, m < R, from bit `at` on.
+template <int R, int NB>
+__device__ __forceinline__ uint32_t band_bits(const StftArgs& a, uint32_t kb, int at) {
+  uint32_t band = 0;
+#pragma unroll
+  for (int m = 0; m < R; ++m)
+    if (kb + uint32_t(m * NB) - a.klo <= a.khi - a.klo) band |= 1u << (at + m);
+  return band;
+}
+
+// Windows that do not overlap (S >= T), or overlap little enough that reading the shared
+// frames again, from L2 for the most part, costs less than the walking kernel's moves (the
+// autotuner times both). One thread per (window, pixel) for T <= 32, one CTA per (window,
+// tile of BT pixels) above: the frames come straight from the queue to registers (whole
+// 64- or 128-byte runs of a frame, up to 32 of them in flight per thread) and are transformed
+// there, with one exchange through shared memory for T >= 64 and none below, as in the
+// spatial passes. Bound by the queue's reads; where windows overlap, by L2's. (Frames
+// copied to padded rows in shared memory, in 1 or 2 buffers, and transformed there by one
+// warp per row were slower at every T: 86 windows of 1024 x 512, T = 128, S = 48, took 1.69 ms
+// walking and 1.00 this way; 512 windows of 256 x 256, T = 32, S = 8, 3.1 and 0.89.)
 template <int T, bool POST>
-__global__ void __launch_bounds__(WinCfg<T, false>::NT, 1) k_stft_winp(StftArgs a) {
-  using Lw = WarpLayout<T>;
-  using Wc = WinCfg<T, false>;
-  constexpr int NT = Wc::NT, LP = Lw::LP, PW = Lw::PW, BT = Wc::BT, WR = Wc::WR;
-  extern __shared__ __align__(16) unsigned char smem_winp[];
-  float2* rows0 = reinterpret_cast<float2*>(smem_winp);  // buffer b at rows0 + b BT WR
-  float2* tw = rows0 + 2 * BT * WR;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int pl = lane / LP, jl = lane % LP;
-  const int px = warp * PW + pl;
+__global__ void __launch_bounds__(256) k_stft_px(StftArgs a) {
+  const uint32_t HW = a.W * a.H;  // a multiple of 256
+  const uint32_t blocks = HW / 256, w = blockIdx.x / blocks, p = (blockIdx.x % blocks) * 256 + threadIdx.x;
+  const float2* tq = static_cast<const float2*>(a.tq.base) + p;
+  uint32_t g = a.tq.slot0 + w * a.S;
+  while (g >= a.tq.cap) g -= a.tq.cap;
+  float2 v[T];
+#pragma unroll
+  for (int t = 0; t < T; ++t) {
+    v[t] = tq[size_t(g) * HW];
+    if (++g == a.tq.cap) g = 0;
+  }
+  MomAcc acc{band_bits<T, 1>(a, 0, 0), 0.f, 0.f, 0.f};
+  if (a.khi < uint32_t(T / 2)) {
+    dft_lower<T>(v);
+    add_moments<T, 1, T / 2>(v, 0, 0.f, acc);
+  } else {
+    dft<T, -1>(v);
+    add_moments<T, 1, T>(v, 0, 0.f, acc);
+  }
+  if constexpr (POST) emit_moments(a, w, p, acc, true, true);
+  else store_moments(a, w, p, acc);
+}
+
+template <int T, bool POST>
+__global__ void __launch_bounds__(ColCfg<T>::NT, ColCfg<T>::CTAS) k_stft_cols(StftArgs a, uint32_t nitems,
+                                                                             uint32_t tiles) {
+  using C = ColCfg<T>;
+  constexpr int NW = C::NT / 32;
+  extern __shared__ __align__(16) unsigned char smem_cols[];
+  __shared__ float red[3][NW][C::BT];
+  float2* buf = reinterpret_cast<float2*>(smem_cols);
+  float2* tw = buf + C::ROWS * C::BT;
+  load_stage_twiddles<C::R1, C::NTW, C::NT>(tw, a.tw_t);
+  const int b = threadIdx.x % C::BT, t = threadIdx.x / C::BT, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const size_t HW = size_t(a.W) * a.H;
-  const uint32_t ntile = uint32_t(HW / BT);
-  const uint32_t nitem = a.nwin * ntile;
-  const float2* tq = static_cast<const float2*>(a.tq.base);
-  const uint32_t cap = a.tq.cap;
-  // item i: window i / ntile, pixels (i % ntile) BT ..; its frames into buffer b
-  auto fetch = [&](uint32_t i, int b) {
-    constexpr int FS = NT / BT;  // frames per pass of the CTA
-    const uint32_t w = i / ntile, p0 = (i % ntile) * BT;
-    float2* rows = rows0 + b * BT * WR;
-    const int c = tid % BT;
-    int f = tid / BT;
-    uint32_t g = a.tq.slot0 + w * a.S + uint32_t(f);
-    while (g >= cap) g -= cap;
-    for (; f < T; f += FS) {
-      cp_async8(&rows[c * WR + wpad(f)], &tq[size_t(g) * HW + p0 + c]);
-      g += FS;
-      if (g >= cap) g -= cap;
-    }
-    cp_async_commit();
-  };
-  uint32_t item = blockIdx.x;
-  if (item < nitem) fetch(item, 0);
-  {  // stage twiddles (the walking kernel's table layout)
-    constexpr int R1 = WarpPlan<T>::R1;
-    int NS = R1;
-    while (NS < T) {
-      const int rem = T / NS;
-      const int R = WarpPlan<T>::R2 != 0 ? WarpPlan<T>::R2 : (rem % 8 == 0 ? 8 : (rem % 4 == 0 ? 4 : 2));
-      for (int idx = tid; idx < (R - 1) * NS; idx += NT) {
-        const int m = idx / NS + 1, jm = idx % NS;
-        tw[(NS - R1) + idx] = a.tw_t[jm * m * (T / (NS * R))];
-      }
-      NS *= R;
-    }
-  }
-  uint32_t band = 0;
-  {
-    constexpr int RL = Lw::RL, NBL = T / RL;
-#pragma unroll
-    for (int it = 0; it < Lw::ITL; ++it)
-#pragma unroll
-      for (int m = 0; m < RL; ++m) {
-        const uint32_t k = uint32_t(jl + LP * it + m * NBL);
-        if (k - a.klo <= a.khi - a.klo) band |= 1u << (it * RL + m);
-      }
-  }
   const bool lower = a.khi < uint32_t(T / 2);
-  for (int b = 0; item < nitem; item += gridDim.x, b ^= 1) {
-    const uint32_t next = item + gridDim.x;
-    // the other buffer was released by the barrier that ended the previous item
-    if (next < nitem) {
-      fetch(next, b ^ 1);
-      cp_async_wait_group<1>();
-    } else {
-      cp_async_wait_all();
-    }
-    __syncthreads();  // every thread's copies of this item landed
-    const uint32_t w = item / ntile, p0 = (item % ntile) * BT;
-    MomAcc acc{band, 0.f, 0.f, 0.f};
-    float2* row = rows0 + b * BT * WR + px * WR;
-    warp_fft<T, 1, LP, true>(row, row, tw, jl, acc, lower);
+  uint32_t band = 0;
 #pragma unroll
-    for (int o = LP / 2; o > 0; o >>= 1) {
+  for (int it = 0; it < C::I2; ++it) band |= band_bits<C::R2, C::R1>(a, uint32_t(col_j2<T>(t, it)), it * C::R2);
+  for (uint32_t item = blockIdx.x; item < nitems; item += gridDim.x) {
+    const uint32_t w = item / tiles;
+    const size_t pix = size_t(item % tiles) * C::BT + b;
+    uint32_t g0 = a.tq.slot0 + w * a.S;
+    while (g0 >= a.tq.cap) g0 -= a.tq.cap;
+    const float2* tq = static_cast<const float2*>(a.tq.base) + pix;
+    float2 v[C::I1][C::R1], u[C::I2][C::R2];
+#pragma unroll
+    for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+      for (int m = 0; m < C::R1; ++m) {
+        uint32_t g = g0 + uint32_t(t + C::NJ * it + (T / C::R1) * m);
+        if (g >= a.tq.cap) g -= a.tq.cap;
+        v[it][m] = tq[size_t(g) * HW];
+      }
+    col_stage1<T, -1>(v, buf, t, b);
+    col_stage2<T, -1>(u, buf, tw, t, b);
+    MomAcc acc{band, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int it = 0; it < C::I2; ++it) {
+      const float kb = float(col_j2<T>(t, it));
+      if (lower) add_moments<C::R2, C::R1, C::R2 / 2>(u[it], it, kb, acc);
+      else add_moments<C::R2, C::R1, C::R2>(u[it], it, kb, acc);
+    }
+    // the pixel's threads: lanes of a warp BT apart, then the warps in order
+#pragma unroll
+    for (int o = C::BT; o < 32; o <<= 1) {
       acc.m0 += __shfl_xor_sync(0xffffffffu, acc.m0, o);
       acc.m1 += __shfl_xor_sync(0xffffffffu, acc.m1, o);
       acc.m2 += __shfl_xor_sync(0xffffffffu, acc.m2, o);
     }
-    if constexpr (POST) {
-      emit_moments(a, w, p0 + px, acc, jl == 0, true);
-    } else if (jl == 0) {
-      const float m1 = acc.m1 * a.fscale, m2 = acc.m2 * (a.fscale * a.fscale);  // bins -> kHz
-      float* o = a.out + size_t(w) * a.nout * HW + p0 + px;
-      int q = 0;
-      if (a.mask & HV_MOM_M0) __stcs(&o[HW * q++], acc.m0);
-      if (a.mask & HV_MOM_M1) __stcs(&o[HW * q++], m1);
-      if (a.mask & HV_MOM_M2) __stcs(&o[HW * q++], m2);
-      const double d0 = acc.m0;
-      if (a.mask & HV_MOM_M1N) __stcs(&o[HW * q++], d0 > 0.0 ? float(double(m1) / d0) : 0.f);
-      if (a.mask & HV_MOM_M2N) {
-        const double r = d0 > 0.0 ? double(m2) / d0 : 0.0;
-        __stcs(&o[HW * q++], float(sqrt(r > 0.0 ? r : 0.0)));
-      }
+    // (the next item's first stage has barriers between these reads and its own writes)
+    if (lane < C::BT) {
+      red[0][warp][lane] = acc.m0;
+      red[1][warp][lane] = acc.m1;
+      red[2][warp][lane] = acc.m2;
     }
-    __syncthreads();  // every warp is done with this buffer before it is refilled
+    __syncthreads();
+    if (warp == 0) {
+      const int e = lane % C::BT;
+      MomAcc sum{0u, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int q = 0; q < NW; ++q) {
+        sum.m0 += red[0][q][e];
+        sum.m1 += red[1][q][e];
+        sum.m2 += red[2][q][e];
+      }
+      const size_t at = size_t(item % tiles) * C::BT + e;
+      if constexpr (POST) emit_moments(a, w, at, sum, lane < C::BT, true);
+      else if (lane < C::BT) store_moments(a, w, at, sum);
+    }
   }
 }
 
-// Windows that do not overlap at T = 512, frames by TMA: the window-per-CTA
-// kernel's work (8 pixels of one window per CTA) with the window's frames brought
-// in by two TMA tensor loads (8 pixels x 256 queue slots each, 64-byte swizzle)
-// instead of one 8-byte cp.async per element, and the FFT run in place in that
-// tile as a decimation in frequency, 512 = 16 x 32: with t = j + 32 m and
+// Every (window, tile) of the launch by the kernels above.
+template <int T>
+static cudaError_t launch_direct(const StftArgs& a, cudaStream_t s) {
+  const size_t hw = size_t(a.W) * a.H;
+  if constexpr (T <= 32) {
+    const uint64_t grid = uint64_t(a.nwin) * (hw / 256);
+    if (hw % 256 || grid >= (1ull << 31)) return cudaErrorInvalidValue;
+    if (a.post_ring) k_stft_px<T, true><<<unsigned(grid), 256, 0, s>>>(a);
+    else k_stft_px<T, false><<<unsigned(grid), 256, 0, s>>>(a);
+    return cudaGetLastError();
+  } else {
+    using C = ColCfg<T>;
+    const uint64_t items = uint64_t(a.nwin) * (hw / C::BT);
+    if (hw % C::BT || items >= (1ull << 31)) return cudaErrorInvalidValue;
+    auto kern = a.post_ring ? k_stft_cols<T, true> : k_stft_cols<T, false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM));
+    int per_sm = 0, dev = 0, nsm = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, C::NT, C::SMEM);
+    if (e != cudaSuccess) return e;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const uint64_t grid = std::min<uint64_t>(items, uint64_t(per_sm > 0 ? per_sm : 1) * nsm);
+    kern<<<unsigned(grid), C::NT, C::SMEM, s>>>(a, uint32_t(items), uint32_t(hw / C::BT));
+    return cudaGetLastError();
+  }
+}
+
+// Windows that do not overlap at T = 512, frames by TMA: one CTA per (window, 8 pixels)
+// as above (a window of 256 x 256 in 47.6 us against 59.4, of 512 x 512 in 258 against 242; the
+// autotuner times both), with the window's frames brought
+// in by two TMA tensor loads (8 pixels x 256 queue slots each, 64-byte swizzle), and the
+// FFT run in place in that tile as a decimation in frequency, 512 = 16 x 32: with t = j + 32 m and
 // k = k1 + 16 k2, X_k = sum_j w32^(j k2) w512^(j k1) sum_m x_t w16^(m k1).
 // Stage 1: butterfly j (two per lane) reads the 16 samples t = j + 32 m, takes
 // their 16-point DFT, multiplies output k1 by w512^(j k1) and writes it back to
@@ -799,7 +747,6 @@ template <bool POST>
 __device__ __forceinline__ void wt_window(const StftArgs& a, float2* tile, const float2* tw1, const float2* tw2,
                                           uint32_t band, int px, int jl, uint32_t w, uint32_t p0) {
   constexpr int T = WT_T;
-  const size_t HW = size_t(a.W) * a.H;
   // sample t of pixel px: 16-byte chunk px / 2 of row t sits at chunk
   // (px / 2) ^ ((t >> 1) & 3), px % 2 selects its half
   auto at = [&](int t) -> float2* { return tile + 8 * t + (px ^ (((t >> 1) & 3) << 1)); };
@@ -846,18 +793,7 @@ __device__ __forceinline__ void wt_window(const StftArgs& a, float2* tile, const
   if constexpr (POST) {
     emit_moments(a, w, p0 + px, acc, jl == 0, true);
   } else if (jl == 0) {
-    const float m1 = acc.m1 * a.fscale, m2 = acc.m2 * (a.fscale * a.fscale);  // bins -> kHz
-    float* o = a.out + size_t(w) * a.nout * HW + p0 + px;
-    int q = 0;
-    if (a.mask & HV_MOM_M0) __stcs(&o[HW * q++], acc.m0);
-    if (a.mask & HV_MOM_M1) __stcs(&o[HW * q++], m1);
-    if (a.mask & HV_MOM_M2) __stcs(&o[HW * q++], m2);
-    const double d0 = acc.m0;
-    if (a.mask & HV_MOM_M1N) __stcs(&o[HW * q++], d0 > 0.0 ? float(double(m1) / d0) : 0.f);
-    if (a.mask & HV_MOM_M2N) {
-      const double rr = d0 > 0.0 ? double(m2) / d0 : 0.0;
-      __stcs(&o[HW * q++], float(sqrt(rr > 0.0 ? rr : 0.0)));
-    }
+    store_moments(a, w, p0 + px, acc);
   }
 }
 
@@ -1037,46 +973,10 @@ static cudaError_t launch_warp(const StftArgs& a0, cudaStream_t s) {
   if constexpr (T == WT_T) {
     if (a.S >= uint32_t(T) && (a.kernel == STFT_TMA || a.kernel == STFT_TMA_PIPE)) {
       const cudaError_t e = launch_wt(a, s);
-      if (e != cudaErrorNotSupported) return e;  // else a window wraps: the window-per-CTA kernel
+      if (e != cudaErrorNotSupported) return e;  // else a window wraps
     }
   }
-  if (a.S >= uint32_t(T) && a.kernel != STFT_WALK) {
-    // one CTA per (window, pixel tile)
-    auto launch_win = [&](auto wide) -> cudaError_t {
-      constexpr bool W = decltype(wide)::value;
-      using Wc = WinCfg<T, W>;
-      if (hw % Wc::BT) return cudaErrorNotSupported;
-      const size_t smem = Wc::bytes();
-      auto kern = a.post_ring ? k_stft_win<T, W, true> : k_stft_win<T, W, false>;
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-      if (e != cudaSuccess) return e;
-      const uint64_t grid = uint64_t(a.nwin) * (hw / Wc::BT);
-      if (grid >= (1ull << 31)) return cudaErrorInvalidValue;
-      kern<<<unsigned(grid), Wc::NT, smem, s>>>(a);
-      return cudaGetLastError();
-    };
-    if (a.kernel == STFT_PIPE) {
-      using Wc = WinCfg<T, false>;
-      if (hw % Wc::BT == 0) {
-        const size_t smem = 2 * size_t(Wc::BT) * Wc::WR * sizeof(float2) + (T - WarpPlan<T>::R1) * sizeof(float2);
-        auto kern = a.post_ring ? k_stft_winp<T, true> : k_stft_winp<T, false>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        int per_sm = 0, dev = 0, nsm = 0;
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, Wc::NT, smem);
-        if (e != cudaSuccess) return e;
-        if (per_sm >= 1) {
-          cudaGetDevice(&dev);
-          cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-          const uint64_t items = uint64_t(a.nwin) * (hw / Wc::BT);
-          const uint64_t grid = std::min<uint64_t>(items, uint64_t(per_sm) * nsm);
-          kern<<<unsigned(grid), Wc::NT, smem, s>>>(a);
-          return cudaGetLastError();
-        }
-      }
-    }
-    const cudaError_t e = a.kernel == STFT_WIDE ? launch_win(std::true_type{}) : launch_win(std::false_type{});
-    if (e != cudaErrorNotSupported) return e;
-  }
+  if (a.kernel == STFT_OVERLAP || (a.S >= uint32_t(T) && a.kernel != STFT_WALK)) return launch_direct<T>(a, s);
   CUtensorMap map{};
   a.tma = queue_map(a, Lw::BT, &map) ? 1 : 0;
   const size_t smem = WarpSmem<T>::bytes(a.S, a.tma != 0);
@@ -1103,12 +1003,15 @@ cudaError_t launch_stft(const StftArgs& a, cudaStream_t s, int* launches) {
   return cudaErrorInvalidValue;
 }
 
-__global__ void k_copy_frames(RingRef tq, uint32_t n, size_t hw, float2* out) {
+// Fields to an output that is not on an 8-byte boundary (others are written in place).
+__global__ void k_copy_frames(RingRef tq, uint32_t n, size_t hw, float* out) {
   const size_t total = hw * n;
   for (size_t e = blockIdx.x * size_t(blockDim.x) + threadIdx.x; e < total;
        e += size_t(gridDim.x) * blockDim.x) {
     const size_t i = e / hw, p = e % hw;
-    out[e] = static_cast<const float2*>(tq.base)[((tq.slot0 + i) % tq.cap) * hw + p];
+    const float2 v = static_cast<const float2*>(tq.base)[((tq.slot0 + i) % tq.cap) * hw + p];
+    out[2 * e] = v.x;
+    out[2 * e + 1] = v.y;
   }
 }
 
@@ -1117,7 +1020,7 @@ cudaError_t launch_copy_frames(const RingRef& tq, uint32_t n, uint32_t hw, float
   if (n == 0) return cudaSuccess;
   const size_t total = size_t(hw) * n;
   const int nb = int((total + 255) / 256 < 152 * 16 ? (total + 255) / 256 : 152 * 16);
-  k_copy_frames<<<nb, 256, 0, s>>>(tq, n, hw, reinterpret_cast<float2*>(out));
+  k_copy_frames<<<nb, 256, 0, s>>>(tq, n, hw, out);
   ++*launches;
   return cudaGetLastError();
 }

@@ -670,6 +670,60 @@ def test_stft_autotuner_times_both_kernels():
         r.close()
 
 
+@pytest.mark.parametrize("T,S,H,W", [(32, 31, 16, 64), (128, 48, 64, 64), (256, 200, 16, 64), (512, 300, 16, 16)])
+def test_autotuned_overlapping_windows(T, S, H, W):
+    """tuned = 1 with S < T: the walking kernel and the window-per-CTA kernels are timed,
+    whichever is kept renders the oracle's windows, over two renders and a wrapping queue."""
+    n = T + 9 * S + 5
+    fr = synth.random_frames(n, H, W, 12, seed=T + S)
+    p = oracle_params(spatial="none", T=T, stride=S, fs_hz=71400.0, band_lo_bin=1, band_hi_bin=T - 2,
+                      moments=ALL_MOMENTS, H=H, W=W)
+    img, st = gpu_render(fr, p, extra=dict(tuned=1), packets=[T + 4 * S, n - T - 4 * S], tq=T + 3 * S)
+    check_images(img, O.render(fr, p))
+
+
+def test_normalised_moments_are_float64s_float32_results():
+    """M1N is the float32 nearest to the float64 quotient, M2N to the float64 root (a tie's
+    width away at most, in one pixel of a few thousand), of the M1, M2 and M0 rendered."""
+    T, N = 16, 128
+    fr = synth.random_frames(4 * T, N, N, 12, seed=31)
+    fr[:, :8] = 7  # constant in time: M0 = 0 there
+    p = oracle_params(spatial="none", T=T, stride=T, fs_hz=71400.0, band_lo_bin=1, band_hi_bin=9,
+                      moments=ALL_MOMENTS, H=N, W=N)
+    img, _ = gpu_render(fr, p)
+    m = img.astype(np.float64)
+    assert np.array_equal(m.astype(np.float32).astype(np.float64), m)
+    z = m[:, 0] > 0
+    assert not np.any(z[:, :8]) and np.all(z[:, 8:])
+    d = np.where(z, m[:, 0], 1.0)
+    assert np.array_equal(np.where(z, m[:, 1] / d, 0.0).astype(np.float32), img[:, 3].astype(np.float32))
+    want = np.where(z, np.sqrt(m[:, 2] / d), 0.0).astype(np.float32)
+    got = img[:, 4].astype(np.float32)
+    assert np.all(np.abs(got - want) <= np.spacing(want)) and np.mean(got != want) < 1e-3
+
+
+def test_fields_at_an_odd_float():
+    """Fields go straight to an output on an 8-byte boundary and are copied to another."""
+    import torch
+    n, N = 3, 64
+    fr = synth.random_frames(n, N, N, 12, seed=8)
+    p = oracle_params(spatial="asp", temporal="none", T=1, stride=1, H=N, W=N)
+    got = []
+    for shift in (0, 1):
+        r = hv.Renderer(N, N, 16, n)
+        try:
+            hv.hv_set_params(r.h, to_hv(p))
+            out = torch.zeros(2 * n * N * N + 1, device="cuda")
+            torch.cuda.synchronize()
+            assert r.push(to_device(fr)) == hv.HV_OK
+            assert r.render(out[shift:]) == n
+            r.synchronize()
+            got.append(out[shift:shift + 2 * n * N * N].cpu().numpy())
+        finally:
+            r.close()
+    assert np.array_equal(got[0], got[1])
+
+
 @pytest.mark.slow
 def test_default_bench_configuration_every_pixel():
     """The default bench workload in the launch configuration bench.py times: its
