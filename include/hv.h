@@ -98,7 +98,8 @@ typedef struct {
                                  inclusive, descending eigenvalue)                     */
   int32_t precision;          /* PCA covariance arithmetic, HV_PREC_*                  */
   int32_t tuned;              /* 1 = tuned form (spatial kernels chosen by timing)    */
-  uint32_t spatial_chunk;     /* frames per spatial launch (0 = automatic)             */
+  uint32_t spatial_chunk;     /* frames per spatial launch (0 = automatic); launches of a
+                                 longer run go side by side, each with scratch of its own */
   uint32_t spatial_kernel;    /* HV_SK_*: which spatial kernels (default automatic):
                                  multi-pass, persistent multi-pass (sides from 64 up,
                                  where both are the same register-direct passes), the

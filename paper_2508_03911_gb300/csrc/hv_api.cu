@@ -57,6 +57,10 @@ struct hv_handle {
   float2* s2 = nullptr;
   size_t s1_bytes = 0, s2_bytes = 0;
   uint32_t chunk = 0;
+  uint32_t sp_lanes = 1;                   // multi-pass launches side by side, each with its part of s1 / s2
+  cudaStream_t sp_stream[kSpLanes - 1] = {};  // lanes 1 ..; lane 0 is the handle's stream
+  cudaEvent_t ev_fork = nullptr, ev_join[kSpLanes - 1] = {};
+  uint32_t strip_fit[kStripKernels * kStripSides] = {};  // see SpatialArgs::fit
   int sp_cluster = 0;         // 1: whole-frame cluster kernel
   int sp_fused = 0;           // 1: fused transform (s1 / s2 are rings of kFusedRing frames)
   int inject = HV_INJECT_NONE;  // pending fault injection (hv_debug_inject)
@@ -344,6 +348,23 @@ hv_status ensure(hv_handle* h, void** p, size_t* have, size_t need) {
   return HV_OK;
 }
 
+// Scratch of the multi-pass transform: `chunk` frames for each of the launches side by side,
+// as many as runs of up to `frames` frames fill and 1 GB holds, one where there is no memory
+// for more; `least` frames in all.
+hv_status size_scratch(hv_handle* h, int spatial, size_t fbytes, uint32_t chunk, uint32_t frames, uint32_t least) {
+  const size_t fit = (size_t(1) << 30) / (chunk * fbytes), runs = (size_t(frames) + chunk - 1) / chunk;
+  uint32_t lanes = uint32_t(std::max<size_t>(1, std::min<size_t>({kSpLanes, fit, runs})));
+  for (;; lanes = 1) {
+    const size_t need = std::max<size_t>(size_t(lanes) * chunk, least) * fbytes;
+    hv_status s = ensure(h, reinterpret_cast<void**>(&h->s1), &h->s1_bytes, need);
+    if (s == HV_OK && spatial == HV_SPATIAL_ASP)
+      s = ensure(h, reinterpret_cast<void**>(&h->s2), &h->s2_bytes, need);
+    h->sp_lanes = lanes;
+    if (s == HV_OK || lanes == 1) return s;
+    cudaGetLastError();
+  }
+}
+
 hv_status tune_spatial(hv_handle* h);
 hv_status tune_temporal(hv_handle* h);
 
@@ -370,26 +391,24 @@ hv_status apply_pending(hv_handle* h) {
   Q = std::max(Q, d.T);
   s = ensure(h, reinterpret_cast<void**>(&h->tq), &h->tq_bytes, size_t(Q) * fbytes);
   if (s != HV_OK) return s;
-  // frames per launch: 256 MB of fields (at 256 x 256 ASP 0.55, 0.46, 0.41, 0.37 us a frame
-  // for 32, 48, 160 and 512 MB: a launch's ramp and tail weigh more than the L2 hits that
-  // a small launch's intermediates get)
-  uint32_t chunk = p.spatial_chunk ? p.spatial_chunk : std::max<uint32_t>(1, uint32_t((size_t(256) << 20) / fbytes));
+  // frames per launch: 64 MB of fields, and up to four launches side by side, since the
+  // ramp and the tail of one then fall into the others' middles. Us a frame by MB a launch:
+  // 256 x 256 ASP one launch at a time 0.77, 0.53, 0.45, 0.39 for 16, 32, 64 and 256, four
+  // side by side 0.333, 0.348, 0.345, 0.348; 512 x 512 Fresnel 1.81, 1.48, 1.47 for 32, 64, 256
+  // against 1.28, 1.26, 1.29; 1024 x 1024 ASP 12.5, 10.9, 9.3 against 10.1, 9.5, 9.0
+  uint32_t chunk = p.spatial_chunk ? p.spatial_chunk : std::max<uint32_t>(1, uint32_t((size_t(64) << 20) / fbytes));
   if (p.spatial_chunk == 0) chunk = std::min(chunk, Q);
   chunk = std::min<uint32_t>(chunk, 1024);
   const bool fused = p.spatial_kernel == HV_SK_FUSED;
-  const size_t sbytes = size_t(fused ? std::max(chunk, kFusedRing) : chunk) * fbytes;
   if (fused) {
     s = ensure(h, reinterpret_cast<void**>(&h->fused_ctr), &h->fused_ctr_bytes,
                (1 + kFusedPasses * size_t(kFusedRing)) * sizeof(unsigned));
     if (s != HV_OK) return s;
   }
+  h->sp_lanes = 1;
   if (p.spatial != HV_SPATIAL_NONE) {
-    s = ensure(h, reinterpret_cast<void**>(&h->s1), &h->s1_bytes, sbytes);
+    s = size_scratch(h, p.spatial, fbytes, chunk, Q, fused ? kFusedRing : 0);
     if (s != HV_OK) return s;
-    if (p.spatial == HV_SPATIAL_ASP) {
-      s = ensure(h, reinterpret_cast<void**>(&h->s2), &h->s2_bytes, sbytes);
-      if (s != HV_OK) return s;
-    }
   }
   s = build_tables(h, p);
   if (s != HV_OK) return s;
@@ -610,6 +629,25 @@ bool cluster_ok(const hv_handle* h) {
          (h->cur.spatial == HV_SPATIAL_ASP || h->cur.spatial == HV_SPATIAL_FRESNEL);
 }
 
+// Lanes 1 .. lanes - 1 wait for the handle's stream; lane 0 is the handle's stream itself.
+cudaError_t fork_lanes(hv_handle* h, uint32_t lanes) {
+  cudaError_t e = lanes > 1 ? cudaEventRecord(h->ev_fork, h->stream) : cudaSuccess;
+  for (uint32_t i = 1; i < lanes && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(h->sp_stream[i - 1], h->ev_fork, 0);
+  return e;
+}
+
+// The handle's stream waits for every lane, also after a failed launch (e, which it returns).
+cudaError_t join_lanes(hv_handle* h, uint32_t lanes, cudaError_t e) {
+  for (uint32_t i = 1; i < lanes; ++i) {
+    cudaError_t j = cudaEventRecord(h->ev_join[i - 1], h->sp_stream[i - 1]);
+    if (j == cudaSuccess) j = cudaStreamWaitEvent(h->stream, h->ev_join[i - 1], 0);
+    if (e == cudaSuccess) e = j;
+  }
+  return e;
+}
+
+cudaStream_t lane_stream(hv_handle* h, uint32_t lane) { return lane ? h->sp_stream[lane - 1] : h->stream; }
+
 // Spatial transform of frames r0 .. r1 - 1, whose raw frames are at `raw` (frame
 // r0 at slot raw.slot0). The fields go to the time queue, whose slots follow the frame
 // numbers, or to `out`, where frame out0 is slot 0.
@@ -617,8 +655,12 @@ hv_status propagate_run(hv_handle* h, uint64_t r0, uint64_t r1, RingRef raw, flo
   // the cluster kernel needs no scratch, the fused transform keeps its intermediates
   // in rings: one persistent launch for all frames
   const bool whole = (h->sp_cluster && cluster_ok(h)) || h->sp_fused;
-  const uint64_t step = whole ? r1 - r0 : h->chunk;
-  for (uint64_t a = r0; a < r1; a += step) {
+  const uint64_t nruns = whole ? 1 : (r1 - r0 + h->chunk - 1) / h->chunk;
+  const uint64_t step = (r1 - r0 + nruns - 1) / nruns;
+  const uint32_t lanes = uint32_t(std::min<uint64_t>(nruns, h->sp_lanes));
+  uint32_t lane = 0;
+  cudaError_t e = fork_lanes(h, lanes);
+  for (uint64_t a = r0; a < r1 && e == cudaSuccess; a += step, lane = (lane + 1) % lanes) {
     const uint32_t n = uint32_t(std::min<uint64_t>(step, r1 - a));
     SpatialArgs sa{};
     sa.err = h->dev_err;
@@ -629,8 +671,10 @@ hv_status propagate_run(hv_handle* h, uint64_t r0, uint64_t r1, RingRef raw, flo
     sa.n = n;
     sa.raw = RingRef{raw.base, raw.cap, uint32_t((raw.slot0 + (a - r0)) % raw.cap)};
     sa.tq = out ? RingRef{out + (a - out0) * h->W * h->H, n, 0} : RingRef{h->tq, h->Q, uint32_t(a % h->Q)};
-    sa.scratch1 = h->s1;
-    sa.scratch2 = h->s2;
+    const size_t part = whole ? 0 : size_t(lane) * h->chunk * h->W * h->H;
+    sa.scratch1 = h->s1 + part;
+    sa.scratch2 = h->s2 + part;
+    sa.fit = h->strip_fit;
     sa.tw_w = h->tw + tw_offset(h->W);
     sa.tw_h = h->tw + tw_offset(h->H);
     sa.asp_ht = h->asp_ht;
@@ -647,11 +691,12 @@ hv_status propagate_run(hv_handle* h, uint64_t r0, uint64_t r1, RingRef raw, flo
       h->inject = HV_INJECT_NONE;
     }
     int launches = 0;
-    cudaError_t e = launch_spatial(sa, h->stream, &launches);
+    e = launch_spatial(sa, lane_stream(h, lane), &launches);
     h->st.kernel_launches += launches;
-    if (e != cudaSuccess) return cuda_fail(h, e, "spatial transform launch");
-    h->st.frames_propagated += n;
+    if (e == cudaSuccess) h->st.frames_propagated += n;
   }
+  e = join_lanes(h, lanes, e);
+  if (e != cudaSuccess) return cuda_fail(h, e, "spatial transform launch");
   return HV_OK;
 }
 
@@ -721,13 +766,9 @@ hv_status tune_spatial(hv_handle* h) {
     if (c.kind == 4 && ensure(h, reinterpret_cast<void**>(&h->fused_ctr), &h->fused_ctr_bytes,
                               (1 + kFusedPasses * size_t(kFusedRing)) * sizeof(unsigned)) != HV_OK)
       continue;
-    if (c.kind != 2) {
-      const size_t need = size_t(c.kind == 4 ? kFusedRing : ch) * fbytes;
-      if (ensure(h, reinterpret_cast<void**>(&h->s1), &h->s1_bytes, need) != HV_OK) continue;
-      if (h->cur.spatial == HV_SPATIAL_ASP &&
-          ensure(h, reinterpret_cast<void**>(&h->s2), &h->s2_bytes, need) != HV_OK)
-        continue;
-    }
+    if (c.kind != 2 && size_scratch(h, h->cur.spatial, fbytes, c.kind == 4 ? kFusedRing : ch, c.kind == 4 ? 1 : n,
+                                    0) != HV_OK)
+      continue;
     h->sp_cluster = c.kind == 2;
     h->sp_fused = c.kind == 4;
     h->chunk = (c.kind == 2 || c.kind == 4) ? h->chunk : ch;
@@ -746,7 +787,9 @@ hv_status tune_spatial(hv_handle* h) {
     h->st.frames_propagated = before;  // tuning work is not rendering work
     const float us_per_frame = 1000.f * ms / (2.f * n);
     t.candidate_us_per_frame[ci] = us_per_frame;
-    if (us_per_frame < best) {
+    // the fused transform's one launch weighs less on short runs than the passes' many: kept
+    // unless they are a tenth faster
+    if (us_per_frame < (c.kind == 4 ? 1.1f * best : best)) {
       best = us_per_frame;
       best_kind = c.kind;
       best_chunk = (c.kind == 2 || c.kind == 4) ? best_chunk : ch;
@@ -758,12 +801,9 @@ hv_status tune_spatial(hv_handle* h) {
   h->sp_fused = best_kind == 4;
   h->chunk = best_chunk;
   // the chosen kernels' scratch: chunk frames (multi-pass), the rings (fused)
-  if (best_kind != 2) {
-    const size_t need = size_t(best_kind == 4 ? std::max(best_chunk, kFusedRing) : best_chunk) * fbytes;
-    if (ensure(h, reinterpret_cast<void**>(&h->s1), &h->s1_bytes, need) != HV_OK ||
-        (h->cur.spatial == HV_SPATIAL_ASP && ensure(h, reinterpret_cast<void**>(&h->s2), &h->s2_bytes, need) != HV_OK))
-      return HV_ERR_NOMEM;
-  }
+  if (best_kind != 2 &&
+      size_scratch(h, h->cur.spatial, fbytes, best_chunk, h->Q, best_kind == 4 ? kFusedRing : 0) != HV_OK)
+    return HV_ERR_NOMEM;
   t.spatial_kernel = best_kind == 2 ? HV_SK_CLUSTER
                      : (best_kind == 3 ? HV_SK_PERSISTENT : (best_kind == 4 ? HV_SK_FUSED : HV_SK_MULTIPASS));
   t.spatial_chunk = best_chunk;
@@ -1231,6 +1271,11 @@ hv_status hv_open(const hv_open_desc* desc, hv_handle** out) {
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_cov[i], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_eig[i], cudaEventDisableTiming);
   }
+  for (uint32_t i = 0; i + 1 < kSpLanes && e == cudaSuccess; ++i) {
+    e = cudaStreamCreateWithFlags(&h->sp_stream[i], cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_join[i], cudaEventDisableTiming);
+  }
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_pushed, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_consumed, cudaEventDisableTiming);
   for (int i = 0; i < hv_handle::NCONS && e == cudaSuccess; ++i)
@@ -1463,6 +1508,14 @@ hv_status hv_close(hv_handle* h) {
     if (h->ev_cov[i]) cudaEventDestroy(h->ev_cov[i]);
     if (h->ev_eig[i]) cudaEventDestroy(h->ev_eig[i]);
   }
+  for (uint32_t i = 0; i + 1 < kSpLanes; ++i) {
+    if (h->sp_stream[i]) {
+      cudaStreamSynchronize(h->sp_stream[i]);
+      cudaStreamDestroy(h->sp_stream[i]);
+    }
+    if (h->ev_join[i]) cudaEventDestroy(h->ev_join[i]);
+  }
+  if (h->ev_fork) cudaEventDestroy(h->ev_fork);
   if (h->ev_pushed) cudaEventDestroy(h->ev_pushed);
   if (h->ev_consumed) cudaEventDestroy(h->ev_consumed);
   for (auto& e : h->cons_ev)
@@ -1530,7 +1583,7 @@ hv_status hv_set_postprocess(hv_handle* h, const hv_post* p) {
 // ------------------------------------------------------------- autofocus
 
 // Frames [n][H][W] in device memory as a ring for the pass kernels.
-static SpatialArgs af_args(const hv_handle* h, const void* frames, uint32_t n) {
+static SpatialArgs af_args(hv_handle* h, const void* frames, uint32_t n) {
   SpatialArgs sa{};
   sa.err = h->dev_err;
   sa.spatial = HV_SPATIAL_ASP;  // no chirp in the column pass
@@ -1540,6 +1593,7 @@ static SpatialArgs af_args(const hv_handle* h, const void* frames, uint32_t n) {
   sa.raw = RingRef{const_cast<void*>(frames), n, 0};
   sa.scratch1 = h->s1;
   sa.scratch2 = h->s2;
+  sa.fit = h->strip_fit;
   sa.tw_w = h->tw + tw_offset(h->W);
   sa.tw_h = h->tw + tw_offset(h->H);
   return sa;

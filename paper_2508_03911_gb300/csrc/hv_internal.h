@@ -44,8 +44,13 @@ struct SpatialArgs {
   int use_fused;
   uint32_t ring;
   unsigned* fused_ctr;
+  uint32_t* fit;        // host table [kStripKernels][kStripSides] kept by the caller: CTAs of a strip
+                        // kernel that fit the device at once, 0 where not asked yet (NULL: no table)
   int stall;            // fault injection (tests): the fused row items wait on a condition nothing sets
 };
+constexpr uint32_t kStripKernels = 9, kStripSides = 5;  // sides 64 .. 1024
+// Multi-pass launches of one run that are queued side by side.
+constexpr uint32_t kSpLanes = 4;
 cudaError_t launch_spatial(const SpatialArgs& a, cudaStream_t s, int* launches);
 bool spatial_cluster_supported(const SpatialArgs& a);
 // Register-direct passes for sides 64 .. 1024 (ASP needs asp_h).

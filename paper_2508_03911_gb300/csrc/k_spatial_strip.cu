@@ -25,7 +25,9 @@
 // block-wide passes that staged each strip of 16 lines in shared memory (two strips per
 // CTA, so one or two CTAs per SM from 512 points on): 256 x 256 ASP 0.53 -> 0.37, Fresnel
 // 0.33 -> 0.31; 512 x 512 3.14 -> 1.89 and 1.65 -> 1.36; 1024 x 1024 17.0 -> 8.9 and
-// 8.4 -> 6.1; 128 x 128 0.139 -> 0.107 and 0.081 -> 0.083.
+// 8.4 -> 6.1; 128 x 128 0.139 -> 0.107 and 0.081 -> 0.083. Callers with more frames than one
+// launch takes queue up to four launches side by side: 0.33 and 0.24, 1.68 and 1.22, 8.9 and
+// 5.5 for 256, 512 and 1024.
 #include "strip_dev.cuh"
 #include "hv_internal.h"
 #include "../../include/hv.h"
@@ -435,17 +437,29 @@ __global__ void __launch_bounds__(RowCfg<L>::NT) k_strip_cells(SpatialArgs a, ui
   }
 }
 
-// Persistent grid: every CTA that fits at once, no more than the items.
+// Row of SpatialArgs::fit.
+enum StripKernel { COLS_ASP, COLS, ICOLS, ROWS_ASP, ROWS_FFT, ROWS_FWD, ROWS_INV, ICOLS_SUMS, CELLS };
+static_assert(CELLS + 1 == kStripKernels, "one row per kernel");
+
+constexpr uint32_t side_index(int L) { return L == 64 ? 0 : 1 + side_index(L / 2); }
+
+// Persistent grid: every CTA that fits at once, no more than the items. How many fit is asked
+// once per caller's table (the two queries and the attribute took longer than the launch).
 template <class K, class... Args>
-cudaError_t launch_resident(K kern, int nt, size_t smem, uint32_t ctas, cudaStream_t s, Args... args) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-  if (e != cudaSuccess) return e;
-  int per_sm = 0, dev = 0, nsm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem);
-  if (e != cudaSuccess) return e;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const uint32_t most = uint32_t(per_sm > 0 ? per_sm : 1) * uint32_t(nsm);
+cudaError_t launch_resident(const SpatialArgs& a, StripKernel row, int L, K kern, int nt, size_t smem, uint32_t ctas,
+                            cudaStream_t s, Args... args) {
+  uint32_t* fit = a.fit ? a.fit + row * kStripSides + side_index(L) : nullptr;
+  uint32_t most = fit ? *fit : 0;
+  if (most == 0) {
+    int per_sm = 0, dev = 0, nsm = 0;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    most = uint32_t(per_sm > 0 ? per_sm : 1) * uint32_t(nsm);
+    if (fit) *fit = most;
+  }
   kern<<<ctas < most ? ctas : most, nt, smem, s>>>(args...);
   return cudaGetLastError();
 }
@@ -454,14 +468,14 @@ template <int L, bool ASP>
 cudaError_t cols(const SpatialArgs& a, cudaStream_t s) {
   using C = ColCfg<L>;
   const uint32_t strips = a.W / (ASP ? 2 * C::BT : C::BT), items = strips * a.n;
-  return launch_resident(k_strip_cols<L, ASP>, C::NT, C::SMEM, items, s, a, items, strips);
+  return launch_resident(a, ASP ? COLS_ASP : COLS, L, k_strip_cols<L, ASP>, C::NT, C::SMEM, items, s, a, items, strips);
 }
 
 template <int L>
 cudaError_t icols(const SpatialArgs& a, cudaStream_t s) {
   using C = ColCfg<L>;
   const uint32_t strips = a.W / C::BT, items = strips * a.n;
-  return launch_resident(k_strip_icols<L>, C::NT, C::SMEM, items, s, a, items, strips);
+  return launch_resident(a, ICOLS, L, k_strip_icols<L>, C::NT, C::SMEM, items, s, a, items, strips);
 }
 
 template <int L>
@@ -470,10 +484,10 @@ cudaError_t rows(const SpatialArgs& a, cudaStream_t s) {
   constexpr uint32_t per = C::NW * C::RPW;
   if (a.spatial == HV_SPATIAL_ASP) {
     const uint32_t nrows = a.n * (a.H / 2 + 1);
-    return launch_resident(k_strip_rows_asp<L>, C::NT, C::SMEM, (nrows + per - 1) / per, s, a, nrows);
+    return launch_resident(a, ROWS_ASP, L, k_strip_rows_asp<L>, C::NT, C::SMEM, (nrows + per - 1) / per, s, a, nrows);
   }
   const uint32_t nrows = a.n * a.H;
-  return launch_resident(k_strip_rows_fft<L>, C::NT, C::SMEM, (nrows + per - 1) / per, s, a, nrows);
+  return launch_resident(a, ROWS_FFT, L, k_strip_rows_fft<L>, C::NT, C::SMEM, (nrows + per - 1) / per, s, a, nrows);
 }
 
 #define HV_BY_SIDE(side, fn)             \
@@ -491,7 +505,7 @@ cudaError_t rows_fwd(const SpatialArgs& a, cudaStream_t s) {
   using C = RowCfg<L>;
   constexpr uint32_t per = C::NW * C::RPW;
   const uint32_t nrows = a.n * (a.H / 2 + 1);
-  return launch_resident(k_strip_rows_fwd<L>, C::NT, C::SMEM, (nrows + per - 1) / per, s, a, nrows);
+  return launch_resident(a, ROWS_FWD, L, k_strip_rows_fwd<L>, C::NT, C::SMEM, (nrows + per - 1) / per, s, a, nrows);
 }
 
 template <int L>
@@ -499,20 +513,20 @@ cudaError_t rows_inv(const SpatialArgs& a, const float2* h, uint32_t nz, cudaStr
   using C = RowCfg<L>;
   constexpr uint32_t per = C::NW * C::RPW;
   const uint32_t nrows = nz * a.n * (a.H / 2 + 1);
-  return launch_resident(k_strip_rows_inv<L>, C::NT, C::SMEM, (nrows + per - 1) / per, s, a, h, nrows);
+  return launch_resident(a, ROWS_INV, L, k_strip_rows_inv<L>, C::NT, C::SMEM, (nrows + per - 1) / per, s, a, h, nrows);
 }
 
 template <int L>
 cudaError_t icols_sums(const SpatialArgs& a, uint32_t nz, cudaStream_t s) {
   using C = ColCfg<L>;
   const uint32_t strips = a.W / C::BT, items = strips * a.n * nz;
-  return launch_resident(k_strip_icols_sums<L>, C::NT, C::SMEM, items, s, a, items, strips);
+  return launch_resident(a, ICOLS_SUMS, L, k_strip_icols_sums<L>, C::NT, C::SMEM, items, s, a, items, strips);
 }
 
 template <int L>
 cudaError_t cells(const SpatialArgs& a, cudaStream_t s) {
   const uint32_t strips = a.H / (2 * CellCfg<L>::SR), items = strips * a.n;
-  return launch_resident(k_strip_cells<L>, RowCfg<L>::NT, CellCfg<L>::SMEM, items, s, a, items, strips);
+  return launch_resident(a, CELLS, L, k_strip_cells<L>, RowCfg<L>::NT, CellCfg<L>::SMEM, items, s, a, items, strips);
 }
 
 }  // namespace

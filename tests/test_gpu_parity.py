@@ -131,6 +131,20 @@ def test_persistent_multipass_parity(H, W, spatial, bits):
         assert rel_l2(img[i], ref[i]) <= FIELD_TOL, (i, rel_l2(img[i], ref[i]))
 
 
+@pytest.mark.parametrize("H,W,spatial,n,chunk", [(64, 64, "asp", 23, 5), (64, 128, "fresnel", 9, 4),
+                                                 (32, 32, "asp", 11, 2), (256, 64, "asp", 37, 1)])
+def test_launches_side_by_side(H, W, spatial, n, chunk):
+    """A run cut into launches that go side by side (two to four at once, the last ones
+    shorter, many more launches than lanes) gives the fields of one launch, frame for frame,
+    over a wrapping input ring and in-place device packets, render after render."""
+    fr = synth.random_frames(n, H, W, 12, seed=n + chunk)
+    p = oracle_params(spatial=spatial, z_m=0.3, temporal="none", T=1, stride=1, H=H, W=W)
+    one, _ = gpu_render(fr, p, extra=dict(spatial_chunk=n))
+    for kw in (dict(), dict(packets=[n // 2, n - n // 2], queue=(n + 1) // 2 + 1), dict(in_place=True)):
+        img, _ = gpu_render(fr, p, extra=dict(spatial_chunk=chunk), **kw)
+        assert np.array_equal(img, one)
+
+
 @pytest.mark.parametrize("H,W,spatial,bits,n", [(64, 1024, "asp", 8, 1), (1024, 128, "asp", 12, 3),
                                                 (512, 64, "fresnel", 8, 2), (512, 512, "asp", 8, 2),
                                                 (1024, 256, "fresnel", 12, 2), (64, 64, "asp", 12, 1),
