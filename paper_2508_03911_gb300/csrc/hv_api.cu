@@ -1615,16 +1615,24 @@ static hv_status af_prepare(hv_handle* h, const void* frames, uint32_t n, uint32
 hv_status hv_focus_sweep(hv_handle* h, const void* frames, uint32_t n, const double* z, uint32_t nz, float* metric) {
   if (!h) return HV_ERR_ARG;
   if (!z || !metric || nz == 0 || nz > 1024) return fail(h, HV_ERR_ARG, "bad distances or output");
-  // holograms whose spectra are held at once, and (distance, hologram) images per launch:
-  // 256 MB of them (64 distances x 64 holograms of 256 x 256 in 1612, 1346, 1281 and 1141 us
-  // with 32, 64, 128 and 256 MB)
+  // holograms whose spectra are held at once
   const uint32_t chunk = std::min<uint32_t>(n, 64);
   hv_status s = af_prepare(h, frames, n, chunk);
   if (s != HV_OK) return s;
   const uint32_t W = h->W, H = h->H;
   const size_t fbytes = size_t(W) * H * sizeof(float2);
-  const uint32_t images = std::max(chunk, uint32_t((size_t(256) << 20) / fbytes));
-  s = ensure(h, reinterpret_cast<void**>(&h->s2), &h->s2_bytes, images * fbytes);
+  // (distance, hologram) images per launch, 64 MB of them, and launches side by side (64
+  // distances x 64 holograms of 256 x 256: 898 us; one launch at a time with 64, 128 and 256 MB
+  // 1346, 1281 and 1141)
+  const uint32_t images = std::max(chunk, uint32_t((size_t(64) << 20) / fbytes));
+  const uint32_t steps = (nz + images / chunk - 1) / (images / chunk);
+  uint32_t lanes = uint32_t(std::max<size_t>(1, std::min<size_t>({kSpLanes, steps, (size_t(1) << 30) / (images * fbytes)})));
+  s = ensure(h, reinterpret_cast<void**>(&h->s2), &h->s2_bytes, lanes * images * fbytes);
+  if (s != HV_OK && lanes > 1) {
+    cudaGetLastError();
+    lanes = 1;
+    s = ensure(h, reinterpret_cast<void**>(&h->s2), &h->s2_bytes, images * fbytes);
+  }
   if (s != HV_OK) return s;
   const hv_params& p = h->cur;
   // transfer functions H_j, rows ky = 0 .. H/2 (1/(W H) folded in, DC bin zero)
@@ -1666,12 +1674,16 @@ hv_status hv_focus_sweep(hv_handle* h, const void* frames, uint32_t n, const dou
     cudaError_t e = launch_strip_spectrum(sa, h->stream);
     h->st.kernel_launches += 2;
     const uint32_t zc = std::max<uint32_t>(1, images / sa.n);
-    for (uint32_t j = 0; j < nz && e == cudaSuccess; j += zc) {
+    if (e == cudaSuccess) e = fork_lanes(h, lanes);
+    float2* const scratch2 = sa.scratch2;
+    for (uint32_t j = 0, lane = 0; j < nz && e == cudaSuccess; j += zc, lane = (lane + 1) % lanes) {
+      sa.scratch2 = scratch2 + size_t(lane) * images * W * H;
       sa.tam_acc = h->sw_acc + (size_t(a) * nz + j) * 2;
       sa.tam_stride = nz * 2;
-      e = launch_strip_sweep(sa, h->sw_tables + j * per, std::min(zc, nz - j), h->stream);
+      e = launch_strip_sweep(sa, h->sw_tables + j * per, std::min(zc, nz - j), lane_stream(h, lane));
       h->st.kernel_launches += 2;
     }
+    e = join_lanes(h, lanes, e);
     if (e != cudaSuccess) return cuda_fail(h, e, "focus sweep passes");
   }
   cudaError_t e = launch_tamura_finish(h->sw_acc, n * nz, W * H, metric, h->stream);
