@@ -16,7 +16,7 @@
 //                  float32 phase of the long-window eigensolver (T > 64, one
 //                  window): parallel cyclic (round-robin) two-sided Jacobi on one
 //                  16-CTA cluster, or cooperative on a quarter of the SMs
-//   k_gemm_c64     float64 congruence C' = Vf^H C Vf
+//   k_congruence   C' = Vf^H C Vf in pairs of float32
 //   k_jacobi_refine cooperative refinement sweeps on C' over all SMs: float64
 //                  diagonal and V, float32 off-diagonal entries
 //   k_jacobi_small both phases for T <= 64, one CTA per window, C and V in
@@ -151,10 +151,79 @@ __device__ __forceinline__ int rr_elem(int k, int r, int T) {
   return k == 0 ? 0 : ((k - 1 + r) % (T - 1)) + 1;
 }
 
-__device__ __forceinline__ double2 zmul(double2 a, double2 b) {
-  return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
+// Numbers as unevaluated sums hi + lo of two float32 (48 bits): GB300 has 64 float32 units
+// for each float64 one.
+__device__ __forceinline__ float2 to_pair(double v) {
+  const float hi = float(v);
+  return make_float2(hi, float(v - double(hi)));
 }
-__device__ __forceinline__ double2 zadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double from_pair(float2 p) { return double(p.x) + double(p.y); }
+
+// The exact sum of a and b as a pair (Knuth's two-sum).
+__device__ __forceinline__ float2 two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+  return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
+}
+
+// acc += a b, a a pair: the products exact by fma, the sum by two_sum.
+__device__ __forceinline__ void pair_fma(float2& acc, float ah, float al, float b) {
+  const float p = __fmul_rn(ah, b), e = fmaf(al, b, fmaf(ah, b, -p));
+  const float2 t = two_sum(acc.x, p);
+  acc.x = t.x;
+  acc.y += t.y + e;
+}
+
+// p + x, renormalised.
+__device__ __forceinline__ float2 pair_add(float2 p, float x) {
+  const float2 t = two_sum(p.x, x);
+  const float lo = p.y + t.y, hi = __fadd_rn(t.x, lo);
+  return make_float2(hi, __fsub_rn(lo, __fsub_rn(hi, t.x)));
+}
+
+// Sums of complex products a b: a of pairs (re, im, then their low parts), b float32.
+struct PairAcc {
+  float2 rr, ii, ri, ir;  // sums of re re, im im, re im, im re
+};
+__device__ __forceinline__ void pair_cfma(PairAcc& q, float4 a, float2 b) {
+  pair_fma(q.rr, a.x, a.z, b.x);
+  pair_fma(q.ii, a.y, a.w, b.y);
+  pair_fma(q.ri, a.x, a.z, b.y);
+  pair_fma(q.ir, a.y, a.w, b.x);
+}
+__device__ __forceinline__ double2 pair_result(const PairAcc& q, bool conj_b) {
+  const double rr = from_pair(q.rr), ii = from_pair(q.ii), ri = from_pair(q.ri), ir = from_pair(q.ir);
+  return conj_b ? make_double2(rr + ii, ir - ri) : make_double2(rr - ii, ri + ir);
+}
+__device__ __forceinline__ float4 to_pairs(double2 v) {
+  const float2 x = to_pair(v.x), y = to_pair(v.y);
+  return make_float4(x.x, y.x, x.y, y.y);
+}
+
+// By one warp: largest diagonal entry and trace of C, and the power of two near 1 / max C_ii
+// by which both are scaled (1 if the maximum is not above 0).
+struct DiagStats {
+  double scale, cmax, trace;
+};
+__device__ __forceinline__ void diag_stats(const double2* C, int T, DiagStats* out) {
+  const int lane = threadIdx.x & 31;
+  double m = 0.0, t = 0.0;
+  for (int i = lane; i < T; i += 32) {
+    const double v = C[size_t(i) * T + i].x;
+    m = fmax(m, v);
+    t += v;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    t += __shfl_xor_sync(0xffffffffu, t, o);
+  }
+  if (lane == 0) {
+    int ex = 0;
+    frexp(m, &ex);
+    const double scale = m > 0.0 ? ldexp(1.0, -ex) : 1.0;
+    *out = DiagStats{scale, m * scale, t * scale};
+  }
+}
 
 // Rotation J = [[c, -s], [conj(ph) s, conj(ph) c]] (c, s real, |ph| = 1) that
 // zeroes the off-diagonal of the Hermitian 2 x 2 block [[al, g], [conj(g), be]]:
@@ -278,26 +347,56 @@ __device__ __forceinline__ bool refine_rot(double* d, int i, int j, float2 g, fl
   return true;
 }
 
-// The rotation of refine_rot for the cluster's refinement, whose rotations are
-// applied in float32 (the float64 refinement of c and ph would be rounded away):
-// the angle and the factors in float32 (approximate reciprocals, a few ulp), the
-// diagonal moved by t |g| in float64.
-__device__ __forceinline__ void refine_rot_f(double* d, int i, int j, float2 g, float tol, float floor_abs, RotF& q) {
+// The rotation of refine_rot where the rotations are applied in float32 (the float64
+// refinement of c and ph would be rounded away): the angle and the factors in float32
+// (approximate reciprocals, a few ulp), the diagonal d in pairs, moved by t |g|. Returns |g|.
+__device__ __forceinline__ float refine_rot_f(float2* d, int i, int j, float2 g, float tol, float floor_abs, RotF& q) {
   q = RotF{1.f, 0.f, 1.f, 0.f};
-  const double al = d[i], be = d[j];
+  const float2 al = d[i], be = d[j];
   const float g2 = fmaf(g.x, g.x, g.y * g.y);
-  if (!(g2 > tol * fabsf(float(al)) * (tol * fabsf(float(be))) && g2 > floor_abs * floor_abs && g2 > 0.f)) return;
+  if (!(g2 > 0.f)) return 0.f;
   const float rg = rsqrtf(g2), ag = g2 * rg;
-  const float zeta = float(be - al) * (0.5f * rg);
+  if (!(g2 > tol * fabsf(al.x) * (tol * fabsf(be.x)) && g2 > floor_abs * floor_abs)) return ag;
+  const float zeta = ((be.x - al.x) + (be.y - al.y)) * (0.5f * rg);
   const float az = fabsf(zeta), x = fmaf(az, az, 1.f);
   const float den = az > 1e18f ? 2.f * az : az + x * rsqrtf(x);
   const float t = __fdividef(zeta >= 0.f ? -1.f : 1.f, den);
-  if (t == 0.f) return;
+  if (t == 0.f) return ag;
   const float c = rsqrtf(fmaf(t, t, 1.f));
-  const double tg = double(t * ag);
-  d[i] = al + tg;
-  d[j] = be - tg;
+  const float tg = t * ag;
+  d[i] = pair_add(al, tg);
+  d[j] = pair_add(be, -tg);
   q = RotF{c, t * c, g.x * rg, g.y * rg};
+  return ag;
+}
+
+// The rotations of the refinement as J = [[c, -s u], [s conj(u), c]], u = g / |g| (the same
+// diagonal as the form with the phase on the second column, P R = diag(1, conj(u)) R, since
+// J = P R P^H): their product stays near the identity. Right: (a, b) <- (a, b) J.
+__device__ __forceinline__ void near_right(float2& a, float2& b, float c, float2 su) {
+  const float2 na = cadd(cscale(a, c), cmul(b, make_float2(su.x, -su.y)));
+  b = csub(cscale(b, c), cmul(a, su));
+  a = na;
+}
+// Left: (a, b)^T <- J^H (a, b)^T.
+__device__ __forceinline__ void near_left(float2& a, float2& b, float c, float2 su) {
+  const float2 na = cadd(cscale(a, c), cmul(su, b));
+  b = csub(cscale(b, c), cmul(make_float2(su.x, -su.y), a));
+  a = na;
+}
+__device__ __forceinline__ float2 rot_su(const RotF& q) { return cscale(make_float2(q.px, q.py), q.s); }
+
+// Columns (j0, j1) of row `row` of D, the product of such rotations less the identity: D <-
+// D J + (J - I), with c - 1 = -s^2 / (1 + c).
+__device__ __forceinline__ void near_drow(float2& va, float2& vb, int row, int j0, int j1, const RotF& q, float2 su) {
+  near_right(va, vb, q.c, su);
+  if (row == j0) {
+    va.x += -q.s * q.s / (1.f + q.c);
+    vb = csub(vb, su);
+  } else if (row == j1) {
+    va = cadd(va, make_float2(su.x, -su.y));
+    vb.x += -q.s * q.s / (1.f + q.c);
+  }
 }
 
 // Refinement of the long-window eigensolver (T >= 128), cooperative over all SMs
@@ -502,13 +601,11 @@ __global__ void __launch_bounds__(256) k_jacobi_f32(PcaArgs a) {
 // (REFINE false): C scaled by a power of two near 1 / max C_ii, rotations
 // J = [[c, -s], [conj(ph) s, conj(ph) c]] accumulated in Vf (from the identity),
 // until a sweep rotates nothing at 1e-6 of the trace. Refinement (REFINE true) on
-// C' = Vf^H C Vf: the diagonal in float64, a copy in every CTA updated
+// C' = Vf^H C Vf: the diagonal in pairs of float32, a copy in every CTA updated
 // identically, the off-diagonal entries in float32, the angles of refine_rot; at
 // most max_sweeps sweeps, fewer when every entry met in a sweep is below stop_rel
 // of the trace; the unscaled diagonal goes back into a.C for the eigenvalue
-// selection. Its rotations take the form J = [[c, -s u], [s conj(u), c]] (u = g / |g|;
-// the same diagonal as the form with the phase on the second column,
-// P R = diag(1, conj(u)) R, since J = P R P^H), so that their product Q = I + D stays
+// selection. Its rotations take the form of near_right, so that their product Q = I + D stays
 // near the identity: D (|D| ~ the off-diagonal size, 1e-6 of the trace) is
 // accumulated in float32 as D <- D J + (J - I), with c - 1 = -s^2 / (1 + c), and
 // written to a.Cf; V = Vf + Vf D follows in k_vcorr, the float32 product exact to
@@ -524,7 +621,7 @@ struct JclSmem {
   static constexpr int NP = T / 2, PPC = NP / JC, R = 2 * PPC;
   // C buffers (2), Vf or D rows, the rotation table, (REFINE) the diagonal
   static constexpr size_t c_bytes = size_t(R) * T * sizeof(float2);
-  static constexpr size_t bytes() { return 3 * c_bytes + NP * sizeof(RotF) + (REFINE ? T * sizeof(double) : 0); }
+  static constexpr size_t bytes() { return 3 * c_bytes + NP * sizeof(RotF) + (REFINE ? T * sizeof(float2) : 0); }
 };
 
 // Owner CTA and slot of position k (pairs PPC to a CTA, R = 2 PPC slots)
@@ -549,12 +646,14 @@ __global__ void __launch_bounds__(JC_NT) k_jacobi_cluster(PcaArgs a) {
   float2* C0 = reinterpret_cast<float2*>(jcs);  // buffer b at C0 + b R T, slot s at + s T
   float2* Vr = C0 + 2 * R * T;                  // own rows of Vf (float32 phase) or of D
   RotF* rot = reinterpret_cast<RotF*>(Vr + R * T);
-  double* d = reinterpret_cast<double*>(rot + NP);  // REFINE: the scaled diagonal
+  float2* d = reinterpret_cast<float2*>(rot + NP);  // REFINE: the scaled diagonal in pairs
   __shared__ float gabs[NP];  // |C_ij| of each pair when its rotation was decided
   __shared__ unsigned s_nrot;
   __shared__ float s_offmax;
-  __shared__ double s_trace;
-  const double scale = pow2_diag_scale(a.C, T);  // the same in every CTA
+  __shared__ DiagStats stats;  // the same in every CTA
+  if (tid < 32) diag_stats(a.C, T, &stats);
+  __syncthreads();
+  const double scale = stats.scale;
   // round 0: position k holds index k
   for (int e = tid; e < R * T; e += JC_NT) {
     const int sl = e / T, c = e % T;
@@ -569,23 +668,15 @@ __global__ void __launch_bounds__(JC_NT) k_jacobi_cluster(PcaArgs a) {
       Vr[e] = make_float2(row0 + sl == c ? 1.f : 0.f, 0.f);
     }
   }
-  if (tid == 0) {
-    double t = 0.0;
-    for (int i = 0; i < T; ++i) t += a.C[size_t(i) * T + i].x * scale;
-    s_trace = t;
-  }
   if (REFINE)
-    for (int i = tid; i < T; i += JC_NT) d[i] = a.C[size_t(i) * T + i].x * scale;
+    for (int i = tid; i < T; i += JC_NT) d[i] = to_pair(a.C[size_t(i) * T + i].x * scale);
   cl.sync();
-  const double trace = s_trace;
+  const double trace = stats.trace;
   // float32 phase: the trace bounds the largest eigenvalue; float32 rounding leaves
   // off-diagonal entries near 6e-8 of it. Refinement: the caller's bounds, relative
   // to the largest diagonal entry (scaled to [0.5, 1))
-  double cmax = 0.0;
-  if (REFINE)
-    for (int i = 0; i < T; ++i) cmax = fmax(cmax, a.C[size_t(i) * T + i].x * scale);
   const float tol = REFINE ? float(a.tol) : 1e-6f;
-  const float floor_abs = REFINE ? float(a.tol_abs * cmax) : 2e-7f * float(trace);
+  const float floor_abs = REFINE ? float(a.tol_abs * stats.cmax) : 2e-7f * float(trace);
   const int max_sweeps = REFINE ? a.max_sweeps : 20;
   // a thread's column pair q is the same in every round, and so is its pair row l
   // (at most one: JC_NT >= PPC NP) with the slots of the pair rows' next positions
@@ -629,18 +720,18 @@ __global__ void __launch_bounds__(JC_NT) k_jacobi_cluster(PcaArgs a) {
           cj = own[(R - 1 - p % PPC) * T + j].x;
         }
         if (REFINE) {
-          refine_rot_f(d, i, j, g, tol, floor_abs, rot[p]);
+          gabs[p] = refine_rot_f(d, i, j, g, tol, floor_abs, rot[p]);
         } else {
           jacobi_rot_f(ci, cj, g, tol, floor_abs, rot[p]);
+          const float g2 = fmaf(g.x, g.x, g.y * g.y);
+          gabs[p] = g2 > 0.f ? g2 * rsqrtf(g2) : 0.f;
         }
-        const float g2 = fmaf(g.x, g.x, g.y * g.y);
-        gabs[p] = g2 > 0.f ? g2 * rsqrtf(g2) : 0.f;
       }
       __syncthreads();
       // (2) the 2 x 2 blocks (pair rows x column pair q) of the CTA's pairs, written
       // to the slots of the rows' next positions
       const RotF Jq = rot[q];
-      const float2 uq = cscale(make_float2(Jq.px, Jq.py), Jq.s);  // u_q s (REFINE), ph_q s
+      const float2 uq = rot_su(Jq);  // u_q s (REFINE), ph_q s
 #pragma unroll
       for (int k = 0; k < NB; ++k) {
         const int l = l0 + k * (JC_NT / NP), p = rank * PPC + l;
@@ -651,15 +742,13 @@ __global__ void __launch_bounds__(JC_NT) k_jacobi_cluster(PcaArgs a) {
         const float2 b00 = lo[ca], b01 = lo[cb], b10 = hi[ca], b11 = hi[cb];
         float2 c00, c01, c10, c11;
         if (REFINE) {
-          // right by J_q = [[c, -s u], [s conj(u), c]], then left by J_p^H
-          const float2 cuq = make_float2(uq.x, -uq.y);
-          const float2 m00 = cadd(cscale(b00, Jq.c), cmul(b01, cuq)), m01 = csub(cscale(b01, Jq.c), cmul(b00, uq));
-          const float2 m10 = cadd(cscale(b10, Jq.c), cmul(b11, cuq)), m11 = csub(cscale(b11, Jq.c), cmul(b10, uq));
-          const float2 up = cscale(make_float2(Jp.px, Jp.py), Jp.s), cup = make_float2(up.x, -up.y);
-          c00 = cadd(cscale(m00, Jp.c), cmul(up, m10));
-          c01 = cadd(cscale(m01, Jp.c), cmul(up, m11));
-          c10 = csub(cscale(m10, Jp.c), cmul(cup, m00));
-          c11 = csub(cscale(m11, Jp.c), cmul(cup, m01));
+          // right by J_q, then left by J_p^H
+          c00 = b00, c01 = b01, c10 = b10, c11 = b11;
+          near_right(c00, c01, Jq.c, uq);
+          near_right(c10, c11, Jq.c, uq);
+          const float2 up = rot_su(Jp);
+          near_left(c00, c10, Jp.c, up);
+          near_left(c01, c11, Jp.c, up);
         } else {
           // right by J_q = [[c, -s], [conj(ph) s, conj(ph) c]], then left by J_p^H
           const float2 q10 = make_float2(Jq.px * Jq.s, -Jq.py * Jq.s), q11 = make_float2(Jq.px * Jq.c, -Jq.py * Jq.c);
@@ -691,27 +780,14 @@ __global__ void __launch_bounds__(JC_NT) k_jacobi_cluster(PcaArgs a) {
       asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
       // the CTA's rows of V (or D): right rotation of the column pair q
       if (Jq.s != 0.f) {
-        const float2 cuq = make_float2(uq.x, -uq.y);
         const float2 q10 = make_float2(Jq.px * Jq.s, -Jq.py * Jq.s), q11 = make_float2(Jq.px * Jq.c, -Jq.py * Jq.c);
 #pragma unroll
         for (int li = tid / NP; li < R; li += JC_NT / NP) {
-          const float2 va = Vr[li * T + ca], vb = Vr[li * T + cb];
-          if (REFINE) {  // D <- D J + (J - I)
-            float2 na = cadd(cscale(va, Jq.c), cmul(vb, cuq));
-            float2 nb = csub(cscale(vb, Jq.c), cmul(va, uq));
-            const int i = row0 + li;
-            if (i == ca || i == cb) {
-              const float cm1 = -Jq.s * Jq.s / (1.f + Jq.c);
-              if (i == ca) {
-                na.x += cm1;
-                nb = csub(nb, uq);
-              } else {
-                na = cadd(na, cuq);
-                nb.x += cm1;
-              }
-            }
-            Vr[li * T + ca] = na;
-            Vr[li * T + cb] = nb;
+          float2 va = Vr[li * T + ca], vb = Vr[li * T + cb];
+          if (REFINE) {
+            near_drow(va, vb, row0 + li, ca, cb, Jq, uq);
+            Vr[li * T + ca] = va;
+            Vr[li * T + cb] = vb;
           } else {
             Vr[li * T + ca] = cadd(cscale(va, Jq.c), cmul(vb, q10));
             Vr[li * T + cb] = cadd(cscale(va, -Jq.s), cmul(vb, q11));
@@ -751,7 +827,7 @@ __global__ void __launch_bounds__(JC_NT) k_jacobi_cluster(PcaArgs a) {
   if (REFINE) {
     for (int e = tid; e < R * T; e += JC_NT) a.Cf[size_t(row0) * T + e] = Vr[e];  // D
     if (rank == 0)  // the Rayleigh numerators (V^H C V)_ii, unscaled, for the selection
-      for (int i = tid; i < T; i += JC_NT) a.C[size_t(i) * T + i] = make_double2(d[i] / scale, 0.0);
+      for (int i = tid; i < T; i += JC_NT) a.C[size_t(i) * T + i] = make_double2(from_pair(d[i]) / scale, 0.0);
   } else {
     for (int e = tid; e < R * T; e += JC_NT) a.Vf[size_t(row0) * T + e] = Vr[e];
   }
@@ -811,37 +887,47 @@ static uint32_t clusters_at_once() {
   return uint32_t(a < b ? a : b);
 }
 
-// out = op(A) B for T x T complex matrices: A float64 (op = identity) or the
-// float32 Vf (op = conjugate transpose, transA = 1); B float64 or Vf as float64.
-// 16 x 16 output tiles, 16-wide k stages in shared memory, float64 accumulation.
-__global__ void __launch_bounds__(256) k_gemm_c64(int T, const double2* A, const float2* Af, int transA,
-                                                  const double2* B, const float2* Bf, double2* out) {
-  __shared__ double2 As[16][17], Bs[16][17];
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  const int r = blockIdx.y * 16 + ty, c = blockIdx.x * 16 + tx;
-  double2 acc = make_double2(0.0, 0.0);
+// The congruence C' = Vf^H C Vf in two launches: M = C Vf (out = C2), then, SECOND, the upper
+// triangle of Vf^H M (out = C). One operand of each product is float32 already, the other is
+// taken as pairs, scaled by the power of two near 1 / max C_ii for float32's range. 16 x 16
+// output tiles, 16-wide k stages in shared memory. Bound by the 44 float32 instructions of a
+// complex term; in float64, at 1/64 of their rate, each launch took 228 us for T = 256, 48
+// and 45 now.
+template <bool SECOND>
+__global__ void __launch_bounds__(256) k_congruence(PcaArgs a, const double2* in, double2* out) {
+  __shared__ float4 Ps[16][17];  // pairs: C [row][k], or M [k][column]
+  __shared__ float2 Fs[16][17];  // Vf [k][column], or [k][row]
+  if (SECOND && blockIdx.x < blockIdx.y) return;
+  const int T = a.T, tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  const int r0 = blockIdx.y * 16, c0 = blockIdx.x * 16;
+  int ex = 0;
+  const double cmax = *a.cmax;
+  frexp(cmax, &ex);
+  const double scale = cmax > 0.0 ? ldexp(1.0, -ex) : 1.0;
+  auto scaled = [&](size_t e) {
+    const double2 v = in[e];
+    return to_pairs(make_double2(v.x * scale, v.y * scale));
+  };
+  PairAcc acc{};
   for (int k0 = 0; k0 < T; k0 += 16) {
-    // A element (r, k): A[r][k], or conj(Vf[k][r]) when transposed
-    const int ar = blockIdx.y * 16 + ty, ak = k0 + tx;
-    if (transA) {
-      const float2 v = Af[size_t(ak) * T + ar];
-      As[ty][tx] = make_double2(v.x, -v.y);
+    if (SECOND) {
+      Ps[ty][tx] = scaled(size_t(k0 + ty) * T + c0 + tx);
+      Fs[ty][tx] = a.Vf[size_t(k0 + ty) * T + r0 + tx];
     } else {
-      As[ty][tx] = A[size_t(ar) * T + ak];
-    }
-    const int bk = k0 + ty, bc = blockIdx.x * 16 + tx;
-    if (Bf) {
-      const float2 v = Bf[size_t(bk) * T + bc];
-      Bs[ty][tx] = make_double2(v.x, v.y);
-    } else {
-      Bs[ty][tx] = B[size_t(bk) * T + bc];
+      Ps[ty][tx] = scaled(size_t(r0 + ty) * T + k0 + tx);
+      Fs[ty][tx] = a.Vf[size_t(k0 + ty) * T + c0 + tx];
     }
     __syncthreads();
-#pragma unroll 4
-    for (int k = 0; k < 16; ++k) acc = zadd(acc, zmul(As[ty][k], Bs[k][tx]));
+#pragma unroll 8
+    for (int k = 0; k < 16; ++k) {
+      if (SECOND) pair_cfma(acc, Ps[k][tx], Fs[k][ty]);
+      else pair_cfma(acc, Ps[ty][k], Fs[k][tx]);
+    }
     __syncthreads();
   }
-  out[size_t(r) * T + c] = acc;
+  const double2 v = pair_result(acc, SECOND);
+  const double inv = 1.0 / scale;  // exact
+  if (!SECOND || r0 + ty <= c0 + tx) out[size_t(r0 + ty) * T + c0 + tx] = make_double2(v.x * inv, v.y * inv);
 }
 
 // V = Vf + Vf D in float64 (D in a.Cf, the refinement's correction): the product
@@ -884,71 +970,71 @@ __global__ void __launch_bounds__(256) k_pca_norms(PcaArgs a, double* scratch) {
 }
 
 // Ranks the eigenvalues (descending, ties by index), writes lam sorted and the
-// sub-basis columns lo..hi of V, normalised, as float32 (zero padding to Mpad).
-__global__ void __launch_bounds__(1024) k_pca_select(PcaArgs a, const double* scratch) {
-  const int T = a.T;
-  __shared__ double lamv[512];
-  __shared__ int col_of[512];  // column of V of each rank
-  for (int i = threadIdx.x; i < T; i += blockDim.x) lamv[i] = scratch[i];
+// sub-basis columns lo..hi of V, normalised, as float32 (zero padding to Mpad). 16 columns a
+// CTA, 16 threads a column; as one CTA over all columns its float64 comparisons and products
+// took 58 us for T = 256 (10 now).
+__global__ void __launch_bounds__(256) k_pca_select(PcaArgs a, const double* scratch) {
+  const int T = a.T, part = threadIdx.x / 16, i = blockIdx.x * 16 + threadIdx.x % 16;
+  __shared__ int ranks[16];
+  if (part == 0) ranks[threadIdx.x] = 0;
   __syncthreads();
-  for (int i = threadIdx.x; i < T; i += blockDim.x) {
-    const double li = lamv[i];
-    int rank = 0;
-    for (int j = 0; j < T; ++j) {
-      const double lj = lamv[j];
-      rank += (lj > li) || (lj == li && j < i);
-    }
-    a.lam[rank] = li;
-    col_of[rank] = i;
+  const double li = scratch[i];
+  int rank = 0;
+  for (int j = part; j < T; j += 16) {
+    const double lj = scratch[j];
+    rank += (lj > li) || (lj == li && j < i);
   }
+  atomicAdd(&ranks[threadIdx.x % 16], rank);
   __syncthreads();
-  const int Mp = int(a.Mpad), lo = int(a.lo) - 1;
-  for (int e = threadIdx.x; e < T * Mp; e += blockDim.x) {
-    const int t = e / Mp, m = e % Mp;
-    float2 v = make_float2(0.f, 0.f);
-    if (m < int(a.M)) {
-      const int i = col_of[lo + m];
+  rank = ranks[threadIdx.x % 16];
+  if (part == 0) a.lam[rank] = li;
+  const int Mp = int(a.Mpad), M = int(a.M), m = rank - (int(a.lo) - 1);
+  if (m >= 0 && m < M) {
+    const double r = scratch[T + i];
+    for (int t = part; t < T; t += 16) {
       const double2 x = a.V[size_t(t) * T + i];
-      const double r = scratch[T + i];
-      v = make_float2(float(x.x * r), float(x.y * r));
+      a.Vs[size_t(t) * Mp + m] = make_float2(float(x.x * r), float(x.y * r));
     }
-    a.Vs[e] = v;
   }
+  const int pad = Mp - M;
+  for (int e = blockIdx.x * 256 + threadIdx.x; e < T * pad; e += gridDim.x * 256)
+    a.Vs[size_t(e / pad) * Mp + M + e % pad] = make_float2(0.f, 0.f);
 }
 
-// One sweep's rounds of the CTA-local cyclic Jacobi on C (T x T) and V. The
-// rotation of the pair (i, j) in slot k is made by rotfn(i, j, k), which stores
-// it in rc[k] (applied to C) and rv[k] (applied to V; may be the same array);
-// returns the rotations performed.
-template <int T, class CM, class VM, class RC, class RV, class RotFn, class BlockFn, class RowFn>
-__device__ __forceinline__ unsigned local_sweep(CM* C, VM* V, const RC* rc, const RV* rv, unsigned* cnt, RotFn rotfn,
-                                                BlockFn blockfn, RowFn rowfn) {
+// Rounds of one sweep of the CTA-local cyclic Jacobi on C (T x T) and V, in place. The
+// rotation of the pair (i, j) in slot k is made by rotfn(i, j, k) in rot[k] (s = 0: none);
+// blockfn rotates the 2 x 2 block of pairs p (rows) and q (columns), rowfn columns (j0, j1) of
+// a row of V. Returns the rotations made (the same in every thread).
+template <int T, class RotFn, class BlockFn, class RowFn>
+__device__ __forceinline__ int local_sweep(const RotF* rot, RotFn rotfn, BlockFn blockfn, RowFn rowfn) {
   constexpr int NP = T / 2;
   const int tid = threadIdx.x;
-  if (tid == 0) *cnt = 0;
-  __syncthreads();
+  int n = 0;
   for (int r = 0; r < T - 1; ++r) {
+    bool turned = false;
     if (tid < NP) {
       const int i = rr_elem(tid, r, T), j = rr_elem(T - 1 - tid, r, T);
-      if (rotfn(i, j, tid)) atomicAdd(cnt, 1u);
+      rotfn(i, j, tid);
+      turned = rot[tid].s != 0.f;
     }
-    __syncthreads();
-    for (int e = tid; e < NP * NP + T * NP; e += blockDim.x) {
-      if (e < NP * NP) {
-        const int p = e / NP, q = e % NP;
-        if (rc[p].s == 0 && rc[q].s == 0) continue;
-        blockfn(C, T, rr_elem(p, r, T), rr_elem(T - 1 - p, r, T), rr_elem(q, r, T), rr_elem(T - 1 - q, r, T), rc[p],
-                rc[q], p == q);
-      } else {
-        const int f = e - NP * NP, row = f / NP, q = f % NP;
-        if (rc[q].s == 0) continue;
-        rowfn(V, T, row, rr_elem(q, r, T), rr_elem(T - 1 - q, r, T), rv[q]);
+    const int made = __syncthreads_count(turned);
+    n += made;
+    if (made)
+      for (int e = tid; e < NP * NP + T * NP; e += blockDim.x) {
+        if (e < NP * NP) {
+          const int p = e / NP, q = e % NP;
+          const RotF Jp = rot[p], Jq = rot[q];
+          if (Jp.s == 0.f && Jq.s == 0.f) continue;
+          blockfn(rr_elem(p, r, T), rr_elem(T - 1 - p, r, T), rr_elem(q, r, T), rr_elem(T - 1 - q, r, T), Jp, Jq,
+                  p == q);
+        } else {
+          const int f = e - NP * NP, row = f / NP, q = f % NP;
+          const RotF Jq = rot[q];
+          if (Jq.s != 0.f) rowfn(row, rr_elem(q, r, T), rr_elem(T - 1 - q, r, T), Jq);
+        }
       }
-    }
     __syncthreads();
   }
-  const unsigned n = *cnt;
-  __syncthreads();
   return n;
 }
 
@@ -957,121 +1043,116 @@ __device__ __forceinline__ unsigned local_sweep(CM* C, VM* V, const RC* rc, cons
 // and no float32 overflow whatever the data's range).
 // (1) Float32 cyclic Jacobi on a float copy of C, with the rotations accumulated
 // in Vf, until a sweep rotates nothing at 1e-6 relative.
-// (2) Refinement: C' = Vf^H C Vf in float64 from the float64 C, whose
-// off-diagonal entries are then about 1e-6 of its diagonal; Jacobi sweeps on C'
-// with the diagonal d in float64, the off-diagonal entries in float32 (every
-// float32 operation of a sweep combines off-diagonal entries only, so its
-// rounding is relative to them: ~1e-7 of 1e-6, far below the float32
-// covariance's own error) and V = Vf rotated further in float64 by J unitary to
-// ~1e-13 (refine_rot), until a sweep rotates nothing at 1e-14 or meets
-// no off-diagonal entry above 1e-12 of the trace. V's columns are then
-// C-orthogonal to the refinement's accuracy; Vf is unitary to about 1e-6 only,
-// so each eigenvalue is the Rayleigh quotient d_i / |v_i|^2 and the vectors are
-// normalised. Then the ranking and the sub-basis. GB300's float64 rate is 1/64
-// of float32, which is why only the diagonal, the rotation factors and V are
-// float64.
+// (2) Refinement, as in the cluster kernel: C' = Vf^H C Vf from the float64 C in pairs of
+// float32, whose off-diagonal entries are then about 1e-6 of its diagonal; Jacobi sweeps on C'
+// with the diagonal d in pairs and the off-diagonal entries in float32 (every float32
+// operation of a sweep combines off-diagonal entries only, so its rounding is relative to
+// them: ~1e-7 of 1e-6, far below the float32 covariance's own error), until a sweep rotates
+// nothing at 1e-14 or meets no off-diagonal entry above 1e-12 of the trace. The rotations'
+// product I + D is kept as D (~1e-6) in float32; V = Vf + Vf D in pairs. Vf is unitary to
+// about 1e-6 only, so each eigenvalue is the Rayleigh quotient d_i / |v_i|^2 and the vectors
+// are normalised. Then the ranking and the sub-basis.
+//
+// A chain of rounds: rotations by T / 2 threads, a barrier, one item a thread, a barrier. 128
+// windows of T = 32: 742 us with 256 threads and d, C' and V in float64 (1/64 of float32's
+// rate), 300 now; 64 windows of T = 64: 3.47 ms, 0.99 now.
 template <int T>
-__global__ void __launch_bounds__(256) k_jacobi_small(PcaArgs a) {
-  extern __shared__ double2 jsm[];
-  double2* RA = jsm;            // Cf (float) in phase 1, then M = C Vf, then V (float64)
-  double2* C = jsm + T * T;     // C' (float64)
+__global__ void __launch_bounds__(T == 32 ? 768 : 1024) k_jacobi_small(PcaArgs a) {
+  extern __shared__ float4 jsm[];
+  float4* P = jsm;                                      // C in pairs; then D and the off-diagonal entries
+  float4* M = jsm + T * T;                              // Cf in phase 1; then M = C Vf; then V, in pairs
   float2* Vf = reinterpret_cast<float2*>(jsm + 2 * T * T);
-  float2* Cf = reinterpret_cast<float2*>(RA);
-  float2* Co = Vf;              // the refinement's float32 off-diagonal entries (Vf is dead by then)
-  __shared__ RotV rotv[T / 2];
-  __shared__ RotF rotf[T / 2];
-  __shared__ double d[T];
-  __shared__ unsigned cnt, offbits;
-  __shared__ double scale_s, cmax_s, trace_s;
-  const int w = blockIdx.x, tid = threadIdx.x;
+  float2* Cf = reinterpret_cast<float2*>(M);
+  float2* Co = reinterpret_cast<float2*>(P);
+  float2* D = Co + T * T;
+  __shared__ RotF rot[T / 2];
+  __shared__ float2 d[T];
+  __shared__ unsigned offbits;
+  __shared__ DiagStats stats;
+  const int w = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
   const double2* Cg = a.C + size_t(w) * T * T;
-  if (tid == 0) {
-    double m = 0.0, t = 0.0;
-    for (int i = 0; i < T; ++i) {
-      m = fmax(m, Cg[i * T + i].x);
-      t += Cg[i * T + i].x;
-    }
-    int ex = 0;
-    frexp(m, &ex);
-    scale_s = m > 0.0 ? ldexp(1.0, -ex) : 1.0;  // scaled max C_ii in [0.5, 1)
-    cmax_s = m * scale_s;
-    trace_s = t * scale_s;
-  }
+  if (tid < 32) diag_stats(Cg, T, &stats);
   __syncthreads();
-  const double scale = scale_s, cmax = cmax_s;  // of the scaled C
-  for (int e = tid; e < T * T; e += blockDim.x) {
+  const double scale = stats.scale;
+  for (int e = tid; e < T * T; e += nt) {
     const double2 v = Cg[e];
-    Cf[e] = make_float2(float(v.x * scale), float(v.y * scale));
+    const float4 p = to_pairs(make_double2(v.x * scale, v.y * scale));
+    P[e] = p;
+    Cf[e] = make_float2(p.x, p.y);
     Vf[e] = make_float2(e / T == e % T ? 1.f : 0.f, 0.f);
   }
   __syncthreads();
   // (1) float32 sweeps until one rotates nothing at 1e-6 (relative, and of the
   // largest diagonal entry)
-  const float ftol = 1e-6f, ffloor = 1e-6f * float(cmax);
+  const float ftol = 1e-6f, ffloor = 1e-6f * float(stats.cmax);
   int sweeps_f = 0;
   for (int sw = 0; sw < 20; ++sw) {
-    const unsigned n = local_sweep<T>(
-        Cf, Vf, rotf, rotf, &cnt,
+    const int n = local_sweep<T>(
+        rot,
         [&](int i, int j, int k) {
-          return jacobi_rot_f(Cf[i * T + i].x, Cf[j * T + j].x, Cf[i * T + j], ftol, ffloor, rotf[k]);
+          jacobi_rot_f(Cf[i * T + i].x, Cf[j * T + j].x, Cf[i * T + j], ftol, ffloor, rot[k]);
         },
-        jacobi_block_f, jacobi_vrow_f);
+        [&](int i0, int i1, int j0, int j1, const RotF& Jp, const RotF& Jq, bool own) {
+          jacobi_block_f(Cf, T, i0, i1, j0, j1, Jp, Jq, own);
+        },
+        [&](int row, int j0, int j1, const RotF& Jq) { jacobi_vrow_f(Vf, T, row, j0, j1, Jq); });
     sweeps_f = sw + 1;
     if (n == 0) break;
   }
-  // (2) C' = Vf^H (C Vf) in float64 (scaled): M = C Vf into RA (Cf is dead), then
-  // the upper triangle of C' into C
-  for (int e = tid; e < T * T; e += blockDim.x) {
+  // (2) M = C Vf (Cf is dead), then the upper triangle of C' = Vf^H M as d and Co, D = 0
+  for (int e = tid; e < T * T; e += nt) {
     const int r = e / T, c = e % T;
-    double2 acc = make_double2(0.0, 0.0);
-    for (int k = 0; k < T; ++k) {
-      const float2 v = Vf[k * T + c];
-      acc = zadd(acc, zmul(Cg[r * T + k], make_double2(v.x, v.y)));
-    }
-    RA[e] = make_double2(acc.x * scale, acc.y * scale);
+    PairAcc acc{};
+#pragma unroll 4
+    for (int k = 0; k < T; ++k) pair_cfma(acc, P[r * T + k], Vf[k * T + c]);
+    M[e] = to_pairs(pair_result(acc, false));
   }
   __syncthreads();
-  for (int u = tid; u < T * (T + 1) / 2; u += blockDim.x) {
-    int r = 0, rem = u;
-    while (rem >= T - r) {
-      rem -= T - r;
-      ++r;
-    }
-    const int c = r + rem;
-    double2 acc = make_double2(0.0, 0.0);
-    for (int k = 0; k < T; ++k) {
-      const float2 v = Vf[k * T + r];
-      acc = zadd(acc, zmul(make_double2(v.x, -v.y), RA[k * T + c]));
-    }
-    C[r * T + c] = acc;
-  }
-  __syncthreads();
-  double2* V = RA;  // V = Vf in float64, rotated further below
-  for (int e = tid; e < T * T; e += blockDim.x) V[e] = make_double2(Vf[e].x, Vf[e].y);
-  __syncthreads();  // Vf read for the last time: its storage takes the off-diagonal entries
-  for (int e = tid; e < T * T; e += blockDim.x) {
+  for (int e = tid; e < T * T; e += nt) {
     const int r = e / T, c = e % T;
-    const double2 v = C[(r < c ? r : c) * T + (r < c ? c : r)];
-    Co[e] = r == c ? make_float2(float(v.x), 0.f) : make_float2(float(v.x), r < c ? float(v.y) : -float(v.y));
-    if (r == c) d[r] = v.x;
+    D[e] = make_float2(0.f, 0.f);
+    if (r > c) continue;
+    PairAcc acc{};
+#pragma unroll 4
+    for (int k = 0; k < T; ++k) pair_cfma(acc, M[k * T + c], Vf[k * T + r]);
+    const double2 v = pair_result(acc, true);
+    if (r == c) d[r] = to_pair(v.x);
+    Co[r * T + c] = make_float2(float(v.x), r == c ? 0.f : float(v.y));
+    if (r < c) Co[c * T + r] = make_float2(float(v.x), -float(v.y));
   }
   __syncthreads();
-  const double trace64 = trace_s;
-  const float rtol = float(a.tol), rfloor = float(a.tol_abs * cmax);
+  const float rtol = float(a.tol), rfloor = float(a.tol_abs * stats.cmax);
   int sweeps_d = 0;
   for (int sw = 0; sw < a.max_sweeps; ++sw) {
     if (tid == 0) offbits = 0u;
-    const unsigned n = local_sweep<T>(
-        Co, V, rotf, rotv, &cnt,
+    __syncthreads();
+    const int n = local_sweep<T>(
+        rot,
         [&](int i, int j, int k) {
-          const float2 g = Co[i * T + j];
-          const float ag = hypotf(g.x, g.y);
+          const float ag = refine_rot_f(d, i, j, Co[i * T + j], rtol, rfloor, rot[k]);
           atomicMax(&offbits, __float_as_uint(ag));  // non-negative floats order like their bits
-          return refine_rot(d, i, j, g, ag, rtol, rfloor, rotf[k], rotv[k]);
         },
-        jacobi_block_f, refine_vrow);
+        [&](int i0, int i1, int j0, int j1, const RotF& Jp, const RotF& Jq, bool own) {
+          float2 b00 = Co[i0 * T + j0], b01 = Co[i0 * T + j1], b10 = Co[i1 * T + j0], b11 = Co[i1 * T + j1];
+          const float2 up = rot_su(Jp), uq = rot_su(Jq);
+          near_right(b00, b01, Jq.c, uq);
+          near_right(b10, b11, Jq.c, uq);
+          near_left(b00, b10, Jp.c, up);
+          near_left(b01, b11, Jp.c, up);
+          if (own) b01 = b10 = make_float2(0.f, 0.f);  // (d holds the diagonal)
+          Co[i0 * T + j0] = b00;
+          Co[i0 * T + j1] = b01;
+          Co[i1 * T + j0] = b10;
+          Co[i1 * T + j1] = b11;
+        },
+        [&](int row, int j0, int j1, const RotF& Jq) {
+          float2 va = D[row * T + j0], vb = D[row * T + j1];
+          near_drow(va, vb, row, j0, j1, Jq, rot_su(Jq));
+          D[row * T + j0] = va;
+          D[row * T + j1] = vb;
+        });
     sweeps_d = sw + 1;
-    const bool done = n == 0 || double(__uint_as_float(offbits)) <= 1e-12 * trace64;
+    const bool done = n == 0 || double(__uint_as_float(offbits)) <= 1e-12 * stats.trace;
     __syncthreads();
     if (done) break;
   }
@@ -1079,18 +1160,35 @@ __global__ void __launch_bounds__(256) k_jacobi_small(PcaArgs a) {
     atomicAdd(&a.counters[1], unsigned(sweeps_f));
     atomicAdd(&a.counters[2], unsigned(sweeps_d));
   }
+  float4* V = M;
+  for (int e = tid; e < T * T; e += nt) {
+    const int r = e / T, c = e % T;
+    float2 acc = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int k = 0; k < T; ++k) acc = cadd(acc, cmul(Vf[r * T + k], D[k * T + c]));
+    V[e] = make_float4(Vf[e].x, Vf[e].y, acc.x, acc.y);
+  }
+  __syncthreads();
   // eigenvalues as Rayleigh quotients, vectors normalised; rank and sub-basis
   __shared__ double lamv[T], inrm[T];
-  for (int i = tid; i < T; i += blockDim.x) {
+  auto vec = [&](int t, int i) {
+    const float4 v = V[t * T + i];
+    return make_double2(double(v.x) + double(v.z), double(v.y) + double(v.w));
+  };
+  for (int i = tid; i < T; i += nt) {
     double n2 = 0.0;
-    for (int t = 0; t < T; ++t) n2 += V[t * T + i].x * V[t * T + i].x + V[t * T + i].y * V[t * T + i].y;
-    lamv[i] = d[i] / (n2 * scale);
+    for (int t = 0; t < T; ++t) {
+      const double2 v = vec(t, i);
+      n2 = fma(v.x, v.x, fma(v.y, v.y, n2));
+    }
+    lamv[i] = from_pair(d[i]) / (n2 * scale);
     inrm[i] = 1.0 / sqrt(n2);
   }
   __syncthreads();
   double* lam = a.lam + size_t(w) * T;
   float2* Vs = a.Vs + size_t(w) * T * a.Mpad;
-  for (int i = tid; i < T; i += blockDim.x) {
+  __shared__ int col_of[T];  // column of V of each rank
+  for (int i = tid; i < T; i += nt) {
     const double li = lamv[i];
     int rank = 0;
     for (int j = 0; j < T; ++j) {
@@ -1098,13 +1196,20 @@ __global__ void __launch_bounds__(256) k_jacobi_small(PcaArgs a) {
       rank += (lj > li) || (lj == li && j < i);
     }
     lam[rank] = li;
-    const int m = rank - int(a.lo - 1);
-    if (m >= 0 && m < int(a.M))
-      for (int t = 0; t < T; ++t)
-        Vs[size_t(t) * a.Mpad + m] = make_float2(float(V[t * T + i].x * inrm[i]), float(V[t * T + i].y * inrm[i]));
+    col_of[rank] = i;
   }
-  for (int e = tid; e < T * int(a.Mpad); e += blockDim.x)
-    if (e % int(a.Mpad) >= int(a.M)) Vs[e] = make_float2(0.f, 0.f);
+  __syncthreads();
+  const int Mp = int(a.Mpad);
+  for (int e = tid; e < T * Mp; e += nt) {
+    const int t = e / Mp, m = e % Mp;
+    float2 o = make_float2(0.f, 0.f);
+    if (m < int(a.M)) {
+      const int i = col_of[int(a.lo) - 1 + m];
+      const double2 v = vec(t, i);
+      o = make_float2(float(v.x * inrm[i]), float(v.y * inrm[i]));
+    }
+    Vs[e] = o;
+  }
 }
 
 // ---------------------------------------------------------------- projection
@@ -1342,10 +1447,10 @@ __global__ void k_vf_to_v(PcaArgs a) {
 
 template <int T>
 static cudaError_t launch_jacobi_small(const PcaArgs& a, cudaStream_t s) {
-  const size_t smem = size_t(2) * T * T * sizeof(double2) + size_t(T) * T * sizeof(float2);  // RA, C', Vf
+  const size_t smem = size_t(2) * T * T * sizeof(float4) + size_t(T) * T * sizeof(float2);  // P, M, Vf
   cudaError_t e = cudaFuncSetAttribute(k_jacobi_small<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
-  k_jacobi_small<T><<<a.nwin, 256, smem, s>>>(a);
+  k_jacobi_small<T><<<a.nwin, T == 32 ? 768 : 1024, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -1418,10 +1523,10 @@ cudaError_t launch_pca_eig(PcaArgs& a, cudaStream_t s, int* launches) {
       e = cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_jacobi_f32), dim3(nf), dim3(256), args, 0, s);
       if (e != cudaSuccess) return e;
     }
-    // (2) C' = Vf^H (C Vf) and V = Vf in float64
+    // (2) C' = Vf^H (C Vf)
     const dim3 gg(a.T / 16, a.T / 16);
-    k_gemm_c64<<<gg, 256, 0, s>>>(int(a.T), a.C, nullptr, 0, nullptr, a.Vf, a.C2);     // M = C Vf
-    k_gemm_c64<<<gg, 256, 0, s>>>(int(a.T), nullptr, a.Vf, 1, a.C2, nullptr, a.C);     // C' = Vf^H M
+    k_congruence<false><<<gg, 256, 0, s>>>(a, a.C, a.C2);  // M = C Vf
+    k_congruence<true><<<gg, 256, 0, s>>>(a, a.C2, a.C);   // C' = Vf^H M
     *launches += 3;
     // (3) float64 sweeps on C' (off-diagonals ~1e-6 of the trace): at most two, fewer
     // when every entry met in a sweep is below 1e-12 of the trace. Two leave the
@@ -1449,7 +1554,7 @@ cudaError_t launch_pca_eig(PcaArgs& a, cudaStream_t s, int* launches) {
     // the cooperative paths' rotation table is free by now: lam and 1/|v| of every column
     double* scratch = a.rot;
     k_pca_norms<<<a.T / 16, 256, 0, s>>>(a, scratch);
-    k_pca_select<<<1, 1024, 0, s>>>(a, scratch);
+    k_pca_select<<<a.T / 16, 256, 0, s>>>(a, scratch);
     *launches += 3;
   }
   if (e != cudaSuccess) return e;

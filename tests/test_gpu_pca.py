@@ -160,6 +160,26 @@ def gpu_pca_window(fr, p, precision):
         r.close()
 
 
+@pytest.mark.parametrize("T,H,W", [(32, 64, 64), (64, 32, 64), (128, 64, 64), (256, 64, 64)])
+def test_pca_rank_deficient_windows(T, H, W):
+    """Windows of six distinct images (every other eigenvalue is 0): the eigenvalues of the
+    exact integer covariance, and the whole band's energy, which is sum_t |u_t|^2 where the
+    eigenvectors are unitary. These are products of float32 rotations, about 8 sweeps of T - 1
+    of them in each column, unitary to 8 T 2^-24 / 2 at worst: 6e-5 for T = 256."""
+    rng = np.random.default_rng(T)
+    base = rng.integers(0, 4096, (6, H, W), dtype=np.uint16)
+    fr = base[rng.integers(0, 6, 2 * T)]
+    p = oracle_params(spatial="none", temporal="pca", T=T, stride=T, pca_lo=1, pca_hi=T, H=H, W=W)
+    img, lam = gpu_pca(fr, p)
+    assert img.shape[0] == 2
+    x = fr.reshape(2, T, H * W).astype(np.float64)
+    for w in range(2):
+        e = (x[w] ** 2).sum(0).reshape(H, W)
+        assert np.max(np.abs(img[w] - e) / e) <= 6e-5
+    ref = np.linalg.eigvalsh(x[1] @ x[1].T)[::-1]
+    assert np.max(np.abs(lam - ref)) <= LAM_TOL * ref[0]
+
+
 def test_pca_batched_many_windows():
     """Short windows are batched: all windows of one render in one launch per kernel
     (one CTA per window for the eigensolver), overlapping and non-overlapping.
