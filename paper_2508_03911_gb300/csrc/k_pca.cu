@@ -390,12 +390,10 @@ __device__ __forceinline__ float2 rot_su(const RotF& q) { return cscale(make_flo
 // D J + (J - I), with c - 1 = -s^2 / (1 + c).
 __device__ __forceinline__ void near_drow(float2& va, float2& vb, int row, int j0, int j1, const RotF& q, float2 su) {
   near_right(va, vb, q.c, su);
-  if (row == j0) {
-    va.x += -q.s * q.s / (1.f + q.c);
-    vb = csub(vb, su);
-  } else if (row == j1) {
-    va = cadd(va, make_float2(su.x, -su.y));
-    vb.x += -q.s * q.s / (1.f + q.c);
+  if (row == j0 || row == j1) {
+    const float cm1 = __fdividef(-q.s * q.s, 1.f + q.c);
+    if (row == j0) va.x += cm1, vb = csub(vb, su);
+    else va = cadd(va, make_float2(su.x, -su.y)), vb.x += cm1;
   }
 }
 
@@ -591,10 +589,12 @@ __global__ void __launch_bounds__(256) k_jacobi_f32(PcaArgs a) {
 // so the left rotation of a row mixes it with a local row. Rows are double
 // buffered: round r reads buffer r & 1 and writes each new row straight into the
 // slot of its next position in buffer (r + 1) & 1 -- of the same CTA, except for
-// two rows a round that go to a neighbour's shared memory. A round: (1) every CTA
-// reads each pair's off-diagonal entry (and in the float32 phase both diagonal
-// entries) from the owners' shared memory and computes all rotations itself (a
-// deterministic function of the same data, so all CTAs agree); (2) it rotates the
+// two rows a round that go to a neighbour's shared memory, and the entries that
+// decide the next round's rotations also into a record of 16 bytes at the pair's next
+// owner. A round: (1) every CTA reads all records (128 bytes in a run from each owner;
+// straight from the rows, 3 scattered reads a pair, they took 0.43 of 1.89 us a round for
+// T = 256) and computes all rotations itself (a deterministic function of the same
+// data, so all CTAs agree); (2) it rotates the
 // 2 x 2 blocks of its pairs' rows (left by the pair's rotation, right by each
 // column pair's) and the column pairs of its rows of V (CTA c owns rows c R ..
 // c R + R - 1 of V, which do not move); (3) one cluster barrier. Float32 phase
@@ -619,9 +619,9 @@ constexpr int JC_NT = 512;
 template <int T, bool REFINE>
 struct JclSmem {
   static constexpr int NP = T / 2, PPC = NP / JC, R = 2 * PPC;
-  // C buffers (2), Vf or D rows, the rotation table, (REFINE) the diagonal
+  // C buffers (2), Vf or D rows, the rotation table, pair records (2), (REFINE) the diagonal
   static constexpr size_t c_bytes = size_t(R) * T * sizeof(float2);
-  static constexpr size_t bytes() { return 3 * c_bytes + NP * sizeof(RotF) + (REFINE ? T * sizeof(float2) : 0); }
+  static constexpr size_t bytes() { return 3 * c_bytes + NP * sizeof(RotF) + 2 * PPC * sizeof(float4) + (REFINE ? T * sizeof(float2) : 0); }
 };
 
 // Owner CTA and slot of position k (pairs PPC to a CTA, R = 2 PPC slots)
@@ -646,7 +646,9 @@ __global__ void __launch_bounds__(JC_NT) k_jacobi_cluster(PcaArgs a) {
   float2* C0 = reinterpret_cast<float2*>(jcs);  // buffer b at C0 + b R T, slot s at + s T
   float2* Vr = C0 + 2 * R * T;                  // own rows of Vf (float32 phase) or of D
   RotF* rot = reinterpret_cast<RotF*>(Vr + R * T);
-  float2* d = reinterpret_cast<float2*>(rot + NP);  // REFINE: the scaled diagonal in pairs
+  // own pairs' off-diagonal entry and two diagonal entries in round r, buffer r & 1
+  float4* rec = reinterpret_cast<float4*>(rot + NP);
+  float2* d = reinterpret_cast<float2*>(rec + 2 * PPC);  // REFINE: the scaled diagonal in pairs
   __shared__ float gabs[NP];  // |C_ij| of each pair when its rotation was decided
   __shared__ unsigned s_nrot;
   __shared__ float s_offmax;
@@ -668,6 +670,12 @@ __global__ void __launch_bounds__(JC_NT) k_jacobi_cluster(PcaArgs a) {
       Vr[e] = make_float2(row0 + sl == c ? 1.f : 0.f, 0.f);
     }
   }
+  if (tid < PPC) {
+    const int i = rank * PPC + tid, j = T - 1 - i;
+    const double2 g = a.C[size_t(i) * T + j];
+    rec[tid] = make_float4(float(g.x * scale), float(g.y * scale), float(a.C[size_t(i) * T + i].x * scale),
+                           float(a.C[size_t(j) * T + j].x * scale));
+  }
   if (REFINE)
     for (int i = tid; i < T; i += JC_NT) d[i] = to_pair(a.C[size_t(i) * T + i].x * scale);
   cl.sync();
@@ -681,13 +689,18 @@ __global__ void __launch_bounds__(JC_NT) k_jacobi_cluster(PcaArgs a) {
   // a thread's column pair q is the same in every round, and so is its pair row l
   // (at most one: JC_NT >= PPC NP) with the slots of the pair rows' next positions
   constexpr int NB = (PPC * NP + JC_NT - 1) / JC_NT;  // pair blocks per thread: pair rows l0 + k JC_NT / NP
-  static_assert(JC_NT % NP == 0 && NB <= 2, "pair blocks per thread");
+  static_assert(JC_NT % NP == 0 && NB <= 2 && PPC % 2 == 0, "pair blocks per thread");
   const int q = tid % NP, l0 = tid / NP;
+  // outermost first: their rows are those that go to a neighbour, and on their way longest
+  auto pair_row = [&](int k) {
+    const int g = l0 + k * (JC_NT / NP);
+    return g >= PPC ? PPC : (g & 1 ? PPC - 1 - g / 2 : g / 2);
+  };
   float2* nlo[NB];  // buffer 0 of the slot of the next position of each pair row
   float2* nhi[NB];
 #pragma unroll
   for (int k = 0; k < NB; ++k) {
-    const int l = l0 + k * (JC_NT / NP);
+    const int l = pair_row(k);
     nlo[k] = nhi[k] = nullptr;
     if (l >= PPC) continue;
     const int p = rank * PPC + l, klo = p, khi = T - 1 - p;
@@ -708,21 +721,15 @@ __global__ void __launch_bounds__(JC_NT) k_jacobi_cluster(PcaArgs a) {
     float offmax = 0.f;
     for (int r = 0; r < T - 1; ++r) {
       const float2* Cs = C0 + cur * R * T;
-      // (1) every pair's rotation, from its owner's rows
+      // (1) every pair's rotation, from its owner's record
       if (tid < NP) {
-        const int p = tid, i = ri, j = rj;
-        const float2* own = cl.map_shared_rank(Cs, p / PPC);
-        const float2* lo = own + (p % PPC) * T;
-        const float2 g = lo[j];
-        float ci = 0.f, cj = 0.f;
-        if (!REFINE) {
-          ci = lo[i].x;
-          cj = own[(R - 1 - p % PPC) * T + j].x;
-        }
+        const int p = tid;
+        const float4 in = cl.map_shared_rank(rec, p / PPC)[cur * PPC + p % PPC];
+        const float2 g = make_float2(in.x, in.y);
         if (REFINE) {
-          gabs[p] = refine_rot_f(d, i, j, g, tol, floor_abs, rot[p]);
+          gabs[p] = refine_rot_f(d, ri, rj, g, tol, floor_abs, rot[p]);
         } else {
-          jacobi_rot_f(ci, cj, g, tol, floor_abs, rot[p]);
+          jacobi_rot_f(in.z, in.w, g, tol, floor_abs, rot[p]);
           const float g2 = fmaf(g.x, g.x, g.y * g.y);
           gabs[p] = g2 > 0.f ? g2 * rsqrtf(g2) : 0.f;
         }
@@ -734,7 +741,7 @@ __global__ void __launch_bounds__(JC_NT) k_jacobi_cluster(PcaArgs a) {
       const float2 uq = rot_su(Jq);  // u_q s (REFINE), ph_q s
 #pragma unroll
       for (int k = 0; k < NB; ++k) {
-        const int l = l0 + k * (JC_NT / NP), p = rank * PPC + l;
+        const int l = pair_row(k), p = rank * PPC + l;
         if (l >= PPC) continue;
         const RotF Jp = rot[p];
         const float2* lo = Cs + l * T;
@@ -773,6 +780,18 @@ __global__ void __launch_bounds__(JC_NT) k_jacobi_cluster(PcaArgs a) {
         dlo[cb] = c01;
         dhi[ca] = c10;
         dhi[cb] = c11;
+        // the next round's records: pair n joins positions n and T-1-n, held now by positions
+        // n+1 and T-n (0, 1 for n = 0; T/2, T/2+1 for n = T/2-1)
+        auto next = [&](int n) { return cl.map_shared_rank(rec, n / PPC) + (cur ^ 1) * PPC + n % PPC; };
+        if (q == p - 2) *reinterpret_cast<float2*>(next(p - 1)) = c01;
+        if (p == 0 && q == 1) *reinterpret_cast<float2*>(next(0)) = c00;
+        if (p == NP - 1 && q == NP - 2) *reinterpret_cast<float2*>(next(NP - 1)) = c11;
+        if (!REFINE && q == p) {
+          if (p == 1) next(0)->w = c00.x;
+          else next(p == 0 ? 0 : p - 1)->z = c00.x;
+          if (p == NP - 1) next(NP - 1)->z = c11.x;
+          else next(p + 1)->w = c11.x;
+        }
       }
       // (3) this CTA's new rows are written (some into a neighbour) and its reads of the
       // round done: arrive on the cluster barrier, rotate the local rows of V while
