@@ -417,9 +417,13 @@ hv_status apply_pending(hv_handle* h) {
     const bool batched = d.T <= 64 && p.precision == HV_PREC_FP32;
     const uint32_t NW = batched ? 128 : 1;  // windows per launch
     // batched (T <= 64): 2048-pixel chunks, one partial T x T matrix per chunk and window;
-    // otherwise up to 64 chunks of the tiled covariance
+    // otherwise chunks of the tiled covariance: at most 64 of at least 1,024 pixels, or of
+    // 256 pixels up to four CTAs per SM where there are few tiles (T = 128 of 128 x 128: 16
+    // chunks of 3 tiles 208 us and 7 to sum them, 64 chunks 74 and 21)
+    const size_t nt = (d.T + 63) / 64, tiles = nt * (nt + 1) / 2;
     uint32_t nchunks = batched ? uint32_t(std::max<size_t>(1, hw / 2048))
-                               : uint32_t(std::min<size_t>(64, std::max<size_t>(1, hw / 1024)));
+                               : uint32_t(std::max(std::min<size_t>(64, std::max<size_t>(1, hw / 1024)),
+                                                   std::min<size_t>(hw / 256, 4 * 152 / tiles)));
     uint32_t chunk = uint32_t((hw + nchunks - 1) / nchunks);
     chunk = (chunk + 63) / 64 * 64;
     nchunks = uint32_t((hw + chunk - 1) / chunk);

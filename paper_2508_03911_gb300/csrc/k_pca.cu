@@ -1326,20 +1326,23 @@ static cudaError_t launch_project(const PcaArgs& a, float* out, cudaStream_t s) 
 
 // -------------------------------------------------- covariance of short windows
 //
-// T <= 64: a group of (T/4)^2 threads covers the whole T x T matrix with 4 x 4
-// complex tiles (thread (ta, tb): rows 4 ta.., columns 4 tb..); the CTA's
-// 256 / (T/4)^2 groups take alternate pixels of each staged strip. A strip is
-// SP pixels of all T frames of the window, [t][p] in shared memory (row stride
-// SP + 1), fetched with cp.async into one of two buffers while the other is
-// used. The groups' sums are added in shared memory and each CTA writes its
-// partial matrix part[window][cta][T][T]; a second kernel sums them in float64.
+// T <= 64: a group of threads covers one triangle of the T x T matrix with 4 x 4 complex
+// tiles: thread (ta, tb), ta <= tb, rows ta + T/4 i and columns tb + T/4 j, so that the
+// rows that neighbouring threads read lie one row stride apart, in different banks (rows
+// 4 ta + i met in the same banks two or four at a time). The CTA's groups (7 of 36 threads
+// for T = 32, 2 of 136 for T = 64) take alternate pixels of each staged strip. A strip is
+// SP pixels of all T frames of the window, [t][p] in shared memory (row stride SP + 1),
+// fetched with cp.async into one of two buffers while the other is used. The groups' sums
+// are added in shared memory and each CTA writes its partial matrix part[window][cta][T][T]
+// (upper triangle); a second kernel sums them in float64. 128 windows of 256 x 256, T = 32:
+// 1040 us before, 991 now; 64 windows, T = 64, over all 256 tiles: 2940 us before, 2016 now.
 constexpr int CS_SP = 64;
 
-// Groups of k_cov_small<T> (tiles per group: the upper triangle's for T = 32) and
-// its dynamic shared memory: two strip buffers, or the groups' partial matrices
-// at the end, whichever is larger.
+// Threads and groups of k_cov_small<T> and its dynamic shared memory: two strip buffers, or
+// the groups' partial matrices at the end, whichever is larger.
+__host__ __device__ constexpr int cov_small_threads(int T) { return T == 64 ? 288 : 256; }
 __host__ __device__ constexpr int cov_small_groups(int T) {
-  return 256 / (T == 32 ? (T / 4) * (T / 4 + 1) / 2 : (T / 4) * (T / 4));
+  return cov_small_threads(T) / ((T / 4) * (T / 4 + 1) / 2);
 }
 __host__ __device__ constexpr size_t cov_small_smem(int T) {
   const size_t strips = size_t(2) * T * (CS_SP + 1), red = size_t(cov_small_groups(T)) * T * T;
@@ -1347,25 +1350,17 @@ __host__ __device__ constexpr size_t cov_small_smem(int T) {
 }
 
 template <int T>
-__global__ void __launch_bounds__(256) k_cov_small(PcaArgs a) {
-  // T = 32: only the 36 tiles on or above the diagonal (ta <= tb), 7 groups in 252
-  // threads; T = 64: all 256 tiles, one group (the reduction reads the upper triangle)
-  constexpr bool UPPER = T == 32;
-  constexpr int TG = T / 4, GT = UPPER ? TG * (TG + 1) / 2 : TG * TG, G = 256 / GT, LDX = CS_SP + 1;
-  static_assert(G == cov_small_groups(T), "groups");
+__global__ void __launch_bounds__(cov_small_threads(T)) k_cov_small(PcaArgs a) {
+  constexpr int NT = cov_small_threads(T), TG = T / 4, GT = TG * (TG + 1) / 2, G = NT / GT, LDX = CS_SP + 1;
   extern __shared__ float2 xs[];  // cov_small_smem(T): 2 buffers of T x LDX, later G x T x T
   const int tid = threadIdx.x, g = tid / GT, r = tid % GT;
   const bool active = g < G;
-  int ta = r / TG, tb = r % TG;
-  if constexpr (UPPER) {  // r-th tile of the upper triangle, row by row
-    int rr = r;
-    ta = 0;
-    while (rr >= TG - ta) {
-      rr -= TG - ta;
-      ++ta;
-    }
-    tb = ta + rr;
+  int ta = 0, tb = r;  // r-th tile of the upper triangle, row by row
+  while (tb >= TG - ta) {
+    tb -= TG - ta;
+    ++ta;
   }
+  tb += ta;
   const size_t hw = size_t(a.W) * a.H;
   const uint32_t z = blockIdx.y;
   const size_t p_begin = size_t(blockIdx.x) * a.chunk;
@@ -1374,7 +1369,7 @@ __global__ void __launch_bounds__(256) k_cov_small(PcaArgs a) {
   auto issue = [&](int sidx, int buf) {
     float2* d = xs + buf * T * LDX;
     const size_t q0 = p_begin + size_t(sidx) * CS_SP;
-    for (int e = tid; e < T * CS_SP; e += 256) {
+    for (int e = tid; e < T * CS_SP; e += NT) {
       const int t = e / CS_SP, p = e % CS_SP;
       if (q0 + p < p_end) {
         const float2* src = win_frame(a, z, t, hw) + q0 + p;
@@ -1401,9 +1396,9 @@ __global__ void __launch_bounds__(256) k_cov_small(PcaArgs a) {
     for (int p = active ? g : CS_SP; p < CS_SP; p += G) {
       float2 u[4], v[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) u[i] = x[(4 * ta + i) * LDX + p];
+      for (int i = 0; i < 4; ++i) u[i] = x[(ta + TG * i) * LDX + p];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = x[(4 * tb + j) * LDX + p];
+      for (int j = 0; j < 4; ++j) v[j] = x[(tb + TG * j) * LDX + p];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -1421,10 +1416,14 @@ __global__ void __launch_bounds__(256) k_cov_small(PcaArgs a) {
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) red[(size_t(g) * T + 4 * ta + i) * T + 4 * tb + j] = acc[i][j];
+      for (int j = 0; j < 4; ++j) {  // entry (row, col), or its mirror where that lies above the diagonal
+        const int row = ta + TG * i, col = tb + TG * j;
+        if (row <= col) red[(size_t(g) * T + row) * T + col] = acc[i][j];
+        else if (ta != tb) red[(size_t(g) * T + col) * T + row] = make_float2(acc[i][j].x, -acc[i][j].y);
+      }
   __syncthreads();
   float2* out = a.partials + (size_t(z) * gridDim.x + blockIdx.x) * T * T;
-  for (int e = tid; e < T * T; e += 256) {
+  for (int e = tid; e < T * T; e += NT) {
     float2 s = red[e];
     for (int q = 1; q < G; ++q) {
       const float2 v = red[size_t(q) * T * T + e];
@@ -1496,7 +1495,7 @@ cudaError_t launch_pca_cov(PcaArgs& a, cudaStream_t s, int* launches) {
       k_cov_small<32><<<gs, 256, smem, s>>>(a);
     } else {
       cudaFuncSetAttribute(k_cov_small<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-      k_cov_small<64><<<gs, 256, smem, s>>>(a);
+      k_cov_small<64><<<gs, cov_small_threads(64), smem, s>>>(a);
     }
     k_cov_small_reduce<<<unsigned((size_t(a.nwin) * a.T * a.T + 255) / 256), 256, 0, s>>>(a, a.nchunks);
     *launches += 2;
