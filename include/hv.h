@@ -114,7 +114,7 @@ typedef struct {
   int32_t stft_kernel;        /* STFT kernel for windows that do not overlap (S >= T;
                                  overlapping windows take the walking kernel unless 0):
                                  0 = automatic (the autotuner's choice when tuned = 1,
-                                 else the walking kernel launched once per window),
+                                 else the window kernel where S >= T),
                                  HV_STFT_WALK, HV_STFT_WINDOW (HV_STFT_WINDOW_WIDE and
                                  HV_STFT_WINDOW_PIPELINED run the same kernel),
                                  HV_STFT_WINDOW_TMA or HV_STFT_WINDOW_TMA_PIPELINED

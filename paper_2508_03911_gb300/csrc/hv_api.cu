@@ -565,17 +565,20 @@ hv_status apply_pending(hv_handle* h) {
   h->tuning = hv_tuning{};
   h->tuning.spatial_chunk = chunk;
   h->tuning.spatial_kernel = p.spatial_kernel == HV_SK_AUTO ? HV_SK_MULTIPASS : int32_t(p.spatial_kernel);
-  // STFT kernel for windows that do not overlap: the caller's, the autotuner's (tuned),
-  // else the walking kernel launched once per window (the plain form)
-  h->stft_kernel = p.stft_kernel == 0 || p.stft_kernel == HV_STFT_WALK     ? STFT_WALK
-                   : p.stft_kernel == HV_STFT_WINDOW_TMA           ? STFT_TMA
-                   : p.stft_kernel == HV_STFT_WINDOW_TMA_PIPELINED ? STFT_TMA_PIPE
-                                                                   : STFT_WINDOW;
+  // STFT kernel: the caller's (for windows that do not overlap; others walk), the
+  // autotuner's (tuned, below), else the window kernel where windows do not overlap (faster
+  // than walking at every T: 0.69 against 1.34 us a window of 256 x 256 at T = 8, 183 against
+  // 277 at T = 1024) and the walking kernel where they do
+  const int32_t asked = p.stft_kernel != 0 ? p.stft_kernel : (d.S >= d.T ? HV_STFT_WINDOW : HV_STFT_WALK);
+  h->stft_kernel = asked == HV_STFT_WALK                   ? STFT_WALK
+                   : asked == HV_STFT_WINDOW_TMA           ? STFT_TMA
+                   : asked == HV_STFT_WINDOW_TMA_PIPELINED ? STFT_TMA_PIPE
+                                                           : STFT_WINDOW;
   if (p.tuned && p.spatial_kernel == HV_SK_AUTO) {
     s = tune_spatial(h);  // rewrites the tuning record
     if (s != HV_OK) return s;
   }
-  h->tuning.stft_kernel = p.stft_kernel == 0 ? HV_STFT_WALK : p.stft_kernel;
+  h->tuning.stft_kernel = asked;
   if (p.tuned && p.stft_kernel == 0 && p.temporal == HV_TEMPORAL_STFT) {
     s = tune_temporal(h);
     if (s != HV_OK) return s;
@@ -1199,18 +1202,7 @@ hv_status enqueue_windows(hv_handle* h, float* dst, uint32_t nw, bool capturing)
       sa.post_sums = pa.renorm ? pa.sums : nullptr;
       e = launch_post_zero(pa, nw, h->stream);
     }
-    if (e == cudaSuccess && (h->cur.tuned || h->cur.stft_kernel != 0)) {
-      e = launch_stft(sa, h->stream, &launches);
-    } else if (e == cudaSuccess) {
-      // plain form: the walking kernel, one launch per window
-      sa.nwin = 1;
-      for (uint32_t w = 0; w < nw && e == cudaSuccess; ++w) {
-        sa.tq = RingRef{h->tq, h->Q, uint32_t((h->next_win + uint64_t(w) * S) % h->Q)};
-        sa.out = dst + size_t(w) * h->win_floats;
-        sa.post_count = pa.count + w;
-        e = launch_stft(sa, h->stream, &launches);
-      }
-    }
+    if (e == cudaSuccess) e = launch_stft(sa, h->stream, &launches);
   }
   if (e == cudaSuccess && h->post_active) {
     e = launch_post(dst, nw, pa, h->stream, &launches);
