@@ -57,6 +57,7 @@ struct hv_handle {
   float2* s2 = nullptr;
   size_t s1_bytes = 0, s2_bytes = 0;
   uint32_t chunk = 0;
+  uint32_t chunk_least = 0;                // a run shorter than four chunks is cut finer, down to this
   uint32_t sp_lanes = 1;                   // multi-pass launches side by side, each with its part of s1 / s2
   cudaStream_t sp_stream[kSpLanes - 1] = {};  // lanes 1 ..; lane 0 is the handle's stream
   cudaEvent_t ev_fork = nullptr, ev_join[kSpLanes - 1] = {};
@@ -348,11 +349,19 @@ hv_status ensure(hv_handle* h, void** p, size_t* have, size_t need) {
   return HV_OK;
 }
 
+// Launches that a run of n frames is cut into: of `chunk` frames at most, and where these are
+// fewer than go side by side, of chunk_least at least (n = 64 and 128 at 256 x 256 ASP: 0.53 and
+// 0.45 us a frame as one launch, 0.47 and 0.38 as two and four; n = 32 at 512 x 512 2.33, 2.10)
+uint64_t launches_of_run(const hv_handle* h, uint64_t n, uint64_t chunk, uint32_t lanes) {
+  const uint64_t least = std::max<uint64_t>(1, std::min<uint64_t>(h->chunk_least, chunk));
+  return std::max((n + chunk - 1) / chunk, std::min<uint64_t>(lanes, n / least));
+}
+
 // Scratch of the multi-pass transform: `chunk` frames for each of the launches side by side,
 // as many as runs of up to `frames` frames fill and 1 GB holds, one where there is no memory
 // for more; `least` frames in all.
 hv_status size_scratch(hv_handle* h, int spatial, size_t fbytes, uint32_t chunk, uint32_t frames, uint32_t least) {
-  const size_t fit = (size_t(1) << 30) / (chunk * fbytes), runs = (size_t(frames) + chunk - 1) / chunk;
+  const size_t fit = (size_t(1) << 30) / (chunk * fbytes), runs = launches_of_run(h, frames, chunk, kSpLanes);
   uint32_t lanes = uint32_t(std::max<size_t>(1, std::min<size_t>({kSpLanes, fit, runs})));
   for (;; lanes = 1) {
     const size_t need = std::max<size_t>(size_t(lanes) * chunk, least) * fbytes;
@@ -399,6 +408,7 @@ hv_status apply_pending(hv_handle* h) {
   uint32_t chunk = p.spatial_chunk ? p.spatial_chunk : std::max<uint32_t>(1, uint32_t((size_t(64) << 20) / fbytes));
   if (p.spatial_chunk == 0) chunk = std::min(chunk, Q);
   chunk = std::min<uint32_t>(chunk, 1024);
+  h->chunk_least = p.spatial_chunk ? chunk : std::max<uint32_t>(1, uint32_t((size_t(16) << 20) / fbytes));
   const bool fused = p.spatial_kernel == HV_SK_FUSED;
   if (fused) {
     s = ensure(h, reinterpret_cast<void**>(&h->fused_ctr), &h->fused_ctr_bytes,
@@ -662,7 +672,7 @@ hv_status propagate_run(hv_handle* h, uint64_t r0, uint64_t r1, RingRef raw, flo
   // the cluster kernel needs no scratch, the fused transform keeps its intermediates
   // in rings: one persistent launch for all frames
   const bool whole = (h->sp_cluster && cluster_ok(h)) || h->sp_fused;
-  const uint64_t nruns = whole ? 1 : (r1 - r0 + h->chunk - 1) / h->chunk;
+  const uint64_t nruns = whole ? 1 : launches_of_run(h, r1 - r0, h->chunk, h->sp_lanes);
   const uint64_t step = (r1 - r0 + nruns - 1) / nruns;
   const uint32_t lanes = uint32_t(std::min<uint64_t>(nruns, h->sp_lanes));
   uint32_t lane = 0;

@@ -132,7 +132,8 @@ def test_persistent_multipass_parity(H, W, spatial, bits):
 
 
 @pytest.mark.parametrize("H,W,spatial,n,chunk", [(64, 64, "asp", 23, 5), (64, 128, "fresnel", 9, 4),
-                                                 (32, 32, "asp", 11, 2), (256, 64, "asp", 37, 1)])
+                                                 (32, 32, "asp", 11, 2), (256, 64, "asp", 37, 1),
+                                                 (512, 512, "fresnel", 29, 29)])
 def test_launches_side_by_side(H, W, spatial, n, chunk):
     """A run cut into launches that go side by side (two to four at once, the last ones
     shorter, many more launches than lanes) gives the fields of one launch, frame for frame,
@@ -140,6 +141,8 @@ def test_launches_side_by_side(H, W, spatial, n, chunk):
     fr = synth.random_frames(n, H, W, 12, seed=n + chunk)
     p = oracle_params(spatial=spatial, z_m=0.3, temporal="none", T=1, stride=1, H=H, W=W)
     one, _ = gpu_render(fr, p, extra=dict(spatial_chunk=n))
+    img, _ = gpu_render(fr, p)  # automatic: cut as finely as 16 MB of fields a launch
+    assert np.array_equal(img, one)
     for kw in (dict(), dict(packets=[n // 2, n - n // 2], queue=(n + 1) // 2 + 1), dict(in_place=True)):
         img, _ = gpu_render(fr, p, extra=dict(spatial_chunk=chunk), **kw)
         assert np.array_equal(img, one)
