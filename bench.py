@@ -83,8 +83,7 @@ WORKLOADS = {
         scene="scene_stream_fresnel"),
     "pca_512_t256": dict(
         desc="512x512 uint16 (12-bit) frames, ASP z=0.40 m, PCA over windows of T=256 (stride 256): "
-             "FP32 covariance, Jacobi eigensolver (FP32 sweeps, then refinement with FP64 diagonal and "
-             "eigenvectors), energy of the projection on eigenvectors 2..64; "
+             "FP32 covariance, Jacobi eigensolver (FP32 sweeps, then refinement), energy of the projection on eigenvectors 2..64; "
              "1,024 frames (4 windows) per step",
         N=512, bits=12, spatial="asp", z=0.40, T=256, S=256, fs=20000.0, band=(0, 0),
         moments=(), temporal="pca", pca=(2, 64), batch=1024, batches=1, pool=256,
@@ -462,7 +461,7 @@ def roofline_pca(w, res, peaks, force=None):
     M = w["pca"][1] - w["pca"][0] + 1
     hbm = (peaks or {}).get("hbm_gbs", 6800.0)
     st = {"spatial": prof["spatial_ms"] / nwin, "covariance": prof["pca_cov_ms"] / nwin,
-          "jacobi_fp64": prof["pca_eig_ms"] / nwin, "projection": prof["pca_proj_ms"] / nwin}
+          "jacobi": prof["pca_eig_ms"] / nwin, "projection": prof["pca_proj_ms"] / nwin}
     kern = force or max(st, key=st.get)
     t = st[kern] / 1e3
     if force is None and kern != "covariance" and st["covariance"] > 0:
@@ -491,26 +490,19 @@ def roofline_pca(w, res, peaks, force=None):
         flops, byts = 4.0 * P * T * (T + 1), 8.0 * P * T
     elif kern == "projection":
         flops, byts = 8.0 * P * T * M, 8.0 * P * T
-    elif kern == "jacobi_fp64":
-        sweeps = prof["pca_sweeps"] / nwin
-        sweeps32 = prof.get("pca_sweeps_f32", 0) / nwin
-        per_sweep32 = (T - 1) * (T // 2) ** 2 * 96.0 + (T - 1) * T * (T // 2) * 32.0
-        # float64 work over the whole eigensolver time: the congruence C' = Vf^H C Vf
-        # (M = C Vf, then the upper triangle for T <= 64 or all of it) and the rotations
-        # of V in the refinement sweeps (20 flops per row and pair); the 2 x 2 blocks of
-        # C' are float32 there, and the float32 sweeps before them are bound by barriers
-        per_sweep = (T - 1) * (T // 2) * T * 20.0
-        congruence = 8.0 * T ** 3 + (4.0 * T * T * (T + 1) if T <= 64 else 8.0 * T ** 3)
-        flops = sweeps * per_sweep + congruence
-        byts = 0.0
-        fp64_peak = alu_peaks()["fp64_tflops"]
-        return {"bound": "alu", "achieved": round(flops / t / 1e12, 4), "peak": round(fp64_peak, 3),
-                "unit": "TFLOP/s (FP64)", "frac": round(flops / t / 1e12 / fp64_peak, 4),
-                "traffic": None,
-                "kernel": "eigensolver (FP32 cyclic Jacobi, then refinement: FP64 diagonal and V, FP32 off-diagonal)",
-                "peak_source": alu_peaks()["source"] + "; nominal GB300 FP64 1.25 TFLOP/s",
+    elif kern == "jacobi":
+        # float32 work of both phases' sweeps (2 x 2 blocks, and the rotations of V or of its
+        # correction) and the congruence C' = Vf^H C Vf (M = C Vf, then the upper triangle; its
+        # 48-bit pairs take 5.5 instructions a multiply-add); a chain of rounds bounds it
+        sweeps, sweeps32 = prof["pca_sweeps"] / nwin, prof.get("pca_sweeps_f32", 0) / nwin
+        per_sweep = (T - 1) * (T // 2) ** 2 * 96.0 + (T - 1) * T * (T // 2) * 32.0
+        flops = (sweeps + sweeps32) * per_sweep + 8.0 * T ** 3 + 4.0 * T * T * (T + 1)
+        peak = alu_peaks()["fp32_tflops"]
+        return {"bound": "alu", "achieved": round(flops / t / 1e12, 4), "peak": round(peak, 1),
+                "unit": "TFLOP/s", "frac": round(flops / t / 1e12 / peak, 4), "traffic": None,
+                "kernel": "eigensolver (FP32 cyclic Jacobi, then refinement: diagonal in pairs of FP32)",
+                "peak_source": alu_peaks()["source"],
                 "sweeps_per_window": round(sweeps, 2), "fp32_sweeps_per_window": round(sweeps32, 2),
-                "fp32_flops_per_window": round(sweeps32 * per_sweep32),
                 "stage_ms_per_window": {k: round(v, 4) for k, v in st.items()}}
     else:  # spatial: the S new frames each window propagates
         alg = algorithmic(w)

@@ -245,7 +245,7 @@ typedef struct {
   double pca_cov_ms;          /* PCA: covariance (partials and reduction)           */
   double pca_eig_ms;          /* PCA: Jacobi eigendecomposition and selection       */
   double pca_proj_ms;         /* PCA: projection and energy                         */
-  uint64_t pca_sweeps;        /* PCA: refinement sweeps (float64 diagonal and eigenvectors,
+  uint64_t pca_sweeps;        /* PCA: refinement sweeps (diagonal in pairs of float32,
                                  float32 off-diagonal) summed over recorded windows */
   uint64_t pca_sweeps_f32;    /* PCA: float32 Jacobi sweeps (first phase) summed likewise */
 } hv_profile;

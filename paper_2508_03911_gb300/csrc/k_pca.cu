@@ -3,7 +3,7 @@
 //
 // With X the P x T matrix whose column t is propagated frame t (P = W H):
 //   C = X^H X                      (T x T Hermitian, unnormalised)
-//   C = V diag(lam) V^H            (cyclic complex Jacobi, float64)
+//   C = V diag(lam) V^H            (cyclic complex Jacobi: float32, then refined)
 //   E(p) = sum_{j = lo..hi} |(X v_j)_p|^2, eigenvectors ranked by descending lam.
 //
 // Kernels (all on the handle's stream; windows of T <= 64 frames are batched,
@@ -1546,7 +1546,7 @@ cudaError_t launch_pca_eig(PcaArgs& a, cudaStream_t s, int* launches) {
     k_congruence<false><<<gg, 256, 0, s>>>(a, a.C, a.C2);  // M = C Vf
     k_congruence<true><<<gg, 256, 0, s>>>(a, a.C2, a.C);   // C' = Vf^H M
     *launches += 3;
-    // (3) float64 sweeps on C' (off-diagonals ~1e-6 of the trace): at most two, fewer
+    // (3) refinement sweeps on C' (off-diagonals ~1e-6 of the trace): at most two, fewer
     // when every entry met in a sweep is below 1e-12 of the trace. Two leave the
     // energy image within ~2e-5 of the float64 reference and the eigenvalues within
     // ~3e-8 of the largest (a third and fourth sweep halve the first figure only;
