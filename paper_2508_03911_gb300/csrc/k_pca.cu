@@ -1331,11 +1331,15 @@ static cudaError_t launch_project(const PcaArgs& a, float* out, cudaStream_t s) 
 // rows that neighbouring threads read lie one row stride apart, in different banks (rows
 // 4 ta + i met in the same banks two or four at a time). The CTA's groups (7 of 36 threads
 // for T = 32, 2 of 136 for T = 64) take alternate pixels of each staged strip. A strip is
-// SP pixels of all T frames of the window, [t][p] in shared memory (row stride SP + 1),
-// fetched with cp.async into one of two buffers while the other is used. The groups' sums
-// are added in shared memory and each CTA writes its partial matrix part[window][cta][T][T]
-// (upper triangle); a second kernel sums them in float64. 128 windows of 256 x 256, T = 32:
-// 1040 us before, 991 now; 64 windows, T = 64, over all 256 tiles: 2940 us before, 2016 now.
+// SP pixels of all T frames of the window, [t][p] in shared memory, fetched with cp.async
+// into one of two buffers while the other is used. T = 32: row stride SP + 2, in which also
+// the two groups of a warp, a pixel apart, meet in different banks, and 16-byte copies from
+// addresses kept per thread; T = 64: SP + 1 (16 rows apart in as many banks). The groups'
+// sums are added in shared memory and each CTA writes its partial matrix
+// part[window][cta][T][T] (upper triangle); a second kernel sums them in float64. 128 windows
+// of 256 x 256, T = 32: 1040 us with rows 4 ta + i, 991 with row stride SP + 1 and 8-byte
+// copies, 772 now (67 % of the multiply-add rate); 64 windows, T = 64, over all 256 tiles:
+// 2940 us before, 1920 now.
 constexpr int CS_SP = 64;
 
 // Threads and groups of k_cov_small<T> and its dynamic shared memory: two strip buffers, or
@@ -1344,15 +1348,16 @@ __host__ __device__ constexpr int cov_small_threads(int T) { return T == 64 ? 28
 __host__ __device__ constexpr int cov_small_groups(int T) {
   return cov_small_threads(T) / ((T / 4) * (T / 4 + 1) / 2);
 }
+__host__ __device__ constexpr int cov_small_ldx(int T) { return CS_SP + (T == 32 ? 2 : 1); }
 __host__ __device__ constexpr size_t cov_small_smem(int T) {
-  const size_t strips = size_t(2) * T * (CS_SP + 1), red = size_t(cov_small_groups(T)) * T * T;
+  const size_t strips = size_t(2) * T * cov_small_ldx(T), red = size_t(cov_small_groups(T)) * T * T;
   return (strips > red ? strips : red) * sizeof(float2);
 }
 
 template <int T>
 __global__ void __launch_bounds__(cov_small_threads(T)) k_cov_small(PcaArgs a) {
-  constexpr int NT = cov_small_threads(T), TG = T / 4, GT = TG * (TG + 1) / 2, G = NT / GT, LDX = CS_SP + 1;
-  extern __shared__ float2 xs[];  // cov_small_smem(T): 2 buffers of T x LDX, later G x T x T
+  constexpr int NT = cov_small_threads(T), TG = T / 4, GT = TG * (TG + 1) / 2, G = NT / GT, LDX = cov_small_ldx(T);
+  extern __shared__ __align__(16) float2 xs[];  // cov_small_smem(T): 2 buffers of T x LDX, later G x T x T
   const int tid = threadIdx.x, g = tid / GT, r = tid % GT;
   const bool active = g < G;
   int ta = 0, tb = r;  // r-th tile of the upper triangle, row by row
@@ -1365,18 +1370,34 @@ __global__ void __launch_bounds__(cov_small_threads(T)) k_cov_small(PcaArgs a) {
   const uint32_t z = blockIdx.y;
   const size_t p_begin = size_t(blockIdx.x) * a.chunk;
   const size_t p_end = p_begin + a.chunk < hw ? p_begin + a.chunk : hw;
-  const int nstrips = int((p_end - p_begin + CS_SP - 1) / CS_SP);
+  const int nstrips = p_begin < p_end ? int((p_end - p_begin) / CS_SP) : 0;  // chunk, hw: multiples of CS_SP
+  // T = 32: a thread's frames tid / 32 + 8 k, two pixels each, in 16-byte units from the queue's
+  // base (a queue of 4 G such units holds 64 GB)
+  constexpr bool PAIRS = T == 32;
+  uint32_t off[PAIRS ? 4 : 1];
+  if constexpr (PAIRS)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      uint32_t slot = a.tq.slot0 + z * a.wstride + uint32_t(tid / 32 + 8 * k);
+      while (slot >= a.tq.cap) slot -= a.tq.cap;
+      off[k] = uint32_t((size_t(slot) * hw + p_begin) / 2) + tid % 32;
+    }
   auto issue = [&](int sidx, int buf) {
     float2* d = xs + buf * T * LDX;
-    const size_t q0 = p_begin + size_t(sidx) * CS_SP;
-    for (int e = tid; e < T * CS_SP; e += NT) {
-      const int t = e / CS_SP, p = e % CS_SP;
-      if (q0 + p < p_end) {
+    if constexpr (PAIRS) {
+      const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(&d[(tid / 32) * LDX + 2 * (tid % 32)]));
+      const float4* base = static_cast<const float4*>(a.tq.base) + sidx * (CS_SP / 2);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa + unsigned(8 * k * LDX * 8)), "l"(base + off[k])
+                     : "memory");
+    } else {
+      const size_t q0 = p_begin + size_t(sidx) * CS_SP;
+      for (int e = tid; e < T * CS_SP; e += NT) {
+        const int t = e / CS_SP, p = e % CS_SP;
         const float2* src = win_frame(a, z, t, hw) + q0 + p;
         const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(&d[t * LDX + p]));
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(src) : "memory");
-      } else {
-        d[t * LDX + p] = make_float2(0.f, 0.f);
       }
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
