@@ -73,7 +73,7 @@ def test_gaussian_renorm_accumulate_stft():
 def test_renorm_accumulate_fused_into_the_stft(T, S, form):
     """Without a convolution the STFT epilogue writes the image ring and adds each
     image's sum itself (window-per-CTA kernels for S >= T, the walking kernel for
-    S < T, one launch per window in the plain form); every moment kind, history
+    S < T); every moment kind, history
     across renders and ring wrap-around."""
     H, W = 32, 64
     fr = synth.random_frames(T + 13 * S + 5, H, W, 12, seed=T + S)
