@@ -1712,13 +1712,7 @@ hv_status hv_af_features(hv_handle* h, const void* frames, uint32_t n, void* out
     sa.raw.slot0 = a;
     sa.n = std::min(chunk, n - a);
     uint16_t* dst = static_cast<uint16_t*>(out_bf16) + a * cells;
-    // s2 holds this chunk's cells [n][H/2][W/2] (floats), then its (sum, sum of squares)
-    sa.cells = reinterpret_cast<float*>(h->s2);
-    sa.tam_acc = reinterpret_cast<double*>(h->s2 + (size_t(sa.n) * cells + 1) / 2);
-    sa.tam_stride = 2;
-    cudaError_t e = cudaMemsetAsync(sa.tam_acc, 0, size_t(sa.n) * 2 * sizeof(double), h->stream);
-    if (e == cudaSuccess) e = launch_strip_cells(sa, h->stream);
-    if (e == cudaSuccess) e = launch_af_standardize(sa.cells, sa.tam_acc, 2, sa.n, uint32_t(cells), dst, h->stream);
+    const cudaError_t e = launch_features(sa, dst, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "feature passes");
     h->st.kernel_launches += 3;
   }

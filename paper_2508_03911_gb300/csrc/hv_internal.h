@@ -35,7 +35,7 @@ struct SpatialArgs {
   int use_cluster;      // 1: whole-frame cluster kernel when the size allows it
   double* tam_acc;      // focus sweep: frame i adds (sum |u|, sum |u|^2) at tam_acc + i * tam_stride
   uint32_t tam_stride;
-  float* cells;         // launch_strip_cells output [n][H/2][W/2]
+  float* cells;         // launch_features: [n][H/2][W/2]
   unsigned* err;        // device flags (bit 3: a row pass's wait for its staged strip gave up;
                         // bit 4: a fused-transform wait for another CTA's pass gave up); may be NULL
   // fused transform (one persistent launch for every pass of every frame, 256 x 256):
@@ -48,7 +48,7 @@ struct SpatialArgs {
                         // kernel that fit the device at once, 0 where not asked yet (NULL: no table)
   int stall;            // fault injection (tests): the fused row items wait on a condition nothing sets
 };
-constexpr uint32_t kStripKernels = 9, kStripSides = 5;  // sides 64 .. 1024
+constexpr uint32_t kStripKernels = 8, kStripSides = 5;  // sides 64 .. 1024
 // Multi-pass launches of one run that are queued side by side.
 constexpr uint32_t kSpLanes = 4;
 cudaError_t launch_spatial(const SpatialArgs& a, cudaStream_t s, int* launches);
@@ -62,10 +62,10 @@ cudaError_t launch_spatial_strip(const SpatialArgs& a, cudaStream_t s, int* laun
 // tam_stride + 2 z.
 cudaError_t launch_strip_spectrum(const SpatialArgs& a, cudaStream_t s);
 cudaError_t launch_strip_sweep(const SpatialArgs& a, const float2* h, uint32_t nz, cudaStream_t s);
-// Network-input cells [n][H/2][W/2] of n frames into cells (through scratch1): the centred
-// spectrum's 2 x 2 blocks as log1p(mean |F|) (DC bin as 0), (sum v, sum v^2) of a frame
-// added to tam_acc + frame * tam_stride.
-cudaError_t launch_strip_cells(const SpatialArgs& a, cudaStream_t s);
+// Network input of n frames (sides 64 .. 1024), bfloat16 [n][H/2][W/2], through scratch1 and
+// scratch2: the centred spectrum's 2 x 2 blocks as log1p(mean |F|) (DC bin as 0), less their mean
+// over their deviation.
+cudaError_t launch_features(const SpatialArgs& a, void* out_bf16, cudaStream_t s);
 cudaError_t launch_spatial_cluster(const SpatialArgs& a, cudaStream_t s, int* launches);
 // Fused transform: frames of 256 x 256, ASP or Fresnel; needs ring >= kFusedRing
 // frames in scratch1 (and scratch2 for ASP), fused_ctr and err.
@@ -176,13 +176,8 @@ uint32_t pca_eig_lanes(uint32_t T);
 cudaError_t launch_pca_eig(PcaArgs& a, cudaStream_t s, int* launches);
 cudaError_t launch_pca_proj(PcaArgs& a, float* out, cudaStream_t s, int* launches);
 
-// Autofocus: Tamura coefficients from per-(frame, distance) amplitude sums, and the
-// network input (2 x 2 binned log-magnitude spectrum, standardised, bfloat16).
+// Autofocus: Tamura coefficients from per-(frame, distance) amplitude sums.
 cudaError_t launch_tamura_finish(const double* acc, uint32_t count, uint32_t pixels, float* metric, cudaStream_t s);
-// The network input from the cells and per-frame sums of launch_strip_cells:
-// (v - mean) / deviation per frame, rounded to bfloat16.
-cudaError_t launch_af_standardize(const float* cells, const double* sums, uint32_t sum_stride, uint32_t n,
-                                  uint32_t ncell, void* out_bf16, cudaStream_t s);
 
 // Post-processing of rendered images [window][nout][H][W] (Sec. III-B): periodic
 // K x K convolution into ring slot (count + window) mod R, per-image float64 sums

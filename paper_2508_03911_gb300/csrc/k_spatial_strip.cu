@@ -349,97 +349,9 @@ __global__ void __launch_bounds__(ColCfg<L>::NT, ColCfg<L>::CTAS) k_strip_icols_
   }
 }
 
-// -------------------------------------------------------------- network input
-//
-// Cells of the autofocus network's input: the centred spectrum's 2 x 2 blocks as
-// log1p(mean |F|) (DC bin as 0). |F| of a real frame is symmetric, |F(-k)| = |F(k)|, so S1
-// rows 0 .. H / 2 are enough: a CTA row-transforms rows y0 .. y0 + SR, keeps their |F| in
-// shared memory, and forms the blocks of rows (2r, 2r + 1), and of rows (H - e, H - e + 1)
-// from rows e and e - 1 with the columns mirrored, e even (over all H rows the column and
-// row passes took 64 + 144 us for 512 holograms of 256 x 256; 37 + 71 now).
-template <int L>
-struct CellCfg {
-  static constexpr int SR = L <= 256 ? 32 : 16;  // rows of a strip (one more is transformed)
-  static constexpr size_t SMEM = RowCfg<L>::SMEM + size_t(SR + 1) * L * sizeof(float);
-};
-
-template <int L>
-__global__ void __launch_bounds__(RowCfg<L>::NT) k_strip_cells(SpatialArgs a, uint32_t nitems, uint32_t strips) {
-  using C = RowCfg<L>;
-  constexpr int SR = CellCfg<L>::SR;
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ float red[2][C::NW];
-  float2* tw = reinterpret_cast<float2*>(smem);
-  float* mag = reinterpret_cast<float*>(tw + C::NTW + C::NW * C::RPW * C::RS);  // [SR + 1][L]
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, jl = lane % C::LP, sub = lane / C::LP;
-  float2* rowp = tw + C::NTW + (warp * C::RPW + sub) * C::RS;
-  load_stage_twiddles<C::R1, C::NTW, C::NT>(tw, a.tw_w);
-  const int H = int(a.H);
-  for (uint32_t item = blockIdx.x; item < nitems; item += gridDim.x) {
-    const uint32_t i = item / strips;
-    const int y0 = int(item % strips) * SR;
-    __syncthreads();  // twiddles loaded; the previous strip's cells formed
-    for (int r0 = warp * C::RPW; r0 <= SR; r0 += C::NW * C::RPW) {
-      const int r = r0 + sub <= SR ? r0 + sub : SR;  // a row too many repeats the last
-      const float2* in = a.scratch1 + (size_t(i) * (H / 2 + 1) + y0 + r) * L + jl;
-      float2 v[C::R1];
-#pragma unroll
-      for (int m = 0; m < C::R1; ++m) v[m] = in[C::LP * m];
-      strip_row_fft<L, -1>(v, rowp, tw, jl);
-#pragma unroll
-      for (int m = 0; m < C::R1; ++m)
-        mag[r * L + jl + C::LP * m] = sqrtf(fmaf(v[m].x, v[m].x, v[m].y * v[m].y));
-    }
-    __syncthreads();
-    if (y0 == 0 && threadIdx.x == 0) mag[0] = 0.f;  // DC bin
-    __syncthreads();
-    float* cells = a.cells + size_t(i) * (H / 2) * (L / 2);
-    float s0 = 0.f, s1 = 0.f;
-    // SR / 2 block rows of each kind, L / 2 cells each
-    for (int e = threadIdx.x; e < SR * (L / 2); e += C::NT) {
-      const int q = e % (L / 2), p = e / (L / 2), k = p >> 1;
-      int ky, ra, rb, xa, xb;
-      if (p & 1) {  // rows H - ke, H - ke + 1 from rows ke and ke - 1, ke = y0 + 2 k + 2
-        ra = 2 * k + 2;
-        rb = 2 * k + 1;
-        ky = H - (y0 + ra);
-        xa = (L - 2 * q) & (L - 1);
-        xb = L - 2 * q - 1;
-      } else {
-        ra = 2 * k;
-        rb = 2 * k + 1;
-        ky = y0 + ra;
-        xa = 2 * q;
-        xb = 2 * q + 1;
-      }
-      const float m = ((mag[ra * L + xa] + mag[ra * L + xb]) + mag[rb * L + xa]) + mag[rb * L + xb];
-      const float c = log1pf(0.25f * m);
-      cells[size_t(((ky + H / 2) & (H - 1)) >> 1) * (L / 2) + (((2 * q + L / 2) & (L - 1)) >> 1)] = c;
-      s0 += c;
-      s1 = fmaf(c, c, s1);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-    }
-    if (lane == 0) {
-      red[0][warp] = s0;
-      red[1][warp] = s1;
-    }
-    __syncthreads();
-    if (threadIdx.x < 2) {
-      double t = 0.0;
-#pragma unroll
-      for (int w = 0; w < C::NW; ++w) t += red[threadIdx.x][w];
-      atomicAdd(&a.tam_acc[size_t(i) * a.tam_stride + threadIdx.x], t);
-    }
-  }
-}
-
 // Row of SpatialArgs::fit.
-enum StripKernel { COLS_ASP, COLS, ICOLS, ROWS_ASP, ROWS_FFT, ROWS_FWD, ROWS_INV, ICOLS_SUMS, CELLS };
-static_assert(CELLS + 1 == kStripKernels, "one row per kernel");
+enum StripKernel { COLS_ASP, COLS, ICOLS, ROWS_ASP, ROWS_FFT, ROWS_FWD, ROWS_INV, ICOLS_SUMS };
+static_assert(ICOLS_SUMS + 1 == kStripKernels, "one row per kernel");
 
 constexpr uint32_t side_index(int L) { return L == 64 ? 0 : 1 + side_index(L / 2); }
 
@@ -523,12 +435,6 @@ cudaError_t icols_sums(const SpatialArgs& a, uint32_t nz, cudaStream_t s) {
   return launch_resident(a, ICOLS_SUMS, L, k_strip_icols_sums<L>, C::NT, C::SMEM, items, s, a, items, strips);
 }
 
-template <int L>
-cudaError_t cells(const SpatialArgs& a, cudaStream_t s) {
-  const uint32_t strips = a.H / (2 * CellCfg<L>::SR), items = strips * a.n;
-  return launch_resident(a, CELLS, L, k_strip_cells<L>, RowCfg<L>::NT, CellCfg<L>::SMEM, items, s, a, items, strips);
-}
-
 }  // namespace
 
 bool spatial_strip_supported(const SpatialArgs& a) {
@@ -572,15 +478,6 @@ cudaError_t launch_strip_sweep(const SpatialArgs& a, const float2* h, uint32_t n
   HV_BY_SIDE(a.W, HV_ROWS_INV)
   if (e != cudaSuccess) return e;
   HV_BY_SIDE(a.H, HV_ICOLS_SUMS)
-  return e;
-}
-
-cudaError_t launch_strip_cells(const SpatialArgs& a, cudaStream_t s) {
-  cudaError_t e;
-#define HV_CELLS(L) cells<L>(a, s)
-  HV_BY_SIDE(a.H, HV_COLS_ASP)
-  if (e != cudaSuccess) return e;
-  HV_BY_SIDE(a.W, HV_CELLS)
   return e;
 }
 
