@@ -13,6 +13,10 @@ struct RingRef {
   uint32_t slot0;    // slot of the first frame of the launch
 };
 
+// Index of value `at` of the frame in slot `slot` of a ring of frames of hw values. A ring may
+// hold more than 2^32 of them, and 2^32 pairs (8,192 fields of 1024 x 1024 are 64 GB).
+__host__ __device__ constexpr size_t queue_value(uint32_t slot, size_t hw, size_t at) { return slot * hw + at; }
+
 // Input element kinds of the first spatial pass.
 enum InKind { IN_U8 = 0, IN_U16 = 1 };
 

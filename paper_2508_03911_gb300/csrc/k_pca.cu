@@ -1371,25 +1371,24 @@ __global__ void __launch_bounds__(cov_small_threads(T)) k_cov_small(PcaArgs a) {
   const size_t p_begin = size_t(blockIdx.x) * a.chunk;
   const size_t p_end = p_begin + a.chunk < hw ? p_begin + a.chunk : hw;
   const int nstrips = p_begin < p_end ? int((p_end - p_begin) / CS_SP) : 0;  // chunk, hw: multiples of CS_SP
-  // T = 32: a thread's frames tid / 32 + 8 k, two pixels each, in 16-byte units from the queue's
-  // base (a queue of 4 G such units holds 64 GB)
+  // T = 32: a thread's frames tid / 32 + 8 k, two pixels each
   constexpr bool PAIRS = T == 32;
-  uint32_t off[PAIRS ? 4 : 1];
+  const float4* src[PAIRS ? 4 : 1];
   if constexpr (PAIRS)
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       uint32_t slot = a.tq.slot0 + z * a.wstride + uint32_t(tid / 32 + 8 * k);
       while (slot >= a.tq.cap) slot -= a.tq.cap;
-      off[k] = uint32_t((size_t(slot) * hw + p_begin) / 2) + tid % 32;
+      src[k] = static_cast<const float4*>(a.tq.base) + queue_value(slot, hw, p_begin) / 2 + tid % 32;
     }
   auto issue = [&](int sidx, int buf) {
     float2* d = xs + buf * T * LDX;
     if constexpr (PAIRS) {
       const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(&d[(tid / 32) * LDX + 2 * (tid % 32)]));
-      const float4* base = static_cast<const float4*>(a.tq.base) + sidx * (CS_SP / 2);
 #pragma unroll
       for (int k = 0; k < 4; ++k)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa + unsigned(8 * k * LDX * 8)), "l"(base + off[k])
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa + unsigned(8 * k * LDX * 8)),
+                     "l"(src[k] + sidx * (CS_SP / 2))
                      : "memory");
     } else {
       const size_t q0 = p_begin + size_t(sidx) * CS_SP;

@@ -3,10 +3,11 @@ declares; error paths that need no GPU behave as documented."""
 import ctypes
 import os
 import re
+import subprocess
 
 import pytest
 
-from paper_2508_03911_gb300 import hv
+from paper_2508_03911_gb300 import build, hv
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -57,3 +58,20 @@ def test_params_struct_layout():
     assert hv.hv_params.z_m.offset == 24 and hv.hv_params.fs_hz.offset == 72
     assert hv.hv_params.highpass_cpp.offset == 128 and hv.hv_params.stft_kernel.offset == 136
     assert ctypes.sizeof(hv.hv_open_desc) == 40
+
+
+def test_queue_indices_hold_in_rings_past_64_gb(tmp_path):
+    """The last value of the last of 16,384 fields of 1024 x 1024 (128 GB), past 32 bits also
+    in units of 16 bytes."""
+    src = tmp_path / "q.cpp"
+    src.write_text("""
+        #include "hv_internal.h"
+        constexpr size_t hw = size_t(1) << 20;
+        static_assert(hv::queue_value(16383, hw, hw - 1) == (size_t(1) << 34) - 1, "values");
+        static_assert(hv::queue_value(16383, hw, hw - 64) / 2 == (size_t(1) << 33) - 32, "16-byte units");
+        static_assert(sizeof(hv::queue_value(0, 0, 0)) == 8, "64 bits");
+    """)
+    cuda = os.path.join(os.path.dirname(os.path.dirname(build.nvcc())), "include")
+    r = subprocess.run(["g++", "-std=c++17", "-fsyntax-only", f"-I{build.CSRC}", f"-I{build.INCLUDE}", f"-I{cuda}", str(src)],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
