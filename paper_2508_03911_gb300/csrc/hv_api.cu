@@ -1861,7 +1861,13 @@ hv_status hv_render_group(hv_group* g, const void* const* frames, const uint32_t
     if (in_place) {
       if (!h->borrowed.empty() && h->borrowed.back().first == first) h->borrowed.pop_back();
       const uint64_t keep = std::max(first, h->next_win);
-      if (s == HV_OK && keep < first + nf) s = enqueue_frames(h, frames[i], uint32_t(keep - first), first, nf);
+      if (s == HV_OK && keep < first + nf) {
+        s = enqueue_frames(h, frames[i], uint32_t(keep - first), first, nf);
+        // the slots of these frames are free after their copy, not after the spatial stage
+        // that read them where they were (a graph's event comes behind the whole step)
+        for (int k = 0; k < hv_handle::NCONS; ++k) h->cons_hi[k] = std::min(h->cons_hi[k], keep);
+        if (s == HV_OK && !graph) s = note_consumed(h);
+      }
     }
     if (s != HV_OK) break;
     n_windows[i] = nw;
