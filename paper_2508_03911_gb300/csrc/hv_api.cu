@@ -344,7 +344,10 @@ hv_status ensure(hv_handle* h, void** p, size_t* have, size_t need) {
   *p = nullptr;
   *have = 0;
   cudaError_t e = cudaMalloc(p, need);
-  if (e != cudaSuccess) return fail(h, HV_ERR_NOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // reported here: not an error of the launches that follow
+    return fail(h, HV_ERR_NOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  }
   *have = need;
   return HV_OK;
 }
@@ -370,12 +373,23 @@ hv_status size_scratch(hv_handle* h, int spatial, size_t fbytes, uint32_t chunk,
       s = ensure(h, reinterpret_cast<void**>(&h->s2), &h->s2_bytes, need);
     h->sp_lanes = lanes;
     if (s == HV_OK || lanes == 1) return s;
-    cudaGetLastError();
   }
 }
 
+bool cluster_ok(const hv_handle* h);
 hv_status tune_spatial(hv_handle* h);
 hv_status tune_temporal(hv_handle* h);
+
+// The scratch of the settings in force: an autofocus call that found no memory for its own
+// has left less of it, or none.
+hv_status keep_scratch(hv_handle* h) {
+  if (h->cur.spatial == HV_SPATIAL_NONE || (h->sp_cluster && cluster_ok(h))) return HV_OK;
+  const size_t fbytes = size_t(h->W) * h->H * sizeof(float2);
+  const uint32_t least = h->sp_fused ? kFusedRing : 0;
+  const size_t need = std::max<size_t>(size_t(h->sp_lanes) * h->chunk, least) * fbytes;
+  if (h->s1_bytes >= need && (h->cur.spatial != HV_SPATIAL_ASP || h->s2_bytes >= need)) return HV_OK;
+  return size_scratch(h, h->cur.spatial, fbytes, h->chunk, h->Q, least);
+}
 
 // Apply the pending settings (window boundary).
 hv_status apply_pending(hv_handle* h) {
@@ -950,6 +964,7 @@ hv_status post_apply(hv_handle* h) {
 // Settings and post-processing settings in force for the next windows.
 hv_status settle(hv_handle* h) {
   hv_status s = apply_pending(h);
+  if (s == HV_OK) s = keep_scratch(h);
   return s == HV_OK ? post_apply(h) : s;
 }
 
@@ -1635,7 +1650,6 @@ hv_status hv_focus_sweep(hv_handle* h, const void* frames, uint32_t n, const dou
   uint32_t lanes = uint32_t(std::max<size_t>(1, std::min<size_t>({kSpLanes, steps, (size_t(1) << 30) / (images * fbytes)})));
   s = ensure(h, reinterpret_cast<void**>(&h->s2), &h->s2_bytes, lanes * images * fbytes);
   if (s != HV_OK && lanes > 1) {
-    cudaGetLastError();
     lanes = 1;
     s = ensure(h, reinterpret_cast<void**>(&h->s2), &h->s2_bytes, images * fbytes);
   }

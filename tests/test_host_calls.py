@@ -1,5 +1,7 @@
 """Host code of the library against a CUDA runtime that only writes calls down: the order of
 copies on several streams, scratch after an allocation that failed, calls that failed half way."""
+import pytest
+
 from tests._fake_cuda import run, unordered_copies
 
 RING = """
@@ -26,3 +28,37 @@ def test_pushes_follow_the_copy_of_a_groups_last_frames():
     slots on the copy stream."""
     for graph in (False, True):
         assert unordered_copies(run(RING % dict(graph=graph))) == []
+
+
+SWEEP = """
+import numpy as np
+N, MB = 512, 1 << 20
+r = hv.Renderer(N, N, 16, 256)
+r.set_params(N, N, spatial="asp", T=128, stride=128, fs=20000.0, band=(1, 2))
+fr, out = Dev((128, N, N), 2), Dev((1, N, N), 4)
+def render():
+    log()
+    assert r.push(fr) == hv.HV_OK and r.render(out) == 1
+    return [l[1:] for l in log() if l[0] == "scratch"]
+before = render()
+fake.fake_fail_malloc(%(least)d * MB, %(times)d)
+try:
+    hv.hv_focus_sweep(r.h, Dev((64, N, N), 2), np.linspace(0.1, 0.6, 64), Dev((64, 64), 4))
+    status = 0
+except hv.HvError as e:
+    status = e.status
+fake.fake_fail_malloc(0, 0)
+print(json.dumps([status, before, render()]))
+"""
+
+
+@pytest.mark.parametrize("least,times,status", [(400, 1, 0), (100, 2, -4)])
+def test_renders_after_a_sweep_without_memory(least, times, status):
+    """A sweep of 64 holograms of 512 x 512 asks for 512 MB where a render has 256. With memory
+    for fewer images, and without any for it, a later render's launches stay in their scratch."""
+    got, before, after = run(SWEEP % dict(least=least, times=times))
+    assert got == status
+    for launches in (before, after):
+        assert len(launches) >= 3
+        for w, h, n, spatial, room1, room2 in launches:
+            assert room1 >= n * w * (h // 2 + 1) * 8 and room2 >= n * w * h * 8
