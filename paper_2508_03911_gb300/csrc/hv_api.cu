@@ -1620,15 +1620,21 @@ static SpatialArgs af_args(hv_handle* h, const void* frames, uint32_t n) {
   return sa;
 }
 
-static hv_status af_prepare(hv_handle* h, const void* frames, uint32_t n, uint32_t chunk) {
+// Settings applied, arguments checked: frames of sides 64 .. 1024.
+static hv_status af_prepare(hv_handle* h, const void* frames, uint32_t n) {
   if (!frames || n == 0) return fail(h, HV_ERR_ARG, "frames is NULL or n = 0");
   if (!h->has_params && !h->pending) return fail(h, HV_ERR_STATE, "no settings");
   HV_CU(h, cudaSetDevice(h->device));
   hv_status s = apply_pending(h);
   if (s != HV_OK) return s;
   if (h->W < 64 || h->H < 64) return fail(h, HV_ERR_UNSUPPORTED, "autofocus needs sides in [64, 1024]");
+  return HV_OK;
+}
+
+// Scratch of `chunk` frames in each buffer.
+static hv_status af_scratch(hv_handle* h, uint32_t chunk) {
   const size_t need = size_t(chunk) * h->W * h->H * sizeof(float2);
-  s = ensure(h, reinterpret_cast<void**>(&h->s1), &h->s1_bytes, need);
+  hv_status s = ensure(h, reinterpret_cast<void**>(&h->s1), &h->s1_bytes, need);
   if (s == HV_OK) s = ensure(h, reinterpret_cast<void**>(&h->s2), &h->s2_bytes, need);
   return s;
 }
@@ -1638,7 +1644,8 @@ hv_status hv_focus_sweep(hv_handle* h, const void* frames, uint32_t n, const dou
   if (!z || !metric || nz == 0 || nz > 1024) return fail(h, HV_ERR_ARG, "bad distances or output");
   // holograms whose spectra are held at once
   const uint32_t chunk = std::min<uint32_t>(n, 64);
-  hv_status s = af_prepare(h, frames, n, chunk);
+  hv_status s = af_prepare(h, frames, n);
+  if (s == HV_OK) s = af_scratch(h, chunk);
   if (s != HV_OK) return s;
   const uint32_t W = h->W, H = h->H;
   const size_t fbytes = size_t(W) * H * sizeof(float2);
@@ -1715,10 +1722,12 @@ hv_status hv_focus_sweep(hv_handle* h, const void* frames, uint32_t n, const dou
 hv_status hv_af_features(hv_handle* h, const void* frames, uint32_t n, void* out_bf16) {
   if (!h) return HV_ERR_ARG;
   if (!out_bf16) return fail(h, HV_ERR_ARG, "output is NULL");
+  hv_status s = af_prepare(h, frames, n);
+  if (s != HV_OK) return s;
   // frames per pass: the feature kernel runs one CTA per frame, so a chunk
   // should cover every SM several times (512 frames: 512 MB of spectra at 256^2)
   const uint32_t chunk = std::max<uint32_t>(64, std::min<uint32_t>(512, uint32_t((size_t(256) << 20) / (size_t(h->W) * h->H * sizeof(float2)))));
-  hv_status s = af_prepare(h, frames, n, std::min(n, chunk));
+  s = af_scratch(h, std::min(n, chunk));
   if (s != HV_OK) return s;
   const size_t cells = size_t(h->W / 2) * (h->H / 2);
   for (uint32_t a = 0; a < n; a += chunk) {

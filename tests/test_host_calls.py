@@ -62,3 +62,14 @@ def test_renders_after_a_sweep_without_memory(least, times, status):
         assert len(launches) >= 3
         for w, h, n, spatial, room1, room2 in launches:
             assert room1 >= n * w * (h // 2 + 1) * 8 and room2 >= n * w * h * 8
+
+
+def test_features_as_a_handles_first_call():
+    """Settings are applied by the call itself: the launch size follows from them."""
+    assert run("""
+r = hv.Renderer(256, 256, 16, 256)
+r.set_params(256, 256, spatial="asp", T=16, stride=16, fs=20000.0, band=(1, 2))
+log()
+hv.hv_af_features(r.h, Dev((200, 256, 256), 2), Dev((200, 128, 128), 2))
+print(json.dumps([l[3] for l in log() if l[0] == "scratch"]))
+""") == [200, 200]
