@@ -1811,6 +1811,37 @@ hv_status hv_group_open(hv_handle* const* handles, uint32_t n, void* stream, int
   return HV_OK;
 }
 
+// What a step of a group changes of a member on the host.
+struct Counters {
+  uint64_t pushed, next_win, propagated, post_count;
+  hv_stats st;
+  std::deque<hv_handle::Borrowed> borrowed;
+  bool pca_has_lam;
+  uint32_t pca_last_nwin;
+  const double* pca_lam_last;
+  int inject;
+  uint64_t cons_hi[hv_handle::NCONS];
+};
+static Counters counters(const hv_handle* h) {
+  Counters c{h->pushed, h->next_win, h->propagated, h->post_count, h->st, h->borrowed,
+             h->pca_has_lam, h->pca_last_nwin, h->pca_lam_last, h->inject, {}};
+  std::copy(std::begin(h->cons_hi), std::end(h->cons_hi), std::begin(c.cons_hi));
+  return c;
+}
+static void restore(hv_handle* h, const Counters& c) {
+  h->pushed = c.pushed;
+  h->next_win = c.next_win;
+  h->propagated = c.propagated;
+  h->post_count = c.post_count;
+  h->st = c.st;
+  h->borrowed = c.borrowed;
+  h->pca_has_lam = c.pca_has_lam;
+  h->pca_last_nwin = c.pca_last_nwin;
+  h->pca_lam_last = c.pca_lam_last;
+  h->inject = c.inject;
+  std::copy(std::begin(c.cons_hi), std::end(c.cons_hi), std::begin(h->cons_hi));
+}
+
 hv_status hv_render_group(hv_group* g, const void* const* frames, const uint32_t* n_frames, float* const* outs,
                           const size_t* out_capacity_floats, uint32_t* n_windows) {
   if (!g) return HV_ERR_ARG;
@@ -1841,6 +1872,14 @@ hv_status hv_render_group(hv_group* g, const void* const* frames, const uint32_t
   }
   const bool graph = g->use_graph;
   const auto t0 = std::chrono::steady_clock::now();
+  // of a graph that is not launched nothing runs: every member's counters as they are now
+  std::vector<Counters> before;
+  if (graph)
+    for (auto* h : g->hs) before.push_back(counters(h));
+  auto undo = [&] {
+    for (uint32_t i = 0; i < before.size(); ++i) restore(g->hs[i], before[i]);
+    for (uint32_t i = 0; i < n; ++i) n_windows[i] = 0;
+  };
   if (graph) {
     HV_GCU(g, cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaEventRecord(g->ev_fork, g->stream);
@@ -1884,12 +1923,19 @@ hv_status hv_render_group(hv_group* g, const void* const* frames, const uint32_t
     if (in_place) {
       if (!h->borrowed.empty() && h->borrowed.back().first == first) h->borrowed.pop_back();
       const uint64_t keep = std::max(first, h->next_win);
-      if (s == HV_OK && keep < first + nf) {
-        s = enqueue_frames(h, frames[i], uint32_t(keep - first), first, nf);
+      // (after a failure too, unless nothing runs: the frames are queued, as pushed ones are)
+      if (keep < first + nf && (s == HV_OK || !graph)) {
+        const hv_status c = enqueue_frames(h, frames[i], uint32_t(keep - first), first, nf);
         // the slots of these frames are free after their copy, not after the spatial stage
         // that read them where they were (a graph's event comes behind the whole step)
         for (int k = 0; k < hv_handle::NCONS; ++k) h->cons_hi[k] = std::min(h->cons_hi[k], keep);
+        if (s == HV_OK) s = c;
         if (s == HV_OK && !graph) s = note_consumed(h);
+        if (c != HV_OK) {  // not queued
+          h->st.frames_pushed -= first + nf - keep;
+          h->pushed = keep;
+          h->propagated = std::min(h->propagated, keep);
+        }
       }
     }
     if (s != HV_OK) break;
@@ -1906,6 +1952,7 @@ hv_status hv_render_group(hv_group* g, const void* const* frames, const uint32_t
     const cudaError_t ec = cudaStreamEndCapture(g->stream, &gr);
     if (s != HV_OK || ec != cudaSuccess) {
       if (gr) cudaGraphDestroy(gr);
+      undo();
       if (s == HV_OK) return gfail(g, HV_ERR_CUDA, std::string("stream capture: ") + cudaGetErrorString(ec));
       for (auto* h : g->hs)
         if (!h->err.empty()) return gfail(g, s, h->err);
@@ -1926,13 +1973,18 @@ hv_status hv_render_group(hv_group* g, const void* const* frames, const uint32_t
       if (ei != cudaSuccess) {
         cudaGraphDestroy(gr);
         g->exec = nullptr;
+        undo();
         return gfail(g, HV_ERR_CUDA, std::string("cudaGraphInstantiate: ") + cudaGetErrorString(ei));
       }
       ++g->st.graph_instantiations;
     }
     cudaGraphDestroy(gr);
     g->st.capture_us_last = std::chrono::duration<double, std::micro>(std::chrono::steady_clock::now() - t0).count();
-    HV_GCU(g, cudaGraphLaunch(g->exec, g->stream));
+    const cudaError_t el = cudaGraphLaunch(g->exec, g->stream);
+    if (el != cudaSuccess) {
+      undo();
+      return gfail(g, HV_ERR_CUDA, std::string("cudaGraphLaunch: ") + cudaGetErrorString(el));
+    }
     ++g->st.graph_launches;
   } else if (s != HV_OK) {
     for (auto* h : g->hs)

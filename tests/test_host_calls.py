@@ -73,3 +73,31 @@ log()
 hv.hv_af_features(r.h, Dev((200, 256, 256), 2), Dev((200, 128, 128), 2))
 print(json.dumps([l[3] for l in log() if l[0] == "scratch"]))
 """) == [200, 200]
+
+
+FAILED_STEP = """
+W = H = 64
+rs = [hv.Renderer(W, H, 8, 16) for _ in range(2)]
+for r in rs:
+    r.set_params(W, H, spatial="asp", T=8, stride=4, fs=20000.0, band=(1, 2))
+g = hv.hv_group_open([r.h for r in rs], use_graph=%(graph)s)
+fr, outs = [Dev((12, H, W), 1) for _ in rs], [Dev((8, H, W), 4) for _ in rs]
+log()
+fake.fake_fail_launch(b"k_stft", 1)
+try:
+    hv.hv_render_group(g, fr, outs)
+    failed = False
+except hv.HvError:
+    failed = True
+copied = sum(l[4] for l in log() if l[0] == "copy" and fr[0].p <= l[3] < fr[0].p + 12 * W * H)
+pushed = [r.stats()["frames_pushed"] for r in rs]
+windows = [r.render(o) for r, o in zip(rs, outs)]
+print(json.dumps([failed, pushed, copied // (W * H), windows]))
+"""
+
+
+def test_a_failed_group_step_keeps_no_frames_it_has_not():
+    """The first member's STFT does not launch. Without a graph its frames are queued all the
+    same, copied, and a render takes them; of a graph nothing runs, so no member has frames."""
+    assert run(FAILED_STEP % dict(graph=False)) == [True, [12, 0], 12, [2, 0]]
+    assert run(FAILED_STEP % dict(graph=True)) == [True, [0, 0], 0, [0, 0]]
