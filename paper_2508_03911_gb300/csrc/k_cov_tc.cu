@@ -294,12 +294,11 @@ __global__ void __launch_bounds__(TC_NT, 1) k_cov_tc(PcaArgs a) {
   }
 }
 
-// C from the chunk partials of G (float64 sums); V = I; largest diagonal.
+// C from the chunk partials of G (float64 sums); largest diagonal.
 __global__ void k_cov_tc_reduce(PcaArgs a) {
   const int T = int(a.T), BF = T < 128 ? T : 128, ntiles = int(a.tc_ntiles);
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < T * T; e += gridDim.x * blockDim.x) {
     const int r = e / T, c = e % T;
-    a.V[e] = make_double2(r == c ? 1.0 : 0.0, 0.0);
     if (r > c) continue;
     const int ti = r / 64, tj = c / BF;
     int t = 0;

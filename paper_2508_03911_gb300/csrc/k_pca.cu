@@ -11,7 +11,7 @@
 //   k_cov_fp32     split-K covariance: each CTA multiplies a 64 x 64 tile of the
 //                  upper triangle over one pixel chunk (float32 FMA), partials
 //                  written per chunk (deterministic, no atomics)
-//   k_cov_reduce   sums the chunk partials in float64 -> C (full Hermitian), V = I
+//   k_cov_reduce   sums the chunk partials in float64 -> C (full Hermitian)
 //   k_jacobi_cluster, k_jacobi_f32
 //                  float32 phase of the long-window eigensolver (T > 64, one
 //                  window): parallel cyclic (round-robin) two-sided Jacobi on one
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(256) k_cov_fp32(PcaArgs a) {
     for (int j = 0; j < nI; ++j) out[(ty + 16 * i) * TS + tx + 16 * j] = acc[i][j];
 }
 
-// C[a][b] = sum over chunks (float64), mirrored to the lower triangle; V = I.
+// C[a][b] = sum over chunks (float64), mirrored to the lower triangle.
 __global__ void k_cov_reduce(PcaArgs a) {
   const int T = a.T, TS = T < COV_TS ? T : COV_TS, nT = T / TS, ntile_up = nT * (nT + 1) / 2;
   for (int ew = blockIdx.x * blockDim.x + threadIdx.x; ew < int(a.nwin) * T * T; ew += gridDim.x * blockDim.x) {
@@ -121,7 +121,6 @@ __global__ void k_cov_reduce(PcaArgs a) {
     const int r = e / T, c = e % T;
     double2* Cw = a.C + size_t(w) * T * T;
     const float2* Pw = a.partials + size_t(w) * a.nchunks * ntile_up * TS * TS;
-    if (w == 0) a.V[e] = make_double2(r == c ? 1.0 : 0.0, 0.0);
     if (r > c) continue;
     const int ta = r / TS, tb = c / TS;
     const int up = ta * nT - ta * (ta - 1) / 2 + (tb - ta);

@@ -74,11 +74,10 @@ def test_pca_parity(H, W, T, S, lohi, spatial):
 
 
 def test_pca_long_windows_pipelined():
-    """Five overlapping long windows (T = 128, S = 64) in one render: the eigensolver
-    of each window runs on a second stream beside the next window's covariance and
-    the previous window's projection, the windows alternating between two buffer
-    sets; every window's image and the last window's eigenvalues against the
-    oracle."""
+    """Five overlapping long windows (T = 128, S = 64) in one render: the eigensolvers run on
+    streams of their own beside later windows' covariances and earlier windows' projections,
+    the windows taking turns at as many buffer sets as eigensolvers fit the device; every
+    window's image and the last window's eigenvalues against the oracle."""
     H = W = 64
     T, S = 128, 64
     fr = synth.random_frames(T + 4 * S + 9, H, W, 12, seed=77)
@@ -86,6 +85,24 @@ def test_pca_long_windows_pipelined():
     img, lam = gpu_pca(fr, p)
     ref = oracle_windows(fr, p)
     assert img.shape[0] == len(ref) == 5
+    for w, rw in enumerate(ref):
+        e = rel_l2(img[w], rw["E"])
+        assert e <= IMAGE_TOL, (w, e)
+    lam_ref = ref[-1]["lam"]
+    assert np.max(np.abs(lam - lam_ref)) <= LAM_TOL * lam_ref[0]
+
+
+def test_pca_windows_of_512_frames_pipelined():
+    """Three windows in one render where one eigensolver runs at a time, all on the same
+    scratch (T = 512, cooperative): the covariance of the next window, beside it, touches none of
+    it. All components but the first, the static part's, whose eigenvalue stands far apart."""
+    H = W = 64
+    T, S = 512, 256
+    fr = synth.random_frames(T + 2 * S, H, W, 12, seed=78)
+    p = oracle_params(spatial="none", temporal="pca", T=T, stride=S, pca_lo=2, pca_hi=T, H=H, W=W)
+    img, lam = gpu_pca(fr, p)
+    ref = oracle_windows(fr, p)
+    assert img.shape[0] == len(ref) == 3
     for w, rw in enumerate(ref):
         e = rel_l2(img[w], rw["E"])
         assert e <= IMAGE_TOL, (w, e)
