@@ -15,6 +15,7 @@
 
 #include <mutex>
 
+#include "quotient.h"
 #include "strip_dev.cuh"
 #include "hv_internal.h"
 #include "../../include/hv.h"
@@ -283,26 +284,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity) {
     if (ok) return true;
     if (clock64() - t0 > (1ll << 32)) return false;
   }
-}
-
-// float(double(a) / double(b)): the float32 quotient is the same number, since float64 keeps
-// more than twice float32's digits and two bits (results below the normal range apart, which
-// float64 rounds twice). Float64 instructions run at 1/64 of the float32 rate, and one lane
-// in 4 to 16 writes: M1N and M2N took 0.1 ms per window of 1024 x 512 in float64.
-__device__ __forceinline__ float quotient(float a, float b) { return __fdiv_rn(a, b); }
-
-// float(sqrt(double(a) / double(b))) for a >= 0, b > 0: the quotient as a float32 pair (its
-// remainder exact by fma), one Newton step of the root on the pair; the float64 form
-// outside the range where the pair holds.
-__device__ __forceinline__ float root_of_quotient(float a, float b) {
-  const float q = __fdiv_rn(a, b);
-  if (!(a > 1e-25f && b > 1e-25f && b < 1e25f && q > 1e-25f && q < 1e25f)) {
-    const double r = double(a) / double(b);
-    return float(sqrt(r > 0.0 ? r : 0.0));
-  }
-  const float lo = __fdiv_rn(fmaf(-q, b, a), b);
-  const float s = __fsqrt_rn(q);
-  return fmaf(0.5f * __frcp_rn(s), fmaf(-s, s, q) + lo, s);
 }
 
 // Post-processing fused into the moment epilogue: the moments of pixel `pix` for
