@@ -849,3 +849,25 @@ def test_window_per_cta_stft_paper_asp_shape():
                       band_lo_bin=klo, band_hi_bin=khi, moments=("M0", "M1", "M2"), H=256, W=256)
     img, _ = gpu_render(fr, p, extra=dict(spatial_kernel="fused", stft_kernel="window"))
     check_images(img, O.render(fr, p))
+
+
+@pytest.mark.parametrize("T,N,bars", [(16, 256, (6.52e-8, 7.18e-8)), (32, 256, (7.4e-8, 8.1e-8)),
+                                      (256, 128, (7.05e-8, 7.5e-8)), (1024, 128, (9.75e-8, 7.85e-8))])
+def test_rounding_of_windows_from_registers(T, N, bars):
+    """M0 and M1N of noise against float64, relative to the 2-norm. The frames are fixed and the
+    kernel's arithmetic deterministic: the bars lie half way between its errors (those of the
+    walking kernel, or less) and those of one DFT and one running sum per thread: (6.47, 7.01) and
+    (6.56, 7.35) e-8 for T = 16, (6.49, 7.21) and (8.32, 9.06) for 32, (6.93, 7.31) and (7.17, 7.70)
+    for 256, (9.48, 7.24) and (10.0, 8.46) for 1024."""
+    fr = synth.random_frames(2 * T, N, N, 12, seed=T)
+    hi = T // 2 - 1
+    p = oracle_params(spatial="none", T=T, stride=T, fs_hz=71400.0, band_lo_bin=1, band_hi_bin=hi,
+                      moments=("M0", "M1N"), H=N, W=N)
+    img, _ = gpu_render(fr, p)
+    for q in range(2):
+        ref = []
+        for w in range(2):
+            P = np.abs(np.fft.fft(fr[w * T:(w + 1) * T].astype(np.float64), axis=0)[1:hi + 1]) ** 2
+            f = np.arange(1, hi + 1).reshape(-1, 1, 1) * (71.4 / T)
+            ref.append((f * P).sum(0) / P.sum(0) if q else P.sum(0))
+        assert max(rel_l2(img[w, q], ref[w]) for w in range(2)) <= bars[q], q
