@@ -871,3 +871,17 @@ def test_rounding_of_windows_from_registers(T, N, bars):
             f = np.arange(1, hi + 1).reshape(-1, 1, 1) * (71.4 / T)
             ref.append((f * P).sum(0) / P.sum(0) if q else P.sum(0))
         assert max(rel_l2(img[w, q], ref[w]) for w in range(2)) <= bars[q], q
+
+
+@pytest.mark.parametrize("N,bar", [(512, 5.2e-8), (1024, 6.2e-8)])
+def test_rounded_constants_of_long_transforms(N, bar):
+    """The projection of a Fresnel field onto the float64 one falls short by what rounded constants
+    lose: 4.3e-8 (512 x 512) and 4.5e-8, 6.2e-8 and 8.0e-8 where the last stage of the 32-point DFT
+    takes them as float32. The bars lie half way."""
+    fr = synth.random_frames(2, N, N, 12, seed=N + 7)
+    p = oracle_params(spatial="fresnel", z_m=0.3, temporal="none", T=1, stride=1, H=N, W=N)
+    img, _ = gpu_render(fr, p)
+    ref = oracle_fields(fr, p)
+    for i in range(2):
+        gain = np.vdot(ref[i], np.asarray(img[i], np.complex128)).real / np.vdot(ref[i], ref[i]).real - 1.0
+        assert abs(gain) <= bar, gain
