@@ -362,10 +362,10 @@ uint64_t launches_of_run(const hv_handle* h, uint64_t n, uint64_t chunk, uint32_
 
 // Scratch of the multi-pass transform: `chunk` frames for each of the launches side by side,
 // as many as runs of up to `frames` frames fill and 1 GB holds, one where there is no memory
-// for more; `least` frames in all.
+// for more; `least` frames in all, for the fused transform, whose frames take one launch.
 hv_status size_scratch(hv_handle* h, int spatial, size_t fbytes, uint32_t chunk, uint32_t frames, uint32_t least) {
   const size_t fit = (size_t(1) << 30) / (chunk * fbytes), runs = launches_of_run(h, frames, chunk, kSpLanes);
-  uint32_t lanes = uint32_t(std::max<size_t>(1, std::min<size_t>({kSpLanes, fit, runs})));
+  uint32_t lanes = least ? 1 : uint32_t(std::max<size_t>(1, std::min<size_t>({kSpLanes, fit, runs})));
   for (;; lanes = 1) {
     const size_t need = std::max<size_t>(size_t(lanes) * chunk, least) * fbytes;
     hv_status s = ensure(h, reinterpret_cast<void**>(&h->s1), &h->s1_bytes, need);
@@ -432,6 +432,10 @@ hv_status apply_pending(hv_handle* h) {
   h->sp_lanes = 1;
   if (p.spatial != HV_SPATIAL_NONE) {
     s = size_scratch(h, p.spatial, fbytes, chunk, Q, fused ? kFusedRing : 0);
+    if (s == HV_ERR_NOMEM && p.spatial_chunk == 0 && chunk * fbytes > (size_t(32) << 20)) {
+      chunk = uint32_t((size_t(32) << 20) / fbytes);
+      s = size_scratch(h, p.spatial, fbytes, chunk, Q, fused ? kFusedRing : 0);
+    }
     if (s != HV_OK) return s;
   }
   s = build_tables(h, p);
@@ -859,7 +863,10 @@ hv_status tune_temporal(hv_handle* h) {
     nwin = std::min<uint32_t>((h->Q - T) / S + 1,
                               std::max<uint32_t>(nwin, std::min<uint32_t>(64, uint32_t((size_t(64) << 20) / (h->nout * hw)))));
   float* out = nullptr;
-  HV_CU(h, cudaMalloc(&out, size_t(nwin) * h->nout * hw * sizeof(float)));
+  if (cudaMalloc(&out, size_t(nwin) * h->nout * hw * sizeof(float)) != cudaSuccess) {
+    cudaGetLastError();
+    return HV_OK;  // no room for a trial: the default kernel
+  }
   cudaEvent_t e0, e1;
   HV_CU(h, cudaEventCreate(&e0));
   HV_CU(h, cudaEventCreate(&e1));

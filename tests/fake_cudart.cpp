@@ -17,7 +17,7 @@ namespace {
 std::string g_log, g_out;
 std::map<size_t, size_t> g_live;  // address -> bytes
 std::map<const void*, std::string> g_name;
-size_t g_next = size_t(1) << 32, g_fail_from = 0;
+size_t g_next = size_t(1) << 32, g_fail_from = 0, g_fail_to = 0;
 int g_fail_malloc = 0, g_fail_launch = 0;
 std::string g_fail_kernel;
 cudaError_t g_last = cudaSuccess;
@@ -72,15 +72,15 @@ const char* fake_log() {
   g_log.clear();
   return g_out.c_str();
 }
-// The next `times` allocations of `from` bytes or more fail.
-void fake_fail_malloc(size_t from, int times) { g_fail_from = from, g_fail_malloc = times; }
+// The next `times` allocations of `from` to `to` bytes fail.
+void fake_fail_malloc(size_t from, size_t to, int times) { g_fail_from = from, g_fail_to = to, g_fail_malloc = times; }
 // The next `times` launches of a kernel whose name holds `part` fail.
 void fake_fail_launch(const char* part, int times) { g_fail_kernel = part, g_fail_launch = times; }
 size_t fake_room(size_t p) { return room(reinterpret_cast<void*>(p)); }
 
 cudaError_t cudaMalloc(void** p, size_t n) {
   *p = nullptr;
-  if (g_fail_malloc > 0 && n >= g_fail_from) {
+  if (g_fail_malloc > 0 && n >= g_fail_from && n <= g_fail_to) {
     --g_fail_malloc;
     return err(cudaErrorMemoryAllocation);
   }

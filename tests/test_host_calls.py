@@ -41,13 +41,13 @@ def render():
     assert r.push(fr) == hv.HV_OK and r.render(out) == 1
     return [l[1:] for l in log() if l[0] == "scratch"]
 before = render()
-fake.fake_fail_malloc(%(least)d * MB, %(times)d)
+fake.fake_fail_malloc(%(least)d * MB, 1 << 40, %(times)d)
 try:
     hv.hv_focus_sweep(r.h, Dev((64, N, N), 2), np.linspace(0.1, 0.6, 64), Dev((64, 64), 4))
     status = 0
 except hv.HvError as e:
     status = e.status
-fake.fake_fail_malloc(0, 0)
+fake.fake_fail_malloc(0, 0, 0)
 print(json.dumps([status, before, render()]))
 """
 
@@ -101,3 +101,39 @@ def test_a_failed_group_step_keeps_no_frames_it_has_not():
     same, copied, and a render takes them; of a graph nothing runs, so no member has frames."""
     assert run(FAILED_STEP % dict(graph=False)) == [True, [12, 0], 12, [2, 0]]
     assert run(FAILED_STEP % dict(graph=True)) == [True, [0, 0], 0, [0, 0]]
+
+
+SHORT = """
+MB = 1 << 20
+r = hv.Renderer(%(side)d, %(side)d, 16, %(cap)d)
+r.set_params(%(side)d, %(side)d, fs=20000.0, band=(1, 2), moments=("M0", "M1"), %(kw)s)
+out = Dev((64, 2, %(side)d, %(side)d), 4)
+assert r.push(Dev((%(cap)d, %(side)d, %(side)d), 2)) == hv.HV_OK
+log()
+fake.fake_fail_malloc(%(low)d, %(high)d, 100)
+nw = r.render(out)
+lines = log()
+print(json.dumps([nw, [l[2] // MB for l in lines if l[0] == "malloc"], [l[3] for l in lines if l[0] == "scratch"]]))
+"""
+
+
+def test_overlapping_windows_tuned_without_memory_for_the_trial():
+    """No memory for the images that the STFT kernels are timed with (64 windows of two images):
+    the default kernel renders."""
+    nw, _, _ = run(SHORT % dict(side=256, cap=1024, low=64 * 2 * 65536 * 4, high=64 * 2 * 65536 * 4,
+                                kw='spatial="none", T=128, stride=16, tuned=1'))
+    assert nw == 57
+
+
+def test_default_launches_without_64_mb():
+    """Where 64 MB of fields a launch do not fit, 32 MB do: 16 frames of 512 x 512."""
+    nw, sizes, frames = run(SHORT % dict(side=512, cap=200, low=60 << 20, high=300 << 20,
+                                         kw='spatial="asp", T=128, stride=128'))
+    assert nw == 1 and sizes.count(32) == 2 and max(frames) == 16
+
+
+def test_fused_transform_takes_no_scratch_for_launches_side_by_side():
+    """One launch for all frames: 64 MB, a launch's frames, and not four times that."""
+    _, sizes, _ = run(SHORT % dict(side=256, cap=480, low=1, high=0,
+                                   kw='spatial="fresnel", T=128, stride=128, spatial_kernel="fused"'))
+    assert 64 in sizes and 256 not in sizes
