@@ -1494,16 +1494,15 @@ def main():
             "gpu_launches": res["launches"],
             "clocks": res["clocks"],
             "form": "plain" if args.form == "plain" else "tuned",
-            "tuning": {"spatial_kernel": {1: "multipass", 2: "cluster", 3: "persistent", 4: "fused"}.get(
+            "tuning": {"spatial_kernel": {1: "multipass", 2: "cluster", 4: "fused"}.get(
                            res["tuning"]["spatial_kernel"], "multipass"),
                        "frames_per_launch": ("every frame of a render" if res["tuning"]["spatial_kernel"] in (2, 4)
                                              else res["tuning"]["spatial_chunk"]),
                        "candidates_us_per_frame": dict(zip(
                            ["mp16", "mp32", "mp64", "mp128", "mp256", "pp64", "pp128", "pp256",
-                            "pp512", "cluster", "fused"],
+                            "mp512", "cluster", "fused"],
                            [round(v, 4) for v in res["tuning"]["candidate_us_per_frame"][:11]])),
-                       "stft_kernel": {1: "walk", 2: "window", 3: "window_wide", 4: "window_pipelined",
-                                       5: "window_tma", 6: "window_tma_pipelined"}.get(
+                       "stft_kernel": {1: "walk", 2: "window", 5: "window_tma", 6: "window_tma_pipelined"}.get(
                            res["tuning"].get("stft_kernel"), "walk"),
                        "stft_candidates_us_per_window": dict(zip(
                            ["walk", "window", "window_wide", "window_pipelined", "window_tma",

@@ -203,15 +203,16 @@ hv_status hv_pca_eigenvalues(const hv_handle* h, double* out, uint32_t n);
  * applied by timing each candidate on the handle's own buffers. */
 typedef struct {
   int32_t tuned;                    /* 1 once the autotuner has run                   */
-  int32_t spatial_kernel;           /* HV_SK_MULTIPASS, _CLUSTER, _PERSISTENT or _FUSED */
+  int32_t spatial_kernel;           /* HV_SK_MULTIPASS (a persistent selection's too, the
+                                       same passes), _CLUSTER or _FUSED               */
   uint32_t spatial_chunk;           /* frames per multi-pass launch                   */
-  int32_t stft_kernel;              /* HV_STFT_WALK, _WINDOW, _WINDOW_WIDE,
-                                       _WINDOW_PIPELINED, _WINDOW_TMA or
+  int32_t stft_kernel;              /* the kernel that runs: HV_STFT_WALK, _WINDOW (a wide
+                                       or pipelined selection's too), _WINDOW_TMA or
                                        _WINDOW_TMA_PIPELINED                          */
   float candidate_us_per_frame[12]; /* measured us per frame: multi-pass with 16, 32, 64,
-                                       128, 256 frames per launch; persistent
-                                       multi-pass with 64, 128, 256 (the same passes as
-                                       multi-pass, not timed again) and 512; the cluster
+                                       128, 256 frames per launch; 64, 128, 256 again
+                                       (the persistent selection, the same passes, not
+                                       timed again) and 512; the cluster
                                        kernel; the fused transform (0 where not
                                        applicable)                                    */
   float stft_us_per_window[6];      /* measured us per window of the STFT kernels:

@@ -592,7 +592,8 @@ hv_status apply_pending(hv_handle* h) {
   h->sp_fused = fused ? 1 : 0;
   h->tuning = hv_tuning{};
   h->tuning.spatial_chunk = chunk;
-  h->tuning.spatial_kernel = p.spatial_kernel == HV_SK_AUTO ? HV_SK_MULTIPASS : int32_t(p.spatial_kernel);
+  h->tuning.spatial_kernel =
+      p.spatial_kernel == HV_SK_CLUSTER || p.spatial_kernel == HV_SK_FUSED ? int32_t(p.spatial_kernel) : HV_SK_MULTIPASS;
   // STFT kernel: the caller's (for windows that do not overlap; others walk), the
   // autotuner's (tuned, below), else the window kernel where windows do not overlap (faster
   // than walking at every T: 0.69 against 1.34 us a window of 256 x 256 at T = 8, 183 against
@@ -606,7 +607,11 @@ hv_status apply_pending(hv_handle* h) {
     s = tune_spatial(h);  // rewrites the tuning record
     if (s != HV_OK) return s;
   }
-  h->tuning.stft_kernel = asked;
+  // the kernel that runs: windows that overlap walk, the TMA-fed ones are T = 512's
+  h->tuning.stft_kernel = h->stft_kernel == STFT_WALK || d.S < d.T ? HV_STFT_WALK
+                          : h->stft_kernel == STFT_TMA && d.T == 512      ? HV_STFT_WINDOW_TMA
+                          : h->stft_kernel == STFT_TMA_PIPE && d.T == 512 ? HV_STFT_WINDOW_TMA_PIPELINED
+                                                                          : HV_STFT_WINDOW;
   if (p.tuned && p.stft_kernel == 0 && p.temporal == HV_TEMPORAL_STFT) {
     s = tune_temporal(h);
     if (s != HV_OK) return s;
@@ -839,8 +844,7 @@ hv_status tune_spatial(hv_handle* h) {
   if (best_kind != 2 &&
       size_scratch(h, h->cur.spatial, fbytes, best_chunk, h->Q, best_kind == 4 ? kFusedRing : 0) != HV_OK)
     return HV_ERR_NOMEM;
-  t.spatial_kernel = best_kind == 2 ? HV_SK_CLUSTER
-                     : (best_kind == 3 ? HV_SK_PERSISTENT : (best_kind == 4 ? HV_SK_FUSED : HV_SK_MULTIPASS));
+  t.spatial_kernel = best_kind == 2 ? HV_SK_CLUSTER : (best_kind == 4 ? HV_SK_FUSED : HV_SK_MULTIPASS);
   t.spatial_chunk = best_chunk;
   t.tuned = 1;
   h->tuning = t;

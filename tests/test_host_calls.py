@@ -137,3 +137,20 @@ def test_fused_transform_takes_no_scratch_for_launches_side_by_side():
     _, sizes, _ = run(SHORT % dict(side=256, cap=480, low=1, high=0,
                                    kw='spatial="fresnel", T=128, stride=128, spatial_kernel="fused"'))
     assert 64 in sizes and 256 not in sizes
+
+
+def test_tuning_record_names_the_kernels_that_run():
+    """Selections that other kernels serve, and windows that overlap."""
+    assert run("""
+got = []
+for kw in (dict(spatial_kernel="persistent"), dict(spatial_kernel="cluster"), dict(stft_kernel="window_wide"),
+           dict(stft_kernel="window_pipelined"), dict(stft_kernel="window_tma"), dict(stft_kernel="window", stride=64),
+           dict(stride=64), dict()):
+    r = hv.Renderer(256, 256, 16, 256)
+    r.set_params(256, 256, **dict(dict(spatial="asp", T=128, stride=128, fs=20000.0, band=(1, 2)), **kw))
+    assert r.push(Dev((256, 256, 256), 2)) == hv.HV_OK
+    r.render(Dev((4, 1, 256, 256), 4))
+    t = hv.hv_get_tuning(r.h)
+    got.append([t["spatial_kernel"], t["stft_kernel"]])
+print(json.dumps(got))
+""") == [[1, 2], [2, 2], [1, 2], [1, 2], [1, 2], [1, 1], [1, 1], [1, 2]]
