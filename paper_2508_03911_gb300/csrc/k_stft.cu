@@ -161,7 +161,7 @@ __device__ __forceinline__ void dft_lower(float2* v) {
 // (every Qth output) added in pairs: where few threads hold a pixel, one running sum rounds more
 // than the sums of the walking kernel's lanes (k_stft_cols against it with one part and the
 // warps in order: M1N of T = 256, 512, 1024 8.9e-8, 9.5e-8, 9.5e-8 off against 8.0e-8, 8.5e-8,
-// 8.6e-8; 8.2e-8, 8.1e-8, 8.1e-8 with parts).
+// 8.6e-8; 8.2e-8, 8.1e-8, 8.2e-8 with parts).
 template <int R, int NB, int MO, int Q = 1>
 __device__ __forceinline__ void add_moments(const float2* v, int it, float kb, MomAcc& acc) {
   float s0[Q], s1[Q], s2[Q];
@@ -680,12 +680,19 @@ __global__ void __launch_bounds__(ColCfg<T>::NT, ColCfg<T>::CTAS) k_stft_cols(St
       }
     col_stage1<T, -1>(v, buf, t, b);
     col_stage2<T, -1>(u, buf, tw, t, b);
-    MomAcc acc{band, 0.f, 0.f, 0.f};
+    MomAcc part2[C::I2];  // each butterfly by itself: a sum of moments rounds once, one carried on thrice
 #pragma unroll
     for (int it = 0; it < C::I2; ++it) {
       const float kb = float(col_j2<T>(t, it));
-      if (lower) add_moments<C::R2, C::R1, C::R2 / 2, sum_parts(C::R2 / 2)>(u[it], it, kb, acc);
-      else add_moments<C::R2, C::R1, C::R2, sum_parts(C::R2)>(u[it], it, kb, acc);
+      part2[it] = MomAcc{band, 0.f, 0.f, 0.f};
+      if (lower) add_moments<C::R2, C::R1, C::R2 / 2, sum_parts(C::R2 / 2)>(u[it], it, kb, part2[it]);
+      else add_moments<C::R2, C::R1, C::R2, sum_parts(C::R2)>(u[it], it, kb, part2[it]);
+    }
+    MomAcc acc = part2[0];
+    if constexpr (C::I2 == 2) {
+      acc.m0 += part2[1].m0;
+      acc.m1 += part2[1].m1;
+      acc.m2 += part2[1].m2;
     }
     // the pixel's threads: lanes of a warp BT apart, then the warps
 #pragma unroll
