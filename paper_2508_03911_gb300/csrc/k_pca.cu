@@ -26,6 +26,7 @@
 #include <cooperative_groups.h>
 
 #include "fft_dev.cuh"
+#include "pair_dev.cuh"
 #include "hv_internal.h"
 #include "../../include/hv.h"
 
@@ -150,19 +151,12 @@ __device__ __forceinline__ int rr_elem(int k, int r, int T) {
   return k == 0 ? 0 : ((k - 1 + r) % (T - 1)) + 1;
 }
 
-// Numbers as unevaluated sums hi + lo of two float32 (48 bits): GB300 has 64 float32 units
-// for each float64 one.
+// Pairs of float32 (pair_dev.cuh) from and to float64.
 __device__ __forceinline__ float2 to_pair(double v) {
   const float hi = float(v);
   return make_float2(hi, float(v - double(hi)));
 }
 __device__ __forceinline__ double from_pair(float2 p) { return double(p.x) + double(p.y); }
-
-// The exact sum of a and b as a pair (Knuth's two-sum).
-__device__ __forceinline__ float2 two_sum(float a, float b) {
-  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-  return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
-}
 
 // acc += a b, a a pair: the products exact by fma, the sum by two_sum.
 __device__ __forceinline__ void pair_fma(float2& acc, float ah, float al, float b) {
@@ -170,13 +164,6 @@ __device__ __forceinline__ void pair_fma(float2& acc, float ah, float al, float 
   const float2 t = two_sum(acc.x, p);
   acc.x = t.x;
   acc.y += t.y + e;
-}
-
-// p + x, renormalised.
-__device__ __forceinline__ float2 pair_add(float2 p, float x) {
-  const float2 t = two_sum(p.x, x);
-  const float lo = p.y + t.y, hi = __fadd_rn(t.x, lo);
-  return make_float2(hi, __fsub_rn(lo, __fsub_rn(hi, t.x)));
 }
 
 // Sums of complex products a b: a of pairs (re, im, then their low parts), b float32.
@@ -1439,7 +1426,8 @@ __global__ void __launch_bounds__(cov_small_threads(T)) k_cov_small(PcaArgs a) {
   }
   asm volatile("cp.async.wait_all;\n" ::: "memory");
   __syncthreads();
-  // groups' sums in shared memory (reusing the strip buffers: G x T x T <= 2 x T x LDX)
+  // groups' sums in shared memory, over the strip buffers
+  static_assert(cov_small_smem(T) >= size_t(G) * T * T * sizeof(float2), "room for every group");
   float2* red = xs;
   if (active)
 #pragma unroll

@@ -9,6 +9,7 @@
 // moving average then reads the slots it needs, so every window of the call is
 // averaged in parallel. Without a convolution the STFT epilogue writes the slots
 // and their sums itself, and only the average runs here.
+#include "pair_dev.cuh"
 #include "hv_internal.h"
 
 namespace hv {
@@ -17,21 +18,9 @@ namespace {
 
 constexpr int PY = 16;  // rows of a convolution tile; TX = 16, 32 or 64 columns, 4 per thread
 
-// A float32 pair hi + lo (about 48 bits): float64 instructions run at 1/64 of the
-// float32 rate, and one conversion and five shuffled additions of them per pixel took
-// most of the kernel's time (see below).
-struct F2 {
-  float hi, lo;
-};
-__device__ __forceinline__ F2 two_sum(float a, float b) {  // exact: hi + lo = a + b
-  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
-  return F2{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
-}
-__device__ __forceinline__ F2 add(F2 a, F2 b) {
-  const F2 s = two_sum(a.hi, b.hi);
-  const float e = __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)), h = __fadd_rn(s.hi, e);
-  return F2{h, __fsub_rn(e, __fsub_rn(h, s.hi))};
-}
+// Sums and scales in pairs of float32 (pair_dev.cuh): one conversion to float64 and five
+// shuffled additions of it per pixel took most of the kernel's time (see below).
+
 // ring[slot][m][y][x] = sum_{a,b} k[a][b] img[(y + a - c) mod H][(x + b - c) mod W]
 // for image m of window w (slot = (count + w) mod R); K = 0 copies. Re-normalising,
 // the tile's sum goes into one of the slot image's partial sums.
@@ -88,11 +77,11 @@ __global__ void __launch_bounds__(TX / 4 * PY) k_post_conv(const float* __restri
   *reinterpret_cast<float4*>(a.ring + (size_t(slot) * a.nout + m) * hw + size_t(ty0 + ly) * a.W + tx0 + lx) =
       make_float4(v[0], v[1], v[2], v[3]);
   if (a.renorm) {
-    F2 t = add(two_sum(v[0], v[1]), two_sum(v[2], v[3]));
+    float2 t = pair_add(two_sum(v[0], v[1]), two_sum(v[2], v[3]));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
-      t = add(t, F2{__shfl_xor_sync(0xffffffffu, t.hi, o), __shfl_xor_sync(0xffffffffu, t.lo, o)});
-    double d = double(t.hi) + double(t.lo);
+      t = pair_add(t, make_float2(__shfl_xor_sync(0xffffffffu, t.x, o), __shfl_xor_sync(0xffffffffu, t.y, o)));
+    double d = double(t.x) + double(t.y);
     if (__any_sync(0xffffffffu, !isfinite(d))) {  // an infinity or NaN, or a sum past the largest float
       d = (double(v[0]) + double(v[1])) + (double(v[2]) + double(v[3]));
 #pragma unroll

@@ -56,7 +56,6 @@ __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-// all but the newest N committed groups complete
 
 __device__ __forceinline__ int wpad(int i) { return i + (i >> 4); }
 
@@ -203,7 +202,6 @@ __host__ __device__ constexpr int sum_parts(int MO) { return MO >= 16 ? 4 : (MO 
 template <int T, int NS, int LP>
 __device__ __forceinline__ void warp_fft(const float2* win, float2* work, const float2* tw, int jl,
                                          MomAcc& acc, bool lower) {
-  // WP: the window itself is stored padded (sample t at t + t / 16)
   constexpr int R = WarpPlan<T>::template radix<NS>();
   constexpr int NB = T / R;
   static_assert(NB % LP == 0, "lanes per pixel must divide the butterflies");

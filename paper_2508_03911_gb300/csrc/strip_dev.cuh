@@ -142,73 +142,73 @@ __device__ __forceinline__ void load_raw_strip(const SpatialArgs& a, size_t fram
   using C = ColCfg<L>;
   const uint32_t W = a.W;
   const bool u8 = a.in_kind == IN_U8;
-      if constexpr (ASP) {
-        const size_t x = size_t(s) * (2 * C::BT) + 2 * b;
-        const size_t at = frame + x;
-        if (u8) {
-          const unsigned char* p = static_cast<const unsigned char*>(a.raw.base) + at;
-          if ((reinterpret_cast<uintptr_t>(a.raw.base) & 1) == 0) {
-  #pragma unroll
-            for (int it = 0; it < C::I1; ++it)
-  #pragma unroll
-              for (int m = 0; m < C::R1; ++m) {
-                const uint32_t q =
-                    *reinterpret_cast<const uint16_t*>(p + size_t(t + C::NJ * it + (L / C::R1) * m) * W);
-                v[it][m] = make_float2(float(q & 0xffu), float(q >> 8));
-              }
-          } else {
-  #pragma unroll
-            for (int it = 0; it < C::I1; ++it)
-  #pragma unroll
-              for (int m = 0; m < C::R1; ++m) {
-                const unsigned char* q = p + size_t(t + C::NJ * it + (L / C::R1) * m) * W;
-                v[it][m] = make_float2(float(q[0]), float(q[1]));
-              }
-          }
-        } else {
-          const uint16_t* p = static_cast<const uint16_t*>(a.raw.base) + at;
-          if ((reinterpret_cast<uintptr_t>(a.raw.base) & 3) == 0) {
-  #pragma unroll
-            for (int it = 0; it < C::I1; ++it)
-  #pragma unroll
-              for (int m = 0; m < C::R1; ++m) {
-                const uint32_t q =
-                    *reinterpret_cast<const uint32_t*>(p + size_t(t + C::NJ * it + (L / C::R1) * m) * W);
-                v[it][m] = make_float2(float(q & 0xffffu), float(q >> 16));
-              }
-          } else {
-  #pragma unroll
-            for (int it = 0; it < C::I1; ++it)
-  #pragma unroll
-              for (int m = 0; m < C::R1; ++m) {
-                const uint16_t* q = p + size_t(t + C::NJ * it + (L / C::R1) * m) * W;
-                v[it][m] = make_float2(float(q[0]), float(q[1]));
-              }
-          }
-        }
-      } else {
-        const size_t x = size_t(s) * C::BT + b;
-        const float2 cx = __ldg(&a.chirp_x[x]);
-        float r[C::I1][C::R1];
-        if (u8) {
-          const unsigned char* p = static_cast<const unsigned char*>(a.raw.base) + frame + x;
-  #pragma unroll
-          for (int it = 0; it < C::I1; ++it)
-  #pragma unroll
-            for (int m = 0; m < C::R1; ++m) r[it][m] = float(p[size_t(t + C::NJ * it + (L / C::R1) * m) * W]);
-        } else {
-          const uint16_t* p = static_cast<const uint16_t*>(a.raw.base) + frame + x;
-  #pragma unroll
-          for (int it = 0; it < C::I1; ++it)
-  #pragma unroll
-            for (int m = 0; m < C::R1; ++m) r[it][m] = float(p[size_t(t + C::NJ * it + (L / C::R1) * m) * W]);
-        }
-  #pragma unroll
+  if constexpr (ASP) {
+    const size_t x = size_t(s) * (2 * C::BT) + 2 * b;
+    const size_t at = frame + x;
+    if (u8) {
+      const unsigned char* p = static_cast<const unsigned char*>(a.raw.base) + at;
+      if ((reinterpret_cast<uintptr_t>(a.raw.base) & 1) == 0) {
+#pragma unroll
         for (int it = 0; it < C::I1; ++it)
-  #pragma unroll
-          for (int m = 0; m < C::R1; ++m)
-            v[it][m] = cscale(cmul(__ldg(&a.chirp_y[t + C::NJ * it + (L / C::R1) * m]), cx), r[it][m]);
+#pragma unroll
+          for (int m = 0; m < C::R1; ++m) {
+            const uint32_t q =
+                *reinterpret_cast<const uint16_t*>(p + size_t(t + C::NJ * it + (L / C::R1) * m) * W);
+            v[it][m] = make_float2(float(q & 0xffu), float(q >> 8));
+          }
+      } else {
+#pragma unroll
+        for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+          for (int m = 0; m < C::R1; ++m) {
+            const unsigned char* q = p + size_t(t + C::NJ * it + (L / C::R1) * m) * W;
+            v[it][m] = make_float2(float(q[0]), float(q[1]));
+          }
       }
+    } else {
+      const uint16_t* p = static_cast<const uint16_t*>(a.raw.base) + at;
+      if ((reinterpret_cast<uintptr_t>(a.raw.base) & 3) == 0) {
+#pragma unroll
+        for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+          for (int m = 0; m < C::R1; ++m) {
+            const uint32_t q =
+                *reinterpret_cast<const uint32_t*>(p + size_t(t + C::NJ * it + (L / C::R1) * m) * W);
+            v[it][m] = make_float2(float(q & 0xffffu), float(q >> 16));
+          }
+      } else {
+#pragma unroll
+        for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+          for (int m = 0; m < C::R1; ++m) {
+            const uint16_t* q = p + size_t(t + C::NJ * it + (L / C::R1) * m) * W;
+            v[it][m] = make_float2(float(q[0]), float(q[1]));
+          }
+      }
+    }
+  } else {
+    const size_t x = size_t(s) * C::BT + b;
+    const float2 cx = __ldg(&a.chirp_x[x]);
+    float r[C::I1][C::R1];
+    if (u8) {
+      const unsigned char* p = static_cast<const unsigned char*>(a.raw.base) + frame + x;
+#pragma unroll
+      for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+        for (int m = 0; m < C::R1; ++m) r[it][m] = float(p[size_t(t + C::NJ * it + (L / C::R1) * m) * W]);
+    } else {
+      const uint16_t* p = static_cast<const uint16_t*>(a.raw.base) + frame + x;
+#pragma unroll
+      for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+        for (int m = 0; m < C::R1; ++m) r[it][m] = float(p[size_t(t + C::NJ * it + (L / C::R1) * m) * W]);
+    }
+#pragma unroll
+    for (int it = 0; it < C::I1; ++it)
+#pragma unroll
+      for (int m = 0; m < C::R1; ++m)
+        v[it][m] = cscale(cmul(__ldg(&a.chirp_y[t + C::NJ * it + (L / C::R1) * m]), cx), r[it][m]);
+  }
 }
 
 // Row FFTs: LP lanes carry a row (lane jl holds elements jl + LP m in v[m]), RPW rows
