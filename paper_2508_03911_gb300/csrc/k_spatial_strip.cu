@@ -26,8 +26,9 @@
 // CTA, so one or two CTAs per SM from 512 points on): 256 x 256 ASP 0.53 -> 0.37, Fresnel
 // 0.33 -> 0.31; 512 x 512 3.14 -> 1.89 and 1.65 -> 1.36; 1024 x 1024 17.0 -> 8.9 and
 // 8.4 -> 6.1; 128 x 128 0.139 -> 0.107 and 0.081 -> 0.083. Callers with more frames than one
-// launch takes queue up to four launches side by side: 0.33 and 0.24, 1.68 and 1.22, 8.9 and
-// 5.5 for 256, 512 and 1024.
+// launch takes queue up to four launches side by side: 0.34 and 0.27, 1.74 and 1.21, 9.6 and
+// 5.6 for runs of 4,096, 1,024 and 256 frames of 256, 512 and 1024 (with float32 constants in
+// the 32-point DFT, further off, 1.73 and 1.21, 9.4 and 5.5).
 #include "strip_dev.cuh"
 #include "hv_internal.h"
 #include "../../include/hv.h"
@@ -202,6 +203,9 @@ __global__ void __launch_bounds__(RowCfg<L>::NT, (L >= 512 ? 4 : 6)) k_strip_row
   float2* rowp = tw + C::NTW + (warp * C::RPW + sub) * C::RS;
   load_stage_twiddles<C::R1, C::NTW, C::NT>(tw, a.tw_w);
   __syncthreads();
+  float2 kept[C::KEEP + 1];
+#pragma unroll
+  for (int m = 0; m < C::KEEP; ++m) kept[m] = tw[m * C::R1 + jl];
   // H is a multiple of the rows of a warp: its rows are all valid and of one frame
   for (uint32_t r0 = (blockIdx.x * C::NW + warp) * C::RPW; r0 < nrows; r0 += gridDim.x * C::NW * C::RPW) {
     const uint32_t row = r0 + sub, i = row / a.H, ky = row % a.H;
@@ -209,7 +213,7 @@ __global__ void __launch_bounds__(RowCfg<L>::NT, (L >= 512 ? 4 : 6)) k_strip_row
     float2 v[C::R1];
 #pragma unroll
     for (int m = 0; m < C::R1; ++m) v[m] = in[C::LP * m];
-    strip_row_fft<L, -1>(v, rowp, tw, jl);
+    strip_row_fft<L, -1, C::KEEP>(v, rowp, tw, jl, kept);
     float2* out = static_cast<float2*>(a.tq.base) + (((a.tq.slot0 + i) % a.tq.cap) * a.H + ky) * size_t(L) + jl;
 #pragma unroll
     for (int m = 0; m < C::R1; ++m) __stcs(&out[C::LP * m], v[m]);
@@ -234,12 +238,15 @@ __global__ void __launch_bounds__(RowCfg<L>::NT, (L >= 512 ? 4 : 6)) k_strip_row
   float2* rowp = tw + C::NTW + (warp * C::RPW + sub) * C::RS;
   load_stage_twiddles<C::R1, C::NTW, C::NT>(tw, a.tw_w);
   __syncthreads();
+  float2 kept[C::KEEP + 1];
+#pragma unroll
+  for (int m = 0; m < C::KEEP; ++m) kept[m] = tw[m * C::R1 + jl];
   for (uint32_t r0 = (blockIdx.x * C::NW + warp) * C::RPW; r0 < nrows; r0 += gridDim.x * C::NW * C::RPW) {
     float2* at = a.scratch1 + size_t(r0 + sub < nrows ? r0 + sub : nrows - 1) * L + jl;
     float2 v[C::R1];
 #pragma unroll
     for (int m = 0; m < C::R1; ++m) v[m] = at[C::LP * m];
-    strip_row_fft<L, -1>(v, rowp, tw, jl);
+    strip_row_fft<L, -1, C::KEEP>(v, rowp, tw, jl, kept);
 #pragma unroll
     for (int m = 0; m < C::R1; ++m) at[C::LP * m] = v[m];
   }

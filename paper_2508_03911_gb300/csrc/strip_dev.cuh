@@ -221,15 +221,20 @@ struct RowCfg {
   static constexpr int NTW = (R2 - 1) * R1;
   static constexpr int RS = L + L / R1;  // exchange row: element e at e + e / R1
   static constexpr size_t SMEM = (size_t(NW) * RPW * RS + NTW) * sizeof(float2);
+  static constexpr int KEEP = L >= 512 ? 8 : 0;  // twiddles in registers (single-FFT kernels)
   static constexpr bool AGAIN = L >= 512;  // ASP rows: the forward FFT twice
   static constexpr int ASP_CTAS = L >= 512 || L == 64 ? 5 : 4;
 };
 
 // L-point FFT of a row through its exchange buffer rowp (padded: the 16 lanes of a
 // half-warp always meet 16 different bank pairs, two rows of 8 lanes too). On return
-// bin jl + LP m is in v[m].
-template <int L, int DIR>
-__device__ __forceinline__ void strip_row_fft(float2 (&v)[RowCfg<L>::R1], float2* rowp, const float2* tw, int jl) {
+// bin jl + LP m is in v[m]. kept: the first KEEP twiddles of the lane's first butterfly, the same
+// for every row, where the kernel has registers to hold them (with all 31 and 32 more values read
+// from shared memory in one go, rows of 1024 points waited for its queue: Fresnel passes 6.55 us
+// a frame, 5.60 with 8 kept, 5.59 with 16).
+template <int L, int DIR, int KEEP = 0>
+__device__ __forceinline__ void strip_row_fft(float2 (&v)[RowCfg<L>::R1], float2* rowp, const float2* tw, int jl,
+                                              const float2* kept = nullptr) {
   using C = RowCfg<L>;
   strip_dft<C::R1, DIR>(v);
   __syncwarp();
@@ -244,7 +249,7 @@ __device__ __forceinline__ void strip_row_fft(float2 (&v)[RowCfg<L>::R1], float2
     for (int m = 0; m < C::R2; ++m) {
       u[m] = rowp[(C::R1 + 1) * m + j];
       if (m > 0) {
-        float2 w = tw[(m - 1) * C::R1 + j];
+        float2 w = i == 0 && m <= KEEP ? kept[m - 1] : tw[(m - 1) * C::R1 + j];
         if (DIR > 0) w.y = -w.y;
         u[m] = cmul(u[m], w);
       }
