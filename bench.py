@@ -568,6 +568,13 @@ def roofline(w, res, peaks):
     if t_tm < t_sp and w["N"] == 256 and w["spatial"] == "asp":
         kern = "k_spatial_fused (every spatial pass, one launch per render)" if tun.get("spatial_kernel") == 4 \
             else kern
+        if tun.get("spatial_kernel") == 1 and w["bits"] > 8:
+            kern = "k_strip_cols, k_strip_rows_asp, k_strip_icols (spatial passes)"
+            v = profiled_traffic("strip_passes_asp_256.md", ["k_spatial_strip.cu", "strip_dev.cuh", "fft_dev.cuh"])
+            if v is not None:
+                traffic = int(v * frames_per_render / 256)
+                traffic_per = ("render (all spatial pass launches; cold-cache 256-frame ncu capture of each pass "
+                               "alone, scaled to the render's frames)")
         if tun.get("spatial_kernel") == 4 and w["bits"] > 8:
             v = profiled_traffic("spatial_fused_asp_256.md", ["k_spatial_pp.cu", "fft_dev.cuh"])
             if v is not None:

@@ -93,3 +93,15 @@ def test_roofline_names_the_dominant_kernel_and_takes_only_its_own_profile():
     assert r["kernel"].startswith("k_spatial_fused") and r["bound"] == "alu"
     assert r["traffic"] == int(fused * 4096 / 1024)
     assert r["frac"] > 0 and abs(r["frac"] - r["achieved"] / r["peak"]) < 1e-3
+
+
+def test_roofline_takes_the_strip_passes_traffic_where_they_run():
+    b = _bench()
+    b._ALU.update(fp32_tflops=76.5, fp64_tflops=1.25, source="test figures")
+    strips = b.profiled_traffic("strip_passes_asp_256.md", ["k_spatial_strip.cu", "strip_dev.cuh", "fft_dev.cuh"])
+    assert strips  # the committed summary matches the committed sources
+    prof = {"renders": 1, "frames": 4096, "spatial_ms": 1.35, "temporal_ms": 0.39}
+    for sk, want in ((1, strips * 16), (2, None)):
+        r = b.roofline(b.WORKLOADS[b.DEFAULT], {"prof": prof, "frames_per_step": 4096,
+                                                "tuning": {"stft_kernel": 5, "spatial_kernel": sk}}, {"hbm_gbs": 6784.8})
+        assert r["traffic"] == want and r["kernel"].startswith("k_strip_cols" if want else "spatial passes")
