@@ -278,6 +278,8 @@ hv_status validate(const hv_handle* h, const hv_params& p, Derived& d, std::stri
   return HV_OK;
 }
 
+hv_status ensure(hv_handle* h, void** p, size_t* have, size_t need);
+
 // exp(i a) in float64, rounded to float
 float2 cis(double a) { return make_float2(float(std::cos(a)), float(std::sin(a))); }
 
@@ -286,11 +288,8 @@ hv_status build_tables(hv_handle* h, const hv_params& p) {
   const uint32_t W = p.width, H = p.height;
   // [Hᵀ: W H][chirp x: W][chirp y: H][H row-major: W H]
   const size_t need = (2 * size_t(W) * H + W + H) * sizeof(float2);
-  if (need > h->table_bytes) {
-    dfree(h->asp_ht);
-    HV_CU(h, cudaMalloc(&h->asp_ht, need));
-    h->table_bytes = need;
-  }
+  hv_status s = ensure(h, reinterpret_cast<void**>(&h->asp_ht), &h->table_bytes, need);
+  if (s != HV_OK) return s;
   h->chirp = h->asp_ht + size_t(W) * H;
   std::vector<float2> host(2 * size_t(W) * H + W + H, make_float2(0.f, 0.f));
   const size_t rowmajor = size_t(W) * H + W + H;

@@ -154,3 +154,26 @@ for kw in (dict(spatial_kernel="persistent"), dict(spatial_kernel="cluster"), di
     got.append([t["spatial_kernel"], t["stft_kernel"]])
 print(json.dumps(got))
 """) == [[1, 2], [2, 2], [1, 2], [1, 2], [1, 2], [1, 1], [1, 1], [1, 2]]
+
+
+def test_tables_after_an_allocation_that_failed():
+    """Larger frames whose tables do not fit, then smaller ones: the tables are allocated again."""
+    status, null = run("""
+MB = 1 << 20
+r = hv.Renderer(1024, 1024, 8, 16)
+def use(side):
+    r.set_params(side, side, spatial="asp", T=8, stride=8, fs=20000.0, band=(1, 2))
+    assert r.push(Dev((8, side, side), 1)) == hv.HV_OK
+    return r.render(Dev((1, 1, side, side), 4))
+assert use(512) == 1
+fake.fake_fail_malloc(16 * MB, 17 * MB, 1)  # two tables of 1024 x 1024 values and the chirps
+try:
+    use(1024)
+    status = 0
+except hv.HvError as e:
+    status = e.status
+log()
+assert use(256) == 1
+print(json.dumps([status, sum(1 for l in log() if l[0] == "copy" and l[2] < 4096)]))
+""")
+    assert status == -4 and null == 0
