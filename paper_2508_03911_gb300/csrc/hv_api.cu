@@ -1677,6 +1677,7 @@ hv_status hv_focus_sweep(hv_handle* h, const void* frames, uint32_t n, const dou
   std::vector<double> key = {double(W), double(H), p.lambda_m, p.pitch_x_m, p.pitch_y_m};
   key.insert(key.end(), z, z + nz);
   if (key != h->sw_key) {
+    h->sw_key.clear();  // the tables of the sweep before go
     s = ensure(h, reinterpret_cast<void**>(&h->sw_tables), &h->sw_bytes, per * nz * sizeof(float2));
     if (s != HV_OK) return s;
     std::vector<float2> host(per * nz);

@@ -177,3 +177,29 @@ assert use(256) == 1
 print(json.dumps([status, sum(1 for l in log() if l[0] == "copy" and l[2] < 4096)]))
 """)
     assert status == -4 and null == 0
+
+
+def test_a_sweep_after_one_without_memory_for_its_tables():
+    """The transfer functions of the sweep before the failed one are gone: formed again."""
+    status, copied = run("""
+import numpy as np
+N = 256
+r = hv.Renderer(N, N, 16, 4)
+r.set_params(N, N, spatial="asp", T=8, stride=8, fs=20000.0, band=(1, 2))
+fr, out = Dev((4, N, N), 2), Dev((4, 512), 4)
+table = N * (N // 2 + 1) * 8
+def sweep(nz):
+    log()
+    hv.hv_focus_sweep(r.h, fr, np.linspace(0.1, 0.6, nz), out)
+    return sum(l[4] for l in log() if l[0] == "copy")
+sweep(8)
+assert sweep(8) == 0
+fake.fake_fail_malloc(512 * table, 512 * table, 1)
+try:
+    sweep(512)
+    status = 0
+except hv.HvError as e:
+    status = e.status
+print(json.dumps([status, sweep(8) // table]))
+""")
+    assert status == -4 and copied == 8
