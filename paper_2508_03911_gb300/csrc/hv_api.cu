@@ -586,6 +586,9 @@ hv_status apply_pending(hv_handle* h) {
   h->nout = d.nout;
   h->win_floats = d.win_floats;
   h->Q = Q;
+  // queue flush: the next window starts at the first unconsumed frame and is propagated
+  // entirely with the new settings (also where their tuning fails below)
+  h->propagated = h->next_win;
   h->chunk = chunk;
   h->sp_cluster = p.spatial_kernel == HV_SK_CLUSTER ? 1 : 0;
   h->sp_fused = fused ? 1 : 0;
@@ -615,9 +618,6 @@ hv_status apply_pending(hv_handle* h) {
     s = tune_temporal(h);
     if (s != HV_OK) return s;
   }
-  // queue flush: the next window starts at the first unconsumed frame and is
-  // propagated entirely with the new settings
-  h->propagated = h->next_win;
   return HV_OK;
 }
 

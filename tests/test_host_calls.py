@@ -203,3 +203,28 @@ except hv.HvError as e:
 print(json.dumps([status, sweep(8) // table]))
 """)
     assert status == -4 and copied == 8
+
+
+def test_settings_whose_tuning_failed_flush_the_queue():
+    """A window half of whose frames were propagated with the settings before: all of them are
+    again, also where the autotuner found no memory and the call before said so."""
+    status, frames = run("""
+MB, N = 1 << 20, 512
+r = hv.Renderer(N, N, 16, 64)
+kw = dict(spatial="asp", T=32, stride=16, fs=20000.0, band=(1, 2))
+out = Dev((1, 1, N, N), 4)
+r.set_params(N, N, **kw)
+assert r.push(Dev((64, N, N), 2)) == hv.HV_OK and r.render(out) == 1
+r.set_params(N, N, z=0.2, tuned=1, **kw)
+fake.fake_fail_malloc(30 * MB, 1 << 40, 1000)
+try:
+    r.render(out)
+    status = 0
+except hv.HvError as e:
+    status = e.status
+fake.fake_fail_malloc(0, 0, 0)
+before = r.stats()["frames_propagated"]
+assert r.render(out) == 1
+print(json.dumps([status, r.stats()["frames_propagated"] - before]))
+""")
+    assert status == -4 and frames == 32
