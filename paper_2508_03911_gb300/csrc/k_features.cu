@@ -8,12 +8,12 @@
 //            and bin it in a kernel of its own.
 //
 // Persistent CTAs that stage their next strip by cp.async while they transform one, over all
-// H rows and with the transforms of a real column one at a time. The bfloat16 result turns a
-// float32 error into a whole unit where a value lies near the middle of two neighbours, and
-// that carries into the network: with two columns to a complex line, rows 0 .. H / 2 only and
-// the mirrored cells from the same |F| (k_strip_cells, 108 us against 208 for 512 holograms of
-// 256 x 256), 6,330 of 8.4 million inputs differed from the float64 result's bfloat16 instead of
-// 4,650, and the network's answer was 7.7e-5 off instead of 6.1e-5.
+// H rows and with the transforms of a real column one at a time: 512 holograms of 256 x 256 in
+// 68 + 145 us, bound by issue and the stages' barriers. Half of the spectrum, from two real
+// columns to a complex line, with the mirrored cells from the same |F|, took 37 + 71, but a
+// bfloat16 result turns a float32 error into a whole unit where a value lies near the middle of
+// two, and that carries into the network: 6,330 of 8.4 million inputs differed from the float64
+// result's bfloat16 instead of 4,650, and the network's answer was 7.7e-5 off instead of 6.1e-5.
 #include <cuda_bf16.h>
 
 #include "pp_dev.cuh"

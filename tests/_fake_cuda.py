@@ -16,8 +16,6 @@ import ctypes as C, json, sys
 sys.path.insert(0, %(root)r)
 fake = C.CDLL(%(fake)r, mode=C.RTLD_GLOBAL)
 fake.fake_log.restype = C.c_char_p
-fake.fake_room.restype = C.c_size_t
-fake.fake_room.argtypes = [C.c_size_t]
 fake.fake_fail_malloc.argtypes = [C.c_size_t, C.c_size_t, C.c_int]
 fake.fake_fail_launch.argtypes = [C.c_char_p, C.c_int]
 from paper_2508_03911_gb300 import hv

@@ -76,7 +76,6 @@ const char* fake_log() {
 void fake_fail_malloc(size_t from, size_t to, int times) { g_fail_from = from, g_fail_to = to, g_fail_malloc = times; }
 // The next `times` launches of a kernel whose name holds `part` fail.
 void fake_fail_launch(const char* part, int times) { g_fail_kernel = part, g_fail_launch = times; }
-size_t fake_room(size_t p) { return room(reinterpret_cast<void*>(p)); }
 
 cudaError_t cudaMalloc(void** p, size_t n) {
   *p = nullptr;
